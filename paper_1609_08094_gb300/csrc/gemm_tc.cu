@@ -108,110 +108,113 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_kernel(const __grid_co
     constexpr uint32_t idesc_m = (1u << 4) | ((uint32_t)(BM >> 4) << 24);
 
     if (warp == 0) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int last_phase[MAX_STAGES];
-            for (int s = 0; s < MAX_STAGES; s++) last_phase[s] = -1;
-            bool ok = true;
-            bool inject = wv.inject_stall != 0 && blockIdx.x == 0;
-            SegCache sc;
-            seg_reset(sc);
-            for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
-                const Item w = decode(wv, it, sc);
-                if (w.diag) continue;
-                const InstDesc &d = *sc.d;
-                const int o = d.dm.o, kv = d.kv, ko = d.ko, nch = num_chunks(d);
-                const int kch = ROW_BYTES / (d.kind == 1 ? 4 : 2);
-                const int s = w.s, pp = w.p, q = w.q;
-                const int cb = w.bt * d.pb, cc = w.ct * d.pc, ca = w.n * d.brows;
-                const uint32_t stage_tx = d.stage_tx;
-                for (int ch = 0; ch < nch; ch++) {
-                    if (!mbar_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
-                        fail(&abort_sh, wv.err, DERR_TIMEOUT_EMPTY);
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t full = smem_u32(&bar_full[stage]);
-                    mbar_expect_tx(full, stage_tx);
-                    last_phase[stage] = (int)phase;
-                    const uint32_t sA = sbase + stage * stage_bytes, sAl = sA + A_BYTES;
-                    const uint32_t sB = sAl + A_BYTES, sBl = sB + b_plane;
-                    int seg, kk;
-                    if (ch < kv) { seg = 0; kk = ch; }
-                    else if (ch < 2 * kv) { seg = 1; kk = ch - kv; }
-                    else if (ch < 2 * kv + ko) { seg = 2; kk = ch - 2 * kv; }
-                    else { seg = 3; kk = ch - 2 * kv - ko; }
-                    const int k0 = kk * kch;
-                    int amap, aslice, bmap, brow;
-                    switch (seg) {
-                        case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; brow = s * o + pp; break;
-                        case 1: amap = MAP_G_SWP; aslice = pp; bmap = MAP_T2R; brow = s * o + q; break;
-                        case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; brow = q * o + s; break;
-                        default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; brow = pp * o + s; break;
-                    }
-                    if (inject) {
-                        inject = false;
-                        last_phase[stage] = -1;  // nothing in flight: the consumer's wait must expire
-                    } else {
-                        tma_load_4d(sA, &d.maps[amap][0], full, k0, cc, cb, aslice);
-                        tma_load_4d(sAl, &d.maps[amap][1], full, k0, cc, cb, aslice);
-                        tma_load_3d(sB, &d.maps[bmap][0], full, k0, ca, brow);
-                        tma_load_3d(sBl, &d.maps[bmap][1], full, k0, ca, brow);
-                    }
-                    if (++stage == nst) { stage = 0; phase ^= 1u; }
+        int stage = 0;
+        uint32_t phase = 0;
+        int last_phase[MAX_STAGES];
+        for (int s = 0; s < MAX_STAGES; s++) last_phase[s] = -1;
+        bool ok = true;
+        bool inject = wv.inject_stall != 0 && blockIdx.x == 0;
+        SegCache sc;
+        seg_reset(sc);
+        for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
+            const Item w = decode(wv, it, sc);
+            if (uni((int)w.diag)) continue;
+            const InstDesc *d = uni(sc.d);
+            const int o = uni(d->dm.o), kv = uni(d->kv), ko = uni(d->ko), nch = 2 * kv + 2 * ko;
+            const int kch = uni(ROW_BYTES / (d->kind == 1 ? 4 : 2));
+            const int s = uni(w.s), pp = uni(w.p), q = uni(w.q);
+            const int cb = uni(w.bt * d->pb), cc = uni(w.ct * d->pc), ca = uni(w.n * d->brows);
+            const uint32_t stage_tx = uni(d->stage_tx);
+            for (int ch = 0; ch < nch; ch++) {
+                if (!wait_warp(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
+                    if (lane == 0) fail(&abort_sh, wv.err, DERR_TIMEOUT_EMPTY);
+                    ok = false;
+                    break;
                 }
-            }
-            if (!ok) {  // let this CTA's copies in flight land before exiting
-                for (int s = 0; s < nst; s++) {
-                    if (last_phase[s] < 0) continue;
-                    const uint64_t t0 = gtimer();
-                    while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
-                           gtimer() - t0 < WAIT_LIMIT_NS) {
+                const uint32_t full = smem_u32(&bar_full[stage]);
+                last_phase[stage] = (int)phase;
+                const uint32_t sA = sbase + stage * stage_bytes, sAl = sA + A_BYTES;
+                const uint32_t sB = sAl + A_BYTES, sBl = sB + b_plane;
+                int seg, kk;
+                if (ch < kv) { seg = 0; kk = ch; }
+                else if (ch < 2 * kv) { seg = 1; kk = ch - kv; }
+                else if (ch < 2 * kv + ko) { seg = 2; kk = ch - 2 * kv; }
+                else { seg = 3; kk = ch - 2 * kv - ko; }
+                const int k0 = kk * kch;
+                int amap, aslice, bmap, brow;
+                switch (seg) {
+                    case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; brow = s * o + pp; break;
+                    case 1: amap = MAP_G_SWP; aslice = pp; bmap = MAP_T2R; brow = s * o + q; break;
+                    case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; brow = q * o + s; break;
+                    default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; brow = pp * o + s; break;
+                }
+                if (elect_one()) {
+                    mbar_expect_tx(full, stage_tx);
+                    if (!inject) {
+                        tma_load_4d(sA, &d->maps[amap][0], full, k0, cc, cb, aslice);
+                        tma_load_4d(sAl, &d->maps[amap][1], full, k0, cc, cb, aslice);
+                        tma_load_3d(sB, &d->maps[bmap][0], full, k0, ca, brow);
+                        tma_load_3d(sBl, &d->maps[bmap][1], full, k0, ca, brow);
                     }
+                }
+                __syncwarp();
+                if (inject) {
+                    inject = false;
+                    last_phase[stage] = -1;  // nothing in flight: the consumer's wait must expire
+                }
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
+            }
+        }
+        if (!ok && lane == 0) {  // let this CTA's copies in flight land before exiting
+            for (int s = 0; s < nst; s++) {
+                if (last_phase[s] < 0) continue;
+                const uint64_t t0 = gtimer();
+                while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
+                       gtimer() - t0 < WAIT_LIMIT_NS) {
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            MmaRing rg;
-            rg.full0 = smem_u32(&bar_full[0]);
-            rg.empty0 = smem_u32(&bar_empty[0]);
-            rg.hfull0 = smem_u32(&bar_hfull[0]);
-            rg.hempty0 = smem_u32(&bar_hempty[0]);
-            rg.lo0 = desc_lo(sbase);
-            rg.step = stage_bytes >> 4;
-            rg.a16 = A_BYTES >> 4;
-            rg.b16 = b_plane >> 4;
-            rg.nst = nst;
-            rg.stage = 0;
-            rg.phase = 0;
-            rg.hblk = 0;
-            SegCache sc;
-            seg_reset(sc);
-            for (int64_t it = blockIdx.x; it < wv.n_gemm; it += gridDim.x) {
-                const Item w = decode(wv, it, sc);
-                if (w.diag) continue;
-                const InstDesc &d = *sc.d;
-                const int kv = d.kv, ko = d.ko, nch = 2 * kv + 2 * ko, kind = d.kind;
-                const bool dh = kind == 2 && (d.dm.dp & 31) != 0, lh = kind == 2 && (d.dm.lp & 31) != 0;
-                const int nvalid = min(d.brows, d.dm.v - w.n * d.brows);
-                const int N = (nvalid + 15) / 16 * 16;
-                const uint32_t fmt = kind == 1 ? 2u : 1u;
-                const uint32_t idesc = idesc_m | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17);
-                // the small hi*lo and lo*hi products of each chunk are issued as it
-                // lands, the dominant hi*hi products of the K block last, so that the
-                // truncation of every instruction acts on the smallest possible
-                // accumulator; each stage is released right after its last product
-                int code = 0;
-                const bool good = kind == 1
-                    ? mma_item<1, 1>(rg, tmem, idesc, nch, -1, -1, -1, -1, &abort_sh, &code)
-                    : mma_item<2, 1>(rg, tmem, idesc, nch, dh ? kv - 1 : -1, dh ? 2 * kv - 1 : -1,
-                                     lh ? 2 * kv + ko - 1 : -1, lh ? nch - 1 : -1, &abort_sh, &code);
-                if (!good) {
-                    fail(&abort_sh, wv.err, code);
-                    break;
-                }
+        MmaRing rg;
+        rg.full0 = smem_u32(&bar_full[0]);
+        rg.empty0 = smem_u32(&bar_empty[0]);
+        rg.hfull0 = smem_u32(&bar_hfull[0]);
+        rg.hempty0 = smem_u32(&bar_hempty[0]);
+        rg.lo0 = desc_lo(sbase);
+        rg.step = stage_bytes >> 4;
+        rg.a16 = A_BYTES >> 4;
+        rg.b16 = b_plane >> 4;
+        rg.nst = nst;
+        rg.stage = 0;
+        rg.phase = 0;
+        rg.hblk = 0;
+        const uint32_t tm = uni(tmem);
+        SegCache sc;
+        seg_reset(sc);
+        for (int64_t it = blockIdx.x; it < wv.n_gemm; it += gridDim.x) {
+            const Item w = decode(wv, it, sc);
+            if (uni((int)w.diag)) continue;
+            const InstDesc *d = uni(sc.d);
+            const int kv = uni(d->kv), ko = uni(d->ko), nch = 2 * kv + 2 * ko, kind = uni(d->kind);
+            const int v = uni(d->dm.v), o = uni(d->dm.o), kch = ROW_BYTES / (kind == 1 ? 4 : 2);
+            // the last chunk of a segment holds one K step of data (half a chunk) or two
+            const bool dh = v - (kv - 1) * kch <= kch / 2, lh = o - (ko - 1) * kch <= kch / 2;
+            const int nvalid = uni(min(d->brows, v - w.n * d->brows));
+            const int N = (nvalid + 15) / 16 * 16;
+            const uint32_t fmt = kind == 1 ? 2u : 1u;
+            const uint32_t idesc = idesc_m | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17);
+            const int dt0 = dh ? kv - 1 : -1, dt1 = dh ? 2 * kv - 1 : -1;
+            const int lt0 = lh ? 2 * kv + ko - 1 : -1, lt1 = lh ? nch - 1 : -1;
+            // the small hi*lo and lo*hi products of each chunk are issued as it
+            // lands, the dominant hi*hi products of the K block last, so that the
+            // truncation of every instruction acts on the smallest possible
+            // accumulator; each stage is released right after its last product
+            int code = 0;
+            const bool good = kind == 1 ? mma_item<1, 1>(rg, tm, idesc, nch, dt0, dt1, lt0, lt1, &abort_sh, &code)
+                                        : mma_item<2, 1>(rg, tm, idesc, nch, dt0, dt1, lt0, lt1, &abort_sh, &code);
+            if (!good) {
+                if (lane == 0) fail(&abort_sh, wv.err, code);
+                break;
             }
         }
     } else {
@@ -301,12 +304,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_kernel(const __grid_co
 //
 // Two CTAs of a thread-block cluster (one per SM of an SM pair) compute one
 // M = 256 tile: each loads its own 128-pair A tile and half of the B tile
-// (N/2 rows of a), and one thread of the even CTA ("leader") issues
+// (N/2 rows of a), and one lane of the even CTA ("leader") issues
 // tcgen05.mma.cta_group::2, which reads A and B from both CTAs' shared memory
 // and accumulates each CTA's 128 rows in that CTA's tensor memory.  Per K
 // chunk an SM then ingests 16 KB of A and N/2 x 128 bytes of B (32 KB at
 // N = 256) instead of 48 KB, for the same tensor work per SM: the per-SM
 // operand-ingest rate, not the tensor pipe, bounds the single-SM kernel.
+//
+// A ring stage holds one K block: two chunks side by side in 128-byte rows
+// (128-byte swizzle), so a block is four copies and one wait instead of eight
+// and two.  A probe of the copy engine alone moved 28 bytes/clk per SM with
+// 8 KB copies of 64-byte rows and 56 with 16 KB copies of 128-byte rows: the
+// copies cost a fixed time each.
 //
 // The pair's two 128-pair tiles are consecutive tiles of the flattened
 // (b tile, c tile) list of a group: work item = (task, tile pair, group,
@@ -326,6 +335,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_kernel(const __grid_co
 // Teardown: a cluster barrier (every role of both CTAs ends after bounded
 // waits), then both CTAs free the pair's tensor memory.
 constexpr int PAIR_HEMPTY_ARRIVALS = 2 * (EPI_THREADS / 32);
+constexpr int PAIR_ROW = 2 * ROW_BYTES;   // one K block (two chunks) per shared-memory row, 128-byte swizzle
+constexpr int PAIR_A = BM * PAIR_ROW;     // 16 KB per A plane
 
 struct PairItem {
     Item it;
@@ -385,9 +396,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
     const uint32_t rank = cluster_rank(), cid = cluster_id(), ncl = cluster_count();
     const bool leader = rank == 0;
     const uint32_t sbase = (smem_u32(smem_dyn) + 1023u) & ~1023u;
-    const uint32_t b_half = (uint32_t)wv.tc_brows / 2;                       // B rows per CTA
-    const uint32_t b_plane = (b_half * ROW_BYTES + 1023u) & ~1023u;
-    const uint32_t stage_bytes = 2u * A_BYTES + 2u * b_plane;
+    const uint32_t b_plane = (uint32_t)wv.tc_brows / 2 * PAIR_ROW;  // B rows per CTA: a multiple of 16
+    const uint32_t stage_bytes = 2u * PAIR_A + 2u * b_plane;
     const int nst = min(MAX_STAGES, (int)(RING_BYTES / stage_bytes));
     const uint32_t peer_abort = peer_addr(smem_u32((const void *)&abort_sh), rank ^ 1u);
 
@@ -420,81 +430,86 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
     constexpr uint32_t idesc_m = (1u << 4) | ((uint32_t)(2 * BM >> 4) << 24);
 
     if (warp == 0) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int last_phase[MAX_STAGES];
-            for (int s = 0; s < MAX_STAGES; s++) last_phase[s] = -1;
-            bool ok = true;
-            bool inject = wv.inject_stall != 0 && cid == 0 && leader;
-            SegCache sc;
-            seg_reset(sc);
-            for (int64_t it = cid; it < wv.n_gemm && ok; it += ncl) {
-                const PairItem pw = decode_pair(wv, it, sc, rank);
-                const Item &w = pw.it;
-                if (w.diag) continue;
-                const InstDesc &d = *sc.d;
-                const int o = d.dm.o, kv = d.kv, ko = d.ko, nch = num_chunks(d);
-                const int kch = ROW_BYTES / (d.kind == 1 ? 4 : 2);
-                const int s = w.s, pp = w.p, q = w.q;
-                const int nvalid = min(d.brows, d.dm.v - w.n * d.brows);
-                const int N = (nvalid + 15) / 16 * 16;
-                const int cb = w.bt * d.pb, cc = w.ct * d.pc, ca = w.n * d.brows + (int)rank * (N / 2);
-                const uint32_t stage_tx = d.stage_tx;  // both CTAs' bytes
-                for (int ch = 0; ch < nch; ch++) {
-                    if (!mbar_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
-                        fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_EMPTY);
+        int stage = 0;
+        uint32_t phase = 0;
+        int last_phase[MAX_STAGES];
+        for (int s = 0; s < MAX_STAGES; s++) last_phase[s] = -1;
+        bool ok = true;
+        bool inject = wv.inject_stall != 0 && cid == 0 && leader;
+        SegCache sc;
+        seg_reset(sc);
+        for (int64_t it = cid; it < wv.n_gemm && ok; it += ncl) {
+            const PairItem pw = decode_pair(wv, it, sc, rank);
+            const Item &w = pw.it;
+            if (uni((int)w.diag)) continue;
+            const InstDesc *d = uni(sc.d);
+            const int o = uni(d->dm.o), kv = uni(d->kv), ko = uni(d->ko);
+            const int kch = uni(ROW_BYTES / (d->kind == 1 ? 4 : 2));
+            const int s = uni(w.s), pp = uni(w.p), q = uni(w.q);
+            const int nvalid = min(d->brows, d->dm.v - w.n * d->brows);
+            const int N = (nvalid + 15) / 16 * 16;
+            const int cb = uni(w.bt * d->pb), cc = uni(w.ct * d->pc), ca = uni(w.n * d->brows + (int)rank * (N / 2));
+            const uint32_t stage_tx = uni(d->stage_tx);  // both CTAs' bytes
+            for (int seg = 0; seg < 4 && ok; seg++) {
+                const int klen = seg < 2 ? kv : ko;
+                int amap, aslice, bmap, brow;
+                switch (seg) {
+                    case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; brow = s * o + pp; break;
+                    case 1: amap = MAP_G_SWP; aslice = pp; bmap = MAP_T2R; brow = s * o + q; break;
+                    case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; brow = q * o + s; break;
+                    default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; brow = pp * o + s; break;
+                }
+                // two chunks per stage; the second segment of a kind with an odd chunk
+                // count gives its first chunk to the block that the first one left
+                // half full (a stage of its own: the half that is not used is the next
+                // chunk or zero fill), and goes on with whole blocks from chunk 1
+                const bool shift = (seg & 1) && (klen & 1);
+                for (int kk = 0; kk < klen; kk += (shift && kk == 0) ? 1 : 2) {
+                    if (!wait_warp(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
+                        if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_EMPTY);
                         ok = false;
                         break;
                     }
                     const uint32_t full = smem_u32(&bar_full[stage]);
-                    if (leader) mbar_expect_tx(full, stage_tx);
                     const uint32_t full_l = peer_addr(full, 0);
                     last_phase[stage] = (int)phase;
-                    const uint32_t sA = sbase + stage * stage_bytes, sAl = sA + A_BYTES;
-                    const uint32_t sB = sAl + A_BYTES, sBl = sB + b_plane;
-                    int seg, kk;
-                    if (ch < kv) { seg = 0; kk = ch; }
-                    else if (ch < 2 * kv) { seg = 1; kk = ch - kv; }
-                    else if (ch < 2 * kv + ko) { seg = 2; kk = ch - 2 * kv; }
-                    else { seg = 3; kk = ch - 2 * kv - ko; }
+                    const uint32_t sA = sbase + stage * stage_bytes, sAl = sA + PAIR_A;
+                    const uint32_t sB = sAl + PAIR_A, sBl = sB + b_plane;
                     const int k0 = kk * kch;
-                    int amap, aslice, bmap, brow;
-                    switch (seg) {
-                        case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; brow = s * o + pp; break;
-                        case 1: amap = MAP_G_SWP; aslice = pp; bmap = MAP_T2R; brow = s * o + q; break;
-                        case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; brow = q * o + s; break;
-                        default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; brow = pp * o + s; break;
+                    if (elect_one()) {
+                        if (leader) mbar_expect_tx(full, stage_tx);
+                        if (!inject) {
+                            tma_load_4d_pair(sA, &d->maps[amap][0], full_l, k0, cc, cb, aslice);
+                            tma_load_4d_pair(sAl, &d->maps[amap][1], full_l, k0, cc, cb, aslice);
+                            tma_load_3d_pair(sB, &d->maps[bmap][0], full_l, k0, ca, brow);
+                            tma_load_3d_pair(sBl, &d->maps[bmap][1], full_l, k0, ca, brow);
+                        }
                     }
+                    __syncwarp();
                     if (inject) {
                         inject = false;
                         last_phase[stage] = -1;  // the leader's bytes never come: the MMA's wait must expire
-                    } else {
-                        tma_load_4d_pair(sA, &d.maps[amap][0], full_l, k0, cc, cb, aslice);
-                        tma_load_4d_pair(sAl, &d.maps[amap][1], full_l, k0, cc, cb, aslice);
-                        tma_load_3d_pair(sB, &d.maps[bmap][0], full_l, k0, ca, brow);
-                        tma_load_3d_pair(sBl, &d.maps[bmap][1], full_l, k0, ca, brow);
                     }
                     if (++stage == nst) { stage = 0; phase ^= 1u; }
                 }
             }
-            if (!ok) {
-                // let the copies in flight land: the leader sees both CTAs' bytes on
-                // its own full barriers; the peer gives its own copies a fixed time
-                if (leader) {
-                    for (int s = 0; s < nst; s++) {
-                        if (last_phase[s] < 0) continue;
-                        const uint64_t t0 = gtimer();
-                        while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
-                               gtimer() - t0 < WAIT_LIMIT_NS) {
-                        }
+        }
+        if (!ok && lane == 0) {
+            // let the copies in flight land: the leader sees both CTAs' bytes on
+            // its own full barriers; the peer gives its own copies a fixed time
+            if (leader) {
+                for (int s = 0; s < nst; s++) {
+                    if (last_phase[s] < 0) continue;
+                    const uint64_t t0 = gtimer();
+                    while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
+                           gtimer() - t0 < WAIT_LIMIT_NS) {
                     }
                 }
-                spin_ns(1000000ull);
             }
+            spin_ns(1000000ull);
         }
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader) {
             MmaRing rg;
             rg.full0 = smem_u32(&bar_full[0]);
             rg.empty0 = smem_u32(&bar_empty[0]);
@@ -502,40 +517,45 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
             rg.hempty0 = smem_u32(&bar_hempty[0]);
             rg.lo0 = desc_lo(sbase);
             rg.step = stage_bytes >> 4;
-            rg.a16 = A_BYTES >> 4;
+            rg.a16 = PAIR_A >> 4;
             rg.b16 = b_plane >> 4;
             rg.nst = nst;
             rg.stage = 0;
             rg.phase = 0;
             rg.hblk = 0;
+            const uint32_t tm = uni(tmem);
             SegCache sc;
             seg_reset(sc);
             for (int64_t it = cid; it < wv.n_gemm; it += ncl) {
                 const PairItem pw = decode_pair(wv, it, sc, rank);
                 const Item &w = pw.it;
-                if (w.diag) continue;
-                const InstDesc &d = *sc.d;
-                const int kv = d.kv, ko = d.ko, nch = 2 * kv + 2 * ko, kind = d.kind;
-                const bool dh = kind == 2 && (d.dm.dp & 31) != 0, lh = kind == 2 && (d.dm.lp & 31) != 0;
-                const int nvalid = min(d.brows, d.dm.v - w.n * d.brows);
+                if (uni((int)w.diag)) continue;
+                const InstDesc *d = uni(sc.d);
+                const int kv = uni(d->kv), ko = uni(d->ko), kind = uni(d->kind);
+                const int v = uni(d->dm.v), o = uni(d->dm.o), kch = ROW_BYTES / (kind == 1 ? 4 : 2);
+                // the last chunk of a segment holds one K step of data (half a chunk) or two
+                const bool dh = v - (kv - 1) * kch <= kch / 2, lh = o - (ko - 1) * kch <= kch / 2;
+                const int nvalid = uni(min(d->brows, v - w.n * d->brows));
                 const int N = (nvalid + 15) / 16 * 16;
                 const uint32_t fmt = kind == 1 ? 2u : 1u;
                 const uint32_t idesc = idesc_m | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17);
                 int code = 0;
                 const bool good = kind == 1
-                    ? mma_item<1, 2>(rg, tmem, idesc, nch, -1, -1, -1, -1, &abort_sh, &code)
-                    : mma_item<2, 2>(rg, tmem, idesc, nch, dh ? kv - 1 : -1, dh ? 2 * kv - 1 : -1,
-                                     lh ? 2 * kv + ko - 1 : -1, lh ? nch - 1 : -1, &abort_sh, &code);
+                    ? mma_item_wide<1>(rg, tm, idesc, kv, ko, dh, lh, &abort_sh, &code)
+                    : mma_item_wide<2>(rg, tm, idesc, kv, ko, dh, lh, &abort_sh, &code);
                 if (!good) {
-                    fail_pair(&abort_sh, peer_abort, wv.err, code);
+                    if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, code);
                     break;
                 }
             }
-            // every MMA issued by this thread has completed before the pair tears down
-            tc_commit_pair(smem_u32(&bar_fin), (uint16_t)1);
-            const uint64_t t0 = gtimer();
-            while (!mbar_test(smem_u32(&bar_fin), 0u) && gtimer() - t0 < WAIT_LIMIT_NS) {
+            // every MMA issued by this warp's elected lane has completed before the pair tears down
+            if (elect_one()) {
+                tc_commit_pair(smem_u32(&bar_fin), (uint16_t)1);
+                const uint64_t t0 = gtimer();
+                while (!mbar_test(smem_u32(&bar_fin), 0u) && gtimer() - t0 < WAIT_LIMIT_NS) {
+                }
             }
+            __syncwarp();
         }
     } else {
         const int wq = warp & 3;
@@ -655,10 +675,12 @@ cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int 
     d.kv = (v + kch - 1) / kch;
     d.ko = (o + kch - 1) / kch;
     // bytes per stage: one CTA's (single SM), or both CTAs' (the pair's leader expects them all)
-    d.stage_tx = pair ? (uint32_t)(2 * (2 * A_BYTES + 2 * (d.brows / 2) * ROW_BYTES))
+    d.stage_tx = pair ? (uint32_t)(2 * (2 * PAIR_A + 2 * (d.brows / 2) * PAIR_ROW))
                       : (uint32_t)(2 * A_BYTES + 2 * d.brows * ROW_BYTES);
     const uint64_t V = v, O = o;
-    const uint32_t bk = (uint32_t)kch, bpc = (uint32_t)pc, bpb = (uint32_t)pb;
+    // rows of a box: one K chunk (64 bytes), or on SM pairs a K block of two
+    const CUtensorMapSwizzle swz = pair ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    const uint32_t bk = (uint32_t)(pair ? 2 * kch : kch), bpc = (uint32_t)pc, bpb = (uint32_t)pb;
     const uint32_t brows = (uint32_t)(pair ? d.brows / 2 : d.brows);  // B box rows per CTA
     void *hi[4] = {op.G, op.T2K, op.T2R, op.AoN};
     void *lo[4] = {op.Glo, op.T2Klo, op.T2Rlo, op.AoNlo};
@@ -668,39 +690,39 @@ cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int 
             uint64_t dims[4] = {V, V, V, O};
             uint64_t st[3] = {dp * eb, V * dp * eb, V * V * dp * eb};
             uint32_t box[4] = {bk, bpc, bpb, 1};
-            if (!encode(&d.maps[MAP_G_NAT][part], dt, 4, src[0], dims, st, box, err, "G")) return cudaErrorInvalidValue;
+            if (!encode(&d.maps[MAP_G_NAT][part], dt, 4, src[0], dims, st, box, err, "G", swz)) return cudaErrorInvalidValue;
         }
         {   // G swapped: (d, c, b, q) with c = x index, b = y index
             uint64_t dims[4] = {V, V, V, O};
             uint64_t st[3] = {V * dp * eb, dp * eb, V * V * dp * eb};
             uint32_t box[4] = {bk, bpc, bpb, 1};
-            if (!encode(&d.maps[MAP_G_SWP][part], dt, 4, src[0], dims, st, box, err, "G swapped"))
+            if (!encode(&d.maps[MAP_G_SWP][part], dt, 4, src[0], dims, st, box, err, "G swapped", swz))
                 return cudaErrorInvalidValue;
         }
         {   // T2K natural
             uint64_t dims[4] = {O, V, V, O};
             uint64_t st[3] = {lp * eb, V * lp * eb, V * V * lp * eb};
             uint32_t box[4] = {bk, bpc, bpb, 1};
-            if (!encode(&d.maps[MAP_T2K_NAT][part], dt, 4, src[1], dims, st, box, err, "T2K")) return cudaErrorInvalidValue;
+            if (!encode(&d.maps[MAP_T2K_NAT][part], dt, 4, src[1], dims, st, box, err, "T2K", swz)) return cudaErrorInvalidValue;
         }
         {   // T2K swapped
             uint64_t dims[4] = {O, V, V, O};
             uint64_t st[3] = {V * lp * eb, lp * eb, V * V * lp * eb};
             uint32_t box[4] = {bk, bpc, bpb, 1};
-            if (!encode(&d.maps[MAP_T2K_SWP][part], dt, 4, src[1], dims, st, box, err, "T2K swapped"))
+            if (!encode(&d.maps[MAP_T2K_SWP][part], dt, 4, src[1], dims, st, box, err, "T2K swapped", swz))
                 return cudaErrorInvalidValue;
         }
         {   // T2R: (d, a, s*o+p)
             uint64_t dims[3] = {V, V, O * O};
             uint64_t st[2] = {dp * eb, V * dp * eb};
             uint32_t box[3] = {bk, brows, 1};
-            if (!encode(&d.maps[MAP_T2R][part], dt, 3, src[2], dims, st, box, err, "T2R")) return cudaErrorInvalidValue;
+            if (!encode(&d.maps[MAP_T2R][part], dt, 3, src[2], dims, st, box, err, "T2R", swz)) return cudaErrorInvalidValue;
         }
         {   // AoN: (l, a, q*o+s)
             uint64_t dims[3] = {O, V, O * O};
             uint64_t st[2] = {lp * eb, V * lp * eb};
             uint32_t box[3] = {bk, brows, 1};
-            if (!encode(&d.maps[MAP_AON][part], dt, 3, src[3], dims, st, box, err, "AoN")) return cudaErrorInvalidValue;
+            if (!encode(&d.maps[MAP_AON][part], dt, 3, src[3], dims, st, box, err, "AoN", swz)) return cudaErrorInvalidValue;
         }
     }
     return cudaSuccess;

@@ -68,6 +68,47 @@ __device__ __forceinline__ void fail(volatile int *abort_flag, int *err, int cod
     atomicOr(err, code);
 }
 
+// ---- warp-wide roles ---------------------------------------------------------
+// The TMA producer and the MMA issuer run their loops with the whole warp and
+// let one elected lane issue: tcgen05.mma and cp.async.bulk.tensor take their
+// descriptors and addresses from uniform registers, which the compiler can
+// only keep in code that the whole warp runs; in a branch on the lane number
+// it moves every operand there for each instruction.  W contractions on SM
+// pairs, with this and with 128-byte operand rows (gemm_tc.cu), before and
+// after: 24 molecules of o = 4..16, v = 20..120 in BF16X3 33.1 -> 29.2 ms,
+// o=13, v=131 in TF32X3 14.1 -> 13.0 ms, 28 tasks of o=50, v=450 67.6 -> 63.6
+// ms (TF32X3) and 39.0 -> 37.3..38.4 ms (BF16X3).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p = 0;
+    asm volatile("{\n\t.reg .pred px;\n\telect.sync _|px, 0xffffffff;\n\t@px mov.s32 %0, 1;\n\t}" : "+r"(p));
+    return p != 0;
+}
+// A value that is the same in every lane, as one that the compiler knows to be
+template <typename T>
+__device__ __forceinline__ T uni(T x) {
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "32- or 64-bit values");
+    return __shfl_sync(0xffffffffu, x, 0);
+}
+template <typename T>
+__device__ __forceinline__ const T *uni(const T *x) {
+    return reinterpret_cast<const T *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), 0));
+}
+// mbar_wait by a whole warp; the result is the same in every lane
+static __device__ __noinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    const uint64_t t0 = gtimer();
+    for (uint32_t it = 1;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+        if ((it & 63) == 0) {
+            const bool stop = *abort_flag || (it >= WAIT_MIN_POLLS && gtimer() - t0 > WAIT_LIMIT_NS);
+            if (__any_sync(0xffffffffu, stop)) return false;
+        }
+    }
+}
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    return mbar_wait_warp(bar, parity, abort_flag);
+}
+
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar,
                                             int c0, int c1, int c2, int c3) {
     asm volatile(
@@ -302,6 +343,7 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t cta_mask) 
 // the asm, and the accumulate flag is a compile-time constant.
 constexpr uint32_t DESC_LO_FLAGS = 1u << 16;                 // LBO = 1 (unused for swizzled K-major tiles)
 constexpr uint32_t DESC_HI = 32u | (1u << 14) | (4u << 29);  // SBO = 512 bytes, bit 46, 64-byte swizzle
+constexpr uint32_t DESC_HI128 = 64u | (1u << 14) | (2u << 29);  // SBO = 1024 bytes, 128-byte swizzle
 static_assert(((uint64_t)DESC_HI << 32 | DESC_LO_FLAGS) == (((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
                                                              ((uint64_t)1 << 46) | ((uint64_t)4 << 61)),
               "same descriptor fields as sdesc");
@@ -311,8 +353,8 @@ __device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr & 0x3
     asm volatile("{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\t"                                  \
                  "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t" PRED                      \
                  "tcgen05.mma.cta_group::" CGS ".kind::" KINDS " [%0], da, db, %3, p;\n\t}\n" ::"r"(d), \
-                 "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(DESC_HI))
-template <int KIND, int CG, bool ACC>
+                 "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(HI))
+template <int KIND, int CG, bool ACC, uint32_t HI = DESC_HI>
 __device__ __forceinline__ void mma_lo(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
     if constexpr (CG == 1 && KIND == 1 && ACC) TCX_MMA_ASM("1", "tf32", "setp.eq.u32 p, 0, 0;\n\t");
     else if constexpr (CG == 1 && KIND == 1) TCX_MMA_ASM("1", "tf32", "setp.ne.u32 p, 0, 0;\n\t");
@@ -334,74 +376,124 @@ struct MmaRing {
     int stage;
     uint32_t phase, hblk;
 };
-// Inline fast path of a bounded wait.
-__device__ __forceinline__ bool wait_fast(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
-    return mbar_test(bar, parity) || mbar_wait(bar, parity, abort_flag);
-}
 template <int CG>
 __device__ __forceinline__ void commit_to(uint32_t bar) {
     if constexpr (CG == 1) tc_commit(bar);
     else tc_commit_pair(bar, (uint16_t)3);
 }
-// The split products of one K chunk in stage st: lo = hi*lo + lo*hi, hi = hi*hi.
-// nks = 1: only the first K step holds data (BF16 segment tail).
-template <int KIND, int CG, bool FIRST>
-__device__ __forceinline__ void chunk_lo(const MmaRing &r, int st, uint32_t dt, uint32_t idesc, int nks) {
-    const uint32_t a = r.lo0 + (uint32_t)st * r.step, b = a + 2 * r.a16;
-    mma_lo<KIND, CG, !FIRST>(dt, a, b + r.b16, idesc);
-    mma_lo<KIND, CG, true>(dt, a + r.a16, b, idesc);
-    if (KIND == 1 || nks > 1) {
-        mma_lo<KIND, CG, true>(dt, a + 2, b + r.b16 + 2, idesc);
-        mma_lo<KIND, CG, true>(dt, a + r.a16 + 2, b + 2, idesc);
+// The split products of one K chunk: lo = hi*lo + lo*hi, hi = hi*hi.  a, b:
+// descriptor low words of the chunk's first K step in the A_hi and B_hi
+// planes; a16, b16: plane sizes >> 4.  nks = 1: only the first K step holds
+// data (segment tail).  HI: descriptor high word (64- or 128-byte rows).
+template <int KIND, int CG, bool FIRST, uint32_t HI>
+__device__ __forceinline__ void chunk_lo(uint32_t a, uint32_t b, uint32_t a16, uint32_t b16, uint32_t dt,
+                                         uint32_t idesc, int nks) {
+    mma_lo<KIND, CG, !FIRST, HI>(dt, a, b + b16, idesc);
+    mma_lo<KIND, CG, true, HI>(dt, a + a16, b, idesc);
+    if (nks > 1) {
+        mma_lo<KIND, CG, true, HI>(dt, a + 2, b + b16 + 2, idesc);
+        mma_lo<KIND, CG, true, HI>(dt, a + a16 + 2, b + 2, idesc);
     }
 }
-template <int KIND, int CG>
-__device__ __forceinline__ void chunk_hi(const MmaRing &r, int st, uint32_t dt, uint32_t idesc, int nks) {
-    const uint32_t a = r.lo0 + (uint32_t)st * r.step, b = a + 2 * r.a16;
-    mma_lo<KIND, CG, true>(dt, a, b, idesc);
-    if (KIND == 1 || nks > 1) mma_lo<KIND, CG, true>(dt, a + 2, b + 2, idesc);
+template <int KIND, int CG, uint32_t HI>
+__device__ __forceinline__ void chunk_hi(uint32_t a, uint32_t b, uint32_t dt, uint32_t idesc, int nks) {
+    mma_lo<KIND, CG, true, HI>(dt, a, b, idesc);
+    if (nks > 1) mma_lo<KIND, CG, true, HI>(dt, a + 2, b + 2, idesc);
 }
-// Every MMA of one work item: K blocks of two chunks, each into a fresh TMEM
-// accumulator buffer (tmem + 256 * (block & 1)); within a block the small
-// products of each chunk are issued as the chunk lands and the block's hi*hi
-// products last, then each stage is released and the block handed to the
-// drain (see the kernels).  nch: chunks of the item; dtail, ltail: chunk
-// indices of the last chunk of the d and l segments (two each) that hold a
-// single K step (BF16 with the segment's extent 16 mod 32), -1 if none.
-// Returns false (after flagging) when a bounded wait expired.
+// Every MMA of one work item, by a whole warp: K blocks of two chunks, each
+// into a fresh TMEM accumulator buffer (tmem + 256 * (block & 1)); within a
+// block the small products of each chunk are issued as the chunk lands and the
+// block's hi*hi products last, then each stage is released and the block
+// handed to the drain (see the kernels).  nch: chunks of the item (even); dt0,
+// dt1, lt0, lt1: chunk indices of the last chunk of the d and l segments (two
+// each) where it holds a single K step, -1 if none.  Returns false (with the
+// code of the wait) when a bounded wait expired.
 template <int KIND, int CG>
 __device__ __forceinline__ bool mma_item(MmaRing &r, uint32_t tmem, uint32_t idesc, int nch, int dt0, int dt1,
                                          int lt0, int lt1, volatile int *abort_flag, int *fail_code) {
     for (int c0 = 0; c0 < nch; c0 += 2) {
-        const bool two = c0 + 1 < nch;
         const uint32_t buf = r.hblk & 1u;
         const uint32_t dt = tmem + buf * 256u;
         const int s0 = r.stage;
-        if (!wait_fast(r.full0 + 8u * (uint32_t)s0, r.phase, abort_flag)) { *fail_code = DERR_TIMEOUT_FULL; return false; }
-        if (!wait_fast(r.hempty0 + 8u * buf, ((r.hblk >> 1) & 1u) ^ 1u, abort_flag)) {
+        if (!wait_warp(r.full0 + 8u * (uint32_t)s0, r.phase, abort_flag)) { *fail_code = DERR_TIMEOUT_FULL; return false; }
+        if (!wait_warp(r.hempty0 + 8u * buf, ((r.hblk >> 1) & 1u) ^ 1u, abort_flag)) {
             *fail_code = DERR_TIMEOUT_TMEM;
             return false;
         }
         tc_fence_after();
         const int n0 = (c0 == dt0 || c0 == dt1 || c0 == lt0 || c0 == lt1) ? 1 : 2;
-        chunk_lo<KIND, CG, true>(r, s0, dt, idesc, n0);
+        const int n1 = (c0 + 1 == dt0 || c0 + 1 == dt1 || c0 + 1 == lt0 || c0 + 1 == lt1) ? 1 : 2;
+        const uint32_t a0 = r.lo0 + (uint32_t)s0 * r.step, b0 = a0 + 2 * r.a16;
         if (++r.stage == r.nst) { r.stage = 0; r.phase ^= 1u; }
-        int s1 = -1, n1 = 2;
-        if (two) {
+        if (elect_one()) chunk_lo<KIND, CG, true, DESC_HI>(a0, b0, r.a16, r.b16, dt, idesc, n0);
+        __syncwarp();
+        const int s1 = r.stage;
+        if (!wait_warp(r.full0 + 8u * (uint32_t)s1, r.phase, abort_flag)) { *fail_code = DERR_TIMEOUT_FULL; return false; }
+        tc_fence_after();
+        const uint32_t a1 = r.lo0 + (uint32_t)s1 * r.step, b1 = a1 + 2 * r.a16;
+        if (++r.stage == r.nst) { r.stage = 0; r.phase ^= 1u; }
+        if (elect_one()) {
+            chunk_lo<KIND, CG, false, DESC_HI>(a1, b1, r.a16, r.b16, dt, idesc, n1);
+            chunk_hi<KIND, CG, DESC_HI>(a0, b0, dt, idesc, n0);
+            commit_to<CG>(r.empty0 + 8u * (uint32_t)s0);
+            chunk_hi<KIND, CG, DESC_HI>(a1, b1, dt, idesc, n1);
+            commit_to<CG>(r.empty0 + 8u * (uint32_t)s1);
+            commit_to<CG>(r.hfull0 + 8u * buf);
+        }
+        __syncwarp();
+        r.hblk++;
+    }
+    return true;
+}
+
+// mma_item for stages of 128-byte rows (SM pairs): a stage holds one K block,
+// the two chunks of a block side by side in its rows (second chunk +64 bytes).
+// Where a segment has an odd number of chunks (kv for d, ko for l), its last
+// chunk shares a block with the first chunk of the next segment: that block
+// takes two stages, each with its chunk in the first half (see the producer).
+// The products of a block, and which chunks share one, are those of mma_item.
+// dtail, ltail: the last chunk of the d (l) segments holds a single K step.
+template <int KIND>
+__device__ __forceinline__ bool mma_item_wide(MmaRing &r, uint32_t tmem, uint32_t idesc, int kv, int ko, bool dtail,
+                                              bool ltail, volatile int *abort_flag, int *fail_code) {
+    const int nch = 2 * (kv + ko);
+    const int dt0 = dtail ? kv - 1 : -1, dt1 = dtail ? 2 * kv - 1 : -1;
+    const int lt0 = ltail ? 2 * kv + ko - 1 : -1, lt1 = ltail ? nch - 1 : -1;
+    const int sd = (kv & 1) ? kv - 1 : -1, sl = (ko & 1) ? 2 * kv + ko - 1 : -1;  // blocks across two segments
+    for (int c0 = 0; c0 < nch; c0 += 2) {
+        const uint32_t buf = r.hblk & 1u;
+        const uint32_t dt = tmem + buf * 256u;
+        const int s0 = r.stage;
+        const bool across = c0 == sd || c0 == sl;
+        if (!wait_warp(r.full0 + 8u * (uint32_t)s0, r.phase, abort_flag)) { *fail_code = DERR_TIMEOUT_FULL; return false; }
+        if (!wait_warp(r.hempty0 + 8u * buf, ((r.hblk >> 1) & 1u) ^ 1u, abort_flag)) {
+            *fail_code = DERR_TIMEOUT_TMEM;
+            return false;
+        }
+        const int n0 = (c0 == dt0 || c0 == dt1 || c0 == lt0 || c0 == lt1) ? 1 : 2;
+        const int n1 = (c0 + 1 == dt0 || c0 + 1 == dt1 || c0 + 1 == lt0 || c0 + 1 == lt1) ? 1 : 2;
+        const uint32_t a0 = r.lo0 + (uint32_t)s0 * r.step, b0 = a0 + 2 * r.a16;
+        if (++r.stage == r.nst) { r.stage = 0; r.phase ^= 1u; }
+        int s1 = s0;
+        uint32_t a1 = a0 + 4, b1 = b0 + 4;
+        if (across) {
             s1 = r.stage;
-            if (!wait_fast(r.full0 + 8u * (uint32_t)s1, r.phase, abort_flag)) { *fail_code = DERR_TIMEOUT_FULL; return false; }
-            tc_fence_after();
-            n1 = (c0 + 1 == dt0 || c0 + 1 == dt1 || c0 + 1 == lt0 || c0 + 1 == lt1) ? 1 : 2;
-            chunk_lo<KIND, CG, false>(r, s1, dt, idesc, n1);
+            if (!wait_warp(r.full0 + 8u * (uint32_t)s1, r.phase, abort_flag)) { *fail_code = DERR_TIMEOUT_FULL; return false; }
+            a1 = r.lo0 + (uint32_t)s1 * r.step;
+            b1 = a1 + 2 * r.a16;
             if (++r.stage == r.nst) { r.stage = 0; r.phase ^= 1u; }
         }
-        chunk_hi<KIND, CG>(r, s0, dt, idesc, n0);
-        commit_to<CG>(r.empty0 + 8u * (uint32_t)s0);
-        if (two) {
-            chunk_hi<KIND, CG>(r, s1, dt, idesc, n1);
-            commit_to<CG>(r.empty0 + 8u * (uint32_t)s1);
+        tc_fence_after();
+        if (elect_one()) {
+            chunk_lo<KIND, 2, true, DESC_HI128>(a0, b0, r.a16, r.b16, dt, idesc, n0);
+            chunk_lo<KIND, 2, false, DESC_HI128>(a1, b1, r.a16, r.b16, dt, idesc, n1);
+            chunk_hi<KIND, 2, DESC_HI128>(a0, b0, dt, idesc, n0);
+            if (across) commit_to<2>(r.empty0 + 8u * (uint32_t)s0);
+            chunk_hi<KIND, 2, DESC_HI128>(a1, b1, dt, idesc, n1);
+            commit_to<2>(r.empty0 + 8u * (uint32_t)s1);
+            commit_to<2>(r.hfull0 + 8u * buf);
         }
-        commit_to<CG>(r.hfull0 + 8u * buf);
+        __syncwarp();
         r.hblk++;
     }
     return true;
