@@ -28,8 +28,10 @@
 // rows, 64-byte K rows) and S B planes (OZ_N rows of a) with 5-D / 4-D tensor
 // maps whose outermost coordinate is the slice; warp 1 issues the S(S+1)/2
 // slice-pair MMAs (M = 128, N = OZ_N) into the S weight accumulators of a
-// TMEM block of OZ_KB chunks; warps 2-9 drain and accumulate.  Every wait is
-// bounded as in the split-precision kernel.
+// TMEM block of OZ_KB chunks; warps 2-9 drain and accumulate.  Warps 0 and 1 run
+// whole, one elected lane issuing (tc_common.cuh): 52 tasks of o=40, v=300 took
+// 128.7 ms with both in a branch on the lane number and 116.4 ms so.  Every wait
+// is bounded as in the split-precision kernel.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -154,114 +156,116 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) ugemm_oz_kernel(const __grid_co
                                ((uint32_t)(OZ_BM >> 4) << 24);
 
     if (warp == 0) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int last_phase[OZ_STAGES];
-            for (int s = 0; s < OZ_STAGES; s++) last_phase[s] = -1;
-            bool ok = true;
-            bool inject = wv.inject_stall != 0 && blockIdx.x == 0;
-            SegCache sc;
-            seg_reset(sc);
-            for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
-                const Item w = decode(wv, it, sc);
-                if (w.diag) continue;
-                const InstDesc &d = *sc.d;
-                const int o = d.dm.o, kv = d.kv, ko = d.ko, nch = 2 * kv + 2 * ko;
-                const int s = w.s, pp = w.p, q = w.q;
-                const int cb = w.bt * d.pb, cc = w.ct * d.pc, ca = w.n * OZ_N;
-                const uint32_t stage_tx = d.stage_tx;
-                for (int ch = 0; ch < nch; ch++) {
-                    if (!mbar_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
-                        fail(&abort_sh, wv.err, DERR_TIMEOUT_EMPTY);
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t full = smem_u32(&bar_full[stage]);
+        int stage = 0;
+        uint32_t phase = 0;
+        int last_phase[OZ_STAGES];
+        for (int s = 0; s < OZ_STAGES; s++) last_phase[s] = -1;
+        bool ok = true;
+        bool inject = wv.inject_stall != 0 && blockIdx.x == 0;
+        SegCache sc;
+        seg_reset(sc);
+        for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
+            const Item w = decode(wv, it, sc);
+            if (uni((int)w.diag)) continue;
+            const InstDesc *d = uni(sc.d);
+            const int o = uni(d->dm.o), kv = uni(d->kv), ko = uni(d->ko), nch = 2 * kv + 2 * ko;
+            const int s = uni(w.s), pp = uni(w.p), q = uni(w.q);
+            const int cb = uni(w.bt * d->pb), cc = uni(w.ct * d->pc), ca = uni(w.n * OZ_N);
+            const uint32_t stage_tx = uni(d->stage_tx);
+            for (int ch = 0; ch < nch; ch++) {
+                if (!wait_warp(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
+                    if (lane == 0) fail(&abort_sh, wv.err, DERR_TIMEOUT_EMPTY);
+                    ok = false;
+                    break;
+                }
+                const uint32_t full = smem_u32(&bar_full[stage]);
+                last_phase[stage] = (int)phase;
+                const uint32_t sA = sbase + stage * OZ_STAGE, sB = sA + OZ_S * OZ_A;
+                int seg, kk;
+                if (ch < kv) { seg = 0; kk = ch; }
+                else if (ch < 2 * kv) { seg = 1; kk = ch - kv; }
+                else if (ch < 2 * kv + ko) { seg = 2; kk = ch - 2 * kv; }
+                else { seg = 3; kk = ch - 2 * kv - ko; }
+                const int k0 = kk * 32;
+                int amap, aslice, bmap, brow;
+                switch (seg) {
+                    case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; brow = s * o + pp; break;
+                    case 1: amap = MAP_G_SWP; aslice = pp; bmap = MAP_T2R; brow = s * o + q; break;
+                    case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; brow = q * o + s; break;
+                    default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; brow = pp * o + s; break;
+                }
+                if (elect_one()) {
                     mbar_expect_tx(full, stage_tx);
-                    last_phase[stage] = (int)phase;
-                    const uint32_t sA = sbase + stage * OZ_STAGE, sB = sA + OZ_S * OZ_A;
-                    int seg, kk;
-                    if (ch < kv) { seg = 0; kk = ch; }
-                    else if (ch < 2 * kv) { seg = 1; kk = ch - kv; }
-                    else if (ch < 2 * kv + ko) { seg = 2; kk = ch - 2 * kv; }
-                    else { seg = 3; kk = ch - 2 * kv - ko; }
-                    const int k0 = kk * 32;
-                    int amap, aslice, bmap, brow;
-                    switch (seg) {
-                        case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; brow = s * o + pp; break;
-                        case 1: amap = MAP_G_SWP; aslice = pp; bmap = MAP_T2R; brow = s * o + q; break;
-                        case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; brow = q * o + s; break;
-                        default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; brow = pp * o + s; break;
-                    }
-                    if (inject) {
-                        inject = false;
-                        last_phase[stage] = -1;  // nothing in flight: the consumer's wait must expire
-                    } else {
+                    if (!inject) {
                         for (int pl = 0; pl < OZ_S; pl++) {
-                            tma_load_5d(sA + pl * OZ_A, &d.maps[amap][0], full, k0, cc, cb, aslice, pl);
-                            tma_load_4d(sB + pl * OZ_B, &d.maps[bmap][0], full, k0, ca, brow, pl);
+                            tma_load_5d(sA + pl * OZ_A, &d->maps[amap][0], full, k0, cc, cb, aslice, pl);
+                            tma_load_4d(sB + pl * OZ_B, &d->maps[bmap][0], full, k0, ca, brow, pl);
                         }
                     }
-                    if (++stage == OZ_STAGES) { stage = 0; phase ^= 1u; }
                 }
+                __syncwarp();
+                if (inject) {
+                    inject = false;
+                    last_phase[stage] = -1;  // nothing in flight: the consumer's wait must expire
+                }
+                if (++stage == OZ_STAGES) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) {  // let this CTA's copies in flight land before exiting
-                for (int s = 0; s < OZ_STAGES; s++) {
-                    if (last_phase[s] < 0) continue;
-                    const uint64_t t0 = gtimer();
-                    while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
-                           gtimer() - t0 < WAIT_LIMIT_NS) {
-                    }
+        }
+        if (!ok && lane == 0) {  // let this CTA's copies in flight land before exiting
+            for (int s = 0; s < OZ_STAGES; s++) {
+                if (last_phase[s] < 0) continue;
+                const uint64_t t0 = gtimer();
+                while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
+                       gtimer() - t0 < WAIT_LIMIT_NS) {
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            uint32_t hblk = 0;  // blocks of OZ_KB chunks issued: accumulator phase hblk & 1
-            bool ok = true;
-            SegCache sc;
-            seg_reset(sc);
-            for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
-                const Item w = decode(wv, it, sc);
-                if (w.diag) continue;
-                const InstDesc &d = *sc.d;
-                const int kv = d.kv, ko = d.ko, dp = d.dm.dp, lp = d.dm.lp;
-                const int nch = 2 * kv + 2 * ko;
-                for (int c0 = 0; c0 < nch && ok; c0 += OZ_KB) {
-                    const int nb = min(OZ_KB, nch - c0);
-                    for (int cb = 0; cb < nb; cb++) {
-                        const int ch = c0 + cb;
-                        if (!mbar_wait(smem_u32(&bar_full[stage]), phase, &abort_sh)) {
-                            fail(&abort_sh, wv.err, DERR_TIMEOUT_FULL);
-                            ok = false;
-                            break;
-                        }
-                        if (cb == 0 && !mbar_wait(smem_u32(&bar_hempty[0]), (hblk & 1u) ^ 1u, &abort_sh)) {
-                            fail(&abort_sh, wv.err, DERR_TIMEOUT_TMEM);
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint32_t sA = sbase + stage * OZ_STAGE, sB = sA + OZ_S * OZ_A;
-                        const int nks = chunk_ksteps(2, kv, ko, dp, lp, ch);
-                        // descriptor low words (see mma_lo): plane and K-step offsets are
-                        // constants added to the stage's base words.  Every slice product
-                        // is exact in FP32, so their order within a block is free: the
-                        // first K step of every weight first (the block's opening MMA of
-                        // each weight zeroes it), then the second
-                        const uint32_t a0 = desc_lo(sA), b0 = desc_lo(sB);
-                        if (cb == 0) oz_chunk<true>(tmem, a0, b0, idesc, nks);
-                        else oz_chunk<false>(tmem, a0, b0, idesc, nks);
-                        tc_commit(smem_u32(&bar_empty[stage]));  // the stage is free once these MMAs are done
-                        if (++stage == OZ_STAGES) { stage = 0; phase ^= 1u; }
+        int stage = 0;
+        uint32_t phase = 0;
+        uint32_t hblk = 0;  // blocks of OZ_KB chunks issued: accumulator phase hblk & 1
+        bool ok = true;
+        const uint32_t tm = uni(tmem);
+        SegCache sc;
+        seg_reset(sc);
+        for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
+            const Item w = decode(wv, it, sc);
+            if (uni((int)w.diag)) continue;
+            const InstDesc *d = uni(sc.d);
+            const int kv = uni(d->kv), ko = uni(d->ko), dp = uni(d->dm.dp), lp = uni(d->dm.lp);
+            const int nch = 2 * kv + 2 * ko;
+            for (int c0 = 0; c0 < nch && ok; c0 += OZ_KB) {
+                const int nb = min(OZ_KB, nch - c0);
+                for (int cb = 0; cb < nb; cb++) {
+                    const int ch = c0 + cb;
+                    int code = 0;
+                    if (!wait_warp(smem_u32(&bar_full[stage]), phase, &abort_sh)) code = DERR_TIMEOUT_FULL;
+                    else if (cb == 0 && !wait_warp(smem_u32(&bar_hempty[0]), (hblk & 1u) ^ 1u, &abort_sh))
+                        code = DERR_TIMEOUT_TMEM;
+                    if (code) {
+                        if (lane == 0) fail(&abort_sh, wv.err, code);
+                        ok = false;
+                        break;
                     }
-                    if (!ok) break;
-                    tc_commit(smem_u32(&bar_hfull[0]));
-                    hblk++;
+                    tc_fence_after();
+                    const uint32_t sA = sbase + stage * OZ_STAGE, sB = sA + OZ_S * OZ_A;
+                    const int nks = chunk_ksteps(2, kv, ko, dp, lp, ch);
+                    // descriptor low words (see mma_lo): plane and K-step offsets are
+                    // constants added to the stage's base words.  Every slice product
+                    // is exact in FP32, so their order within a block is free: the
+                    // first K step of every weight first (the block's opening MMA of
+                    // each weight zeroes it), then the second
+                    const uint32_t a0 = desc_lo(sA), b0 = desc_lo(sB);
+                    if (elect_one()) {
+                        if (cb == 0) oz_chunk<true>(tm, a0, b0, idesc, nks);
+                        else oz_chunk<false>(tm, a0, b0, idesc, nks);
+                        tc_commit(smem_u32(&bar_empty[stage]));  // the stage is free once these MMAs are done
+                        if (cb == nb - 1) tc_commit(smem_u32(&bar_hfull[0]));
+                    }
+                    __syncwarp();
+                    if (++stage == OZ_STAGES) { stage = 0; phase ^= 1u; }
                 }
+                hblk++;
             }
         }
     } else {

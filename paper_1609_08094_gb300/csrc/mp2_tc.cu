@@ -32,7 +32,9 @@
 // producer, a ring of 3 stages of 8 planes of 128 rows x 64 bytes (64 KB).
 // Warp 1: TMEM allocation (512 columns: G and H of two K blocks) and the MMA
 // issue.  Warps 2-9: two per TMEM lane quarter, 64 columns of G and of H
-// each.  Every mbarrier wait is bounded (wall clock): on expiry the kernel
+// each.  Warps 0 and 1 run whole, one elected lane issuing (tc_common.cuh): o=50,
+// v=450, naux=1500 in BF16X3 took 4.37 ms with both in a branch on the lane
+// number and 3.71 ms so.  Every mbarrier wait is bounded (wall clock): on expiry the kernel
 // sets an error flag, stops all roles, waits (bounded) for its own copies in
 // flight, frees TMEM and returns; the host reports TCORR_ETIMEOUT.
 #include <mutex>
@@ -105,27 +107,27 @@ __global__ void __launch_bounds__(MP_THREADS, 1) mp2_tc_kernel(const __grid_cons
     double ej = 0.0, ek = 0.0;  // epilogue threads: weighted Coulomb and exchange sums
 
     if (warp == 0) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int last_phase[MP_STAGES];
-            for (int s = 0; s < MP_STAGES; s++) last_phase[s] = -1;
-            bool ok = true;
-            for (int64_t it = blockIdx.x; it < a.items && ok; it += gridDim.x) {
-                const int pr = (int)(it / a.ntp), tp = (int)(it % a.ntp);
-                const int i = a.pairs[2 * pr], j = a.pairs[2 * pr + 1];
-                const int A0 = a.tiles[2 * tp] * MP_BM, B0 = a.tiles[2 * tp + 1] * MP_BM;
-                for (int ch = 0; ch < nch; ch++) {
-                    if (!mbar_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
-                        fail(&abort_sh, a.err, DERR_TIMEOUT_EMPTY);
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t full = smem_u32(&bar_full[stage]);
+        int stage = 0;
+        uint32_t phase = 0;
+        int last_phase[MP_STAGES];
+        for (int s = 0; s < MP_STAGES; s++) last_phase[s] = -1;
+        bool ok = true;
+        for (int64_t it = blockIdx.x; it < a.items && ok; it += gridDim.x) {
+            const int pr = (int)(it / a.ntp), tp = (int)(it % a.ntp);
+            const int i = uni(a.pairs[2 * pr]), j = uni(a.pairs[2 * pr + 1]);
+            const int A0 = uni(a.tiles[2 * tp]) * MP_BM, B0 = uni(a.tiles[2 * tp + 1]) * MP_BM;
+            for (int ch = 0; ch < nch; ch++) {
+                if (!wait_warp(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
+                    if (lane == 0) fail(&abort_sh, a.err, DERR_TIMEOUT_EMPTY);
+                    ok = false;
+                    break;
+                }
+                const uint32_t full = smem_u32(&bar_full[stage]);
+                last_phase[stage] = (int)phase;
+                const uint32_t s = sbase + stage * MP_STAGE;
+                const int k0 = ch * kch;
+                if (elect_one()) {
                     mbar_expect_tx(full, (uint32_t)MP_STAGE);
-                    last_phase[stage] = (int)phase;
-                    const uint32_t s = sbase + stage * MP_STAGE;
-                    const int k0 = ch * kch;
                     tma_load_3d(s + P_AI_HI * MP_TILE, &a.map[0], full, k0, A0, i);
                     tma_load_3d(s + P_AI_LO * MP_TILE, &a.map[1], full, k0, A0, i);
                     tma_load_3d(s + P_BJ_HI * MP_TILE, &a.map[0], full, k0, B0, j);
@@ -134,50 +136,50 @@ __global__ void __launch_bounds__(MP_THREADS, 1) mp2_tc_kernel(const __grid_cons
                     tma_load_3d(s + P_AJ_LO * MP_TILE, &a.map[1], full, k0, A0, j);
                     tma_load_3d(s + P_BI_HI * MP_TILE, &a.map[0], full, k0, B0, i);
                     tma_load_3d(s + P_BI_LO * MP_TILE, &a.map[1], full, k0, B0, i);
-                    if (++stage == MP_STAGES) { stage = 0; phase ^= 1u; }
                 }
+                __syncwarp();
+                if (++stage == MP_STAGES) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) {  // let this CTA's copies in flight land before exiting
-                for (int s = 0; s < MP_STAGES; s++) {
-                    if (last_phase[s] < 0) continue;
-                    const uint64_t t0 = gtimer();
-                    while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
-                           gtimer() - t0 < WAIT_LIMIT_NS) {
-                    }
+        }
+        if (!ok && lane == 0) {  // let this CTA's copies in flight land before exiting
+            for (int s = 0; s < MP_STAGES; s++) {
+                if (last_phase[s] < 0) continue;
+                const uint64_t t0 = gtimer();
+                while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
+                       gtimer() - t0 < WAIT_LIMIT_NS) {
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            uint32_t hblk = 0;  // K blocks issued so far: buffer hblk & 1, phase (hblk >> 1) & 1
-            bool ok = true;
-            for (int64_t it = blockIdx.x; it < a.items && ok; it += gridDim.x) {
-                for (int c0 = 0; c0 < nch && ok; c0 += MP_KB) {
-                    const int nb = min(MP_KB, nch - c0);
-                    const uint32_t buf = hblk & 1u;
-                    const uint32_t dG = tmem + buf * (uint32_t)(2 * MP_BM), dH = dG + (uint32_t)MP_BM;
-                    const int st0 = stage;
-                    for (int cb = 0; cb < nb; cb++) {
-                        if (!mbar_wait(smem_u32(&bar_full[stage]), phase, &abort_sh)) {
-                            fail(&abort_sh, a.err, DERR_TIMEOUT_FULL);
-                            ok = false;
-                            break;
-                        }
-                        if (cb == 0 &&
-                            !mbar_wait(smem_u32(&bar_hempty[buf]), ((hblk >> 1) & 1u) ^ 1u, &abort_sh)) {
-                            fail(&abort_sh, a.err, DERR_TIMEOUT_TMEM);
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        // descriptor low words of the stage's planes (see mma_lo): one K
-                        // step of 32 bytes is +2; the block's first products zero D
-                        const uint32_t s = desc_lo(sbase + stage * MP_STAGE);
-                        const uint32_t ai = s + P_AI_HI * (MP_TILE >> 4), bj = s + P_BJ_HI * (MP_TILE >> 4);
-                        const uint32_t aj = s + P_AJ_HI * (MP_TILE >> 4), bi = s + P_BI_HI * (MP_TILE >> 4);
-                        constexpr uint32_t LO = MP_TILE >> 4;  // hi plane -> lo plane
+        int stage = 0;
+        uint32_t phase = 0;
+        uint32_t hblk = 0;  // K blocks issued so far: buffer hblk & 1, phase (hblk >> 1) & 1
+        bool ok = true;
+        const uint32_t tm = uni(tmem);
+        for (int64_t it = blockIdx.x; it < a.items && ok; it += gridDim.x) {
+            for (int c0 = 0; c0 < nch && ok; c0 += MP_KB) {
+                const int nb = min(MP_KB, nch - c0);
+                const uint32_t buf = hblk & 1u;
+                const uint32_t dG = tm + buf * (uint32_t)(2 * MP_BM), dH = dG + (uint32_t)MP_BM;
+                const int st0 = stage;
+                for (int cb = 0; cb < nb; cb++) {
+                    int code = 0;
+                    if (!wait_warp(smem_u32(&bar_full[stage]), phase, &abort_sh)) code = DERR_TIMEOUT_FULL;
+                    else if (cb == 0 && !wait_warp(smem_u32(&bar_hempty[buf]), ((hblk >> 1) & 1u) ^ 1u, &abort_sh))
+                        code = DERR_TIMEOUT_TMEM;
+                    if (code) {
+                        if (lane == 0) fail(&abort_sh, a.err, code);
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    // descriptor low words of the stage's planes (see mma_lo): one K
+                    // step of 32 bytes is +2; the block's first products zero D
+                    const uint32_t s = desc_lo(sbase + stage * MP_STAGE);
+                    const uint32_t ai = s + P_AI_HI * (MP_TILE >> 4), bj = s + P_BJ_HI * (MP_TILE >> 4);
+                    const uint32_t aj = s + P_AJ_HI * (MP_TILE >> 4), bi = s + P_BI_HI * (MP_TILE >> 4);
+                    constexpr uint32_t LO = MP_TILE >> 4;  // hi plane -> lo plane
+                    if (elect_one()) {
                         if (cb == 0) mma_lo<KIND, 1, false>(dG, ai + LO, bj + LO, idesc);
                         else mma_lo<KIND, 1, true>(dG, ai + LO, bj + LO, idesc);
                         mma_lo<KIND, 1, true>(dG, ai, bj + LO, idesc);
@@ -192,12 +194,15 @@ __global__ void __launch_bounds__(MP_THREADS, 1) mp2_tc_kernel(const __grid_cons
                         mma_lo<KIND, 1, true>(dH, aj + LO + 2, bi + LO + 2, idesc);
                         mma_lo<KIND, 1, true>(dH, aj + 2, bi + LO + 2, idesc);
                         mma_lo<KIND, 1, true>(dH, aj + LO + 2, bi + 2, idesc);
-                        if (++stage == MP_STAGES) { stage = 0; phase ^= 1u; }
                     }
-                    if (!ok) break;
-                    // the dominant hi*hi products of the block last; each stage is
-                    // released (commit: arrives once every MMA issued so far has
-                    // completed) right after its last product is issued
+                    __syncwarp();
+                    if (++stage == MP_STAGES) { stage = 0; phase ^= 1u; }
+                }
+                if (!ok) break;
+                // the dominant hi*hi products of the block last; each stage is
+                // released (commit: arrives once every MMA issued so far has
+                // completed) right after its last product is issued
+                if (elect_one()) {
                     int sj = st0;
                     for (int cb = 0; cb < nb; cb++) {
                         const uint32_t s = desc_lo(sbase + sj * MP_STAGE);
@@ -211,8 +216,9 @@ __global__ void __launch_bounds__(MP_THREADS, 1) mp2_tc_kernel(const __grid_cons
                         if (++sj == MP_STAGES) sj = 0;
                     }
                     tc_commit(smem_u32(&bar_hfull[buf]));
-                    hblk++;
                 }
+                __syncwarp();
+                hblk++;
             }
         }
     } else {
