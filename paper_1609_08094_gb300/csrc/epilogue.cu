@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
 // ring of two orbit stages in shared memory.
 //
 // The tensor-core contractions store each group tensor as its term of W in
-// W's own index order, in swizzled 8^3 cubes (tcorr_internal.cuh), so the
+// W's own index order, in 8^3 cubes (tcorr_internal.cuh), so the
 // three cubes that make up one W cube sit at the same cube coordinates and
 // W = C0 + C1 + C2 element by element, and the three terms of a cube are
 // stored side by side.  Per orbit two producer warps fill a free stage, every
@@ -379,8 +379,14 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
 // kernel: one warp issuing 57 copies per orbit took 0.38 ms per task at
 // o=50, v=450 (0.27 ms now; 16-byte cp.async for the small operands was
 // slower still).  Eight compute warps evaluate the orbit held in the other
-// stage meanwhile.  The cube swizzle makes every W read conflict-free, and
-// the index arithmetic per element orbit is a handful of precomputed offsets.
+// stage meanwhile.  The lanes of a warp take the elements of an orbit in a
+// skewed order that makes every read of W, t1 and ovov conflict-free (see the
+// compute warps), and the index arithmetic per element orbit is a handful of
+// precomputed offsets.  Orbits with repeated blocks take the same form.  With
+// swizzled cubes and an element-by-element loop for repeated blocks the kernel
+// took 7.1 ms for 28 tasks of o=50, v=450 (6.6 ms now), 3.93 ms for o=13, v=131
+// (3.01) and 13.7 ms for 24 molecules of v = 20..120 (10.5), where most orbits
+// have repeated blocks.
 //
 // The per-orbit sum over the CTA goes through shared memory in a fixed
 // order, summed by one compute warp per orbit in rotation, with
@@ -441,7 +447,7 @@ struct EpiMeta {
     ff eijk;                     // e_i + e_j + e_k
     int ob[3];                   // blocks A <= B <= C
     int smap[6];                 // slot whose cubes hold slot s's data (the first with its block triple)
-    int kind;                    // 0: no more orbits, 1: three distinct blocks, 2: repeated blocks
+    int kind;                    // 0: no more orbits, 1: three distinct blocks, 2: two equal, 6: all equal
     int v;                       // virtual orbitals of the problem
 };
 
@@ -470,7 +476,6 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
     __shared__ __align__(8) uint64_t bar_full[EPI_STAGES], bar_empty[EPI_STAGES];
     __shared__ __align__(8) uint64_t bar_rfull[2], bar_rempty[2];
     __shared__ __align__(16) float4 red[2][NT];
-    __shared__ int comp[6][6];
     __shared__ volatile int abort_sh;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -485,14 +490,6 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
         }
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (tid < 36) {  // comp[pi][q]: the slot of permutation pi composed with q
-        const int pi = tid / 6, q = tid % 6;
-        const int t0 = perm_pos(pi, perm_pos(q, 0)), t1v = perm_pos(pi, perm_pos(q, 1));
-        int sig = 0;
-        for (int s = 0; s < 6; s++)
-            if (perm_pos(s, 0) == t0 && perm_pos(s, 1) == t1v) sig = s;
-        comp[pi][q] = sig;
     }
     __syncthreads();  // the last CTA-wide barrier: from here on the roles meet only at mbarriers
 
@@ -608,7 +605,7 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
                 m.ob[0] = ob0; m.ob[1] = ob1; m.ob[2] = ob2;
 #pragma unroll
                 for (int s = 0; s < 6; s++) m.smap[s] = smap[s];
-                m.kind = (ob0 < ob1 && ob1 < ob2) ? 1 : 2;
+                m.kind = (ob0 < ob1 && ob1 < ob2) ? 1 : (ob0 == ob2 ? 6 : 2);
                 m.v = v;
                 mbar_expect_tx(full, u_bytes + ev_bytes + (EPI_PRODUCERS == 1 ? ovt1_bytes : 0u));
             }
@@ -671,28 +668,17 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
     }
 
     // ---------------- compute warps ----------------
-    // thread: fixed (b, c) = (lb, lc), a = la0 and la0 + 4 (the 512 element
-    // orbits of a cube with three distinct blocks over 256 threads)
-    const int lb = (tid >> 3) & 7, lc = tid & 7, la0 = tid >> 6;
-    // cube offsets of the six orderings (abc, acb, bac, bca, cab, cba) in C0
-    // and C1 (offd) and in C2 (offd2: its y index innermost)
-    int offd[2][6], offd2[2][6];
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-        const int la = la0 + 4 * h;
-        offd[h][0] = ucube_off(la, lb, lc);
-        offd[h][1] = ucube_off(la, lc, lb);
-        offd[h][2] = ucube_off(lb, la, lc);
-        offd[h][3] = ucube_off(lb, lc, la);
-        offd[h][4] = ucube_off(lc, la, lb);
-        offd[h][5] = ucube_off(lc, lb, la);
-        offd2[h][0] = ucube_off(la, lc, lb);
-        offd2[h][1] = ucube_off(la, lb, lc);
-        offd2[h][2] = ucube_off(lb, lc, la);
-        offd2[h][3] = ucube_off(lb, la, lc);
-        offd2[h][4] = ucube_off(lc, lb, la);
-        offd2[h][5] = ucube_off(lc, la, lb);
-    }
+    // thread: fixed (b, c) = (lb, lc) and two a, la and la ^ 4: the 512 element
+    // orbits of a cube over 256 threads.  Lane 8 j + i of warp w holds lb = i,
+    // lc = i ^ j ^ 4 (w & 1), la = i ^ n(j) ^ (w >> 1) with n = (0, 2, 3, 1): in
+    // each of the six orders of (la, lb, lc) as (slow, middle, fast) index of an
+    // 8^3 cube, and of each pair of them in an 8 x 8 block, the 32 lanes touch
+    // 32 distinct banks (n(j) and n(j) ^ j are both permutations of 0..3).
+    const int li = lane & 7, lj = lane >> 3;
+    const int lb = li, lc = li ^ lj ^ ((warp & 1) << 2), la0 = li ^ ((lj & 1) << 1) ^ ((lj >> 1) * 3) ^ (warp >> 1);
+    // offsets of (slow, middle, fast) = abc, acb, bac, bca, cab, cba
+    const int p_abc = la0 * 64 + lb * 8 + lc, p_acb = la0 * 64 + lc * 8 + lb, p_bac = lb * 64 + la0 * 8 + lc;
+    const int p_bca = lb * 64 + lc * 8 + la0, p_cab = lc * 64 + la0 * 8 + lb, p_cba = lc * 64 + lb * 8 + la0;
     for (int n = 0;; n++) {
         const int stage = n % EPI_STAGES;
         if (!mbar_wait(smem_u32(&bar_full[stage]), (uint32_t)((n / EPI_STAGES) & 1), &abort_sh)) {
@@ -707,17 +693,21 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
         const int v = meta[stage].v;
         const EpiStage &S = stg[stage];
         ff A4 = {0.f, 0.f}, A5 = {0.f, 0.f};
-        if (kind == 1) {
-            // Distinct blocks: each thread takes element orbits, the six orderings
-            // of one (a,b,c) with a in A, b in B, c in C.  Slot q holds the element
-            // with indices ordered as q (slots 0..5 = abc, acb, bac, bca, cab, cba);
-            // even slots 0,3,4, odd slots 1,2,5.  With E and O the sums of W over
-            // the even and odd slots, Z at slot q is 6 w_q + 2E - 4O (q even) or
-            // 6 w_q + 2O - 4E (q odd), and all six share one denominator.  What
-            // depends only on b and c is read once for the thread's two orbits.
+        // Each thread takes element orbits, the six orderings of one (a,b,c) with
+        // a in A, b in B, c in C.  Slot q holds the element with indices ordered
+        // as q (slots 0..5 = abc, acb, bac, bca, cab, cba); even slots 0,3,4, odd
+        // slots 1,2,5.  With E and O the sums of W over the even and odd slots, Z
+        // at slot q is 6 w_q + 2E - 4O (q even) or 6 w_q + 2O - 4E (q odd), and
+        // all six share one denominator.  What depends only on b and c is read
+        // once for the thread's two orbits.  Where blocks repeat, the loop over
+        // (a,b,c) meets every element 2 (two equal blocks) or 6 times (all equal)
+        // -- as often for elements with equal indices, whose six orderings repeat
+        // instead -- and the orbit's sum is divided by that; a slot whose block
+        // triple repeats an earlier one's reads that slot's cube (meta.smap).
+        auto orbits = [&](const float *c0, const float *c1, const float *c2, const float *c3, const float *c4,
+                          const float *c5) {
             const int A0 = ob0 * F8, B0 = ob1 * F8, C0 = ob2 * F8;
 #define OVV(sl, pu, pw, lu, lw) S.ov[sl][pu][pw][(lu) * F8 + (lw)]
-#define WQ(q, h) (S.cube[q][0][offd[h][q]] + S.cube[q][1][offd[h][q]] + S.cube[q][2][offd2[h][q]])
             const float tib = S.t1[0][1][lb], tic = S.t1[0][2][lc];
             const float tjb = S.t1[1][1][lb], tjc = S.t1[1][2][lc];
             const float tkb = S.t1[2][1][lb], tkc = S.t1[2][2][lc];
@@ -729,10 +719,17 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
             const bool bc_in = B0 + lb < v && C0 + lc < v;
 #pragma unroll
             for (int h = 0; h < 2; h++) {
-                const int la = la0 + 4 * h;
-                if (!bc_in || A0 + la >= v) break;  // a grows with h
-                const float w0 = WQ(0, h), w1 = WQ(1, h), w2 = WQ(2, h);
-                const float w3 = WQ(3, h), w4 = WQ(4, h), w5 = WQ(5, h);
+                const int la = la0 ^ (4 * h);
+                if (!bc_in || A0 + la >= v) continue;
+                // W at slot (x, y, z) = C0 + C1 + C2, each with its group's a (x, y, z) innermost
+                const int abc = p_abc ^ (h * 256), acb = p_acb ^ (h * 256), bac = p_bac ^ (h * 32);
+                const int bca = p_bca ^ (h * 4), cab = p_cab ^ (h * 32), cba = p_cba ^ (h * 4);
+                const float w0 = c0[bca] + c0[512 + acb] + c0[1024 + abc];
+                const float w1 = c1[cba] + c1[512 + abc] + c1[1024 + acb];
+                const float w2 = c2[acb] + c2[512 + bca] + c2[1024 + bac];
+                const float w3 = c3[cab] + c3[512 + bac] + c3[1024 + bca];
+                const float w4 = c4[abc] + c4[512 + cba] + c4[1024 + cab];
+                const float w5 = c5[bac] + c5[512 + cab] + c5[1024 + cba];
                 // t1 of occupied i, j, k at a (at b and c above)
                 const float tia = S.t1[0][0][la], tja = S.t1[1][0][la], tka = S.t1[2][0][la];
                 // (j u | k w), (i u | k w), (i u | j w) for the ordered pairs of {a, b, c} that hold a
@@ -759,37 +756,14 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
                 A4 = ff_add(A4, ff_mul(s4, r));
                 A5 = ff_add(A5, ff_mul(s5, r));
             }
-#undef WQ
 #undef OVV
+        };
+        if (kind == 1) {
+            const float *q = S.cube[0][0];
+            orbits(q, q + 1536, q + 3072, q + 4608, q + 6144, q + 7680);
         } else {
-            // blocks repeat: element by element over the distinct slots
-            for (int s = 0; s < 6; s++) {
-                if (meta[stage].smap[s] != s) continue;
-                const int p0 = perm_pos(s, 0), p1 = perm_pos(s, 1), p2 = perm_pos(s, 2);
-                const float *W[6];
-#pragma unroll
-                for (int q = 0; q < 6; q++) W[q] = S.cube[meta[stage].smap[comp[s][q]]][0];
-#define WAT(q, x, y, z) (W[q][ucube_off(x, y, z)] + W[q][512 + ucube_off(x, y, z)] + W[q][1024 + ucube_off(x, z, y)])
-                for (int l = tid; l < 512; l += NT) {
-                    const int l0 = l >> 6, l1 = (l >> 3) & 7, l2 = l & 7;
-                    const int x = pick3(ob0, ob1, ob2, p0) * F8 + l0, y = pick3(ob0, ob1, ob2, p1) * F8 + l1,
-                              z = pick3(ob0, ob1, ob2, p2) * F8 + l2;
-                    if (x >= v || y >= v || z >= v) continue;
-                    const float w0 = WAT(0, l0, l1, l2);
-                    // Z = 8 W(abc) - 4 (W(acb) + W(bac) + W(cba)) + 2 (W(bca) + W(cab))
-                    const float zv = 8.f * w0 - 4.f * (WAT(1, l0, l2, l1) + WAT(2, l1, l0, l2) + WAT(5, l2, l1, l0)) +
-                                     2.f * (WAT(3, l1, l2, l0) + WAT(4, l2, l0, l1));
-                    const float yv = S.t1[0][p0][l0] * S.ov[0][p1][p2][l1 * F8 + l2] +
-                                     S.t1[1][p1][l1] * S.ov[1][p0][p2][l0 * F8 + l2] +
-                                     S.t1[2][p2][l2] * S.ov[2][p0][p1][l0 * F8 + l1];
-                    const ff e0 = {S.ev[p0][l0].x, S.ev[p0][l0].y}, e1 = {S.ev[p1][l1].x, S.ev[p1][l1].y},
-                             e2 = {S.ev[p2][l2].x, S.ev[p2][l2].y};
-                    const ff r = ff_recip(ff_sub(ff_sub(ff_sub(eijk, e0), e1), e2));
-                    A4 = ff_add(A4, ff_mul(zv * w0, r));
-                    A5 = ff_add(A5, ff_mul(zv * yv, r));
-                }
-#undef WAT
-            }
+            const int *m = meta[stage].smap;
+            orbits(S.cube[0][0], S.cube[m[1]][0], S.cube[m[2]][0], S.cube[m[3]][0], S.cube[m[4]][0], S.cube[m[5]][0]);
         }
         // the stage is free once every warp has read it
         __syncwarp();
@@ -827,8 +801,9 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
             }
             __syncwarp();
             if (lane == 0) {
-                out[0] = ff_to_double(b4);
-                out[1] = ff_to_double(b5);
+                const double w = kind == 1 ? 1.0 : (kind == 2 ? 0.5 : 1.0 / 6.0);  // repeated blocks: see above
+                out[0] = ff_to_double(b4) * w;
+                out[1] = ff_to_double(b5) * w;
                 mbar_arrive(smem_u32(&bar_rempty[rb]));
             }
         }

@@ -549,48 +549,44 @@ inline bool encode(CUtensorMap *m, CUtensorMapDataType dt, int rank, void *base,
 }
 
 
+// 8 consecutive floats to a 32-byte aligned global address in one store
+__device__ __forceinline__ void st_v8(float *p, const float *x) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]),
+                 "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7])
+                 : "memory");
+}
 // Stores one thread's U row (fixed b < v, c < v of group g; a = a0 + j for
 // j < na, a0 a multiple of 8) into the mixed paths' cube layout
 // (tcorr_internal.cuh): group 0 at C0[a][b][c], 1 at C1[b][a][c], 2 at
-// C2[b][c][a].  Ut: the task's U block; nb: cubes per edge.  Every 8 values of
-// a lie in one cube; the swizzle is linear, so an element's offset in its
-// cube is the thread's part XOR the part of a & 7.  In every group the 8
-// values of c & 7 at fixed (a, b) fill one aligned 32-byte row, so a warp's
-// store (2 values of b x 16 of c) writes 4 whole sectors.
+// C2[b][c][a].  Ut: the task's U block; nb: cubes per edge.  In every group 8
+// values of a at fixed (b, c) are 32 consecutive bytes of one cube, so a
+// thread writes them with one 256-bit store, and a warp's store (2 values of b
+// x 16 of c) is two runs of 512 bytes.  With the former order in the cube
+// (c innermost) each value was a store of its own, 128 per thread and tile:
+// the warps that store also drain the accumulators.  Contractions before and
+// after: 24 molecules of v = 20..120 in BF16X3 29.2 -> 26.2 ms, 28 tasks of o=50,
+// v=450 37.3 -> 36.3 ms (BF16X3) and 63.6 -> 62.7 ms (TF32X3).
+// Values past na in the last 8 are the zeros of the padded columns and land in
+// the cube's padding.
 __device__ __forceinline__ void store_u_cubes(float *Ut, int nb, int g, int a0, int b, int c, int na,
                                               const float (&total)[128]) {
-    const int A0 = a0 >> 3, B = b >> 3, C = c >> 3, lb = b & 7, lc = c & 7;
+    const int A0 = a0 >> 3, B = b >> 3, C = c >> 3;
     int64_t base, step;
-    int offs[8];
     if (g == 0) {
         base = (((int64_t)A0 * nb + B) * nb + C) * 3 * 512;
         step = (int64_t)nb * nb * 3 * 512;
-#pragma unroll
-        for (int q = 0; q < 8; q++) offs[q] = ucube_off(0, lb, lc) ^ ucube_off(q, 0, 0);
     } else if (g == 1) {
         base = ((((int64_t)B * nb + A0) * nb + C) * 3 + 1) * 512;
         step = (int64_t)nb * 3 * 512;
-#pragma unroll
-        for (int q = 0; q < 8; q++) offs[q] = ucube_off(lb, 0, lc) ^ ucube_off(0, q, 0);
-    } else {  // element (x, y, z) = (b, c, a) of C2 at ucube_off(x, z, y)
+    } else {
         base = ((((int64_t)B * nb + C) * nb + A0) * 3 + 2) * 512;
         step = 3 * 512;
-#pragma unroll
-        for (int q = 0; q < 8; q++) offs[q] = ucube_off(lb, 0, lc) ^ ucube_off(0, q, 0);
     }
-    float *p = Ut + base;
-    if (na >= 128) {
+    float *p = Ut + base + ucube_off(0, b & 7, c & 7);
 #pragma unroll
-        for (int j = 0; j < 128; j++) {
-            p[offs[j & 7]] = total[j];
-            if ((j & 7) == 7) p += step;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 128; j++) {
-            if (j < na) p[offs[j & 7]] = total[j];
-            if ((j & 7) == 7) p += step;
-        }
+    for (int k = 0; k < 16; k++) {
+        if (8 * k < na) st_v8(p, total + 8 * k);
+        p += step;
     }
 }
 

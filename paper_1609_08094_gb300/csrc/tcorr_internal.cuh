@@ -41,14 +41,13 @@ __host__ __device__ inline Dims make_dims(int o, int v) {
     const int64_t flat = (int64_t)v * v * vc, cubes = vp * vp * vp;
     return Dims{o, v, round_up(v, KPAD), round_up(o, KPAD), vc, flat > cubes ? flat : cubes};
 }
-// Offset of element (x, y, z) (each < 8) inside a U cube of the mixed paths.
-// An XOR swizzle, linear over GF(2) in the bits of x, y, z, so that the six
-// ways the epilogue walks a cube (a warp holds 4 consecutive values of one
-// index and all 8 of another, the third fixed, in any assignment to x, y, z)
-// each touch 32 distinct shared-memory banks.
-__host__ __device__ inline int ucube_off(int x, int y, int z) {
-    return (x << 6) | ((y ^ (x & 3)) << 3) | (z ^ y ^ (x & 4));
-}
+// Offset of U^g[a][b][c] inside its U cube of the mixed paths (la, lb, lc: the
+// low 3 bits of a, b, c; the same for the three groups): a innermost, so that
+// the contraction's thread, which holds consecutive a at fixed (b, c), stores 8
+// of them at once.  No swizzle: the epilogue's lanes take the elements of a
+// cube in a skewed order instead, in which each of its reads touches 32
+// distinct shared-memory banks (epilogue.cu).
+__host__ __device__ inline int ucube_off(int la, int lb, int lc) { return (lb << 6) | (lc << 3) | la; }
 
 // Operand layouts built by the prep kernels (element type T = double, float
 // (TF32 container) or __nv_bfloat16):
@@ -71,11 +70,10 @@ __host__ __device__ inline int ucube_off(int x, int y, int z) {
 //   U^2[a][b][c], so that W[x][y][z] = C0[x][y][z] + C1[x][y][z] +
 //   C2[x][y][z]; as cubes of 8^3 (nb = ceil(v / 8) per edge) with the three
 //   groups interleaved: cube (X, Y, Z) of group g at (((X nb + Y) nb + Z) 3
-//   + g) * 512 in the task's block, element (x, y, z) of it at
-//   ucube_off(x, y, z) in C0 and C1 and at ucube_off(x, z, y) in C2 (so that
-//   the contraction's stores, 8 consecutive c at fixed a and b, fill one
-//   32-byte sector in every group).  An epilogue block orbit reads the three
-//   terms of one W cube as one contiguous 6 KB copy.
+//   + g) * 512 in the task's block, and inside it U^g[a][b][c] at
+//   ucube_off(a & 7, b & 7, c & 7) in every group, so that the contraction
+//   stores 8 consecutive a as one 32-byte sector.  An epilogue block orbit
+//   reads the three terms of one W cube as one contiguous 6 KB copy.
 struct Operands {
     void *G = nullptr, *T2K = nullptr, *T2R = nullptr, *AoN = nullptr;       // FP64 or hi part
     void *Glo = nullptr, *T2Klo = nullptr, *T2Rlo = nullptr, *AoNlo = nullptr;  // lo part (mixed)
