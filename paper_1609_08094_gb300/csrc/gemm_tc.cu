@@ -334,43 +334,131 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_kernel(const __grid_co
 //    issued MMAs, and a producer that aborted lets its copies in flight land.
 // Teardown: a cluster barrier (every role of both CTAs ends after bounded
 // waits), then both CTAs free the pair's tensor memory.
+constexpr int PAIR_THREADS = TC_THREADS + 32;  // warp 10: scheduler
 constexpr int PAIR_HEMPTY_ARRIVALS = 2 * (EPI_THREADS / 32);
 constexpr int PAIR_ROW = 2 * ROW_BYTES;   // one K block (two chunks) per shared-memory row, 128-byte swizzle
 constexpr int PAIR_A = BM * PAIR_ROW;     // 16 KB per A plane
+constexpr int PACK_ROWS = 16;             // rows of a B box of packed columns
+constexpr int PACK_BOXES = BN / 2 / PACK_ROWS;  // boxes per CTA and plane at N = 256
+constexpr int PACK_MAX_V = 256;           // packed columns up to this v (see tc_fill_desc)
+constexpr int PACK_BOX_BYTES = PACK_ROWS * PAIR_ROW;
 
-struct PairItem {
-    Item it;
-    bool empty;  // this CTA's tile index lies past the group's tile list
+struct PairCache {
+    SegCache s;
+    const PackRun *runs;
+    const PackEnt *ents;
+    int nrun, r, r_end;  // cached run and the unit after its last
+    PackRun run;
 };
-__device__ __forceinline__ PairItem decode_pair(const Wave &w, int64_t it, SegCache &c, uint32_t rank) {
-    seg_update(w, it, c);
+__device__ __forceinline__ void pair_reset(PairCache &c) { seg_reset(c.s); }
+struct PairItem {
+    int bt, ct;          // this CTA's pair tile
+    int p, q;            // the A side's slices
+    int N;               // columns of the MMAs
+    int pass0, ncol;     // first column (of a, or of the run's packed columns) and valid columns
+    int tb, g, s;        // not packed: task of the segment, group and its s
+    int ent0;            // packed: first entry of the run
+    bool packed;         // entries of a run
+    bool boxes;          // several entries: B in 16-row boxes
+    bool empty;          // this CTA's tile index lies past the group's tile list
+    bool diag;           // i = j = k: no work
+};
+__device__ __forceinline__ PairItem decode_pair(const Wave &w, int64_t it, PairCache &c, uint32_t rank) {
+    const bool fresh = c.s.si < 0 || it >= c.s.end;
+    seg_update(w, it, c.s);
     PairItem r;
-    const int npt = c.nbt * c.nct;
+    const InstDesc &d = *c.s.d;
+    const int npt = c.s.nbt * c.s.nct;
     const int npair = (npt + 1) / 2;
-    int64_t x = it - c.begin;
-    r.it.n = (int)(x % c.npass);  // N pass fastest, then group, then tile pair (as decode)
-    x /= c.npass;
-    r.it.g = (int)(x % 3);
-    x /= 3;
-    const int t = (int)(x % npair) * 2 + (int)rank;
-    r.it.tb = (int)(x / npair);
-    r.empty = t >= npt;
-    r.it.bt = r.empty ? c.nbt : t / c.nct;  // past the list: b >= v, all TMA fill
-    r.it.ct = r.empty ? 0 : t % c.nct;
-    if (r.it.tb != c.tcached) {
-        const int *tk = c.d->tasks + 3 * (c.task0 + r.it.tb);
-        c.ti = tk[0];
-        c.tj = tk[1];
-        c.tk = tk[2];
-        c.tcached = r.it.tb;
+    int tp;
+    if (fresh) {
+        const Seg &sg = w.segs[c.s.si];
+        c.runs = sg.runs;
+        c.ents = sg.ents;
+        c.nrun = sg.nrun;
+        c.r = 0;
+        c.r_end = -1;
     }
-    const int i = c.ti, j = c.tj, k = c.tk;
-    r.it.diag = (i == j && j == k);
-    if (r.it.g == 0) { r.it.s = i; r.it.p = j; r.it.q = k; }
-    else if (r.it.g == 1) { r.it.s = j; r.it.p = i; r.it.q = k; }
-    else { r.it.s = k; r.it.p = i; r.it.q = j; }
+    r.packed = c.nrun != 0;
+    r.boxes = false;
+    if (r.packed) {
+        const int x = (int)(it - c.s.begin);
+        if (x >= c.r_end) {  // units only grow: search forward
+            int lo = c.r, hi = c.nrun - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (c.runs[mid].unit0 <= x) lo = mid; else hi = mid - 1;
+            }
+            c.r = lo;
+            c.run = c.runs[lo];
+            c.r_end = c.run.unit0 + npair * c.run.npass;
+        }
+        const int local = x - c.run.unit0, n = local % c.run.npass;
+        tp = local / c.run.npass;
+        r.boxes = c.run.nent > 1;
+        if (r.boxes) {
+            const int cols = c.run.nent * d.packw;
+            const int width = ((cols + c.run.npass - 1) / c.run.npass + 31) / 32 * 32;
+            r.pass0 = n * width;
+            r.ncol = min(width, cols - r.pass0);
+            r.N = (r.ncol + 31) / 32 * 32;
+        } else {  // v <= 256: one pass
+            r.pass0 = 0;
+            r.ncol = d.dm.v;
+            r.N = (r.ncol + 15) / 16 * 16;
+        }
+        r.ent0 = c.run.ent0;
+        r.p = c.run.p;
+        r.q = c.run.q;
+        r.tb = r.g = r.s = 0;
+        r.diag = false;  // the tables hold no group of a task i = j = k
+    } else {
+        int64_t x = it - c.s.begin;
+        const int n = (int)(x % c.s.npass);  // N pass fastest, then group, then tile pair (as decode)
+        x /= c.s.npass;
+        r.g = (int)(x % 3);
+        x /= 3;
+        tp = (int)(x % npair);
+        r.tb = (int)(x / npair);
+        if (r.tb != c.s.tcached) {
+            const int *tk = d.tasks + 3 * (c.s.task0 + r.tb);
+            c.s.ti = tk[0];
+            c.s.tj = tk[1];
+            c.s.tk = tk[2];
+            c.s.tcached = r.tb;
+        }
+        const int i = c.s.ti, j = c.s.tj, k = c.s.tk;
+        r.diag = (i == j && j == k);
+        r.s = r.g == 0 ? i : (r.g == 1 ? j : k);
+        r.p = r.g == 0 ? j : i;
+        r.q = r.g == 2 ? j : k;
+        r.pass0 = n * d.brows;
+        r.ncol = min(d.brows, d.dm.v - r.pass0);
+        r.N = (r.ncol + 15) / 16 * 16;
+        r.ent0 = 0;
+    }
+    const int t = tp * 2 + (int)rank;
+    r.empty = t >= npt;
+    r.bt = r.empty ? c.s.nbt : t / c.s.nct;  // past the list: b >= v, all TMA fill
+    r.ct = r.empty ? 0 : t % c.s.nct;
     return r;
 }
+// What the roles of a CTA need of an item, written by its scheduler warp.
+struct PairSlot {
+    const InstDesc *d;
+    float *U;               // the segment's U (packed), or the task's
+    int64_t ug3;
+    int end;                // no more items
+    int o, v, kv, ko, kind;
+    int p, q, N, cb, cc;    // A slices, columns, first b and c of this CTA's tile
+    uint32_t stage_tx;      // bytes of a stage, both CTAs'
+    int nbx, boxes;         // B copies per plane and stage; in 16-row boxes?
+    int pc, packed, empty;
+    int g, pass0, ncol;     // not packed: group and columns of a
+    int2 box[PACK_BOXES];   // (s, first a) of the B copies, s = -1 past the valid columns
+    int2 ent[BN / 8];       // packed: (tbg, a) of columns 8 k .. 8 k + 7, a = 2^20 for none
+};
+constexpr int PAIR_SLOTS = 4;
 // abort both CTAs of the pair and raise the device error flag
 __device__ __forceinline__ void fail_pair(volatile int *abort_flag, uint32_t peer_abort_cl, int *err, int code) {
     *abort_flag = 1;
@@ -383,14 +471,15 @@ __device__ __forceinline__ void spin_ns(uint64_t ns) {
     }
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __grid_constant__ Wave wv) {
+__global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_tc_pair_kernel(const __grid_constant__ Wave wv) {
     extern __shared__ __align__(1024) uint8_t smem_dyn[];
     __shared__ __align__(8) uint64_t bar_full[MAX_STAGES], bar_empty[MAX_STAGES];
     __shared__ __align__(8) uint64_t bar_hfull[2], bar_hempty[2];
     __shared__ __align__(8) uint64_t bar_fin;
     __shared__ uint32_t tmem_holder;
     __shared__ volatile int abort_sh;
-    __shared__ SegCache ecache[EPI_THREADS / 32];
+    __shared__ __align__(8) uint64_t bar_sfull[PAIR_SLOTS], bar_sempty[PAIR_SLOTS];
+    __shared__ PairSlot slots[PAIR_SLOTS];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank(), cid = cluster_id(), ncl = cluster_count();
@@ -411,6 +500,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
             mbar_init(smem_u32(&bar_hempty[b]), PAIR_HEMPTY_ARRIVALS);
         }
         mbar_init(smem_u32(&bar_fin), 1);
+        for (int n = 0; n < PAIR_SLOTS; n++) {
+            mbar_init(smem_u32(&bar_sfull[n]), 1);
+            mbar_init(smem_u32(&bar_sempty[n]), (leader ? 2 : 1) + EPI_THREADS / 32);  // producer, drains, MMA issuer
+        }
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -436,29 +529,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
         for (int s = 0; s < MAX_STAGES; s++) last_phase[s] = -1;
         bool ok = true;
         bool inject = wv.inject_stall != 0 && cid == 0 && leader;
-        SegCache sc;
-        seg_reset(sc);
-        for (int64_t it = cid; it < wv.n_gemm && ok; it += ncl) {
-            const PairItem pw = decode_pair(wv, it, sc, rank);
-            const Item &w = pw.it;
-            if (uni((int)w.diag)) continue;
-            const InstDesc *d = uni(sc.d);
-            const int o = uni(d->dm.o), kv = uni(d->kv), ko = uni(d->ko);
-            const int kch = uni(ROW_BYTES / (d->kind == 1 ? 4 : 2));
-            const int s = uni(w.s), pp = uni(w.p), q = uni(w.q);
-            const int nvalid = min(d->brows, d->dm.v - w.n * d->brows);
-            const int N = (nvalid + 15) / 16 * 16;
-            const int cb = uni(w.bt * d->pb), cc = uni(w.ct * d->pc), ca = uni(w.n * d->brows + (int)rank * (N / 2));
-            const uint32_t stage_tx = uni(d->stage_tx);  // both CTAs' bytes
+        for (uint32_t n = 0; ok; n++) {
+            const PairSlot &sl = slots[n % PAIR_SLOTS];
+            if (!wait_warp(smem_u32(&bar_sfull[n % PAIR_SLOTS]), (n / PAIR_SLOTS) & 1u, &abort_sh)) {
+                if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_FULL);
+                ok = false;
+                break;
+            }
+            if (uni(sl.end)) break;
+            const InstDesc *d = uni(sl.d);
+            const int o = uni(sl.o), kv = uni(sl.kv), ko = uni(sl.ko), kch = uni(sl.kind) == 1 ? 16 : 32;
+            const int pp = uni(sl.p), q = uni(sl.q), cb = uni(sl.cb), cc = uni(sl.cc);
+            const int nbx = uni(sl.nbx);
+            const bool boxes = uni(sl.boxes) != 0;
+            const uint32_t stage_tx = uni(sl.stage_tx);
+            int bs[PACK_BOXES], ba[PACK_BOXES];
+#pragma unroll
+            for (int b = 0; b < PACK_BOXES; b++) {
+                bs[b] = uni(sl.box[b].x);
+                ba[b] = uni(sl.box[b].y);
+            }
+            if (lane == 0) mbar_arrive(smem_u32(&bar_sempty[n % PAIR_SLOTS]));
             for (int seg = 0; seg < 4 && ok; seg++) {
                 const int klen = seg < 2 ? kv : ko;
-                int amap, aslice, bmap, brow;
+                // B rows of box b: (bs[b] * bmul + badd) of [o o][v]
+                int amap, aslice, bmap, bmul, badd;
                 switch (seg) {
-                    case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; brow = s * o + pp; break;
-                    case 1: amap = MAP_G_SWP; aslice = pp; bmap = MAP_T2R; brow = s * o + q; break;
-                    case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; brow = q * o + s; break;
-                    default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; brow = pp * o + s; break;
+                    case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; bmul = o; badd = pp; break;
+                    case 1: amap = MAP_G_SWP; aslice = pp; bmap = MAP_T2R; bmul = o; badd = q; break;
+                    case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; bmul = 1; badd = q * o; break;
+                    default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; bmul = 1; badd = pp * o; break;
                 }
+                if (boxes) bmap += MAP_T2R_PK - MAP_T2R;
                 // two chunks per stage; the second segment of a kind with an odd chunk
                 // count gives its first chunk to the block that the first one left
                 // half full (a stage of its own: the half that is not used is the next
@@ -481,8 +583,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
                         if (!inject) {
                             tma_load_4d_pair(sA, &d->maps[amap][0], full_l, k0, cc, cb, aslice);
                             tma_load_4d_pair(sAl, &d->maps[amap][1], full_l, k0, cc, cb, aslice);
-                            tma_load_3d_pair(sB, &d->maps[bmap][0], full_l, k0, ca, brow);
-                            tma_load_3d_pair(sBl, &d->maps[bmap][1], full_l, k0, ca, brow);
+                            if (!boxes) {
+                                tma_load_3d_pair(sB, &d->maps[bmap][0], full_l, k0, ba[0], bs[0] * bmul + badd);
+                                tma_load_3d_pair(sBl, &d->maps[bmap][1], full_l, k0, ba[0], bs[0] * bmul + badd);
+                            } else {
+#pragma unroll
+                                for (int b = 0; b < PACK_BOXES; b++) {
+                                    if (b < nbx) {
+                                        // past the valid columns: a row past the tensor, zero fill
+                                        const int brow = bs[b] < 0 ? o * o : bs[b] * bmul + badd;
+                                        tma_load_3d_pair(sB + b * PACK_BOX_BYTES, &d->maps[bmap][0], full_l, k0, ba[b], brow);
+                                        tma_load_3d_pair(sBl + b * PACK_BOX_BYTES, &d->maps[bmap][1], full_l, k0, ba[b], brow);
+                                    }
+                                }
+                            }
                         }
                     }
                     __syncwarp();
@@ -524,19 +638,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
             rg.phase = 0;
             rg.hblk = 0;
             const uint32_t tm = uni(tmem);
-            SegCache sc;
-            seg_reset(sc);
-            for (int64_t it = cid; it < wv.n_gemm; it += ncl) {
-                const PairItem pw = decode_pair(wv, it, sc, rank);
-                const Item &w = pw.it;
-                if (uni((int)w.diag)) continue;
-                const InstDesc *d = uni(sc.d);
-                const int kv = uni(d->kv), ko = uni(d->ko), kind = uni(d->kind);
-                const int v = uni(d->dm.v), o = uni(d->dm.o), kch = ROW_BYTES / (kind == 1 ? 4 : 2);
+            for (uint32_t n = 0;; n++) {
+                const PairSlot &sl = slots[n % PAIR_SLOTS];
+                if (!wait_warp(smem_u32(&bar_sfull[n % PAIR_SLOTS]), (n / PAIR_SLOTS) & 1u, &abort_sh)) {
+                    if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_FULL);
+                    break;
+                }
+                if (uni(sl.end)) break;
+                const int kv = uni(sl.kv), ko = uni(sl.ko), kind = uni(sl.kind), N = uni(sl.N);
+                const int v = uni(sl.v), o = uni(sl.o), kch = kind == 1 ? 16 : 32;
+                if (lane == 0) mbar_arrive(smem_u32(&bar_sempty[n % PAIR_SLOTS]));
                 // the last chunk of a segment holds one K step of data (half a chunk) or two
                 const bool dh = v - (kv - 1) * kch <= kch / 2, lh = o - (ko - 1) * kch <= kch / 2;
-                const int nvalid = uni(min(d->brows, v - w.n * d->brows));
-                const int N = (nvalid + 15) / 16 * 16;
                 const uint32_t fmt = kind == 1 ? 2u : 1u;
                 const uint32_t idesc = idesc_m | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17);
                 int code = 0;
@@ -557,6 +670,80 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
             }
             __syncwarp();
         }
+    } else if (warp == 2 + EPI_THREADS / 32) {
+        // scheduler: decodes this CTA's items ahead of the other roles
+        PairCache pc;
+        pair_reset(pc);
+        uint32_t n = 0;
+        bool ok = true;
+        for (int64_t it = cid; ok; it += ncl) {
+            const bool end = it >= wv.n_gemm;
+            PairItem w;
+            if (!end) {
+                w = decode_pair(wv, it, pc, rank);
+                if (w.diag) continue;
+            }
+            PairSlot &sl = slots[n % PAIR_SLOTS];
+            if (n >= PAIR_SLOTS &&
+                !wait_warp(smem_u32(&bar_sempty[n % PAIR_SLOTS]), (n / PAIR_SLOTS - 1) & 1u, &abort_sh)) {
+                if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_EMPTY);
+                ok = false;
+                break;
+            }
+            if (!end) {
+                const InstDesc &d = *pc.s.d;
+                if (lane == 0) {
+                    sl.d = &d;
+                    sl.ug3 = 3 * d.dm.ug;
+                    sl.U = static_cast<float *>(wv.U) + pc.s.u_off + w.tb * (3 * d.dm.ug);
+                    sl.o = d.dm.o;
+                    sl.v = d.dm.v;
+                    sl.kv = d.kv;
+                    sl.ko = d.ko;
+                    sl.kind = d.kind;
+                    sl.p = w.p;
+                    sl.q = w.q;
+                    sl.N = w.N;
+                    sl.cb = w.bt * d.pb;
+                    sl.cc = w.ct * d.pc;
+                    sl.nbx = w.boxes ? w.N / (2 * PACK_ROWS) : 1;
+                    sl.stage_tx = w.boxes ? 2u * (2u * PAIR_A + 2u * (uint32_t)(w.N / (2 * PACK_ROWS) * PACK_BOX_BYTES))
+                                          : d.stage_tx;
+                    sl.boxes = w.boxes;
+                    sl.pc = d.pc;
+                    sl.packed = w.packed;
+                    sl.empty = w.empty;
+                    sl.g = w.g;
+                    sl.pass0 = w.pass0;
+                    sl.ncol = w.ncol;
+                }
+                if (!w.boxes) {
+                    if (lane == 0)
+                        sl.box[0] = make_int2(w.packed ? pc.ents[w.ent0].s : w.s, w.pass0 + (int)rank * (w.N / 2));
+                } else if (lane < PACK_BOXES) {
+                    const int x = (int)rank * (w.N / 2) + PACK_ROWS * lane;  // column in the pass
+                    int2 e = make_int2(-1, 0);
+                    if (x < w.ncol && lane < w.N / (2 * PACK_ROWS)) {
+                        const int col = w.pass0 + x, m = col / d.packw;
+                        e = make_int2(pc.ents[w.ent0 + m].s, col - m * d.packw);
+                    }
+                    sl.box[lane] = e;
+                }
+                if (w.packed) {
+                    int2 e = make_int2(0, 1 << 20);
+                    if (8 * lane < w.ncol) {
+                        const int col = w.pass0 + 8 * lane, m = col / d.packw;
+                        e = make_int2(pc.ents[w.ent0 + m].tbg, col - m * d.packw);
+                    }
+                    sl.ent[lane] = e;
+                }
+            }
+            if (lane == 0) sl.end = end;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bar_sfull[n % PAIR_SLOTS]));
+            if (end) break;
+            n++;
+        }
     } else {
         const int wq = warp & 3;
         const int half = (warp - 2) >> 2;
@@ -564,26 +751,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
         const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
         uint32_t hblk = 0;
         bool ok = true;
-        SegCache &cs = ecache[warp - 2];
-        if (lane == 0) seg_reset(cs);
-        __syncwarp();
-        for (int64_t it = cid; it < wv.n_gemm && ok; it += ncl) {
-            SegCache sc = cs;
-            const PairItem pw = decode_pair(wv, it, sc, rank);
-            const Item &w = pw.it;
-            __syncwarp();
-            if (lane == 0) cs = sc;
-            __syncwarp();
-            if (w.diag) continue;
-            const InstDesc &d = *sc.d;
-            const int64_t u_seg = sc.u_off;
-            const int v = d.dm.v;
-            const int nhb = (num_chunks(d) + d.kb - 1) / d.kb;
-            const int lb = row / d.pc, lc = row % d.pc;
-            const int pass0 = w.n * d.brows, pass_end = min(v, pass0 + d.brows);
-            const int N = (pass_end - pass0 + 15) / 16 * 16;
-            const int wh = N > 128 ? 128 : (N > 64 ? 64 : 32);
-            const int nld = wh / 32;
+        for (uint32_t n = 0; ok; n++) {
+            // the item's fields stay in the slot until the store: in registers
+            // they would compete with the 128-column running total
+            const PairSlot &sl = slots[n % PAIR_SLOTS];
+            if (!wait_warp(smem_u32(&bar_sfull[n % PAIR_SLOTS]), (n / PAIR_SLOTS) & 1u, &abort_sh)) {
+                if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_FULL);
+                break;
+            }
+            if (sl.end) break;
+            // the two warps of a lane quarter split the N columns, 32 at a time
+            const int nld = (sl.N / 2 + 31) / 32, nhb = sl.kv + sl.ko;
             float total[128];
 #pragma unroll
             for (int j = 0; j < 128; j++) total[j] = 0.f;
@@ -599,7 +777,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
                 for (int c4 = 0; c4 < 4; c4++) {
                     if (c4 < nld) {
                         uint32_t r[16], r2[16];
-                        const uint32_t ta = tmem + lane_off + buf * (uint32_t)BN + (uint32_t)(half * wh + c4 * 32);
+                        const uint32_t ta = tmem + lane_off + buf * (uint32_t)BN + (uint32_t)(half * nld * 32 + c4 * 32);
                         tc_ld16(ta, r);
                         tc_ld16(ta + 16, r2);
                         tc_wait_ld();
@@ -618,13 +796,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_pair_kernel(const __gr
                 if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_TMEM);
                 break;
             }
-            if (pw.empty) continue;
-            const int b = w.bt * d.pb + lb, c = w.ct * d.pc + lc;
-            if (b < v && c < v) {
-                const int a0 = pass0 + half * wh;  // a multiple of 8
-                float *Ut = static_cast<float *>(wv.U) + u_seg + (int64_t)w.tb * 3 * d.dm.ug;
-                store_u_cubes(Ut, (v + 7) >> 3, w.g, a0, b, c, min(wh, pass_end - a0), total);
+            if (!sl.empty) {
+                const int v = sl.v, pc = sl.pc;
+                const int b = sl.cb + row / pc, c = sl.cc + row % pc;
+                const int nb = (v + 7) >> 3;
+                if (sl.packed) {
+                    // 8 columns at a time: their entry's task and group, and a
+                    const int B = b >> 3, C = c >> 3;
+                    const bool in = b < v && c < v;
+                    const int64_t ug3 = sl.ug3;
+                    float *Ui = sl.U + ucube_off(0, b & 7, c & 7);
+                    const int2 *ent = sl.ent + half * nld * 4;
+#pragma unroll
+                    for (int k = 0; k < 16; k++) {
+                        if (k < nld * 4) {
+                            const int2 e = ent[k];
+                            const int g = e.x & 3, a = e.y, A = a >> 3;
+                            if (in && a < v) {
+                                const int cube = g == 0 ? (A * nb + B) * nb + C
+                                                        : (g == 1 ? (B * nb + A) * nb + C : (B * nb + C) * nb + A);
+                                st_v8(Ui + (e.x >> 2) * ug3 + (cube * 3 + g) * 512, total + 8 * k);
+                            }
+                        }
+                    }
+                } else if (b < v && c < v) {
+                    const int a0 = sl.pass0 + half * nld * 32;  // a multiple of 8
+                    store_u_cubes(sl.U, nb, sl.g, a0, b, c, min(nld * 32, sl.pass0 + sl.ncol - a0), total);
+                }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bar_sempty[n % PAIR_SLOTS]));
         }
     }
     tc_fence_before();
@@ -672,16 +873,19 @@ cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int 
     // width rounded to 16, the peer's half starting at N / 2, a multiple of 8)
     const int wq = pair ? 32 : 16;
     d.brows = round_up((v + d.npass - 1) / d.npass, wq);
+    // SM pairs, v <= PACK_MAX_V: the groups that share (p, q) side by side in passes of up to 256 columns
+    d.packw = pair && v <= PACK_MAX_V ? round_up(v, PACK_ROWS) : 0;
     d.kv = (v + kch - 1) / kch;
     d.ko = (o + kch - 1) / kch;
     // bytes per stage: one CTA's (single SM), or both CTAs' (the pair's leader expects them all)
     d.stage_tx = pair ? (uint32_t)(2 * (2 * PAIR_A + 2 * (d.brows / 2) * PAIR_ROW))
                       : (uint32_t)(2 * A_BYTES + 2 * d.brows * ROW_BYTES);
+    const uint32_t brows = (uint32_t)(pair ? d.brows / 2 : d.brows);  // B box rows per CTA
+    if (d.packw) d.brows = BN;  // the ring holds passes of 256 packed columns
     const uint64_t V = v, O = o;
     // rows of a box: one K chunk (64 bytes), or on SM pairs a K block of two
     const CUtensorMapSwizzle swz = pair ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
     const uint32_t bk = (uint32_t)(pair ? 2 * kch : kch), bpc = (uint32_t)pc, bpb = (uint32_t)pb;
-    const uint32_t brows = (uint32_t)(pair ? d.brows / 2 : d.brows);  // B box rows per CTA
     void *hi[4] = {op.G, op.T2K, op.T2R, op.AoN};
     void *lo[4] = {op.Glo, op.T2Klo, op.T2Rlo, op.AoNlo};
     for (int part = 0; part < 2; part++) {
@@ -717,12 +921,18 @@ cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int 
             uint64_t st[2] = {dp * eb, V * dp * eb};
             uint32_t box[3] = {bk, brows, 1};
             if (!encode(&d.maps[MAP_T2R][part], dt, 3, src[2], dims, st, box, err, "T2R", swz)) return cudaErrorInvalidValue;
+            box[1] = PACK_ROWS;
+            if (d.packw && !encode(&d.maps[MAP_T2R_PK][part], dt, 3, src[2], dims, st, box, err, "T2R packed", swz))
+                return cudaErrorInvalidValue;
         }
         {   // AoN: (l, a, q*o+s)
             uint64_t dims[3] = {O, V, O * O};
             uint64_t st[2] = {lp * eb, V * lp * eb};
             uint32_t box[3] = {bk, brows, 1};
             if (!encode(&d.maps[MAP_AON][part], dt, 3, src[3], dims, st, box, err, "AoN", swz)) return cudaErrorInvalidValue;
+            box[1] = PACK_ROWS;
+            if (d.packw && !encode(&d.maps[MAP_AON_PK][part], dt, 3, src[3], dims, st, box, err, "AoN packed", swz))
+                return cudaErrorInvalidValue;
         }
     }
     return cudaSuccess;
@@ -732,6 +942,8 @@ int64_t tc_units_per_task(const InstDesc &d) {
     const int64_t tiles = (int64_t)d.nbt * d.nct;
     return (int64_t)3 * (d.pair ? (tiles + 1) / 2 : tiles) * d.npass;
 }
+
+int tc_tile_pairs(const InstDesc &d) { return (d.nbt * d.nct + 1) / 2; }
 
 cudaError_t tc_prepare(int) {
     static std::mutex mu;
@@ -761,7 +973,7 @@ static int pair_clusters(int sm_count) {
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)(sm_count / 2 * 2), 1, 1);
-    cfg.blockDim = dim3(TC_THREADS, 1, 1);
+    cfg.blockDim = dim3(PAIR_THREADS, 1, 1);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.attrs = at;
     cfg.numAttrs = 1;
@@ -792,7 +1004,7 @@ cudaError_t launch_ugemm_tc(int prec, int sm_count, const Wave &w, cudaStream_t 
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)(2 * ncl), 1, 1);
-    cfg.blockDim = dim3(TC_THREADS, 1, 1);
+    cfg.blockDim = dim3(PAIR_THREADS, 1, 1);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = st;
     cfg.attrs = at;

@@ -374,6 +374,95 @@ void fill_desc(Exec &ex, Problem &pb, int pbt) {
     }
 }
 
+// The first task (i <= j <= k, lexicographic) with index n of o orbitals
+static void task_at(int o, int64_t n, int &i, int &j, int &k) {
+    for (i = 0;; i++) {
+        const int64_t m = (int64_t)(o - i) * (o - i + 1) / 2;
+        if (n < m) break;
+        n -= m;
+    }
+    for (j = i;; j++) {
+        const int64_t m = o - j;
+        if (n < m) break;
+        n -= m;
+    }
+    k = j + (int)n;
+}
+
+int64_t seg_units(const Problem &pb, Seg &sg, PackTabs &tabs) {
+    PackTabs::Of of;
+    of.run0 = tabs.runs.size();
+    of.ent0 = tabs.ents.size();
+    tabs.of.push_back(of);
+    const InstDesc &d = pb.desc;
+    if (!d.packw) return sg.ntb * pb.gemm_units;
+    // counting sort of the groups (s; p, q) of the tasks by (p, q).  Packed, the
+    // passes are 256 columns wide instead of v, so an SM takes in fewer A rows per
+    // product: with it and the scheduler warp of the pair kernel, o=13, v=131 in
+    // TF32X3 took 12.4 ms (15.8 before), o=10, v=70 1.03 ms (1.42) and 24 molecules
+    // of v = 20..120 28.0 ms (36.7).
+    const int o = pb.dm.o;
+    std::vector<int> at((size_t)o * o + 1, 0);
+    auto each = [&](auto f) {
+        int i, j, k;
+        task_at(o, sg.task0, i, j, k);
+        for (int tb = 0; tb < sg.ntb; tb++) {
+            if (i != k) {
+                f(tb, 0, i, j, k);
+                f(tb, 1, j, i, k);
+                f(tb, 2, k, i, j);
+            }
+            if (++k == o) {
+                if (++j == o) j = ++i;
+                k = j;
+            }
+        }
+    };
+    each([&](int, int, int, int p, int q) { at[(size_t)p * o + q + 1]++; });
+    // Side by side only where that saves passes: a run, where it saves an eighth
+    // of its own (else its groups one by one, with one B copy per plane instead
+    // of one per 16 columns); the segment, where it saves a quarter over all.
+    // In the other order (a tile pair's three groups together) two groups share
+    // each A slice, which counts for more with few entries per run or large v:
+    // 69 consecutive tasks of o=26, v=237 took 9.5 ms so and 9.9 ms in runs.
+    auto passes = [&](int n) { return (int)(((int64_t)n * d.packw + 255) / 256); };
+    int64_t npass = 0, nent = 0;
+    for (size_t m = 0; m < (size_t)o * o; m++) {
+        npass += std::min(at[m + 1], passes(at[m + 1]));
+        nent += at[m + 1];
+    }
+    if (4 * npass > 3 * nent) return sg.ntb * pb.gemm_units;
+    const int npair = tc_tile_pairs(d);
+    int64_t unit = 0;
+    for (size_t m = 0; m < (size_t)o * o; m++) {
+        const int n = at[m + 1], np = passes(n);
+        at[m + 1] += at[m];
+        if (n == 0) continue;
+        const bool side = 8 * np <= 7 * n;
+        for (int e = 0; e < (side ? 1 : n); e++) {
+            tabs.runs.push_back(PackRun{(int)unit, at[m] + e, side ? n : 1, side ? np : 1, (int)(m / o), (int)(m % o)});
+            unit += (int64_t)npair * (side ? np : 1);
+        }
+    }
+    tabs.ents.resize(of.ent0 + at[(size_t)o * o]);
+    each([&](int tb, int g, int s, int p, int q) {
+        tabs.ents[of.ent0 + at[(size_t)p * o + q]++] = PackEnt{tb * 4 + g, s};
+    });
+    sg.nrun = (int)(tabs.runs.size() - of.run0);
+    if (unit > 0x7fffffff) throw Fail{TCORR_EUNSUPPORTED, "too many work units in one wave"};
+    return unit;
+}
+
+void place_tabs(const PackTabs &tabs, std::vector<Seg> &segs, unsigned char *dst, const unsigned char *dev) {
+    const size_t rb = tabs.runs.size() * sizeof(PackRun);
+    if (rb) memcpy(dst, tabs.runs.data(), rb);
+    if (!tabs.ents.empty()) memcpy(dst + rb, tabs.ents.data(), tabs.ents.size() * sizeof(PackEnt));
+    for (size_t n = 0; n < segs.size(); n++) {
+        segs[n].runs = reinterpret_cast<const PackRun *>(dev) + tabs.of[n].run0;
+        segs[n].ents = reinterpret_cast<const PackEnt *>(dev + rb) + tabs.of[n].ent0;
+    }
+}
+
 Plan make_plan(const Exec &ex, const std::vector<Problem *> &pbs, const std::vector<Span> &spans) {
     Plan pl;
     WaveRec cur{0, 0, 0, 0, 0, 0};
@@ -406,10 +495,10 @@ Plan make_plan(const Exec &ex, const std::vector<Problem *> &pbs, const std::vec
             s.epi0 = cur.n_epi;
             s.red0 = cur.n_red;
             s.part_off = p_used;
-            pl.segs.push_back(s);
             cur.nseg++;
             cur.tc_brows = std::max(cur.tc_brows, pb.desc.brows);
-            cur.n_gemm += n * pb.gemm_units;
+            cur.n_gemm += seg_units(pb, s, pl.tabs);
+            pl.segs.push_back(s);
             cur.n_epi += n * pb.norb;
             cur.n_red += n;
             u_used += n * pb.u_task;
@@ -429,7 +518,8 @@ Plan make_plan(const Exec &ex, const std::vector<Problem *> &pbs, const std::vec
 void upload_plan(Exec &ex, Plan &pl, Seg *&d_segs, SumSpan *&d_spans) {
     const size_t seg_b = pl.segs.size() * sizeof(Seg);
     const size_t span_off = (seg_b + 255) / 256 * 256;
-    const size_t total = span_off + pl.sums.size() * sizeof(SumSpan);
+    const size_t tab_off = (span_off + pl.sums.size() * sizeof(SumSpan) + 255) / 256 * 256;
+    const size_t total = tab_off + pl.tabs.bytes();
     if ((int)pl.sums.size() > ex.sums_cap || total > ex.stage_cap) {
         CK(cudaStreamSynchronize(ex.stream));  // the old tables may still be in use
         if ((int)pl.sums.size() > ex.sums_cap) {
@@ -448,6 +538,7 @@ void upload_plan(Exec &ex, Plan &pl, Seg *&d_segs, SumSpan *&d_spans) {
         }
     }
     for (size_t n = 0; n < pl.sums.size(); n++) pl.sums[n].out = ex.d_sums + 3 * n;
+    place_tabs(pl.tabs, pl.segs, ex.h_stage + tab_off, ex.d_stage + tab_off);
     memcpy(ex.h_stage, pl.segs.data(), seg_b);
     memcpy(ex.h_stage + span_off, pl.sums.data(), pl.sums.size() * sizeof(SumSpan));
     CK(cudaMemcpyAsync(ex.d_stage, ex.h_stage, total, cudaMemcpyHostToDevice, ex.stream));
@@ -605,20 +696,32 @@ int tuned_pb(Exec &ex, Problem &pb) {
     Seg *d_seg = nullptr;
     dalloc(ex, d_one, sizeof(InstDesc));
     dalloc(ex, d_seg, sizeof(Seg));
+    unsigned char *d_tab = nullptr;
+    const size_t tab_cap = (size_t)n * 3 * (sizeof(PackRun) + sizeof(PackEnt));  // at most a run per group
+    dalloc(ex, d_tab, tab_cap);
+    Problem cp = pb;
     for (int cand : {8, 4, 16}) {
         InstDesc d = pb.desc;
         std::string msg;
         if (tc_fill_desc(d, pprec, pb.op, cand, TC_KB, ex.pair, msg) != cudaSuccess) continue;
-        Seg s{};
+        std::vector<Seg> sv(1);
+        Seg &s = sv[0];
         s.ntb = (int)n;
         s.task0 = first;
+        cp.desc = d;
+        cp.gemm_units = tc_units_per_task(d);
+        PackTabs tabs;
+        const int64_t units = seg_units(cp, s, tabs);
+        std::vector<unsigned char> ht(tabs.bytes() + 1);
+        place_tabs(tabs, sv, ht.data(), d_tab);
+        CK(cudaMemcpy(d_tab, ht.data(), tabs.bytes(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(d_one, &d, sizeof(InstDesc), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(d_seg, &s, sizeof(Seg), cudaMemcpyHostToDevice));
         Wave w{};
         w.descs = d_one;
         w.segs = d_seg;
         w.nseg = 1;
-        w.n_gemm = n * tc_units_per_task(d);
+        w.n_gemm = units;
         w.U = ex.U;
         w.err = ex.err;
         w.tc_brows = d.brows;
@@ -638,6 +741,7 @@ int tuned_pb(Exec &ex, Problem &pb) {
     cudaEventDestroy(e1);
     dfree(ex, d_one, sizeof(InstDesc));
     dfree(ex, d_seg, sizeof(Seg));
+    dfree(ex, d_tab, tab_cap);
     check_err_flag(ex);
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune_cache[key] = best;

@@ -142,7 +142,16 @@ struct WaveRec {
     int64_t n_gemm, n_epi, n_red;
     int tc_brows;  // largest tensor-core B tile of the wave's problems
 };
+// Tables of the packed segments (PackRun, PackEnt), in the order of the segments
+struct PackTabs {
+    struct Of { size_t run0 = 0, ent0 = 0; };  // a segment's first run and entry
+    std::vector<PackRun> runs;
+    std::vector<PackEnt> ents;
+    std::vector<Of> of;
+    size_t bytes() const { return runs.size() * sizeof(PackRun) + ents.size() * sizeof(PackEnt); }
+};
 struct Plan {
+    PackTabs tabs;
     std::vector<Seg> segs;
     std::vector<WaveRec> waves;
     std::vector<SumSpan> sums;  // span n sums into d_sums[3n .. 3n+2] (out set at upload)
@@ -184,6 +193,11 @@ size_t host_staging_bytes(const Dims &d);
 int model_pb(int v);
 void fill_desc(Exec &ex, Problem &pb, int pbt);
 Plan make_plan(const Exec &ex, const std::vector<Problem *> &pbs, const std::vector<Span> &spans);
+// Work units of the W contraction for the segment sg of pb's tasks; builds the
+// segment's tables when the problem's columns are packed.  One call per segment.
+int64_t seg_units(const Problem &pb, Seg &sg, PackTabs &tabs);
+// Copies the tables to dst (host) and points the segments at their device copy
+void place_tabs(const PackTabs &tabs, std::vector<Seg> &segs, unsigned char *dst, const unsigned char *dev);
 void upload_plan(Exec &ex, Plan &pl, Seg *&d_segs, SumSpan *&d_spans);
 void launch_plan(Exec &ex, const Plan &pl, const Seg *d_segs, const SumSpan *d_spans, cudaStream_t st);
 void check_err_flag(Exec &ex);

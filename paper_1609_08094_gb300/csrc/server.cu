@@ -214,6 +214,7 @@ void launch_wave(tcorr_server_s &s) {
     // segments (one per job) and the sums of the jobs that finish
     std::vector<Seg> segs;
     std::vector<SumSpan> sums;
+    PackTabs tabs;
     std::vector<Job *> finishing, members;
     WaveRec wr{0, 0, 0, 0, 0, 0};
     int64_t u_off = 0, p_off = 0;
@@ -229,10 +230,10 @@ void launch_wave(tcorr_server_s &s) {
         sg.epi0 = wr.n_epi;
         sg.red0 = wr.n_red;
         sg.part_off = p_off;
-        segs.push_back(sg);
         wr.nseg++;
         wr.tc_brows = std::max(wr.tc_brows, j->pb.desc.brows);
-        wr.n_gemm += take[n] * j->pb.gemm_units;
+        wr.n_gemm += seg_units(j->pb, sg, tabs);
+        segs.push_back(sg);
         wr.n_epi += take[n] * j->pb.norb;
         wr.n_red += take[n];
         u_off += take[n] * j->pb.u_task;
@@ -248,14 +249,18 @@ void launch_wave(tcorr_server_s &s) {
     RingSlot &r = s.ring[s.waves_issued % DEPTH];
     const size_t seg_b = segs.size() * sizeof(Seg);
     const size_t span_off = (seg_b + 255) / 256 * 256;
-    const size_t total = span_off + std::max<size_t>(1, sums.size()) * sizeof(SumSpan);
+    const size_t tab_off = (span_off + std::max<size_t>(1, sums.size()) * sizeof(SumSpan) + 255) / 256 * 256;
+    const size_t total = tab_off + tabs.bytes();
     if (total > r.cap) {  // the slot's previous wave has retired (ring discipline)
         dfree(ex, r.d_tab, r.cap);
         hfree(ex, r.h_tab);
-        dalloc(ex, r.d_tab, total);
-        halloc(ex, r.h_tab, total);
-        r.cap = total;
+        r.cap = 0;
+        const size_t cap = std::max<size_t>(total, (size_t)512 << 10);  // above a wave of 4096 tasks
+        dalloc(ex, r.d_tab, cap);
+        halloc(ex, r.h_tab, cap);
+        r.cap = cap;
     }
+    place_tabs(tabs, segs, r.h_tab + tab_off, r.d_tab + tab_off);
     memcpy(r.h_tab, segs.data(), seg_b);
     if (!sums.empty()) memcpy(r.h_tab + span_off, sums.data(), sums.size() * sizeof(SumSpan));
     CK(cudaMemcpyAsync(r.d_tab, r.h_tab, total, cudaMemcpyHostToDevice, ex.stream));

@@ -84,7 +84,8 @@ struct Operands {
 // a single handle has one, a batch one per problem.  Aligned like its tensor
 // maps (alignof(CUtensorMap)), so an array of them keeps every map aligned.
 struct InstDesc {
-    CUtensorMap maps[6][2];   // tensor-core operand maps [G, G swapped, T2K, T2K swapped, T2R, AoN][hi, lo]
+    CUtensorMap maps[8][2];   // tensor-core operand maps [G, G swapped, T2K, T2K swapped, T2R, AoN, and T2R, AoN in
+                              // 16-row boxes for packed columns][hi, lo]
     CUtensorMap emaps[3];     // mixed epilogue row maps for 4-row gathers: ovov 8x8 blocks, t1 rows, eps_v blocks
     Dims dm;
     int pb, pc;               // tensor-core pair tile: pb values of b x pc values of c (pb * pc = 128)
@@ -92,6 +93,7 @@ struct InstDesc {
     int kind;                 // split-precision operand type: 1 = TF32, 2 = BF16 hi + lo
     int pair;                 // tensor-core tiles on SM pairs (cta_group::2, M = 256)
     int nbt, nct, npass, kv, ko, brows;
+    int packw;                // SM pairs, packed columns (PackRun): columns per entry (v rounded to 16), 0: not packed
     uint32_t stage_tx;        // TMA bytes per pipeline stage
     int norb;                 // epilogue block orbits per task (cube edge 8)
     const int *oz_e;          // FP64 emulation: device [2] scale exponents of the A and B operand sides
@@ -106,6 +108,24 @@ struct InstDesc {
 static_assert(alignof(InstDesc) % 64 == 0 && sizeof(InstDesc) % alignof(InstDesc) == 0,
               "tensor maps need (at least) 64-byte alignment in every array element");
 
+// Packed columns of the SM-pair contraction.  The groups (s; p, q) of a
+// segment's tasks that share (p, q) read the same A rows (G[q], G[p], T2K[p],
+// T2K[q]) and differ only in the rows of B that their s selects, so they are
+// computed side by side as the columns of one GEMM: a run is one (p, q) with
+// its entries (one per group, in task order), each packw columns wide, cut
+// into passes of at most 256 columns; or a single group, v columns wide.  Units
+// of a run: tile pairs x passes, passes fastest.
+struct PackRun {
+    int unit0;                // first work unit of the run in its segment
+    int ent0, nent;           // entries
+    int npass;                // column passes
+    int p, q;
+};
+struct PackEnt {
+    int tbg;                  // (task index in the segment) * 4 + group
+    int s;
+};
+
 // A contiguous run of one instance's tasks inside one launch ("wave").
 // The prefix counts let every kernel find its segment by binary search.
 struct Seg {
@@ -117,6 +137,9 @@ struct Seg {
     int64_t epi0;             // prefix of epilogue items (task, block orbit)
     int64_t red0;             // prefix of tasks
     int64_t part_off;         // double offset of the segment's orbit partials [ntb][norb][2]
+    const PackRun *runs;      // packed columns: device tables (nrun runs), else NULL
+    const PackEnt *ents;
+    int nrun;
 };
 
 // last segment s with key(s) <= x (segments sorted by key, key(0) = 0)
@@ -193,7 +216,10 @@ bool tc_supported(int cc_major, int cc_minor);
 // the operand layouts in op; pb in {4, 8, 16}, kb in {1, 2}
 // pair: tiles on SM pairs (2-CTA clusters, M = 256; B boxes of brows / 2 rows)
 cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int kb, bool pair, std::string &err);
+// W-contraction work units of a segment of ntb tasks that is not packed; and
+// per column pass of a packed one (tile pairs)
 int64_t tc_units_per_task(const InstDesc &d);
+int tc_tile_pairs(const InstDesc &d);
 // sets the kernel attributes once per process (call before any stream capture)
 cudaError_t tc_prepare(int prec);
 
