@@ -85,6 +85,11 @@ __device__ __forceinline__ ff ff_mul(float x, ff r) {
     const float p = x * r.hi;
     return ff_fast(p, fmaf(x, r.lo, fmaf(x, r.hi, -p)));
 }
+// a * r: as above plus the product with a.lo
+__device__ __forceinline__ ff ff_mul2(ff a, ff r) {
+    const float p = a.hi * r.hi;
+    return ff_fast(p, fmaf(a.lo, r.hi, fmaf(a.hi, r.lo, fmaf(a.hi, r.hi, -p))));
+}
 __device__ __forceinline__ ff ff_of(double x) {  // x rounded to ~48 bits
     const float hi = (float)x;
     return {hi, (float)(x - (double)hi)};
@@ -382,8 +387,8 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
 // stage meanwhile.  The lanes of a warp take the elements of an orbit in a
 // skewed order that makes every read of W, t1 and ovov conflict-free (see the
 // compute warps), and the index arithmetic per element orbit is a handful of
-// precomputed offsets.  Orbits with repeated blocks take the same form.  With
-// swizzled cubes and an element-by-element loop for repeated blocks the kernel
+// precomputed offsets.  Orbits with repeated blocks read the six elements of an
+// element orbit once too.  With swizzled cubes and an element-by-element loop for repeated blocks the kernel
 // took 7.1 ms for 28 tasks of o=50, v=450 (6.6 ms now), 3.93 ms for o=13, v=131
 // (3.01) and 13.7 ms for 24 molecules of v = 20..120 (10.5), where most orbits
 // have repeated blocks.
@@ -447,7 +452,7 @@ struct EpiMeta {
     ff eijk;                     // e_i + e_j + e_k
     int ob[3];                   // blocks A <= B <= C
     int smap[6];                 // slot whose cubes hold slot s's data (the first with its block triple)
-    int kind;                    // 0: no more orbits, 1: three distinct blocks, 2: two equal, 6: all equal
+    int kind;                    // 0: no more orbits, 1: A < B < C, 2: A = B < C, 3: A < B = C, 4: A = B = C
     int v;                       // virtual orbitals of the problem
 };
 
@@ -476,6 +481,7 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
     __shared__ __align__(8) uint64_t bar_full[EPI_STAGES], bar_empty[EPI_STAGES];
     __shared__ __align__(8) uint64_t bar_rfull[2], bar_rempty[2];
     __shared__ __align__(16) float4 red[2][NT];
+    __shared__ short trip[156];
     __shared__ volatile int abort_sh;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -490,6 +496,18 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
         }
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (tid < 64) {  // sorted triples of 0..7 (120), then sorted pairs (36): la | lb << 3 | lc << 6
+        const int x = tid >> 3, y = tid & 7;
+        if (x <= y) {
+            // before (x, y): the triples with a smaller first, then second index
+            int n = 0, m = 0;
+            for (int k = 0; k < x; k++) { n += (8 - k) * (9 - k) / 2; m += 8 - k; }
+            for (int k = x; k < y; k++) n += 8 - k;
+            m += y - x;
+            for (int z = y; z < 8; z++) trip[n + z - y] = (short)(x | y << 3 | z << 6);
+            trip[120 + m] = (short)(x | y << 3);
+        }
     }
     __syncthreads();  // the last CTA-wide barrier: from here on the roles meet only at mbarriers
 
@@ -605,7 +623,7 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
                 m.ob[0] = ob0; m.ob[1] = ob1; m.ob[2] = ob2;
 #pragma unroll
                 for (int s = 0; s < 6; s++) m.smap[s] = smap[s];
-                m.kind = (ob0 < ob1 && ob1 < ob2) ? 1 : (ob0 == ob2 ? 6 : 2);
+                m.kind = ob0 == ob1 ? (ob1 == ob2 ? 4 : 2) : (ob1 == ob2 ? 3 : 1);
                 m.v = v;
                 mbar_expect_tx(full, u_bytes + ev_bytes + (EPI_PRODUCERS == 1 ? ovt1_bytes : 0u));
             }
@@ -694,20 +712,17 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
         const EpiStage &S = stg[stage];
         ff A4 = {0.f, 0.f}, A5 = {0.f, 0.f};
         // Each thread takes element orbits, the six orderings of one (a,b,c) with
-        // a in A, b in B, c in C.  Slot q holds the element with indices ordered
-        // as q (slots 0..5 = abc, acb, bac, bca, cab, cba); even slots 0,3,4, odd
-        // slots 1,2,5.  With E and O the sums of W over the even and odd slots, Z
-        // at slot q is 6 w_q + 2E - 4O (q even) or 6 w_q + 2O - 4E (q odd), and
-        // all six share one denominator.  What depends only on b and c is read
-        // once for the thread's two orbits.  Where blocks repeat, the loop over
-        // (a,b,c) meets every element 2 (two equal blocks) or 6 times (all equal)
-        // -- as often for elements with equal indices, whose six orderings repeat
-        // instead -- and the orbit's sum is divided by that; a slot whose block
-        // triple repeats an earlier one's reads that slot's cube (meta.smap).
-        auto orbits = [&](const float *c0, const float *c1, const float *c2, const float *c3, const float *c4,
-                          const float *c5) {
-            const int A0 = ob0 * F8, B0 = ob1 * F8, C0 = ob2 * F8;
+        // a in A, b in B, c in C; slot q holds the element with indices ordered as
+        // q (slots 0..5 = abc, acb, bac, bca, cab, cba; even slots 0,3,4, odd 1,2,5).
 #define OVV(sl, pu, pw, lu, lw) S.ov[sl][pu][pw][(lu) * F8 + (lw)]
+        const int A0 = ob0 * F8, B0 = ob1 * F8, C0 = ob2 * F8;
+        if (kind == 1) {
+            // Distinct blocks: with E and O the sums of W over the even and odd slots,
+            // Z at slot q is 6 w_q + 2E - 4O (q even) or 6 w_q + 2O - 4E (q odd), and all
+            // six share one denominator.  What depends only on b and c is read once
+            // for the thread's two orbits.
+            const float *c0 = S.cube[0][0], *c1 = S.cube[1][0], *c2 = S.cube[2][0];
+            const float *c3 = S.cube[3][0], *c4 = S.cube[4][0], *c5 = S.cube[5][0];
             const float tib = S.t1[0][1][lb], tic = S.t1[0][2][lc];
             const float tjb = S.t1[1][1][lb], tjc = S.t1[1][2][lc];
             const float tkb = S.t1[2][1][lb], tkc = S.t1[2][2][lc];
@@ -756,15 +771,67 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
                 A4 = ff_add(A4, ff_mul(s4, r));
                 A5 = ff_add(A5, ff_mul(s5, r));
             }
-#undef OVV
-        };
-        if (kind == 1) {
-            const float *q = S.cube[0][0];
-            orbits(q, q + 1536, q + 3072, q + 4608, q + 6144, q + 7680);
         } else {
-            const int *m = meta[stage].smap;
-            orbits(S.cube[0][0], S.cube[m[1]][0], S.cube[m[2]][0], S.cube[m[3]][0], S.cube[m[4]][0], S.cube[m[5]][0]);
+            // Repeated blocks: the element orbits with a <= b where A = B and b <= c
+            // where B = C, so that every element of the distinct cubes is met once;
+            // of an orbit with equal indices only the slots of its distinct elements
+            // count.  Each element's Z W and Z Y are formed in FP32 on their own; the
+            // warps take the orbits in turn (32 each, the first ones by another warp
+            // each time).
+            const int norb = kind == 4 ? 120 : 288;
+            for (int x = ((warp + n) & (EPI_CW - 1)) * 32 + lane; x < norb; x += NT) {
+                const int pr = kind == 4 ? trip[x] : trip[120 + (x >> 3)], l8 = x & 7;
+                const int la = kind == 3 ? l8 : pr & 7;
+                const int lb = kind == 3 ? pr & 7 : (pr >> 3) & 7;
+                const int lc = kind == 4 ? pr >> 6 : (kind == 3 ? (pr >> 3) & 7 : l8);
+                if (A0 + la >= v || B0 + lb >= v || C0 + lc >= v) continue;
+                const int abc = la * 64 + lb * 8 + lc, acb = la * 64 + lc * 8 + lb, bac = lb * 64 + la * 8 + lc;
+                const int bca = lb * 64 + lc * 8 + la, cab = lc * 64 + la * 8 + lb, cba = lc * 64 + lb * 8 + la;
+                const int *m = meta[stage].smap;
+                const float *c0 = S.cube[0][0], *c1 = S.cube[m[1]][0], *c2 = S.cube[m[2]][0];
+                const float *c3 = S.cube[m[3]][0], *c4 = S.cube[m[4]][0], *c5 = S.cube[m[5]][0];
+                float w[6], y[6];
+                w[0] = c0[bca] + c0[512 + acb] + c0[1024 + abc];
+                w[1] = c1[cba] + c1[512 + abc] + c1[1024 + acb];
+                w[2] = c2[acb] + c2[512 + bca] + c2[1024 + bac];
+                w[3] = c3[cab] + c3[512 + bac] + c3[1024 + bca];
+                w[4] = c4[abc] + c4[512 + cba] + c4[1024 + cab];
+                w[5] = c5[bac] + c5[512 + cab] + c5[1024 + cba];
+                const float tia = S.t1[0][0][la], tja = S.t1[1][0][la], tka = S.t1[2][0][la];
+                const float tib = S.t1[0][1][lb], tjb = S.t1[1][1][lb], tkb = S.t1[2][1][lb];
+                const float tic = S.t1[0][2][lc], tjc = S.t1[1][2][lc], tkc = S.t1[2][2][lc];
+                y[0] = tia * OVV(0, 1, 2, lb, lc) + tjb * OVV(1, 0, 2, la, lc) + tkc * OVV(2, 0, 1, la, lb);
+                y[1] = tia * OVV(0, 2, 1, lc, lb) + tjc * OVV(1, 0, 1, la, lb) + tkb * OVV(2, 0, 2, la, lc);
+                y[2] = tib * OVV(0, 0, 2, la, lc) + tja * OVV(1, 1, 2, lb, lc) + tkc * OVV(2, 1, 0, lb, la);
+                y[3] = tib * OVV(0, 2, 0, lc, la) + tjc * OVV(1, 1, 0, lb, la) + tka * OVV(2, 1, 2, lb, lc);
+                y[4] = tic * OVV(0, 0, 1, la, lb) + tja * OVV(1, 2, 1, lc, lb) + tkb * OVV(2, 2, 0, lc, la);
+                y[5] = tic * OVV(0, 1, 0, lb, la) + tjb * OVV(1, 2, 0, lc, la) + tka * OVV(2, 2, 1, lc, lb);
+                // equal indices: a = b makes slots 0 2, 1 3, 4 5 the same, b = c 0 1, 2 4, 3 5
+                const bool ab = kind != 3 && la == lb, bc = kind != 2 && lb == lc;
+                const int count = ab ? (bc ? 1 : 0x13) : (bc ? 0xd : 0x3f);
+                const ff e0 = {S.ev[0][la].x, S.ev[0][la].y}, e1 = {S.ev[1][lb].x, S.ev[1][lb].y},
+                         e2 = {S.ev[2][lc].x, S.ev[2][lc].y};
+                const ff r = ff_recip(ff_sub(ff_sub(ff_sub(eijk, e0), e1), e2));
+                ff n4 = {0.f, 0.f}, n5 = {0.f, 0.f};
+#pragma unroll
+                for (int q = 0; q < 6; q++) {
+                    // the slots of the element's acb, bac, cba, bca and cab
+                    constexpr int P[6][5] = {{1, 2, 5, 3, 4}, {0, 4, 3, 5, 2}, {3, 0, 4, 1, 5},
+                                             {2, 5, 1, 4, 0}, {5, 1, 2, 0, 3}, {4, 3, 0, 2, 1}};
+                    // Z = 8 W(abc) - 4 (W(acb) + W(bac) + W(cba)) + 2 (W(bca) + W(cab))
+                    const float zv = 8.f * w[q] - 4.f * (w[P[q][0]] + w[P[q][1]] + w[P[q][2]]) +
+                                     2.f * (w[P[q][3]] + w[P[q][4]]);
+                    if ((count >> q) & 1) {
+                        const ff s4 = ff_two_sum(n4.hi, zv * w[q]), s5 = ff_two_sum(n5.hi, zv * y[q]);
+                        n4 = {s4.hi, n4.lo + s4.lo};
+                        n5 = {s5.hi, n5.lo + s5.lo};
+                    }
+                }
+                A4 = ff_add(A4, ff_mul2(n4, r));
+                A5 = ff_add(A5, ff_mul2(n5, r));
+            }
         }
+#undef OVV
         // the stage is free once every warp has read it
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bar_empty[stage]));
@@ -801,9 +868,8 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
             }
             __syncwarp();
             if (lane == 0) {
-                const double w = kind == 1 ? 1.0 : (kind == 2 ? 0.5 : 1.0 / 6.0);  // repeated blocks: see above
-                out[0] = ff_to_double(b4) * w;
-                out[1] = ff_to_double(b5) * w;
+                out[0] = ff_to_double(b4);
+                out[1] = ff_to_double(b5);
                 mbar_arrive(smem_u32(&bar_rempty[rb]));
             }
         }

@@ -75,14 +75,34 @@ def test_stores_and_epilogue_reads_agree(v):
         assert w == pytest.approx(U[0][x, y, z] + U[1][y, x, z] + U[2][z, x, y], rel=1e-14, abs=1e-14)
 
 
-@pytest.mark.parametrize("orbit,times", [((0, 1, 2), 1), ((0, 0, 1), 2), ((0, 1, 1), 2), ((1, 1, 1), 6)])
-def test_repeated_blocks_count_every_ordering_equally_often(orbit, times):
-    """Over (a, b, c) in A x B x C with all six orderings each, every element of the orbit's distinct
-    cubes is met `times` times (the divisor of the orbit's sum)."""
-    met = {}
-    for t in itertools.product(range(2), repeat=3):  # 2 values per block are enough
-        e = tuple((orbit[d], t[d]) for d in range(3))
-        for p in PERMS:
-            k = tuple(e[d] for d in p)
-            met[k] = met.get(k, 0) + 1
-    assert set(met.values()) == {times}
+SLOTS = [(0, 1, 2), (0, 2, 1), (1, 0, 2), (1, 2, 0), (2, 0, 1), (2, 1, 0)]  # abc, acb, bac, bca, cab, cba
+
+
+@pytest.mark.parametrize("kind,orbit", [(2, (0, 0, 1)), (3, (0, 1, 1)), (4, (1, 1, 1))])
+def test_repeated_blocks_meet_every_element_once(kind, orbit):
+    """The element orbits and slot masks of the epilogue's repeated-block form."""
+    trip = [(x, y, z) for x in range(8) for y in range(x, 8) for z in range(y, 8)]
+    pair = [(x, y) for x in range(8) for y in range(x, 8)]
+    if kind == 4:
+        els = trip
+    elif kind == 2:
+        els = [(x, y, z) for x, y in pair for z in range(8)]
+    else:
+        els = [(x, y, z) for y, z in pair for x in range(8)]
+    met = []
+    for la, lb, lc in els:
+        ab, bc = kind != 3 and la == lb, kind != 2 and lb == lc
+        count = (1 if bc else 0x13) if ab else (0xd if bc else 0x3f)
+        e = [(orbit[0], la), (orbit[1], lb), (orbit[2], lc)]
+        met += [tuple(e[d] for d in SLOTS[q]) for q in range(6) if count >> q & 1]
+    want = {tuple((p[d], l[d]) for d in range(3)) for p in {tuple(orbit[d] for d in s) for s in SLOTS}
+            for l in itertools.product(range(8), repeat=3)}
+    assert len(met) == len(set(met)) and set(met) == want
+
+
+def test_slot_composition():
+    """P[q]: the slots of acb, bac, cba, bca, cab of the element at slot q."""
+    P = [(1, 2, 5, 3, 4), (0, 4, 3, 5, 2), (3, 0, 4, 1, 5), (2, 5, 1, 4, 0), (5, 1, 2, 0, 3), (4, 3, 0, 2, 1)]
+    for q, s in enumerate(SLOTS):
+        want = [tuple(s[d] for d in SLOTS[k]) for k in (1, 2, 5, 3, 4)]
+        assert [SLOTS[k] for k in P[q]] == want
