@@ -23,22 +23,24 @@
 // side's largest magnitude.  U is stored in the FP64 path's layout and the
 // FP64 epilogue does the rest.
 //
-// Kernel structure (one persistent CTA per SM, 10 warps; the same roles as the
-// split-precision kernel): warp 0 loads per chunk the S A planes (128 pair
-// rows, 64-byte K rows) and S B planes (OZ_N rows of a) with 5-D / 4-D tensor
-// maps whose outermost coordinate is the slice; warp 1 issues the S(S+1)/2
-// slice-pair MMAs (M = 128, N = OZ_N) into the S weight accumulators of a
-// TMEM block of OZ_KB chunks; warps 2-9 drain and accumulate.  Warps 0 and 1 run
-// whole, one elected lane issuing (tc_common.cuh): 52 tasks of o=40, v=300 took
-// 128.7 ms with both in a branch on the lane number and 116.4 ms so.  Every wait
-// is bounded as in the split-precision kernel.
+// Kernel structure: SM pairs (tcgen05 cta_group::2, M = 256), the roles of the
+// split-precision pair kernel (gemm_tc.cu, tc_pair.cuh).  Warp 0 loads per chunk
+// the S A planes (128 pair rows of its CTA, 64-byte K rows, one box) and half of
+// the S B planes (the pass's rows of a); the even CTA's warp 1 issues the
+// S(S+1)/2 slice-pair MMAs into the S weight accumulators of a TMEM block of up
+// to OZ_KB chunks; warps 2-9 drain and accumulate, weight by weight, the
+// conversions after the weight is handed back; warp 10 decodes the items.  Every
+// wait is bounded as in the split-precision kernel.
+// What bounds it: operand ingest (55 KB per chunk and SM) and the MMAs.  52 tasks
+// of o=40, v=300 took 98 ms on single SMs (M = 128, passes of 96 columns for any
+// v, TMEM blocks of 8 chunks whose whole drain the MMAs waited for) and take 71 ms.
 #include <cuda_bf16.h>
 
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
-#include "tc_common.cuh"
+#include "tc_pair.cuh"
 
 namespace tcorr {
 namespace {
@@ -66,94 +68,112 @@ using namespace tcx;
 
 constexpr int OZ_S = 5;          // slices per operand
 constexpr int OZ_BETA = 7;       // bits per slice
-constexpr int OZ_N = 96;         // a columns per item
-constexpr int OZ_THREADS = 320;
-constexpr int OZ_EPI = 256;      // warps 2-9
-constexpr int OZ_BM = 128;       // pair rows per tile
+constexpr int OZ_N = 96;         // most a columns per item
 constexpr int OZ_ROW = 64;       // K bytes per shared-memory row (32 BF16)
-constexpr int OZ_A = OZ_BM * OZ_ROW;        // 8 KB per A plane
-constexpr int OZ_B = OZ_N * OZ_ROW;         // 3 KB per B plane
+constexpr int OZ_A = PAIR_BM * OZ_ROW;      // 8 KB per A plane
+constexpr int OZ_B = OZ_N / 2 * OZ_ROW;     // 3 KB per B plane (half of the columns per CTA)
 constexpr int OZ_STAGE = OZ_S * (OZ_A + OZ_B);
-constexpr int OZ_STAGES = 3;
+constexpr int OZ_STAGES = 4;
 constexpr int OZ_SMEM = OZ_STAGES * OZ_STAGE + 1024;
-constexpr int OZ_HALF = OZ_N / 2;  // columns per epilogue warp
-// One TMEM accumulator block of OZ_S weights x OZ_N columns (single-buffered:
-// a block spans OZ_KB chunks, so its drain is short against its MMAs)
+// One TMEM accumulator block of OZ_S weights x OZ_N columns, handed over weight
+// by weight (below)
 static_assert(OZ_S * OZ_N <= 512, "weight accumulators exceed the 512 TMEM columns");
 static_assert(OZ_A % 1024 == 0 && OZ_B % 1024 == 0, "planes keep the 64-byte swizzle pattern aligned");
-constexpr int OZ_KB = 8;         // K chunks accumulated in TMEM per block (exact, see below)
+constexpr int OZ_KB = 18;        // most K chunks accumulated in TMEM per block (exact, see below)
 // Exactness of a block's weight sums in FP32: |a_1| <= 2^beta, |a_i| <= 2^(beta-1)
-// for i >= 2; weight t = 0 holds the single pair (1, 1), every other weight
-// at most S pairs each with one factor <= 2^(beta-1).
-static_assert(32 * OZ_KB * (1 << (2 * OZ_BETA)) < (1 << 24), "weight (1,1) must stay exact in FP32");
-static_assert(OZ_S * 32 * OZ_KB * (1 << (2 * OZ_BETA - 1)) < (1 << 24), "weight sums must stay exact in FP32");
-static_assert(OZ_HALF % 16 == 0, "the drain loads 16 columns at a time");
-
-
-// The 15 slice products (i + j <= S + 1) of one K chunk into the five weight
-// accumulators (columns t * OZ_N of tmem, t = i + j - 2); a0, b0: descriptor
-// low words of the stage's A and B slice planes.  FIRST: the chunk opens the
-// accumulator block, so each weight's first product zeroes its accumulator.
-template <bool FIRST>
-__device__ __forceinline__ void oz_chunk(uint32_t tmem, uint32_t a0, uint32_t b0, uint32_t idesc, int nks) {
-#pragma unroll
-    for (int t = 0; t < OZ_S; t++) {
-#pragma unroll
-        for (int ia = 0; ia <= t; ia++) {
-            const uint32_t d = tmem + (uint32_t)(t * OZ_N);
-            const uint32_t a = a0 + (uint32_t)((ia * OZ_A) >> 4), b = b0 + (uint32_t)(((t - ia) * OZ_B) >> 4);
-            if (FIRST && ia == 0) mma_lo<2, 1, false>(d, a, b, idesc);
-            else mma_lo<2, 1, true>(d, a, b, idesc);
-        }
-    }
-    if (nks > 1) {
-#pragma unroll
-        for (int t = 0; t < OZ_S; t++) {
-#pragma unroll
-            for (int ia = 0; ia <= t; ia++)
-                mma_lo<2, 1, true>(tmem + (uint32_t)(t * OZ_N), a0 + (uint32_t)((ia * OZ_A) >> 4) + 2,
-                                   b0 + (uint32_t)(((t - ia) * OZ_B) >> 4) + 2, idesc);
-        }
-    }
+// for i >= 2.  Weight t = i + j - 2 holds (1, 1) alone for t = 0, else (1, t+1) and
+// (t+1, 1) and t - 1 pairs of two smaller factors; the largest sum is t = OZ_S - 1's.
+static_assert(32LL * OZ_KB * (1 << (2 * OZ_BETA)) <= (1 << 24), "weight (1,1) must stay exact in FP32");
+static_assert(32LL * OZ_KB * (2 * (1 << (2 * OZ_BETA - 1)) + (OZ_S - 2) * (1 << (2 * OZ_BETA - 2))) <= (1 << 24),
+              "weight sums must stay exact in FP32");
+// chunks per block: the item's nch chunks in as few blocks as exactness allows, evenly
+__host__ __device__ inline int oz_block(int nch) {
+    const int nblk = (nch + OZ_KB - 1) / OZ_KB;
+    return (nch + nblk - 1) / nblk;
 }
 
-__global__ void __launch_bounds__(OZ_THREADS, 1) ugemm_oz_kernel(const __grid_constant__ Wave wv) {
+// The slice products of weight t (i + j = t + 2) of one K chunk into its
+// accumulator (columns t * OZ_N of tmem); a0, b0: descriptor low words of the
+// stage's A and B slice planes.  FIRST: the chunk opens the accumulator block,
+// so the weight's first product zeroes it.
+template <int T, bool FIRST>
+__device__ __forceinline__ void oz_weight(uint32_t tmem, uint32_t a0, uint32_t b0, uint32_t idesc, int nks) {
+    const uint32_t d = tmem + (uint32_t)(T * OZ_N);
+#pragma unroll
+    for (int ia = 0; ia <= T; ia++) {
+        const uint32_t a = a0 + (uint32_t)((ia * OZ_A) >> 4), b = b0 + (uint32_t)(((T - ia) * OZ_B) >> 4);
+        if (FIRST && ia == 0) mma_lo<2, 2, false>(d, a, b, idesc);
+        else mma_lo<2, 2, true>(d, a, b, idesc);
+        if (nks > 1) mma_lo<2, 2, true>(d, a + 2, b + 2, idesc);
+    }
+}
+// one weight of a block's first chunk (waits until it is drained); false on expiry
+template <int T>
+__device__ __forceinline__ bool oz_open(uint32_t tmem, uint32_t a0, uint32_t b0, uint32_t idesc, int nks, uint32_t hfull0,
+                                        uint32_t hempty0, uint32_t parity, bool last, volatile int *abort_flag) {
+    if (!wait_warp(hempty0 + 8u * T, parity, abort_flag)) return false;
+    tc_fence_after();
+    if (elect_one()) {
+        oz_weight<T, true>(tmem, a0, b0, idesc, nks);
+        if (last) tc_commit_pair(hfull0 + 8u * T, (uint16_t)3);
+    }
+    __syncwarp();
+    return true;
+}
+template <int T>
+__device__ __forceinline__ void oz_next(uint32_t tmem, uint32_t a0, uint32_t b0, uint32_t idesc, int nks, uint32_t hfull0,
+                                        bool last) {
+    oz_weight<T, false>(tmem, a0, b0, idesc, nks);
+    if (last) tc_commit_pair(hfull0 + 8u * T, (uint16_t)3);
+}
+
+__global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_oz_kernel(const __grid_constant__ Wave wv) {
     extern __shared__ __align__(1024) uint8_t smem_dyn[];
     __shared__ __align__(8) uint64_t bar_full[OZ_STAGES], bar_empty[OZ_STAGES];
-    __shared__ __align__(8) uint64_t bar_hfull[2], bar_hempty[2];
+    __shared__ __align__(8) uint64_t bar_hfull[OZ_S], bar_hempty[OZ_S];
+    __shared__ __align__(8) uint64_t bar_fin;
+    __shared__ __align__(8) uint64_t bar_sfull[PAIR_SLOTS], bar_sempty[PAIR_SLOTS];
+    __shared__ PairSlot slots[PAIR_SLOTS];
     __shared__ uint32_t tmem_holder;
     __shared__ volatile int abort_sh;
-    __shared__ SegCache ecache[OZ_EPI / 32];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank(), cid = cluster_id(), ncl = cluster_count();
+    const bool leader = rank == 0;
     const uint32_t sbase = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    const uint32_t peer_abort = peer_addr(smem_u32((const void *)&abort_sh), rank ^ 1u);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < OZ_STAGES; s++) {
             mbar_init(smem_u32(&bar_full[s]), 1);
             mbar_init(smem_u32(&bar_empty[s]), 1);
         }
-        for (int b = 0; b < 2; b++) {
-            mbar_init(smem_u32(&bar_hfull[b]), 1);
-            mbar_init(smem_u32(&bar_hempty[b]), OZ_EPI);
+        for (int t = 0; t < OZ_S; t++) {
+            mbar_init(smem_u32(&bar_hfull[t]), 1);
+            mbar_init(smem_u32(&bar_hempty[t]), PAIR_HEMPTY_ARRIVALS);
+        }
+        mbar_init(smem_u32(&bar_fin), 1);
+        for (int n = 0; n < PAIR_SLOTS; n++) {
+            mbar_init(smem_u32(&bar_sfull[n]), 1);
+            mbar_init(smem_u32(&bar_sempty[n]), (leader ? 2 : 1) + PAIR_EPI / 32);  // producer, drains, MMA issuer
         }
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_holder)),
                      "r"(512)
                      : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync_all();  // both CTAs' barriers exist before any remote signal
     tc_fence_after();
     const uint32_t tmem = tmem_holder;
-    // D = F32, A = B = BF16, K-major, M = 128, N = OZ_N
-    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(OZ_N >> 3) << 17) |
-                               ((uint32_t)(OZ_BM >> 4) << 24);
+    // D = F32, A = B = BF16, K-major, M = 256 over the pair
+    constexpr uint32_t idesc_m = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * PAIR_BM >> 4) << 24);
 
     if (warp == 0) {
         int stage = 0;
@@ -161,32 +181,23 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) ugemm_oz_kernel(const __grid_co
         int last_phase[OZ_STAGES];
         for (int s = 0; s < OZ_STAGES; s++) last_phase[s] = -1;
         bool ok = true;
-        bool inject = wv.inject_stall != 0 && blockIdx.x == 0;
-        SegCache sc;
-        seg_reset(sc);
-        for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
-            const Item w = decode(wv, it, sc);
-            if (uni((int)w.diag)) continue;
-            const InstDesc *d = uni(sc.d);
-            const int o = uni(d->dm.o), kv = uni(d->kv), ko = uni(d->ko), nch = 2 * kv + 2 * ko;
-            const int s = uni(w.s), pp = uni(w.p), q = uni(w.q);
-            const int cb = uni(w.bt * d->pb), cc = uni(w.ct * d->pc), ca = uni(w.n * OZ_N);
-            const uint32_t stage_tx = uni(d->stage_tx);
-            for (int ch = 0; ch < nch; ch++) {
-                if (!wait_warp(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
-                    if (lane == 0) fail(&abort_sh, wv.err, DERR_TIMEOUT_EMPTY);
-                    ok = false;
-                    break;
-                }
-                const uint32_t full = smem_u32(&bar_full[stage]);
-                last_phase[stage] = (int)phase;
-                const uint32_t sA = sbase + stage * OZ_STAGE, sB = sA + OZ_S * OZ_A;
-                int seg, kk;
-                if (ch < kv) { seg = 0; kk = ch; }
-                else if (ch < 2 * kv) { seg = 1; kk = ch - kv; }
-                else if (ch < 2 * kv + ko) { seg = 2; kk = ch - 2 * kv; }
-                else { seg = 3; kk = ch - 2 * kv - ko; }
-                const int k0 = kk * 32;
+        bool inject = wv.inject_stall != 0 && cid == 0 && leader;
+        for (uint32_t n = 0; ok; n++) {
+            const PairSlot &sl = slots[n % PAIR_SLOTS];
+            if (!wait_warp(smem_u32(&bar_sfull[n % PAIR_SLOTS]), (n / PAIR_SLOTS) & 1u, &abort_sh)) {
+                if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_FULL);
+                ok = false;
+                break;
+            }
+            if (uni(sl.end)) break;
+            const InstDesc *d = uni(sl.d);
+            const int o = uni(sl.o), kv = uni(sl.kv), ko = uni(sl.ko);
+            const int pp = uni(sl.p), q = uni(sl.q), cb = uni(sl.cb), cc = uni(sl.cc);
+            const int s = uni(sl.box[0].x), ca = uni(sl.box[0].y);
+            const uint32_t stage_tx = uni(sl.stage_tx);
+            if (lane == 0) mbar_arrive(smem_u32(&bar_sempty[n % PAIR_SLOTS]));
+            for (int seg = 0; seg < 4 && ok; seg++) {
+                const int klen = seg < 2 ? kv : ko;
                 int amap, aslice, bmap, brow;
                 switch (seg) {
                     case 0: amap = MAP_G_NAT; aslice = q; bmap = MAP_T2R; brow = s * o + pp; break;
@@ -194,158 +205,210 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) ugemm_oz_kernel(const __grid_co
                     case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; brow = q * o + s; break;
                     default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; brow = pp * o + s; break;
                 }
-                if (elect_one()) {
-                    mbar_expect_tx(full, stage_tx);
-                    if (!inject) {
-                        for (int pl = 0; pl < OZ_S; pl++) {
-                            tma_load_5d(sA + pl * OZ_A, &d->maps[amap][0], full, k0, cc, cb, aslice, pl);
-                            tma_load_4d(sB + pl * OZ_B, &d->maps[bmap][0], full, k0, ca, brow, pl);
-                        }
-                    }
-                }
-                __syncwarp();
-                if (inject) {
-                    inject = false;
-                    last_phase[stage] = -1;  // nothing in flight: the consumer's wait must expire
-                }
-                if (++stage == OZ_STAGES) { stage = 0; phase ^= 1u; }
-            }
-        }
-        if (!ok && lane == 0) {  // let this CTA's copies in flight land before exiting
-            for (int s = 0; s < OZ_STAGES; s++) {
-                if (last_phase[s] < 0) continue;
-                const uint64_t t0 = gtimer();
-                while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
-                       gtimer() - t0 < WAIT_LIMIT_NS) {
-                }
-            }
-        }
-    } else if (warp == 1) {
-        int stage = 0;
-        uint32_t phase = 0;
-        uint32_t hblk = 0;  // blocks of OZ_KB chunks issued: accumulator phase hblk & 1
-        bool ok = true;
-        const uint32_t tm = uni(tmem);
-        SegCache sc;
-        seg_reset(sc);
-        for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
-            const Item w = decode(wv, it, sc);
-            if (uni((int)w.diag)) continue;
-            const InstDesc *d = uni(sc.d);
-            const int kv = uni(d->kv), ko = uni(d->ko), dp = uni(d->dm.dp), lp = uni(d->dm.lp);
-            const int nch = 2 * kv + 2 * ko;
-            for (int c0 = 0; c0 < nch && ok; c0 += OZ_KB) {
-                const int nb = min(OZ_KB, nch - c0);
-                for (int cb = 0; cb < nb; cb++) {
-                    const int ch = c0 + cb;
-                    int code = 0;
-                    if (!wait_warp(smem_u32(&bar_full[stage]), phase, &abort_sh)) code = DERR_TIMEOUT_FULL;
-                    else if (cb == 0 && !wait_warp(smem_u32(&bar_hempty[0]), (hblk & 1u) ^ 1u, &abort_sh))
-                        code = DERR_TIMEOUT_TMEM;
-                    if (code) {
-                        if (lane == 0) fail(&abort_sh, wv.err, code);
+                for (int kk = 0; kk < klen; kk++) {
+                    if (!wait_warp(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_sh)) {
+                        if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_EMPTY);
                         ok = false;
                         break;
                     }
-                    tc_fence_after();
+                    const uint32_t full = smem_u32(&bar_full[stage]);
+                    const uint32_t full_l = peer_addr(full, 0);
+                    last_phase[stage] = (int)phase;
                     const uint32_t sA = sbase + stage * OZ_STAGE, sB = sA + OZ_S * OZ_A;
-                    const int nks = chunk_ksteps(2, kv, ko, dp, lp, ch);
-                    // descriptor low words (see mma_lo): plane and K-step offsets are
-                    // constants added to the stage's base words.  Every slice product
-                    // is exact in FP32, so their order within a block is free: the
-                    // first K step of every weight first (the block's opening MMA of
-                    // each weight zeroes it), then the second
-                    const uint32_t a0 = desc_lo(sA), b0 = desc_lo(sB);
+                    const int k0 = kk * 32;
                     if (elect_one()) {
-                        if (cb == 0) oz_chunk<true>(tm, a0, b0, idesc, nks);
-                        else oz_chunk<false>(tm, a0, b0, idesc, nks);
-                        tc_commit(smem_u32(&bar_empty[stage]));  // the stage is free once these MMAs are done
-                        if (cb == nb - 1) tc_commit(smem_u32(&bar_hfull[0]));
+                        if (leader) mbar_expect_tx(full, stage_tx);
+                        if (!inject) {
+                            // the five A planes in one box; B planes at a fixed pitch, one copy each
+                            tma_load_5d_pair(sA, &d->maps[amap][0], full_l, k0, cc, cb, aslice, 0);
+#pragma unroll
+                            for (int pl = 0; pl < OZ_S; pl++)
+                                tma_load_4d_pair(sB + pl * OZ_B, &d->maps[bmap][0], full_l, k0, ca, brow, pl);
+                        }
                     }
                     __syncwarp();
+                    if (inject) {
+                        inject = false;
+                        last_phase[stage] = -1;  // the leader's bytes never come: the MMA's wait must expire
+                    }
                     if (++stage == OZ_STAGES) { stage = 0; phase ^= 1u; }
                 }
-                hblk++;
             }
         }
+        if (!ok && lane == 0) {
+            // let the copies in flight land: the leader sees both CTAs' bytes on
+            // its own full barriers; the peer gives its own copies a fixed time
+            if (leader) {
+                for (int s = 0; s < OZ_STAGES; s++) {
+                    if (last_phase[s] < 0) continue;
+                    const uint64_t t0 = gtimer();
+                    while (!mbar_test(smem_u32(&bar_full[s]), (uint32_t)last_phase[s]) &&
+                           gtimer() - t0 < WAIT_LIMIT_NS) {
+                    }
+                }
+            }
+            spin_ns(1000000ull);
+        }
+    } else if (warp == 1) {
+        if (leader) {
+            int stage = 0;
+            uint32_t phase = 0;
+            uint32_t hblk = 0;  // accumulator blocks issued
+            bool ok = true;
+            const uint32_t tm = uni(tmem), hfull0 = smem_u32(&bar_hfull[0]), hempty0 = smem_u32(&bar_hempty[0]);
+            for (uint32_t n = 0; ok; n++) {
+                const PairSlot &sl = slots[n % PAIR_SLOTS];
+                if (!wait_warp(smem_u32(&bar_sfull[n % PAIR_SLOTS]), (n / PAIR_SLOTS) & 1u, &abort_sh)) {
+                    if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_FULL);
+                    break;
+                }
+                if (uni(sl.end)) break;
+                const int kv = uni(sl.kv), ko = uni(sl.ko), N = uni(sl.N), nch = 2 * kv + 2 * ko;
+                const int v = uni(sl.v), o = uni(sl.o);
+                if (lane == 0) mbar_arrive(smem_u32(&bar_sempty[n % PAIR_SLOTS]));
+                // a segment's last chunk holds one K step of data (16 values or fewer) or two
+                const bool dh = v - (kv - 1) * 32 <= 16, lh = o - (ko - 1) * 32 <= 16;
+                const uint32_t idesc = idesc_m | ((uint32_t)(N >> 3) << 17);
+                const int kb = oz_block(nch);
+                for (int c0 = 0; c0 < nch && ok; c0 += kb) {
+                    const int c1 = min(c0 + kb, nch);
+                    for (int ch = c0; ch < c1; ch++) {
+                        if (!wait_warp(smem_u32(&bar_full[stage]), phase, &abort_sh)) {
+                            if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_FULL);
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t a0 = desc_lo(sbase + stage * OZ_STAGE), b0 = a0 + (uint32_t)((OZ_S * OZ_A) >> 4);
+                        const bool tail = (dh && (ch == kv - 1 || ch == 2 * kv - 1)) ||
+                                          (lh && (ch == 2 * kv + ko - 1 || ch == nch - 1));
+                        const int nks = tail ? 1 : 2;
+                        const bool last = ch == c1 - 1;
+                        // Every slice product is exact in FP32, so their order within a
+                        // block is free: weight by weight.  A block's first chunk opens each
+                        // weight once the drain has read it from the block before, and its
+                        // last chunk hands each weight over when its products are issued, so
+                        // the drain of one block overlaps the ends of both.
+                        if (ch == c0) {
+                            const uint32_t par = (hblk & 1u) ^ 1u;
+                            ok = oz_open<0>(tm, a0, b0, idesc, nks, hfull0, hempty0, par, last, &abort_sh) &&
+                                 oz_open<1>(tm, a0, b0, idesc, nks, hfull0, hempty0, par, last, &abort_sh) &&
+                                 oz_open<2>(tm, a0, b0, idesc, nks, hfull0, hempty0, par, last, &abort_sh) &&
+                                 oz_open<3>(tm, a0, b0, idesc, nks, hfull0, hempty0, par, last, &abort_sh) &&
+                                 oz_open<4>(tm, a0, b0, idesc, nks, hfull0, hempty0, par, last, &abort_sh);
+                            if (!ok) {
+                                if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_TMEM);
+                                break;
+                            }
+                            if (elect_one()) tc_commit_pair(smem_u32(&bar_empty[stage]), (uint16_t)3);
+                        } else if (elect_one()) {
+                            oz_next<0>(tm, a0, b0, idesc, nks, hfull0, last);
+                            oz_next<1>(tm, a0, b0, idesc, nks, hfull0, last);
+                            oz_next<2>(tm, a0, b0, idesc, nks, hfull0, last);
+                            oz_next<3>(tm, a0, b0, idesc, nks, hfull0, last);
+                            oz_next<4>(tm, a0, b0, idesc, nks, hfull0, last);
+                            tc_commit_pair(smem_u32(&bar_empty[stage]), (uint16_t)3);
+                        }
+                        __syncwarp();
+                        if (++stage == OZ_STAGES) { stage = 0; phase ^= 1u; }
+                    }
+                    hblk++;
+                }
+            }
+            // every MMA issued by this warp's elected lane has completed before the pair tears down
+            if (elect_one()) {
+                tc_commit_pair(smem_u32(&bar_fin), (uint16_t)1);
+                const uint64_t t0 = gtimer();
+                while (!mbar_test(smem_u32(&bar_fin), 0u) && gtimer() - t0 < WAIT_LIMIT_NS) {
+                }
+            }
+            __syncwarp();
+        }
+    } else if (warp == 2 + PAIR_EPI / 32) {
+        pair_scheduler(wv, cid, ncl, rank, slots, bar_sfull, bar_sempty, &abort_sh, peer_abort);
     } else {
         const int wq = warp & 3;              // TMEM lane quarter of this warp
-        const int half = (warp - 2) >> 2;     // column half of each weight block
+        const int half = (warp - 2) >> 2;     // column half of each weight
         const int row = wq * 32 + lane;       // accumulator row = pair in tile
         const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
         uint32_t hblk = 0;
         bool ok = true;
-        SegCache &cs = ecache[warp - 2];
-        if (lane == 0) seg_reset(cs);
-        __syncwarp();
-        for (int64_t it = blockIdx.x; it < wv.n_gemm && ok; it += gridDim.x) {
-            SegCache sc = cs;
-            const Item w = decode(wv, it, sc);
-            __syncwarp();
-            if (lane == 0) cs = sc;
-            __syncwarp();
-            if (w.diag) continue;
-            const InstDesc &d = *sc.d;
-            const int64_t u_seg = sc.u_off;
-            const int v = d.dm.v, vc = d.dm.vc;
-            const int nhb = (num_chunks(d) + OZ_KB - 1) / OZ_KB;
-            const int lb = row / d.pc, lc = row % d.pc;
-            long long tot[OZ_HALF];
+        for (uint32_t n = 0; ok; n++) {
+            const PairSlot &sl = slots[n % PAIR_SLOTS];
+            if (!wait_warp(smem_u32(&bar_sfull[n % PAIR_SLOTS]), (n / PAIR_SLOTS) & 1u, &abort_sh)) {
+                if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_FULL);
+                break;
+            }
+            if (sl.end) break;
+            const int nch = 2 * (sl.kv + sl.ko), kb = oz_block(nch), nhb = (nch + kb - 1) / kb;
+            const int hw = sl.N / 2;          // columns of this warp, a multiple of 8
+            long long tot[OZ_N / 2];
 #pragma unroll
-            for (int j = 0; j < OZ_HALF; j++) tot[j] = 0;
-            for (int hb = 0; hb < nhb; hb++) {
-                int good = 1;
-                if (lane == 0) good = mbar_wait(smem_u32(&bar_hfull[0]), hblk & 1u, &abort_sh) ? 1 : 0;
-                good = __shfl_sync(0xffffffffu, good, 0);
-                __syncwarp();
-                if (!good) { ok = false; break; }
-                tc_fence_after();
+            for (int j = 0; j < OZ_N / 2; j++) tot[j] = 0;
+            for (int hb = 0; hb < nhb && ok; hb++) {
 #pragma unroll
                 for (int t = 0; t < OZ_S; t++) {
-                    const long long wgt = 1LL << (OZ_BETA * (OZ_S - 1 - t));
+                    if (ok) {
+                        ok = wait_warp(smem_u32(&bar_hfull[t]), hblk & 1u, &abort_sh);
+                        if (ok) {
+                            // the weight is free once its columns are in registers: the
+                            // conversions run beside the next block's products
+                            const long long wgt = 1LL << (OZ_BETA * (OZ_S - 1 - t));
+                            uint32_t r[OZ_N / 16][8];
+                            tc_fence_after();
 #pragma unroll
-                    for (int c16 = 0; c16 < OZ_HALF / 16; c16++) {
-                        uint32_t r[16];
-                        tc_ld16(tmem + lane_off + (uint32_t)(t * OZ_N + half * OZ_HALF + c16 * 16), r);
-                        tc_wait_ld();
+                            for (int c8 = 0; c8 < OZ_N / 16; c8++)
+                                if (c8 * 8 < hw)
+                                    tc_ld8(tmem + lane_off + (uint32_t)(t * OZ_N + half * hw + c8 * 8), r[c8]);
+                            tc_wait_ld();
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive_cluster(peer_addr(smem_u32(&bar_hempty[t]), 0));
 #pragma unroll
-                        for (int j = 0; j < 16; j++)
-                            tot[c16 * 16 + j] += (long long)__float2int_rn(__uint_as_float(r[j])) * wgt;
+                            for (int c8 = 0; c8 < OZ_N / 16; c8++)
+                                if (c8 * 8 < hw) {
+#pragma unroll
+                                    for (int j = 0; j < 8; j++)
+                                        tot[c8 * 8 + j] += (long long)__float2int_rn(__uint_as_float(r[c8][j])) * wgt;
+                                }
+                        }
                     }
                 }
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bar_hempty[0]));
                 hblk++;
             }
             if (!ok) {
-                if (lane == 0) fail(&abort_sh, wv.err, DERR_TIMEOUT_TMEM);
+                if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_TMEM);
                 break;
             }
             // U^g[a][b][c] in the FP64 path's layout, each value as a float-float
             // (hi, lo) pair in its 8 bytes (about 48 significant bits), so that the
             // epilogue works on the FP32 pipe; formed from the exact int64 total
             // without the FP64 pipe (int64_to_ff)
-            const int b = w.bt * d.pb + lb, c = w.ct * d.pc + lc;
-            if (b < v && c < v) {
-                const int scale_exp = d.oz_e[0] + d.oz_e[1] - OZ_BETA * (OZ_S + 1);
-                const int a0 = w.n * OZ_N + half * OZ_HALF;
+            const int v = sl.v, pc = sl.pc, vc = round_up(v, UPAD);
+            const int b = sl.cb + row / pc, c = sl.cc + row % pc;
+            if (!sl.empty && b < v && c < v) {
+                const int scale_exp = sl.scale - OZ_BETA * (OZ_S + 1);
+                const int a0 = sl.pass0 + half * hw;
                 const int64_t stride = (int64_t)v * vc;
-                float2 *Ug = static_cast<float2 *>(wv.U) + u_seg + (int64_t)(w.tb * 3 + w.g) * d.dm.ug +
-                             (int64_t)b * vc + c + (int64_t)a0 * stride;
+                float2 *Ug = static_cast<float2 *>(wv.U) + sl.u_off + (int64_t)sl.g * (sl.ug3 / 3) + (int64_t)b * vc + c +
+                             (int64_t)a0 * stride;
 #pragma unroll
-                for (int j = 0; j < OZ_HALF; j++) {
-                    if (a0 + j < v) *Ug = int64_to_ff(tot[j], scale_exp);
+                for (int j = 0; j < OZ_N / 2; j++) {
+                    if (j < hw && a0 + j < v) *Ug = int64_to_ff(tot[j], scale_exp);
                     Ug += stride;
                 }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bar_sempty[n % PAIR_SLOTS]));
         }
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync_all();  // the peer no longer signals this CTA's barriers or reads its operands
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512)
                      : "memory");
     }
 }
@@ -464,21 +527,23 @@ cudaError_t oz_fill_desc(InstDesc &d, const Operands &op, const int *exps, std::
     d.kb = 1;
     d.nbt = (v + pb - 1) / pb;
     d.nct = (v + pc - 1) / pc;
+    d.pair = 1;
+    // passes of equal width, a multiple of 16: each CTA holds half of the columns
     d.npass = (v + OZ_N - 1) / OZ_N;
+    d.brows = round_up((v + d.npass - 1) / d.npass, 16);
     d.kv = (v + 31) / 32;
     d.ko = (o + 31) / 32;
-    d.brows = OZ_N;
-    d.stage_tx = (uint32_t)(OZ_S * (OZ_A + OZ_N * OZ_ROW));
+    d.stage_tx = (uint32_t)(2 * OZ_S * (OZ_A + d.brows / 2 * OZ_ROW));  // both CTAs' bytes
     d.oz_e = exps;
     const uint64_t V = v, O = o, S = OZ_S;
     // plane strides (bytes): one slice plane of each operand layout
     const uint64_t pG = (uint64_t)O * V * V * dp * eb, pT2K = (uint64_t)O * V * V * lp * eb;
     const uint64_t pT2R = (uint64_t)O * O * V * dp * eb, pAoN = (uint64_t)O * O * V * lp * eb;
-    const uint32_t bk = 32, bpc = (uint32_t)pc, bpb = (uint32_t)pb, bn = (uint32_t)OZ_N;
+    const uint32_t bk = 32, bpc = (uint32_t)pc, bpb = (uint32_t)pb, bn = (uint32_t)(d.brows / 2), bs = OZ_S;
     {
         uint64_t dims[5] = {V, V, V, O, S};
         uint64_t st[4] = {dp * eb, V * dp * eb, V * V * dp * eb, pG};
-        uint32_t box[5] = {bk, bpc, bpb, 1, 1};
+        uint32_t box[5] = {bk, bpc, bpb, 1, bs};
         if (!encode(&d.maps[MAP_G_NAT][0], dt, 5, op.G, dims, st, box, err, "G slices")) return cudaErrorInvalidValue;
         uint64_t st2[4] = {V * dp * eb, dp * eb, V * V * dp * eb, pG};
         if (!encode(&d.maps[MAP_G_SWP][0], dt, 5, op.G, dims, st2, box, err, "G slices swapped"))
@@ -487,7 +552,7 @@ cudaError_t oz_fill_desc(InstDesc &d, const Operands &op, const int *exps, std::
     {
         uint64_t dims[5] = {O, V, V, O, S};
         uint64_t st[4] = {lp * eb, V * lp * eb, V * V * lp * eb, pT2K};
-        uint32_t box[5] = {bk, bpc, bpb, 1, 1};
+        uint32_t box[5] = {bk, bpc, bpb, 1, bs};
         if (!encode(&d.maps[MAP_T2K_NAT][0], dt, 5, op.T2K, dims, st, box, err, "T2K slices"))
             return cudaErrorInvalidValue;
         uint64_t st2[4] = {V * lp * eb, lp * eb, V * V * lp * eb, pT2K};
@@ -509,7 +574,7 @@ cudaError_t oz_fill_desc(InstDesc &d, const Operands &op, const int *exps, std::
     return cudaSuccess;
 }
 
-int64_t oz_units_per_task(const InstDesc &d) { return (int64_t)3 * d.nbt * d.nct * d.npass; }
+int64_t oz_units_per_task(const InstDesc &d) { return (int64_t)3 * ((d.nbt * d.nct + 1) / 2) * d.npass; }
 
 cudaError_t oz_prepare() {
     static std::mutex mu;
@@ -522,12 +587,11 @@ cudaError_t oz_prepare() {
 }
 
 cudaError_t launch_ugemm_oz(int sm_count, const Wave &w, cudaStream_t st) {
-    const int grid = (int)std::min<int64_t>(sm_count, w.n_gemm);
-    if (grid <= 0) return cudaSuccess;
+    if (w.n_gemm <= 0) return cudaSuccess;
     const cudaError_t e = oz_prepare();
     if (e != cudaSuccess) return e;
-    ugemm_oz_kernel<<<grid, OZ_THREADS, OZ_SMEM, st>>>(w);
-    return cudaGetLastError();
+    static PairLaunch pl;
+    return pl.launch(ugemm_oz_kernel, PAIR_THREADS, OZ_SMEM, sm_count, w.n_gemm, st, w);
 }
 
 }  // namespace tcorr

@@ -45,7 +45,7 @@
 #include <cstring>
 #include <mutex>
 
-#include "tc_common.cuh"
+#include "tc_pair.cuh"
 
 namespace tcorr {
 namespace {
@@ -334,142 +334,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) ugemm_tc_kernel(const __grid_co
 //    issued MMAs, and a producer that aborted lets its copies in flight land.
 // Teardown: a cluster barrier (every role of both CTAs ends after bounded
 // waits), then both CTAs free the pair's tensor memory.
-constexpr int PAIR_THREADS = TC_THREADS + 32;  // warp 10: scheduler
-constexpr int PAIR_HEMPTY_ARRIVALS = 2 * (EPI_THREADS / 32);
-constexpr int PAIR_ROW = 2 * ROW_BYTES;   // one K block (two chunks) per shared-memory row, 128-byte swizzle
-constexpr int PAIR_A = BM * PAIR_ROW;     // 16 KB per A plane
-constexpr int PACK_ROWS = 16;             // rows of a B box of packed columns
-constexpr int PACK_BOXES = BN / 2 / PACK_ROWS;  // boxes per CTA and plane at N = 256
 constexpr int PACK_MAX_V = 256;           // packed columns up to this v (see tc_fill_desc)
-constexpr int PACK_BOX_BYTES = PACK_ROWS * PAIR_ROW;
-
-struct PairCache {
-    SegCache s;
-    const PackRun *runs;
-    const PackEnt *ents;
-    int nrun, r, r_end;  // cached run and the unit after its last
-    PackRun run;
-};
-__device__ __forceinline__ void pair_reset(PairCache &c) { seg_reset(c.s); }
-struct PairItem {
-    int bt, ct;          // this CTA's pair tile
-    int p, q;            // the A side's slices
-    int N;               // columns of the MMAs
-    int pass0, ncol;     // first column (of a, or of the run's packed columns) and valid columns
-    int tb, g, s;        // not packed: task of the segment, group and its s
-    int ent0;            // packed: first entry of the run
-    bool packed;         // entries of a run
-    bool boxes;          // several entries: B in 16-row boxes
-    bool empty;          // this CTA's tile index lies past the group's tile list
-    bool diag;           // i = j = k: no work
-};
-__device__ __forceinline__ PairItem decode_pair(const Wave &w, int64_t it, PairCache &c, uint32_t rank) {
-    const bool fresh = c.s.si < 0 || it >= c.s.end;
-    seg_update(w, it, c.s);
-    PairItem r;
-    const InstDesc &d = *c.s.d;
-    const int npt = c.s.nbt * c.s.nct;
-    const int npair = (npt + 1) / 2;
-    int tp;
-    if (fresh) {
-        const Seg &sg = w.segs[c.s.si];
-        c.runs = sg.runs;
-        c.ents = sg.ents;
-        c.nrun = sg.nrun;
-        c.r = 0;
-        c.r_end = -1;
-    }
-    r.packed = c.nrun != 0;
-    r.boxes = false;
-    if (r.packed) {
-        const int x = (int)(it - c.s.begin);
-        if (x >= c.r_end) {  // units only grow: search forward
-            int lo = c.r, hi = c.nrun - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (c.runs[mid].unit0 <= x) lo = mid; else hi = mid - 1;
-            }
-            c.r = lo;
-            c.run = c.runs[lo];
-            c.r_end = c.run.unit0 + npair * c.run.npass;
-        }
-        const int local = x - c.run.unit0, n = local % c.run.npass;
-        tp = local / c.run.npass;
-        r.boxes = c.run.nent > 1;
-        if (r.boxes) {
-            const int cols = c.run.nent * d.packw;
-            const int width = ((cols + c.run.npass - 1) / c.run.npass + 31) / 32 * 32;
-            r.pass0 = n * width;
-            r.ncol = min(width, cols - r.pass0);
-            r.N = (r.ncol + 31) / 32 * 32;
-        } else {  // v <= 256: one pass
-            r.pass0 = 0;
-            r.ncol = d.dm.v;
-            r.N = (r.ncol + 15) / 16 * 16;
-        }
-        r.ent0 = c.run.ent0;
-        r.p = c.run.p;
-        r.q = c.run.q;
-        r.tb = r.g = r.s = 0;
-        r.diag = false;  // the tables hold no group of a task i = j = k
-    } else {
-        int64_t x = it - c.s.begin;
-        const int n = (int)(x % c.s.npass);  // N pass fastest, then group, then tile pair (as decode)
-        x /= c.s.npass;
-        r.g = (int)(x % 3);
-        x /= 3;
-        tp = (int)(x % npair);
-        r.tb = (int)(x / npair);
-        if (r.tb != c.s.tcached) {
-            const int *tk = d.tasks + 3 * (c.s.task0 + r.tb);
-            c.s.ti = tk[0];
-            c.s.tj = tk[1];
-            c.s.tk = tk[2];
-            c.s.tcached = r.tb;
-        }
-        const int i = c.s.ti, j = c.s.tj, k = c.s.tk;
-        r.diag = (i == j && j == k);
-        r.s = r.g == 0 ? i : (r.g == 1 ? j : k);
-        r.p = r.g == 0 ? j : i;
-        r.q = r.g == 2 ? j : k;
-        r.pass0 = n * d.brows;
-        r.ncol = min(d.brows, d.dm.v - r.pass0);
-        r.N = (r.ncol + 15) / 16 * 16;
-        r.ent0 = 0;
-    }
-    const int t = tp * 2 + (int)rank;
-    r.empty = t >= npt;
-    r.bt = r.empty ? c.s.nbt : t / c.s.nct;  // past the list: b >= v, all TMA fill
-    r.ct = r.empty ? 0 : t % c.s.nct;
-    return r;
-}
-// What the roles of a CTA need of an item, written by its scheduler warp.
-struct PairSlot {
-    const InstDesc *d;
-    float *U;               // the segment's U (packed), or the task's
-    int64_t ug3;
-    int end;                // no more items
-    int o, v, kv, ko, kind;
-    int p, q, N, cb, cc;    // A slices, columns, first b and c of this CTA's tile
-    uint32_t stage_tx;      // bytes of a stage, both CTAs'
-    int nbx, boxes;         // B copies per plane and stage; in 16-row boxes?
-    int pc, packed, empty;
-    int g, pass0, ncol;     // not packed: group and columns of a
-    int2 box[PACK_BOXES];   // (s, first a) of the B copies, s = -1 past the valid columns
-    int2 ent[BN / 8];       // packed: (tbg, a) of columns 8 k .. 8 k + 7, a = 2^20 for none
-};
-constexpr int PAIR_SLOTS = 4;
-// abort both CTAs of the pair and raise the device error flag
-__device__ __forceinline__ void fail_pair(volatile int *abort_flag, uint32_t peer_abort_cl, int *err, int code) {
-    *abort_flag = 1;
-    st_cluster_u32(peer_abort_cl, 1u);
-    atomicOr(err, code);
-}
-__device__ __forceinline__ void spin_ns(uint64_t ns) {
-    const uint64_t t0 = gtimer();
-    while (gtimer() - t0 < ns) {
-    }
-}
 
 __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_tc_pair_kernel(const __grid_constant__ Wave wv) {
     extern __shared__ __align__(1024) uint8_t smem_dyn[];
@@ -671,79 +536,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_tc_pair_kernel(const __
             __syncwarp();
         }
     } else if (warp == 2 + EPI_THREADS / 32) {
-        // scheduler: decodes this CTA's items ahead of the other roles
-        PairCache pc;
-        pair_reset(pc);
-        uint32_t n = 0;
-        bool ok = true;
-        for (int64_t it = cid; ok; it += ncl) {
-            const bool end = it >= wv.n_gemm;
-            PairItem w;
-            if (!end) {
-                w = decode_pair(wv, it, pc, rank);
-                if (w.diag) continue;
-            }
-            PairSlot &sl = slots[n % PAIR_SLOTS];
-            if (n >= PAIR_SLOTS &&
-                !wait_warp(smem_u32(&bar_sempty[n % PAIR_SLOTS]), (n / PAIR_SLOTS - 1) & 1u, &abort_sh)) {
-                if (lane == 0) fail_pair(&abort_sh, peer_abort, wv.err, DERR_TIMEOUT_EMPTY);
-                ok = false;
-                break;
-            }
-            if (!end) {
-                const InstDesc &d = *pc.s.d;
-                if (lane == 0) {
-                    sl.d = &d;
-                    sl.ug3 = 3 * d.dm.ug;
-                    sl.U = static_cast<float *>(wv.U) + pc.s.u_off + w.tb * (3 * d.dm.ug);
-                    sl.o = d.dm.o;
-                    sl.v = d.dm.v;
-                    sl.kv = d.kv;
-                    sl.ko = d.ko;
-                    sl.kind = d.kind;
-                    sl.p = w.p;
-                    sl.q = w.q;
-                    sl.N = w.N;
-                    sl.cb = w.bt * d.pb;
-                    sl.cc = w.ct * d.pc;
-                    sl.nbx = w.boxes ? w.N / (2 * PACK_ROWS) : 1;
-                    sl.stage_tx = w.boxes ? 2u * (2u * PAIR_A + 2u * (uint32_t)(w.N / (2 * PACK_ROWS) * PACK_BOX_BYTES))
-                                          : d.stage_tx;
-                    sl.boxes = w.boxes;
-                    sl.pc = d.pc;
-                    sl.packed = w.packed;
-                    sl.empty = w.empty;
-                    sl.g = w.g;
-                    sl.pass0 = w.pass0;
-                    sl.ncol = w.ncol;
-                }
-                if (!w.boxes) {
-                    if (lane == 0)
-                        sl.box[0] = make_int2(w.packed ? pc.ents[w.ent0].s : w.s, w.pass0 + (int)rank * (w.N / 2));
-                } else if (lane < PACK_BOXES) {
-                    const int x = (int)rank * (w.N / 2) + PACK_ROWS * lane;  // column in the pass
-                    int2 e = make_int2(-1, 0);
-                    if (x < w.ncol && lane < w.N / (2 * PACK_ROWS)) {
-                        const int col = w.pass0 + x, m = col / d.packw;
-                        e = make_int2(pc.ents[w.ent0 + m].s, col - m * d.packw);
-                    }
-                    sl.box[lane] = e;
-                }
-                if (w.packed) {
-                    int2 e = make_int2(0, 1 << 20);
-                    if (8 * lane < w.ncol) {
-                        const int col = w.pass0 + 8 * lane, m = col / d.packw;
-                        e = make_int2(pc.ents[w.ent0 + m].tbg, col - m * d.packw);
-                    }
-                    sl.ent[lane] = e;
-                }
-            }
-            if (lane == 0) sl.end = end;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bar_sfull[n % PAIR_SLOTS]));
-            if (end) break;
-            n++;
-        }
+        pair_scheduler(wv, cid, ncl, rank, slots, bar_sfull, bar_sempty, &abort_sh, peer_abort);
     } else {
         const int wq = warp & 3;
         const int half = (warp - 2) >> 2;
@@ -805,7 +598,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_tc_pair_kernel(const __
                     const int B = b >> 3, C = c >> 3;
                     const bool in = b < v && c < v;
                     const int64_t ug3 = sl.ug3;
-                    float *Ui = sl.U + ucube_off(0, b & 7, c & 7);
+                    float *Ui = static_cast<float *>(wv.U) + sl.u_off + ucube_off(0, b & 7, c & 7);
                     const int2 *ent = sl.ent + half * nld * 4;
 #pragma unroll
                     for (int k = 0; k < 16; k++) {
@@ -821,7 +614,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_tc_pair_kernel(const __
                     }
                 } else if (b < v && c < v) {
                     const int a0 = sl.pass0 + half * nld * 32;  // a multiple of 8
-                    store_u_cubes(sl.U, nb, sl.g, a0, b, c, min(nld * 32, sl.pass0 + sl.ncol - a0), total);
+                    store_u_cubes(static_cast<float *>(wv.U) + sl.u_off, nb, sl.g, a0, b, c, min(nld * 32, sl.pass0 + sl.ncol - a0), total);
                 }
             }
             __syncwarp();
@@ -957,35 +750,6 @@ cudaError_t tc_prepare(int) {
     return e;
 }
 
-// Co-resident 2-CTA clusters of the pair kernel on the current device (one
-// per SM pair that the cluster scheduler can place), queried once per device.
-static int pair_clusters(int sm_count) {
-    static std::mutex mu;
-    static int cache[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count / 2;
-    std::lock_guard<std::mutex> lk(mu);
-    if (cache[dev] > 0) return cache[dev];
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(sm_count / 2 * 2), 1, 1);
-    cfg.blockDim = dim3(PAIR_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, ugemm_tc_pair_kernel, &cfg) != cudaSuccess || n < 1) {
-        cudaGetLastError();
-        n = sm_count / 2;
-    }
-    cache[dev] = std::min(n, sm_count / 2);
-    return cache[dev];
-}
-
 cudaError_t launch_ugemm_tc(int prec, int sm_count, const Wave &w, cudaStream_t st, bool pair) {
     if (w.n_gemm <= 0) return cudaSuccess;
     if (w.tc_brows < 16 || w.tc_brows > BN || w.tc_brows % (pair ? 32 : 16) != 0) return cudaErrorInvalidValue;
@@ -996,22 +760,8 @@ cudaError_t launch_ugemm_tc(int prec, int sm_count, const Wave &w, cudaStream_t 
         ugemm_tc_kernel<<<grid, TC_THREADS, SMEM_BYTES, st>>>(w);
         return cudaGetLastError();
     }
-    const int ncl = (int)std::min<int64_t>(pair_clusters(sm_count), w.n_gemm);
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(2 * ncl), 1, 1);
-    cfg.blockDim = dim3(PAIR_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, ugemm_tc_pair_kernel, w);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    static PairLaunch pl;
+    return pl.launch(ugemm_tc_pair_kernel, PAIR_THREADS, SMEM_BYTES, sm_count, w.n_gemm, st, w);
 }
 
 }  // namespace tcorr
