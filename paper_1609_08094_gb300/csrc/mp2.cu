@@ -237,7 +237,62 @@ struct tcorr_mp2_s {
     void *ct_hi = nullptr, *ct_lo = nullptr;
     float *eps_vf = nullptr;
     Mp2TcArgs tc{};
+    // Gram form: waves of at most MP2_GRAM_BYTES of g
+    bool gram = false;
+    Mp2GramArgs gr{};
+    std::vector<Mp2Wave> waves;
 };
+
+namespace {
+
+// The Gram form of the split precisions keeps g of a wave in scratch: at most
+// MP2_GRAM_BYTES, which holds at least one pair up to v = MP2_GRAM_MAX_V.
+constexpr int64_t MP2_GRAM_BYTES = (int64_t)1 << 30;
+constexpr int MP2_GRAM_MAX_V = 8192;
+
+// Waves over the pairs i <= j (pair list lexicographic, so that each wave's
+// pairs are consecutive): ni values of i with every j >= the first of them, or
+// one i with some j; and their tiles, skipping those left of the pairs i <= j.
+void mp2_plan_waves(int o, int v, int sm_count, std::vector<Mp2Wave> &waves, std::vector<int2> &tiles, int64_t &g_floats,
+                    int64_t &nparts) {
+    const int64_t cap = MP2_GRAM_BYTES / 4;
+    g_floats = nparts = 0;
+    auto pair_index = [&](int64_t i, int64_t j) { return i * o - i * (i - 1) / 2 + (j - i); };
+    for (int i0 = 0; i0 < o;) {
+        const int64_t row = (int64_t)v * round_up((o - i0) * v, 8);  // floats of one i with every j >= i0
+        const int ni = (int)std::min<int64_t>(o - i0, std::max<int64_t>(1, cap / row));
+        const int nj = row <= cap ? o - i0 : (int)std::max<int64_t>(1, cap / ((int64_t)v * v) - 1);
+        for (int j0 = i0; j0 < o; j0 += nj) {
+            const int j1 = std::min(o, j0 + nj);
+            Mp2Wave w{};
+            w.row0 = (int64_t)i0 * v;
+            w.col0 = (int64_t)j0 * v;
+            w.nrows = ni * v;
+            w.ncols = (j1 - j0) * v;
+            w.ld = round_up(w.ncols, 8);
+            w.tile0 = (int)tiles.size();
+            const int nr = (w.nrows + MP2_GRAM_TILE - 1) / MP2_GRAM_TILE, nc = (w.ncols + MP2_GRAM_TILE - 1) / MP2_GRAM_TILE;
+            // eight row tiles at a time, so that the tiles computed together share
+            // their rows of X in L2
+            for (int r0 = 0; r0 < nr; r0 += 8)
+                for (int c = 0; c < nc; c++)
+                    for (int r = r0; r < std::min(nr, r0 + 8); r++) {
+                        const int64_t last = std::min<int64_t>((int64_t)(c + 1) * MP2_GRAM_TILE, w.ncols) - 1;
+                        if ((w.col0 + last) / v >= (w.row0 + (int64_t)r * MP2_GRAM_TILE) / v) tiles.push_back(make_int2(r, c));
+                    }
+            w.ntile = (int)tiles.size() - w.tile0;
+            w.pair0 = pair_index(i0, j0);
+            w.npair = (int)(ni == 1 ? j1 - j0 : pair_index(i0 + ni - 1, o - 1) + 1 - w.pair0);
+            w.part0 = (int)nparts;
+            nparts += mp2_energy_ctas(sm_count, v, w.npair);
+            g_floats = std::max(g_floats, (int64_t)w.nrows * w.ld);
+            waves.push_back(w);
+        }
+        i0 += ni;
+    }
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -297,10 +352,14 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
         if (h->items > 0x7fffffff) throw Fail{TCORR_EUNSUPPORTED, "too many work items"};
         // partials: one per item (FP64 kernel) or one per persistent CTA (tensor-core kernel)
         h->nparts = split ? std::min<int64_t>(ex.sm_count, h->items) : h->items;
+        std::vector<int2> gram_tiles;
+        int64_t g_floats = 0;
+        h->gram = split && v <= MP2_GRAM_MAX_V;
+        if (h->gram) mp2_plan_waves(o, v, ex.sm_count, h->waves, gram_tiles, g_floats, h->nparts);
         const size_t ct_bytes = (size_t)o * v * h->kp * elem_bytes(op.prec) * (split ? 2 : 1);  // hi + lo
         size_t free_b = 0, total_b = 0;
         CK(cudaMemGetInfo(&free_b, &total_b));
-        const size_t need = ct_bytes + (size_t)h->nparts * 16 + (op.host_inputs ? (size_t)o * v * naux * 8 : 0) +
+        const size_t need = ct_bytes + (size_t)h->nparts * 16 + (size_t)g_floats * 4 + (op.host_inputs ? (size_t)o * v * naux * 8 : 0) +
                             ((size_t)64 << 20);
         if (need > free_b)
             throw Fail{TCORR_ENOMEM, "footprint " + std::to_string(need) + " bytes exceeds free device memory"};
@@ -362,8 +421,25 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
             a.ntp = h->ntp;
             a.items = h->items;
             std::string err;
-            if (mp2_tc_fill(a, op.prec, h->ct_hi, h->ct_lo, o, v, h->kp, err) != cudaSuccess)
+            if (h->gram) {
+                Mp2GramArgs &g = h->gr;
+                g.pairs = h->pairs;
+                g.eps_o = h->eps_o;
+                g.eps_v = h->eps_v;
+                g.eps_vf = h->eps_vf;
+                g.partials = h->partials;
+                g.err = ex.err;
+                g.v = v;
+                int2 *tl2 = nullptr;
+                dalloc(ex, tl2, gram_tiles.size() * sizeof(int2));
+                CK(cudaMemcpy(tl2, gram_tiles.data(), gram_tiles.size() * sizeof(int2), cudaMemcpyHostToDevice));
+                g.tiles = tl2;
+                dalloc(ex, g.g, (size_t)g_floats * sizeof(float));
+                if (mp2_gram_fill(g, op.prec, h->ct_hi, h->ct_lo, o, v, h->kp, err) != cudaSuccess)
+                    throw Fail{TCORR_ECUDA, err};
+            } else if (mp2_tc_fill(a, op.prec, h->ct_hi, h->ct_lo, o, v, h->kp, err) != cudaSuccess) {
                 throw Fail{TCORR_ECUDA, err};
+            }
         }
         CK(cudaStreamSynchronize(ex.stream));
         resolve_timers(ex);
@@ -399,6 +475,11 @@ tcorr_status tcorr_mp2_energy(tcorr_mp2_t h, double *e_out) {
                 Mp2Args a{h->Ct, h->eps_o, h->eps_v, h->pairs, h->tiles, h->v, h->kp, h->ntp, h->partials};
                 mp2_pair_kernel<<<(unsigned)h->items, MNT, 0, ex.stream>>>(a);
                 CK(cudaGetLastError());
+            } else if (h->gram) {
+                for (const Mp2Wave &w : h->waves) {
+                    CK(launch_mp2_gram(ex.prec, ex.sm_count, h->gr, w, ex.stream));
+                    CK(launch_mp2_energy(ex.sm_count, h->gr, w, ex.stream));
+                }
             } else {
                 CK(launch_mp2_tc(ex.prec, ex.sm_count, h->tc, ex.stream));
             }

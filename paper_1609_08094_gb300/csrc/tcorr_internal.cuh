@@ -96,7 +96,7 @@ struct InstDesc {
     int packw;                // SM pairs, packed columns (PackRun): columns per entry (v rounded to 16), 0: not packed
     uint32_t stage_tx;        // TMA bytes per pipeline stage
     int norb;                 // epilogue block orbits per task (cube edge 8)
-    const int *oz_e;          // FP64 emulation: device [2] scale exponents of the A and B operand sides
+    const int *oz_e;          // FP64 emulation (else NULL): device [2] scale exponents of the A and B operand sides
     const void *G, *T2K, *T2R, *AoN;  // FP64 operand layouts (FP64 W contractions)
     const double *eps_o, *eps_v;
     const void *t1, *ovov;    // epilogue copies: FP64, float-float pairs (FP64 emulation) or FP32
@@ -255,6 +255,33 @@ struct Mp2TcArgs {
     int v, nch, ntp;          // nch: K chunks of 64 bytes (set by mp2_tc_fill)
     int64_t items;            // npair * ntp
 };
+// A block of the problem whose g values are formed by one launch and stored:
+// rows (i, a) of an occupied range, columns (j, b) of another, flattened as
+// i v + a and j v + b.
+struct Mp2Wave {
+    int64_t row0, col0;       // first row and column
+    int nrows, ncols, ld;     // extents; row stride of g (floats, a multiple of 8)
+    int tile0, ntile;         // its 256 x 256 tiles in the tile list
+    int64_t pair0;            // its pairs (i, j) in the pair list
+    int npair;
+    int part0;                // first partial of its energy CTAs
+};
+struct Mp2GramArgs {
+    CUtensorMap map[2];       // hi, lo planes of C^T as [o v][kp] (K-major), box {two chunks, 128}
+    const int2 *tiles;        // (row tile, column tile) of every wave, tiles of MP2_GRAM_TILE
+    const int *pairs;         // [npair][2], i <= j
+    const double *eps_o, *eps_v;
+    const float *eps_vf;      // eps_v rounded to FP32
+    float *g;                 // the wave's block
+    double *partials;         // [.][2]: (E_J, E_K) of each energy CTA, pair weights applied
+    int *err;                 // DERR_* flags of bounded waits that expired
+    int v, nblk;              // nblk: K blocks of two chunks (set by mp2_gram_fill)
+};
+constexpr int MP2_GRAM_TILE = 256;
+cudaError_t mp2_gram_fill(Mp2GramArgs &a, int prec, void *hi, void *lo, int o, int v, int kp, std::string &err);
+cudaError_t launch_mp2_gram(int prec, int sm_count, const Mp2GramArgs &a, const Mp2Wave &w, cudaStream_t st);
+int mp2_energy_ctas(int sm_count, int v, int npair);  // partial pairs of a wave
+cudaError_t launch_mp2_energy(int sm_count, const Mp2GramArgs &a, const Mp2Wave &w, cudaStream_t st);
 // Encodes the two operand maps of the planes hi / lo ([o][v][kp], TF32 or BF16)
 // and sets a.nch; kp must be a multiple of the chunk (16 TF32, 32 BF16 values).
 cudaError_t mp2_tc_fill(Mp2TcArgs &a, int prec, void *hi, void *lo, int o, int v, int kp, std::string &err);
