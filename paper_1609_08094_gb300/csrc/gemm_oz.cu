@@ -528,6 +528,7 @@ cudaError_t oz_fill_desc(InstDesc &d, const Operands &op, const int *exps, std::
     d.nbt = (v + pb - 1) / pb;
     d.nct = (v + pc - 1) / pc;
     d.pair = 1;
+    d.tblk = pair_task_block(v, dp, OZ_S * eb);
     // passes of equal width, a multiple of 16: each CTA holds half of the columns
     d.npass = (v + OZ_N - 1) / OZ_N;
     d.brows = round_up((v + d.npass - 1) / d.npass, 16);

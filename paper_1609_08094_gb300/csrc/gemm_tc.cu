@@ -658,6 +658,7 @@ cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int 
     d.kb = kb;
     d.kind = tf ? 1 : 2;
     d.pair = pair ? 1 : 0;
+    d.tblk = pair_task_block(v, dp, 2 * eb);
     d.nbt = (v + pb - 1) / pb;
     d.nct = (v + pc - 1) / pc;
     d.npass = (v + BN - 1) / BN;

@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(MP_THREADS, 1) mp2_tc_kernel(const __grid_cons
 // computes G and H = G^T of diagonal tiles, and takes in 128 KB per K block for
 // the same tensor work: at o=50, v=450, naux=1500 it forms 4.2e8 products x naux
 // against 2.6e8.  There, in BF16X3, the tile-pair kernel took 3.71 ms; the Gram
-// tiles take 1.62 ms (1.25 PFLOP/s of the four products) and the energy pass 0.54.
+// tiles take 1.62 ms (1.88 PFLOP/s of the four products) and the energy pass 0.54.
 // g goes to a scratch of at most 1 GiB (one wave per so much of
 // the problem) in FP32, as the register totals hold it, and the energy kernel
 // reads the two tiles (i, A) x (j, B) and (i, B) x (j, A) that hold g_ab and g_ba.  The accumulation (four products, fresh accumulator per K block,

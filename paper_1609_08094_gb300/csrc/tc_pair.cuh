@@ -28,6 +28,7 @@ struct PairCache {
     const PackRun *runs;
     const PackEnt *ents;
     int nrun, r, r_end;  // cached run and the unit after its last
+    int ntb, tblk;       // tasks of the segment, and of a block
     PackRun run;
 };
 __device__ __forceinline__ void pair_reset(PairCache &c) { seg_reset(c.s); }
@@ -56,6 +57,9 @@ __device__ __forceinline__ PairItem decode_pair(const Wave &w, int64_t it, PairC
         c.runs = sg.runs;
         c.ents = sg.ents;
         c.nrun = sg.nrun;
+        c.ntb = sg.ntb;
+        const int nblk = (c.ntb + d.tblk - 1) / d.tblk;
+        c.tblk = (c.ntb + nblk - 1) / nblk;  // equal blocks
         c.r = 0;
         c.r_end = -1;
     }
@@ -93,13 +97,21 @@ __device__ __forceinline__ PairItem decode_pair(const Wave &w, int64_t it, PairC
         r.tb = r.g = r.s = 0;
         r.diag = false;  // the tables hold no group of a task i = j = k
     } else {
-        int64_t x = it - c.s.begin;
-        const int n = (int)(x % c.s.npass);  // N pass fastest, then group, then tile pair (as decode)
-        x /= c.s.npass;
-        r.g = (int)(x % 3);
-        x /= 3;
-        tp = (int)(x % npair);
-        r.tb = (int)(x / npair);
+        // N pass fastest, then group, then the tasks of a block, then tile pair: the
+        // tasks of a block are neighbours (i, j, k), (i, j, k + 1), ..., whose groups
+        // read the same tiles of G[i] and G[j] (two groups of a task also of G[k]),
+        // and the block's rows of B stay in L2 (pair_task_block)
+        const int64_t x = it - c.s.begin;
+        const int per = 3 * c.s.npass;  // items of a task at one tile pair
+        const int64_t blk = x / ((int64_t)per * npair * c.tblk);
+        const int nt = (int)min((int64_t)c.tblk, c.ntb - blk * c.tblk);
+        const int l = (int)(x - blk * c.tblk * npair * per);
+        tp = l / (nt * per);
+        int y = l - tp * nt * per;
+        const int n = y % c.s.npass;
+        y /= c.s.npass;
+        r.g = y % 3;
+        r.tb = (int)(blk * c.tblk) + y / 3;
         if (r.tb != c.s.tcached) {
             const int *tk = d.tasks + 3 * (c.s.task0 + r.tb);
             c.s.ti = tk[0];
@@ -232,6 +244,14 @@ __device__ __forceinline__ void pair_scheduler(const Wave &wv, uint32_t cid, uin
         if (end) break;
         n++;
     }
+}
+
+// Tasks per block of the item order: so many that the rows of T2R they read
+// (four blocks [v][dp] per task that its neighbours do not) take at most 40 MB of
+// the 126 MB L2, which A and U stream through.
+inline int pair_task_block(int v, int dp, size_t bytes_per_value) {
+    const int64_t per_task = 4 * (int64_t)v * dp * (int64_t)bytes_per_value;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(64, ((int64_t)40 << 20) / per_task));
 }
 
 // Launch of a pair kernel on as many 2-CTA clusters as are co-resident (one

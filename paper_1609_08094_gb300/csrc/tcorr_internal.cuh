@@ -93,6 +93,7 @@ struct InstDesc {
     int kind;                 // split-precision operand type: 1 = TF32, 2 = BF16 hi + lo
     int pair;                 // tensor-core tiles on SM pairs (cta_group::2, M = 256)
     int nbt, nct, npass, kv, ko, brows;
+    int tblk;                 // SM pairs: tasks that go through the tile pairs together (tc_pair.cuh)
     int packw;                // SM pairs, packed columns (PackRun): columns per entry (v rounded to 16), 0: not packed
     uint32_t stage_tx;        // TMA bytes per pipeline stage
     int norb;                 // epilogue block orbits per task (cube edge 8)
