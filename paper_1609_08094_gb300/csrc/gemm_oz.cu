@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_oz_kernel(const __grid_
     }
 }
 
-// ---- slicing ------------------------------------------------------------------------
+// ---- scales ------------------------------------------------------------------------
 // Max |x| over n doubles: non-negative doubles order like their bit patterns.
 __global__ void maxabs_kernel(const double *__restrict__ x, int64_t n, unsigned long long *out) {
     unsigned long long m = 0;
@@ -439,52 +439,6 @@ __global__ void seed_max_kernel(unsigned long long *m, double x) {
     if (threadIdx.x == 0 && blockIdx.x == 0) atomicMax(m, (unsigned long long)__double_as_longlong(fabs(x)));
 }
 
-// out[p][b][c][r] = slice p of scale * in[b*sb + r*sr + c*sc] (r < R), zero for R <= r < Rp,
-// with scale = sign * 2^-e[0] read on the device.
-// Slices: y = scale * x (|y| <= 1 by choice of scale); for p = 0..S-1:
-// y *= 2^beta, a = rint(y), y -= a; all steps exact in FP64.
-constexpr int ST = 32;
-__global__ void __launch_bounds__(256) slice_pad_kernel(const double *__restrict__ in, __nv_bfloat16 *__restrict__ out,
-                                                        int64_t B, int R, int Rp, int64_t C, int64_t sb, int64_t sr,
-                                                        int64_t sc, int64_t ob, int64_t oc, int64_t plane,
-                                                        const int *e, double sign) {
-    __shared__ double tile[ST][ST + 1];
-    const double scale = sign * ldexp(1.0, -e[0]);
-    const int64_t ntc = (C + ST - 1) / ST, ntr = (Rp + ST - 1) / ST;
-    const int64_t ntiles = B * ntc * ntr;
-    for (int64_t tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
-        const int64_t b = tl / (ntc * ntr);
-        const int64_t rem = tl % (ntc * ntr);
-        const int64_t c0 = (rem / ntr) * ST;
-        const int r0 = (int)(rem % ntr) * ST;
-        // load: threads along c when sc == 1, else along r (coalesced either way for the layouts used)
-        for (int e = threadIdx.y; e < ST; e += blockDim.y) {
-            const int64_t cidx = sc == 1 ? c0 + threadIdx.x : c0 + e;
-            const int ridx = sc == 1 ? r0 + e : r0 + threadIdx.x;
-            double x = 0.0;
-            if (cidx < C && ridx < R) x = in[b * sb + (int64_t)ridx * sr + cidx * sc];
-            if (sc == 1) tile[e][threadIdx.x] = x; else tile[threadIdx.x][e] = x;
-        }
-        __syncthreads();
-        for (int e = threadIdx.y; e < ST; e += blockDim.y) {
-            const int64_t cidx = c0 + e;
-            const int ridx = r0 + threadIdx.x;
-            if (cidx < C && ridx < Rp) {
-                double y = tile[threadIdx.x][e] * scale;
-                const int64_t o = b * ob + cidx * oc + ridx;
-#pragma unroll
-                for (int p = 0; p < OZ_S; p++) {
-                    y *= (double)(1 << OZ_BETA);
-                    const double a = rint(y);
-                    y -= a;
-                    out[p * plane + o] = __double2bfloat16(a);
-                }
-            }
-        }
-        __syncthreads();
-    }
-}
-
 }  // namespace
 
 int oz_slices() { return OZ_S; }
@@ -503,17 +457,6 @@ cudaError_t launch_oz_exponents(const unsigned long long *m, int *e, cudaStream_
 
 cudaError_t launch_seed_max(unsigned long long *m, double x, cudaStream_t st) {
     seed_max_kernel<<<1, 32, 0, st>>>(m, x);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_slice_pad(const double *in, void *out, int64_t B, int R, int Rp, int64_t C, int64_t sb,
-                             int64_t sr, int64_t sc, int64_t ob, int64_t oc, int64_t plane, const int *e,
-                             double sign, cudaStream_t st) {
-    const int64_t ntiles = B * ((C + ST - 1) / ST) * ((Rp + ST - 1) / ST);
-    if (ntiles == 0) return cudaSuccess;
-    const unsigned grid = (unsigned)(ntiles < ((int64_t)1 << 22) ? ntiles : ((int64_t)1 << 22));
-    slice_pad_kernel<<<grid, dim3(ST, 8), 0, st>>>(in, static_cast<__nv_bfloat16 *>(out), B, R, Rp, C, sb, sr, sc,
-                                                   ob, oc, plane, e, sign);
     return cudaGetLastError();
 }
 

@@ -387,8 +387,9 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
             // hi and lo planes in TF32 or BF16)
             Timer tm(ex, KC_PREP);
             const int kind = op.prec == TCORR_TF32X3 ? 1 : (op.prec == TCORR_BF16X3 ? 2 : 0);
-            CK(launch_transpose_pad(kind, dC, split ? h->ct_hi : h->Ct, split ? h->ct_lo : nullptr, o, naux, h->kp,
-                                    v, 1, (int64_t)v * o, o, (int64_t)v * h->kp, h->kp, 1.0, ex.stream));
+            CK(launch_transpose_rows(kind, dC, split ? h->ct_hi : h->Ct, split ? h->ct_lo : nullptr, 0, nullptr, false, 1,
+                                     naux, h->kp, (int64_t)v * o, 0, (int64_t)v * o, 0, o, (int64_t)v * h->kp, h->kp,
+                                     ex.stream));
             tm.stop();
         }
         free_tmp(ex, tmp, (size_t)o * v * naux);

@@ -5,12 +5,12 @@
 // the paper's dgemm -> sgemm swap of Sec. 3).
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "tcorr_internal.cuh"
 
 namespace tcorr {
 namespace {
-
-constexpr int TT = 32;  // transpose tile edge
 
 __device__ __forceinline__ float tf32_rn(float x) {
     uint32_t r;
@@ -18,54 +18,192 @@ __device__ __forceinline__ float tf32_rn(float x) {
     return __uint_as_float(r & 0xFFFFE000u);  // TF32 keeps 10 mantissa bits
 }
 
-template <int KIND>
-__device__ __forceinline__ void store_split(void *hi, void *lo, int64_t idx, double x) {
-    if constexpr (KIND == 0) {
-        static_cast<double *>(hi)[idx] = x;
-    } else if constexpr (KIND == 1) {
-        const float h = tf32_rn(static_cast<float>(x));
-        const float l = tf32_rn(static_cast<float>(x - static_cast<double>(h)));
-        static_cast<float *>(hi)[idx] = h;
-        static_cast<float *>(lo)[idx] = l;
+// Where the values of one output row go: kind 0: hi as FP64; 1, 2: hi and lo planes
+// in TF32 (float) or BF16; 3: OZ_PLANES BF16 slice planes `plane` values apart.
+struct RowOut {
+    void *hi, *lo;
+    int64_t plane;
+    const int *e;      // kind 3: the scale exponent, on the device
+    int neg;           // every value with its sign flipped
+};
+constexpr int OZ_PLANES = 5, OZ_BITS = 7;
+__device__ __forceinline__ double flip(double x, int neg) {
+    return __hiloint2double(__double2hiint(x) ^ (neg << 31), __double2loint(x));
+}
+
+// T = x 2^(35 - E) rounded to an integer (half to even) and its digits a_1 .. a_5,
+// a_p = round half to even of what the digits before leave, times 2^7 each.  The
+// same T as from five steps y *= 2^7, a = rint(y), y -= a on y = x 2^-E (the digits
+// differ only where one of those lies within 2^-29 of a tie), on the integer pipe:
+// FP64 arithmetic runs at 1/64 of its rate, and 15 operations per value bounded
+// the pass (o=40, v=300, all layouts: 77.8 ms, now 11.3).
+__device__ __forceinline__ int64_t shift_even(int64_t t, int s) {  // t / 2^s, half to even, 1 <= s <= 62
+    return (t + (((int64_t)1 << (s - 1)) - 1) + ((t >> s) & 1)) >> s;
+}
+__device__ __forceinline__ int64_t oz_fixed(double x, int e) {
+    const int64_t bits = __double_as_longlong(x);
+    const int ex = (int)((bits >> 52) & 0x7ff);
+    const int s = 1075 - 35 + e - ex;
+    // zero and values below any digit; s < 1 is no finite value of this side
+    if (ex == 0 || s > 60 || s < 1) return 0;
+    const int64_t m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
+    // |x| = m 2^(ex - 1075) < 2^e: T = m 2^-s, s >= 18
+    const int64_t t = shift_even(m, s);
+    return bits < 0 ? -t : t;
+}
+
+// x = a + b with a the top 24 bits of x and b the other 29, cut to 23 with the last
+// one sticky, from the bits of x: the FP64 pipe (1/64 of the FP32 rate) bounded
+// this pass when the split was done with FP64 conversions and subtractions (o=50,
+// v=450 in BF16: 55 ms).  False (a and b unset) for zero and for exponents where b
+// would leave FP32's normal range.
+__device__ __forceinline__ bool fp32_parts(double x, float &a, float &b) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int ex = (int)((hi >> 20) & 0x7ff) - 1023;
+    if (ex < -100 || ex > 126) return false;
+    const uint32_t sign = hi & 0x80000000u, rest = lo & 0x1fffffffu;
+    a = __uint_as_float(sign | (uint32_t)(ex + 127) << 23 | (hi & 0xfffffu) << 3 | lo >> 29);
+    const uint32_t base = sign | (uint32_t)(ex + 104) << 23;  // +-2^(ex - 23)
+    b = __uint_as_float(base | rest >> 6 | ((rest & 63u) != 0)) - __uint_as_float(base);
+    return true;
+}
+// x = h + l in TF32: h = x rounded to FP32, then to TF32 (ties away); l = x - h likewise
+__device__ __forceinline__ void split_tf32(double x, float &h, float &l) {
+    float a, b;
+    if (fp32_parts(x, a, b)) {
+        h = tf32_rn(a + b);
+        l = tf32_rn((a - h) + b);  // a - h is exact
     } else {
-        const __nv_bfloat16 h = __double2bfloat16(x);
-        const __nv_bfloat16 l = __double2bfloat16(x - static_cast<double>(__bfloat162float(h)));
-        static_cast<__nv_bfloat16 *>(hi)[idx] = h;
-        static_cast<__nv_bfloat16 *>(lo)[idx] = l;
+        h = tf32_rn(static_cast<float>(x));
+        l = tf32_rn(static_cast<float>(x - static_cast<double>(h)));
+    }
+}
+// x = h + l in BF16, each rounded to nearest even
+__device__ __forceinline__ void split_bf16(double x, __nv_bfloat16 &h, __nv_bfloat16 &l) {
+    float a, b;
+    if (fp32_parts(x, a, b)) {
+        // the rest as a sticky last bit of a: one rounding, as from FP64
+        h = __float2bfloat16_rn(b != 0.f ? __uint_as_float(__float_as_uint(a) | 1u) : a);
+        // x - h = s + b rounded to odd in FP32 (t + err exact), then once to BF16
+        const float s = a - __bfloat162float(h), t = s + b, err = b - (t - s);
+        uint32_t u = __float_as_uint(t);
+        if (err != 0.f) u = (((__float_as_uint(err) ^ u) >> 31) ? u - 1 : u) | 1u;
+        l = __float2bfloat16_rn(__uint_as_float(u));
+    } else {
+        h = __double2bfloat16(x);
+        l = __double2bfloat16(x - static_cast<double>(__bfloat162float(h)));
     }
 }
 
-// One CTA (32 x 8 threads) moves a TT x TT tile: rows r (output-contiguous),
-// columns c (input-contiguous when sc = 1).  Tiles are enumerated flat over
-// (b, c-tile, r-tile) in blockIdx.x (64-bit safe through a grid-stride loop).
+// One value of an output row, and two neighbouring ones (idx even)
 template <int KIND>
-__global__ void __launch_bounds__(256) transpose_pad_kernel(
-    const double *__restrict__ in, void *out_hi, void *out_lo, int64_t B, int R, int Rp,
-    int64_t C, int64_t sb, int64_t sr, int64_t sc, int64_t ob, int64_t oc, double scale) {
-    __shared__ double tile[TT][TT + 1];
-    const int64_t nct = (C + TT - 1) / TT;
-    const int64_t nrt = (Rp + TT - 1) / TT;
-    const int64_t ntiles = B * nct * nrt;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t rt = t % nrt;
-        const int64_t ct = (t / nrt) % nct;
-        const int64_t b = t / (nrt * nct);
-        const int64_t r0 = rt * TT, c0 = ct * TT;
-        // load: column c0+tx, rows r0+ty+8m
-        for (int m = 0; m < TT; m += 8) {
-            const int64_t r = r0 + ty + m, c = c0 + tx;
-            double x = 0.0;
-            if (r < R && c < C) x = scale * in[b * sb + r * sr + c * sc];
-            tile[ty + m][tx] = x;
+__device__ __forceinline__ void store_one(const RowOut &o, int e, int64_t idx, double x) {
+    if constexpr (KIND == 0) {
+        static_cast<double *>(o.hi)[idx] = x;
+    } else if constexpr (KIND == 1) {
+        split_tf32(x, static_cast<float *>(o.hi)[idx], static_cast<float *>(o.lo)[idx]);
+    } else if constexpr (KIND == 2) {
+        split_bf16(x, static_cast<__nv_bfloat16 *>(o.hi)[idx], static_cast<__nv_bfloat16 *>(o.lo)[idx]);
+    } else {
+        int64_t t = oz_fixed(x, e);
+#pragma unroll
+        for (int p = 0; p < OZ_PLANES; p++) {
+            const int s = OZ_BITS * (OZ_PLANES - 1 - p);
+            const int64_t a = s ? shift_even(t, s) : t;
+            t -= a << s;
+            static_cast<__nv_bfloat16 *>(o.hi)[idx + p * o.plane] = __float2bfloat16_rn(static_cast<float>(static_cast<int>(a)));
+        }
+    }
+}
+template <int KIND>
+__device__ __forceinline__ void store_pair(const RowOut &o, int e, int64_t idx, double x0, double x1) {
+    if constexpr (KIND == 0) {
+        *reinterpret_cast<double2 *>(static_cast<double *>(o.hi) + idx) = make_double2(x0, x1);
+    } else if constexpr (KIND == 1) {
+        float2 h, l;
+        split_tf32(x0, h.x, l.x);
+        split_tf32(x1, h.y, l.y);
+        *reinterpret_cast<float2 *>(static_cast<float *>(o.hi) + idx) = h;
+        *reinterpret_cast<float2 *>(static_cast<float *>(o.lo) + idx) = l;
+    } else if constexpr (KIND == 2) {
+        __nv_bfloat162 h, l;
+        split_bf16(x0, h.x, l.x);
+        split_bf16(x1, h.y, l.y);
+        *reinterpret_cast<__nv_bfloat162 *>(static_cast<__nv_bfloat16 *>(o.hi) + idx) = h;
+        *reinterpret_cast<__nv_bfloat162 *>(static_cast<__nv_bfloat16 *>(o.lo) + idx) = l;
+    } else {
+        int64_t t0 = oz_fixed(x0, e), t1 = oz_fixed(x1, e);
+        __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(o.hi) + idx;
+#pragma unroll
+        for (int p = 0; p < OZ_PLANES; p++) {
+            const int s = OZ_BITS * (OZ_PLANES - 1 - p);
+            const int64_t a0 = s ? shift_even(t0, s) : t0, a1 = s ? shift_even(t1, s) : t1;
+            t0 -= a0 << s;
+            t1 -= a1 << s;
+            __nv_bfloat162 d;
+            d.x = __float2bfloat16_rn(static_cast<float>(static_cast<int>(a0)));
+            d.y = __float2bfloat16_rn(static_cast<float>(static_cast<int>(a1)));
+            *reinterpret_cast<__nv_bfloat162 *>(out + p * o.plane) = d;
+        }
+    }
+}
+
+// Rows r of the input become the innermost index of the output:
+//   out[b ob + (c % m) s1 + (c / m) s2 + r] = conv(+-in[b sb + r sr + c]),
+// r < R, zero for R <= r < Rp (Rp even, or the last r of a row without padding).
+// A CTA takes 32 neighbouring c (256-byte reads) and all r (or, where there are few
+// c, some: gridDim.y), 64 at a time through shared memory; each output row gets
+// runs of 64 r.  All layouts of o=50, v=450 (45 GB in, 22 GB out in BF16) took 97 ms
+// when each (x, y) was a transpose of its own d x q with q in 32-wide tiles, after a
+// pass that zeroed the output, and take 23 ms; in FP64 61 and 19 ms.
+constexpr int TC = 32, TR = 64;
+template <int KIND>
+__global__ void __launch_bounds__(256) transpose_rows_kernel(const double *__restrict__ in, const RowOut o, int R, int Rp,
+                                                             int64_t C, int64_t sb, int64_t sr, int64_t ob, uint32_t m,
+                                                             int64_t s1, int64_t s2, int odd) {
+    __shared__ __align__(16) double tile[TC][TR + 2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t nct = (C + TC - 1) / TC;
+    const int e = KIND == 3 ? o.e[0] : 0;
+    const int64_t b = blockIdx.x / nct, c0 = (blockIdx.x - b * nct) * TC;
+    const double *src = in + b * sb + c0 + lane;
+    const bool c_in = c0 + lane < C;
+    for (int r0 = blockIdx.y * TR; r0 < Rp; r0 += gridDim.y * TR) {
+        const int nr = min(TR, Rp - r0);
+#pragma unroll
+        for (int k = 0; k < TR / 8; k++) {
+            const int r = r0 + warp + 8 * k;
+            if (warp + 8 * k < nr) tile[lane][warp + 8 * k] = c_in && r < R ? flip(src[(int64_t)r * sr], o.neg) : 0.0;
         }
         __syncthreads();
-        // store: row c0+ty+8m of the output, element r0+tx
-        for (int m = 0; m < TT; m += 8) {
-            const int64_t c = c0 + ty + m, r = r0 + tx;
-            if (c < C && r < Rp) store_split<KIND>(out_hi, out_lo, b * ob + c * oc + r, tile[tx][ty + m]);
+        // lanes along r, two values each: 8, 16 or 32 lanes per output row
+        const int sh = nr <= 16 ? 3 : (nr <= 32 ? 4 : 5);
+        const int r = 2 * (threadIdx.x & ((1 << sh) - 1));
+        for (int cc = threadIdx.x >> sh; cc < TC; cc += 256 >> sh) {
+            const int64_t c = c0 + cc;
+            if (c >= C || r >= nr) continue;
+            const int64_t row = b * ob + (m == 1 ? c * s2 : (int64_t)((uint32_t)c % m) * s1 + (int64_t)((uint32_t)c / m) * s2) + r0;
+            if (!odd && r + 1 < nr) {
+                store_pair<KIND>(o, e, row + r, tile[cc][r], tile[cc][r + 1]);
+            } else {  // rows that start on odd values, or the last of an odd number
+                store_one<KIND>(o, e, row + r, tile[cc][r]);
+                if (r + 1 < nr) store_one<KIND>(o, e, row + r + 1, tile[cc][r + 1]);
+            }
         }
         __syncthreads();
+    }
+}
+
+// out[row Rp + r] = conv(+-in[row R + r]), zero for R <= r < Rp (Rp even): a warp per row
+template <int KIND>
+__global__ void __launch_bounds__(256) pad_convert_rows_kernel(const double *__restrict__ in, const RowOut o,
+                                                               int64_t rows, int R, int Rp) {
+    const int lane = threadIdx.x & 31;
+    const int e = KIND == 3 ? o.e[0] : 0;
+    for (int64_t row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += (int64_t)gridDim.x * 8) {
+        const double *src = in + row * R;
+        for (int r = 2 * lane; r < Rp; r += 64)
+            store_pair<KIND>(o, e, row * Rp + r, r < R ? flip(src[r], o.neg) : 0.0, r + 1 < R ? flip(src[r + 1], o.neg) : 0.0);
     }
 }
 
@@ -122,23 +260,38 @@ __global__ void pad_rows_kernel(const double *__restrict__ in, float *__restrict
 
 }  // namespace
 
-cudaError_t launch_transpose_pad(int kind, const double *in, void *out_hi, void *out_lo,
-                                 int64_t B, int R, int Rp, int64_t C, int64_t sb, int64_t sr,
-                                 int64_t sc, int64_t ob, int64_t oc, double scale,
-                                 cudaStream_t st) {
-    const int64_t ntiles = B * ((C + TT - 1) / TT) * ((Rp + TT - 1) / TT);
-    if (ntiles == 0) return cudaSuccess;
-    const unsigned grid = (unsigned)(ntiles < (int64_t)1 << 22 ? ntiles : (int64_t)1 << 22);
-    dim3 blk(TT, 8);
-    if (kind == 0)
-        transpose_pad_kernel<0><<<grid, blk, 0, st>>>(in, out_hi, out_lo, B, R, Rp, C, sb, sr, sc,
-                                                      ob, oc, scale);
-    else if (kind == 1)
-        transpose_pad_kernel<1><<<grid, blk, 0, st>>>(in, out_hi, out_lo, B, R, Rp, C, sb, sr, sc,
-                                                      ob, oc, scale);
-    else
-        transpose_pad_kernel<2><<<grid, blk, 0, st>>>(in, out_hi, out_lo, B, R, Rp, C, sb, sr, sc,
-                                                      ob, oc, scale);
+cudaError_t launch_transpose_rows(int kind, const double *in, void *out_hi, void *out_lo, int64_t plane, const int *e,
+                                  bool negate, int64_t B, int R, int Rp, int64_t C, int64_t sb, int64_t sr, int64_t ob,
+                                  int64_t m, int64_t s1, int64_t s2, cudaStream_t st) {
+    const int64_t grid = B * ((C + TC - 1) / TC);
+    if (grid == 0 || Rp == 0) return cudaSuccess;
+    if (grid > 0x7fffffff || (m > 1 && C > 0xffffffffll)) return cudaErrorInvalidValue;
+    const RowOut o{out_hi, out_lo, plane, e, negate ? 1 : 0};
+    // pairs are stored as one: every row has to start on an even value of a plane
+    const size_t pair = kind == 0 ? 16 : (kind == 1 ? 8 : 4);
+    const int odd = ((uintptr_t)out_hi | (uintptr_t)out_lo) % pair != 0 || ob % 2 != 0 || (m > 1 && s1 % 2 != 0) ||
+                    s2 % 2 != 0 || plane % 2 != 0;
+    const int ny = (int)std::min<int64_t>((Rp + TR - 1) / TR, std::max<int64_t>(1, 1024 / grid));
+    const dim3 gd((unsigned)grid, (unsigned)ny);
+#define TR_LAUNCH(K) transpose_rows_kernel<K><<<gd, 256, 0, st>>>(in, o, R, Rp, C, sb, sr, ob, (uint32_t)m, s1, s2, odd)
+    if (kind == 0) TR_LAUNCH(0);
+    else if (kind == 1) TR_LAUNCH(1);
+    else if (kind == 2) TR_LAUNCH(2);
+    else TR_LAUNCH(3);
+#undef TR_LAUNCH
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pad_convert_rows(int kind, const double *in, void *out_hi, void *out_lo, int64_t plane, const int *e,
+                                    bool negate, int64_t rows, int R, int Rp, cudaStream_t st) {
+    if (rows == 0) return cudaSuccess;
+    if (Rp % 2 != 0 || plane % 2 != 0) return cudaErrorInvalidValue;
+    const RowOut o{out_hi, out_lo, plane, e, negate ? 1 : 0};
+    const unsigned grid = (unsigned)(rows / 8 < 8192 ? (rows + 7) / 8 : 8192);
+    if (kind == 0) pad_convert_rows_kernel<0><<<grid, 256, 0, st>>>(in, o, rows, R, Rp);
+    else if (kind == 1) pad_convert_rows_kernel<1><<<grid, 256, 0, st>>>(in, o, rows, R, Rp);
+    else if (kind == 2) pad_convert_rows_kernel<2><<<grid, 256, 0, st>>>(in, o, rows, R, Rp);
+    else pad_convert_rows_kernel<3><<<grid, 256, 0, st>>>(in, o, rows, R, Rp);
     return cudaGetLastError();
 }
 
@@ -163,27 +316,28 @@ cudaError_t launch_epilogue_f32_inputs(const double *t1, const double *ovov, con
 
 
 namespace {
-// Thread per leading index x: the sorted triples x <= y <= z of n values
-// start at offset sum_{x' < x} (n - x')(n - x' + 1) / 2.
+// Thread per (x, y): the sorted triples x <= y <= z of n values with this x and
+// y, in lexicographic order after the T(n) - T(n - x) triples with a smaller first
+// index, T(m) = m (m + 1) (m + 2) / 6, and those with this x and a smaller second.
 __global__ void sorted_triples_kernel(int n, int *out) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= n) return;
-    int64_t off = 0;
-    for (int xp = 0; xp < x; xp++) off += (int64_t)(n - xp) * (n - xp + 1) / 2;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int x = (int)(t / n), y = (int)(t % n);
+    if (x >= n || y < x) return;
+    const int64_t m = n - x, k = n - y, N = n;
+    int64_t off = N * (N + 1) * (N + 2) / 6 - m * (m + 1) * (m + 2) / 6 + m * (m + 1) / 2 - k * (k + 1) / 2;
     int *w = out + 3 * off;
-    for (int y = x; y < n; y++)
-        for (int z = y; z < n; z++) {
-            w[0] = x;
-            w[1] = y;
-            w[2] = z;
-            w += 3;
-        }
+    for (int z = y; z < n; z++) {
+        w[0] = x;
+        w[1] = y;
+        w[2] = z;
+        w += 3;
+    }
 }
 }  // namespace
 
 cudaError_t launch_build_tables(int o, int nb, int *tasks, int *orbits, cudaStream_t st) {
-    sorted_triples_kernel<<<(o + 63) / 64, 64, 0, st>>>(o, tasks);
-    sorted_triples_kernel<<<(nb + 63) / 64, 64, 0, st>>>(nb, orbits);
+    sorted_triples_kernel<<<(unsigned)(((int64_t)o * o + 63) / 64), 64, 0, st>>>(o, tasks);
+    sorted_triples_kernel<<<(unsigned)(((int64_t)nb * nb + 63) / 64), 64, 0, st>>>(nb, orbits);
     return cudaGetLastError();
 }
 

@@ -147,6 +147,40 @@ static void stream_rows(Exec &ex, const double *host, size_t row, int v, F consu
     CK(cudaStreamSynchronize(cp.cs));
 }
 
+// The four operand layouts of a problem (tcorr_internal.cuh) in the given element
+// kind; vvvo on the host is streamed in chunks of d rows.  pG .. pN: slice plane
+// sizes, eA, eB: scale exponents of the two operand sides (FP64 emulation).
+static void layout_g(Exec &ex, Problem &pb, int kind, int64_t pG, const int *eA, const double *vvvo, bool host) {
+    const int o = pb.dm.o, v = pb.dm.v, dp = pb.dm.dp;
+    const int64_t v2 = (int64_t)v * v;
+    const size_t eb = kind == 0 ? 8 : (kind == 1 ? 4 : 2);
+    Operands &op = pb.op;
+    const size_t row = (size_t)v2 * o;  // doubles per d row of vvvo
+    // G[q][xy][d] = vvvo[d][xy][q]: rows d, columns (xy, q); the last rows write the padding
+    auto g_rows = [&](const double *src, int d0, int nr) {
+        char *hi = static_cast<char *>(op.G) + (size_t)d0 * eb;
+        char *lo = op.Glo ? static_cast<char *>(op.Glo) + (size_t)d0 * eb : nullptr;
+        CK(launch_transpose_rows(kind, src, hi, lo, pG, eA, false, 1, nr, d0 + nr == v ? dp - d0 : nr, (int64_t)row, 0,
+                                 (int64_t)row, 0, o, v2 * dp, dp, ex.stream));
+    };
+    if (!host) g_rows(vvvo, 0, v);
+    else stream_rows(ex, vvvo, row, v, g_rows);
+}
+static void layout_small(Exec &ex, Problem &pb, int kind, int64_t pK, int64_t pR, int64_t pN, const int *eA,
+                         const int *eB, const double *dt2, const double *doo) {
+    const int o = pb.dm.o, v = pb.dm.v, dp = pb.dm.dp, lp = pb.dm.lp;
+    const int64_t v2 = (int64_t)v * v;
+    Operands &op = pb.op;
+    // T2K[q][xy][l] = t2[q][l][xy]
+    CK(launch_transpose_rows(kind, dt2, op.T2K, op.T2Klo, pK, eA, false, o, o, lp, v2, (int64_t)o * v2, v2, v2 * lp, 1, 0, lp,
+                             ex.stream));
+    // T2R[spa][d] = t2[spa][d]
+    CK(launch_pad_convert_rows(kind, dt2, op.T2R, op.T2Rlo, pR, eB, false, (int64_t)o * o * v, v, dp, ex.stream));
+    // AoN[qsa][l] = -ooov[l][qsa]
+    CK(launch_transpose_rows(kind, doo, op.AoN, op.AoNlo, pN, eB, true, 1, o, lp, (int64_t)o * o * v, 0,
+                             (int64_t)o * o * v, 0, 1, 0, lp, ex.stream));
+}
+
 // FP64 emulation: the operands as oz_slices() BF16 slice planes under one
 // power-of-two scale per operand side (exponents computed on the device from
 // max |vvvo|, |t2|, |ooov|, so nothing here waits for the device).
@@ -166,7 +200,6 @@ static void build_operands_oz(Exec &ex, Problem &pb, const double *t2, const dou
     dalloc(ex, pb.oz_e, 2 * sizeof(int));
     Timer tm(ex, KC_PREP);
     CK(cudaMemsetAsync(pb.oz_max, 0, 3 * sizeof(unsigned long long), ex.stream));
-    CK(cudaMemsetAsync(op.G, 0, nG * 2 * S, ex.stream));
     double *tmp_t2 = nullptr, *tmp_oo = nullptr;
     const double *dt2 = device_view(ex, t2, (size_t)o * o * v2, host, tmp_t2);
     const double *doo = device_view(ex, ooov, (size_t)o * o * o * v, host, tmp_oo);
@@ -182,25 +215,8 @@ static void build_operands_oz(Exec &ex, Problem &pb, const double *t2, const dou
     CK(launch_maxabs(doo, (int64_t)o * o * o * v, pb.oz_max + 2, ex.stream));
     CK(launch_oz_exponents(pb.oz_max, pb.oz_e, ex.stream));
     const int *eA = pb.oz_e, *eB = pb.oz_e + 1;
-    // G[p][q][xy][d] = slices of vvvo[d][xy][q]
-    if (!host) {
-        CK(launch_slice_pad(vvvo, op.G, v2, v, v, o, o, (int64_t)row, 1, dp, (int64_t)v2 * dp, (int64_t)nG, eA, 1.0,
-                            ex.stream));
-    } else {
-        stream_rows(ex, vvvo, row, v, [&](const double *stage, int d0, int nr) {
-            char *g = static_cast<char *>(op.G) + (size_t)d0 * 2;
-            CK(launch_slice_pad(stage, g, v2, nr, nr, o, o, (int64_t)row, 1, dp, (int64_t)v2 * dp, (int64_t)nG, eA,
-                                1.0, ex.stream));
-        });
-    }
-    // T2K[p][q][xy][l] = slices of t2[q][l][xy]; T2R[p][spa][d] = slices of t2[spa][d]
-    CK(launch_slice_pad(dt2, op.T2K, o, o, lp, v2, (int64_t)o * v2, v2, 1, (int64_t)v2 * lp, lp, (int64_t)nT2K, eA,
-                        1.0, ex.stream));
-    CK(launch_slice_pad(dt2, op.T2R, (int64_t)o * o * v, v, dp, 1, v, 1, 0, dp, 0, (int64_t)nT2R, eB, 1.0,
-                        ex.stream));
-    // AoN[p][qsa][l] = slices of -ooov[l][qsa]
-    CK(launch_slice_pad(doo, op.AoN, 1, o, lp, (int64_t)o * o * v, 0, (int64_t)o * o * v, 1, 0, lp, (int64_t)nAoN,
-                        eB, -1.0, ex.stream));
+    layout_g(ex, pb, 3, (int64_t)nG, eA, vvvo, host);
+    layout_small(ex, pb, 3, (int64_t)nT2K, (int64_t)nT2R, (int64_t)nAoN, eA, eB, dt2, doo);
     tm.stop();
     free_tmp(ex, tmp_t2, (size_t)o * o * v2);
     free_tmp(ex, tmp_oo, (size_t)o * o * o * v);
@@ -232,33 +248,11 @@ void build_operands(Exec &ex, Problem &pb, const double *t2, const double *vvvo,
         dalloc(ex, op.AoNlo, nAoN * eb);
     }
     Timer tm(ex, KC_PREP);
-    // G[q][xy][d] = vvvo[d][xy][q]; staged in chunks of d rows for host inputs
-    CK(cudaMemsetAsync(op.G, 0, nG * eb, ex.stream));
-    if (split) CK(cudaMemsetAsync(op.Glo, 0, nG * eb, ex.stream));
-    const size_t row = (size_t)v2 * o;  // doubles per d row of vvvo
-    if (!host) {
-        CK(launch_transpose_pad(kind, vvvo, op.G, op.Glo, v2, v, v, o, o, (int64_t)row, 1, dp,
-                                (int64_t)v2 * dp, 1.0, ex.stream));
-    } else {
-        stream_rows(ex, vvvo, row, v, [&](const double *stage, int d0, int nr) {
-            char *ghi = static_cast<char *>(op.G) + (size_t)d0 * eb;
-            char *glo = split ? static_cast<char *>(op.Glo) + (size_t)d0 * eb : nullptr;
-            CK(launch_transpose_pad(kind, stage, ghi, glo, v2, nr, nr, o, o, (int64_t)row, 1, dp,
-                                    (int64_t)v2 * dp, 1.0, ex.stream));
-        });
-    }
+    layout_g(ex, pb, kind, 0, nullptr, vvvo, host);
     double *tmp_t2 = nullptr, *tmp_oo = nullptr;
     const double *dt2 = device_view(ex, t2, (size_t)o * o * v2, host, tmp_t2);
-    // T2K[q][xy][l] = t2[q][l][xy]
-    CK(launch_transpose_pad(kind, dt2, op.T2K, op.T2Klo, o, o, lp, v2, (int64_t)o * v2, v2, 1,
-                            (int64_t)v2 * lp, lp, 1.0, ex.stream));
-    // T2R[spa][d] = t2[spa][d]  (row copy with padding: C = 1)
-    CK(launch_transpose_pad(kind, dt2, op.T2R, op.T2Rlo, (int64_t)o * o * v, v, dp, 1, v, 1, 0,
-                            dp, 0, 1.0, ex.stream));
     const double *doo = device_view(ex, ooov, (size_t)o * o * o * v, host, tmp_oo);
-    // AoN[qsa][l] = -ooov[l][qsa]
-    CK(launch_transpose_pad(kind, doo, op.AoN, op.AoNlo, 1, o, lp, (int64_t)o * o * v, 0,
-                            (int64_t)o * o * v, 1, 0, lp, -1.0, ex.stream));
+    layout_small(ex, pb, kind, 0, 0, 0, nullptr, nullptr, dt2, doo);
     tm.stop();
     free_tmp(ex, tmp_t2, (size_t)o * o * v2);
     free_tmp(ex, tmp_oo, (size_t)o * o * o * v);

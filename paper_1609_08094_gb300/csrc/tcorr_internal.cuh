@@ -167,13 +167,17 @@ struct Wave {
 };
 
 // ---- prep.cu -------------------------------------------------------------
-// out[b][c][r] = conv(scale * in[b*sb + r*sr + c*sc]) for r < R; zero for
-// R <= r < Rp; out index b*ob + c*oc + r.  Writes hi (and lo when non-null).
-// kind: 0 = FP64, 1 = TF32 hi+lo (float containers), 2 = BF16 hi+lo.
-cudaError_t launch_transpose_pad(int kind, const double *in, void *out_hi, void *out_lo,
-                                 int64_t B, int R, int Rp, int64_t C,
-                                 int64_t sb, int64_t sr, int64_t sc,
-                                 int64_t ob, int64_t oc, double scale, cudaStream_t st);
+// Element kinds: 0 = FP64 (hi), 1 = TF32 hi and lo planes (float containers), 2 =
+// BF16 hi and lo, 3 = the FP64 emulation's BF16 slice planes (hi: the first plane,
+// `plane` values apart; e: the device scale exponent).  negate: every sign flipped.
+// out[b ob + (c % m) s1 + (c / m) s2 + r] = conv(+-in[b sb + r sr + c]) for
+// r < R and c < C, zero for R <= r < Rp.
+cudaError_t launch_transpose_rows(int kind, const double *in, void *out_hi, void *out_lo, int64_t plane, const int *e,
+                                  bool negate, int64_t B, int R, int Rp, int64_t C, int64_t sb, int64_t sr, int64_t ob,
+                                  int64_t m, int64_t s1, int64_t s2, cudaStream_t st);
+// out[row Rp + r] = conv(+-in[row R + r]) for r < R, zero for R <= r < Rp (even)
+cudaError_t launch_pad_convert_rows(int kind, const double *in, void *out_hi, void *out_lo, int64_t plane, const int *e,
+                                    bool negate, int64_t rows, int R, int Rp, cudaStream_t st);
 // FP32 epilogue inputs, zero padded to vp = 8 nb: t1 as rows [o][vp]; (p x | q z)
 // as [p][q][X][Z][8][8] (8x8 blocks of x, z, each 256 contiguous bytes); eps_v
 // as float-float pairs [vp]
@@ -232,10 +236,6 @@ cudaError_t launch_maxabs(const double *x, int64_t n, unsigned long long *out, c
 cudaError_t launch_seed_max(unsigned long long *m, double x, cudaStream_t st);
 // e[0], e[1]: scale exponents of the A side (m[0] vvvo, m[1] t2) and B side (m[1] t2, m[2] ooov)
 cudaError_t launch_oz_exponents(const unsigned long long *m, int *e, cudaStream_t st);
-// out[p*plane + b*ob + c*oc + r] = slice p of sign * 2^-e[0] * in[b*sb + r*sr + c*sc], r < Rp (zero for r >= R)
-cudaError_t launch_slice_pad(const double *in, void *out, int64_t B, int R, int Rp, int64_t C, int64_t sb,
-                             int64_t sr, int64_t sc, int64_t ob, int64_t oc, int64_t plane, const int *e,
-                             double sign, cudaStream_t st);
 cudaError_t oz_fill_desc(InstDesc &d, const Operands &op, const int *exps, std::string &err);
 int64_t oz_units_per_task(const InstDesc &d);
 cudaError_t oz_prepare();
