@@ -47,6 +47,18 @@ __device__ __forceinline__ int perm_pos(int s, int d) {
 }
 __device__ __forceinline__ int pick3(int a, int b, int c, int k) { return k == 0 ? a : (k == 1 ? b : c); }
 
+// Sorted triples of 0..7 (120 entries), then sorted pairs (36): la | lb << 3 | lc << 6;
+// thread t of 64 writes those that start with (t / 8, t % 8)
+__device__ __forceinline__ void sorted_entry(short *trip, int t) {
+    const int x = t >> 3, y = t & 7;
+    if (x > y) return;
+    int n = 0, m = 0;  // triples, pairs with a smaller first, then second index
+    for (int k = 0; k < x; k++) { n += (8 - k) * (9 - k) / 2; m += 8 - k; }
+    for (int k = x; k < y; k++) n += 8 - k;
+    for (int z = y; z < 8; z++) trip[n + z - y] = (short)(x | y << 3 | z << 6);
+    trip[120 + m + y - x] = (short)(x | y << 3);
+}
+
 // ---- float-float (double-FP32) arithmetic ------------------------------------
 // A value hi + lo with |lo| <= ulp(hi) / 2 carries ~48 significant bits.  The
 // split-precision epilogue forms its denominators, their reciprocals and the
@@ -168,10 +180,11 @@ template <> __device__ __forceinline__ dd eps_vir<dd>(const InstDesc &p, int x) 
     return dd(ff{e.x, e.y});
 }
 
-// FP64 epilogue; TE: cube edge.  Orbits of three distinct blocks take the
-// element-orbit form (the six orderings of one (a,b,c) share one denominator
-// and the E/O expansion of Z, as in the mixed epilogue), orbits with repeated
-// blocks the generic per-element form.  CT = double (FP64 path: U, t1, ovov
+// FP64 epilogue; TE: cube edge.  Element orbits: the six orderings of one (a,b,c)
+// share one denominator and the E/O expansion of Z, as in the mixed epilogue; where
+// blocks repeat, only the orbits with a <= b (b <= c), about half of the warps' work
+// of one element at a time (o=4, v=20: 33 us, now 26; 52 tasks of o=40, v=300 in FP64
+// emulation 18.1 ms, now 16.8).  CT = double (FP64 path: U, t1, ovov
 // in FP64) or dd (FP64 emulation: all of them float-float pairs, so that no
 // operation per element runs on the FP64 pipe).
 template <typename CT, int TE>
@@ -181,8 +194,7 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
     constexpr int TP = TE + 1;               // padded innermost extent
     constexpr int CUBE = TE * TE * TP;       // smem elements per cube
     constexpr int NE = TE * TE * TE;         // elements per cube
-    __shared__ int comp[6][6];
-    __shared__ int distinct[6];
+    __shared__ short trip[156];
     __shared__ double red[NT][2];
 
     const int64_t item = blockIdx.x;
@@ -227,21 +239,7 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
         if (xb < v && yb < v && zb < v)
             rc[it] = __ldg(reinterpret_cast<const double2 *>(U2 + ((int64_t)zb * v + xb) * vc + yb));
     }
-    if (tid < 36) {  // comp[pi][q]: the slot of permutation pi composed with q
-        const int pi = tid / 6, q = tid % 6;
-        const int t0 = perm_pos(pi, perm_pos(q, 0)), t1v = perm_pos(pi, perm_pos(q, 1));
-        int sig = 0;
-        for (int s2 = 0; s2 < 6; s2++)
-            if (perm_pos(s2, 0) == t0 && perm_pos(s2, 1) == t1v) sig = s2;
-        comp[pi][q] = sig;
-    }
-    if (tid >= 64 && tid < 70) {
-        const int t = tid - 64;
-        int d = 1;
-        for (int s2 = 0; s2 < t; s2++)
-            if (OBP(s2, 0) == OBP(t, 0) && OBP(s2, 1) == OBP(t, 1) && OBP(s2, 2) == OBP(t, 2)) d = 0;
-        distinct[t] = d;
-    }
+    if (tid < 64) sorted_entry(trip, tid);
 #pragma unroll
     for (int it = 0; it < 6; it++) {
         const int e2 = tid + it * NT;
@@ -268,7 +266,6 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
     const CT *t1 = static_cast<const CT *>(p.t1);
     const CT *ov = static_cast<const CT *>(p.ovov);
     const CT eijk = CT(p.eps_o[ti] + p.eps_o[tj] + p.eps_o[tkk]);
-    const CT coef[6] = {CT(8), CT(-4), CT(-4), CT(2), CT(2), CT(-4)};
     // ovov rows used by Y: (j y | k z), (i x | k z), (i x | j y)
     const CT *ov_jk = ov + ((int64_t)tj * v * o + tkk) * v;   // [y][z] stride o*v in y
     const CT *ov_ik = ov + ((int64_t)ti * v * o + tkk) * v;   // [x][z]
@@ -332,30 +329,41 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
         }
         kahan_add(s4, c4, double(a4));
         kahan_add(s5, c5, double(a5));
-    } else
-    for (int s = 0; s < 6; s++) {
-        if (!distinct[s]) continue;
+    } else {
+        // repeated blocks: the element orbits with a <= b where A = B and b <= c where
+        // B = C; of one with two equal indices the six slots repeat three elements
+        // (weight 1/2), with three Z vanishes
+        const int kind = ob0 == ob1 ? (ob1 == ob2 ? 4 : 2) : 3;
+        const int norb = kind == 4 ? 120 : 288;
         CT a4 = CT(0), a5 = CT(0);
-        const int X0 = OBP(s, 0) * TE, Y0 = OBP(s, 1) * TE, Z0 = OBP(s, 2) * TE;
-        for (int l = tid; l < NE; l += NT) {
-            const int lv0 = l / (TE * TE), lv1 = (l / TE) % TE, lv2 = l % TE;
-            const int x = X0 + lv0, y = Y0 + lv1, z = Z0 + lv2;
-            if (x >= v || y >= v || z >= v) continue;
-            CT zv = CT(0);
-#pragma unroll
-            for (int q = 0; q < 6; q++) {
-                const int sg = comp[s][q];
-                const int m0 = pick3(lv0, lv1, lv2, perm_pos(q, 0)), m1 = pick3(lv0, lv1, lv2, perm_pos(q, 1)),
-                          m2 = pick3(lv0, lv1, lv2, perm_pos(q, 2));
-                zv += coef[q] * Ws[sg * CUBE + (m0 * TE + m1) * TP + m2];
-            }
-            const CT w0 = Ws[s * CUBE + (lv0 * TE + lv1) * TP + lv2];
-            const CT yv = t1[ti * v + x] * ov_jk[y * ovs + z] + t1[tj * v + y] * ov_ik[x * ovs + z] +
-                          t1[tkk * v + z] * ov_ij[x * ovs + y];
-            const CT dn = eijk - eps_vir<CT>(p, x) - eps_vir<CT>(p, y) - eps_vir<CT>(p, z);
-            const CT r = CT(1) / dn;
-            a4 += zv * w0 * r;
-            a5 += zv * yv * r;
+        for (int x = tid; x < norb; x += NT) {
+            const int pr = kind == 4 ? trip[x] : trip[120 + (x >> 3)], l8 = x & 7;
+            const int la = kind == 3 ? l8 : pr & 7;
+            const int lb = kind == 3 ? pr & 7 : (pr >> 3) & 7;
+            const int lc = kind == 4 ? pr >> 6 : (kind == 3 ? (pr >> 3) & 7 : l8);
+            const int a = ob0 * TE + la, b = ob1 * TE + lb, c = ob2 * TE + lc;
+            if (a >= v || b >= v || c >= v || (a == b && b == c)) continue;
+            const CT w0 = Ws[0 * CUBE + (la * TE + lb) * TP + lc], w1 = Ws[1 * CUBE + (la * TE + lc) * TP + lb];
+            const CT w2 = Ws[2 * CUBE + (lb * TE + la) * TP + lc], w3 = Ws[3 * CUBE + (lb * TE + lc) * TP + la];
+            const CT w4 = Ws[4 * CUBE + (lc * TE + la) * TP + lb], w5 = Ws[5 * CUBE + (lc * TE + lb) * TP + la];
+            const CT tia = t1[ti * v + a], tja = t1[tj * v + a], tka = t1[tkk * v + a];
+            const CT tib = t1[ti * v + b], tjb = t1[tj * v + b], tkb = t1[tkk * v + b];
+            const CT tic = t1[ti * v + c], tjc = t1[tj * v + c], tkc = t1[tkk * v + c];
+            const CT y0 = tia * ov_jk[b * ovs + c] + tjb * ov_ik[a * ovs + c] + tkc * ov_ij[a * ovs + b];
+            const CT y1 = tia * ov_jk[c * ovs + b] + tjc * ov_ik[a * ovs + b] + tkb * ov_ij[a * ovs + c];
+            const CT y2 = tib * ov_jk[a * ovs + c] + tja * ov_ik[b * ovs + c] + tkc * ov_ij[b * ovs + a];
+            const CT y3 = tib * ov_jk[c * ovs + a] + tjc * ov_ik[b * ovs + a] + tka * ov_ij[b * ovs + c];
+            const CT y4 = tic * ov_jk[a * ovs + b] + tja * ov_ik[c * ovs + b] + tkb * ov_ij[c * ovs + a];
+            const CT y5 = tic * ov_jk[b * ovs + a] + tjb * ov_ik[c * ovs + a] + tka * ov_ij[c * ovs + b];
+            const CT E = w0 + w3 + w4, O = w1 + w2 + w5;
+            const CT ww = w0 * w0 + w1 * w1 + w2 * w2 + w3 * w3 + w4 * w4 + w5 * w5;
+            const CT wy = w0 * y0 + w1 * y1 + w2 * y2 + w3 * y3 + w4 * y4 + w5 * y5;
+            const CT q4 = CT(6) * ww + CT(2) * (E * E + O * O) - CT(8) * E * O;
+            const CT q5 = CT(6) * wy + (CT(2) * E - CT(4) * O) * (y0 + y3 + y4) + (CT(2) * O - CT(4) * E) * (y1 + y2 + y5);
+            const CT n = (a == b || b == c) ? CT(2) : CT(1);
+            const CT r = CT(1) / (n * (eijk - eps_vir<CT>(p, a) - eps_vir<CT>(p, b) - eps_vir<CT>(p, c)));
+            a4 += q4 * r;
+            a5 += q5 * r;
         }
         kahan_add(s4, c4, double(a4));
         kahan_add(s5, c5, double(a5));
@@ -497,18 +505,7 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < 64) {  // sorted triples of 0..7 (120), then sorted pairs (36): la | lb << 3 | lc << 6
-        const int x = tid >> 3, y = tid & 7;
-        if (x <= y) {
-            // before (x, y): the triples with a smaller first, then second index
-            int n = 0, m = 0;
-            for (int k = 0; k < x; k++) { n += (8 - k) * (9 - k) / 2; m += 8 - k; }
-            for (int k = x; k < y; k++) n += 8 - k;
-            m += y - x;
-            for (int z = y; z < 8; z++) trip[n + z - y] = (short)(x | y << 3 | z << 6);
-            trip[120 + m] = (short)(x | y << 3);
-        }
-    }
+    if (tid < 64) sorted_entry(trip, tid);
     __syncthreads();  // the last CTA-wide barrier: from here on the roles meet only at mbarriers
 
     if (warp >= EPI_CW) {

@@ -8,7 +8,8 @@
 // GB300's FP64 rate is far below its tensor rates, so this kernel is bound by
 // the FP64 pipe: a register-tiled DFMA GEMM (CTA tile 128 pairs x 32 a, 16
 // outputs per thread, K staged through shared memory in chunks of 8 with a
-// register prefetch of the next chunk).  One flattened grid covers the work
+// register prefetch of the next chunk; 32 pairs and 4 outputs for few units, see
+// f64_tile_pairs).  One flattened grid covers the work
 // units of every segment of a wave (one or many problems).  Operand rows are K-contiguous, so
 // the swapped pair order (c,b) of two segments only changes which rows are
 // read, never the coalescing.
@@ -17,20 +18,19 @@
 namespace tcorr {
 namespace {
 
-constexpr int TP = 128;  // pairs per CTA tile
 constexpr int TA = 32;   // a values per CTA tile
 constexpr int KC = 8;    // K chunk
 constexpr int NT = 256;  // threads
 
-__global__ void __launch_bounds__(NT) ugemm_f64_kernel(const Wave w) {
-    __shared__ __align__(16) double As[KC][TP + 4];
-    __shared__ __align__(16) double Bs[KC][TA + 4];
+// One work unit: a tile of TP pairs x TA values of a of one group
+template <int TP>
+__device__ __forceinline__ void f64_unit(const Wave &w, const Seg &sg, int64_t unit, double (*As)[128 + 4],
+                                         double (*Bs)[TA + 4]) {
+    constexpr int RP = TP / 32;  // pairs per thread
 
-    // work unit -> segment -> (task, group, pair tile, a tile); a tiles fastest,
+    // work unit -> (task, group, pair tile, a tile); a tiles fastest,
     // so the CTAs sharing one pair tile (the large A operand) run back to back
     // and it is read from HBM once, then from L2
-    const int64_t unit = blockIdx.x;
-    const Seg sg = w.segs[seg_find(w.segs, w.nseg, unit, [](const Seg &x) { return x.gemm0; })];
     const InstDesc &d = w.descs[sg.inst];
     const int o = d.dm.o, v = d.dm.v, dp = d.dm.dp, lp = d.dm.lp, vc = d.dm.vc;
     const int64_t v2 = (int64_t)v * v;
@@ -56,16 +56,18 @@ __global__ void __launch_bounds__(NT) ugemm_f64_kernel(const Wave w) {
     const double *T2R = static_cast<const double *>(d.T2R);
     const double *AoN = static_cast<const double *>(d.AoN);
 
-    // A-row loader: row = tid>>1, half = tid&1 (4 doubles each)
-    const int arow = tid >> 1, ahalf = tid & 1;
+    // A-row loader: row = tid>>1, half = tid&1 (4 doubles each); TP = 32: the first 128
+    // threads, row = tid>>2, quarter = tid&3 (2 doubles each)
+    constexpr bool WIDE = TP == 128;
+    const int arow = WIDE ? tid >> 1 : (tid & 127) >> 2, ak = WIDE ? (tid & 1) * 4 : (tid & 3) * 2;
     const int64_t apair = p0 + arow;
-    const bool a_ok = apair < v2;
+    const bool a_ok = apair < v2 && (WIDE || tid < 128);
     const int64_t ab = a_ok ? apair / v : 0, ac = a_ok ? apair % v : 0;
     const int64_t row_nat = ab * v + ac, row_swp = ac * v + ab;
-    // B-row loader: tid < 128: row = tid>>2, quarter = tid&3 (2 doubles each)
+    // B-row loader: half of the threads: row = tid>>2, quarter = tid&3 (2 doubles each)
     const int brow = (tid & 127) >> 2, bq = tid & 3;
     const int ba = a0 + brow;
-    const bool b_ok = (tid < 128) && (ba < v);
+    const bool b_thr = WIDE ? tid < 128 : tid >= 128, b_ok = b_thr && ba < v;
 
     const int KV = round_up(v, KC), KO = round_up(o, KC);
     const int nchunk_v = KV / KC, nchunk_o = KO / KC;
@@ -102,9 +104,9 @@ __global__ void __launch_bounds__(NT) ugemm_f64_kernel(const Wave w) {
         const double *aptr, *bptr;
         src_ptrs(chunk, aptr, bptr);
         if (a_ok) {
-            const double2 *pa = reinterpret_cast<const double2 *>(aptr + ahalf * 4);
+            const double2 *pa = reinterpret_cast<const double2 *>(aptr + ak);
             ra0 = __ldg(pa);
-            ra1 = __ldg(pa + 1);
+            if constexpr (WIDE) ra1 = __ldg(pa + 1);
         } else {
             ra0 = make_double2(0, 0);
             ra1 = make_double2(0, 0);
@@ -113,21 +115,24 @@ __global__ void __launch_bounds__(NT) ugemm_f64_kernel(const Wave w) {
         else rb = make_double2(0, 0);
     };
     auto store_chunk = [&]() {
-        const int k = ahalf * 4;
-        As[k + 0][arow] = ra0.x;
-        As[k + 1][arow] = ra0.y;
-        As[k + 2][arow] = ra1.x;
-        As[k + 3][arow] = ra1.y;
-        if (tid < 128) {
+        if (WIDE || tid < 128) {
+            As[ak + 0][arow] = ra0.x;
+            As[ak + 1][arow] = ra0.y;
+            if constexpr (WIDE) {
+                As[ak + 2][arow] = ra1.x;
+                As[ak + 3][arow] = ra1.y;
+            }
+        }
+        if (b_thr) {
             Bs[bq * 2 + 0][brow] = rb.x;
             Bs[bq * 2 + 1][brow] = rb.y;
         }
     };
 
     const int tp = tid & 31, ta = tid >> 5;
-    double acc[4][4];
+    double acc[RP][4];
 #pragma unroll
-    for (int r = 0; r < 4; r++)
+    for (int r = 0; r < RP; r++)
 #pragma unroll
         for (int c = 0; c < 4; c++) acc[r][c] = 0.0;
 
@@ -137,14 +142,14 @@ __global__ void __launch_bounds__(NT) ugemm_f64_kernel(const Wave w) {
     // (the zero padding of d to a multiple of KC and of l is never multiplied).
     const bool active = a0 + ta * 4 < v;
     auto mma_step = [&](int k) {
-        double av[4], bv[4];
+        double av[RP], bv[4];
 #pragma unroll
-        for (int r = 0; r < 4; r++) av[r] = As[k][tp + 32 * r];
+        for (int r = 0; r < RP; r++) av[r] = As[k][tp + 32 * r];
         const double2 b01 = *reinterpret_cast<const double2 *>(&Bs[k][ta * 4]);
         const double2 b23 = *reinterpret_cast<const double2 *>(&Bs[k][ta * 4 + 2]);
         bv[0] = b01.x; bv[1] = b01.y; bv[2] = b23.x; bv[3] = b23.y;
 #pragma unroll
-        for (int r = 0; r < 4; r++)
+        for (int r = 0; r < RP; r++)
 #pragma unroll
             for (int c = 0; c < 4; c++) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
     };
@@ -178,7 +183,7 @@ __global__ void __launch_bounds__(NT) ugemm_f64_kernel(const Wave w) {
         const int a = a0 + ta * 4 + c;
         if (a >= v) continue;
 #pragma unroll
-        for (int r = 0; r < 4; r++) {
+        for (int r = 0; r < RP; r++) {
             const int64_t pidx = p0 + tp + 32 * r;
             if (pidx >= v2) continue;
             const int64_t b = pidx / v, cc = pidx % v;
@@ -187,11 +192,29 @@ __global__ void __launch_bounds__(NT) ugemm_f64_kernel(const Wave w) {
     }
 }
 
+__global__ void __launch_bounds__(NT) ugemm_f64_kernel(const Wave w) {
+    __shared__ __align__(16) double As[KC][128 + 4];
+    __shared__ __align__(16) double Bs[KC][TA + 4];
+    const int64_t unit = blockIdx.x;
+    const Seg sg = w.segs[seg_find(w.segs, w.nseg, unit, [](const Seg &x) { return x.gemm0; })];
+    if (sg.f64_tp == 128) f64_unit<128>(w, sg, unit, As, Bs);
+    else f64_unit<32>(w, sg, unit, As, Bs);
+}
+
 }  // namespace
 
-int64_t f64_units_per_task(const Dims &dm) {
+// Pairs per tile for a segment of ntb tasks: 128, or 32 where 128 would give fewer
+// than 16 units per SM of 152.  The FP64 pipe is as busy with either (4 or 16 FMAs
+// per thread and K step, each 16 clocks of the SM's pipe), and the finer cut
+// leaves less of the last units over: o=4, v=20 has 192 units of 128 pairs (two on
+// some SMs, one on others) or 624 of 32, 70 and 49 us.
+int f64_tile_pairs(const Dims &dm, int64_t ntb) {
+    return ntb * f64_units_per_task(dm, 128) < 16 * 152 ? 32 : 128;
+}
+
+int64_t f64_units_per_task(const Dims &dm, int tp) {
     const int64_t v2 = (int64_t)dm.v * dm.v;
-    return 3 * ((v2 + TP - 1) / TP) * ((dm.v + TA - 1) / TA);
+    return 3 * ((v2 + tp - 1) / tp) * ((dm.v + TA - 1) / TA);
 }
 
 cudaError_t launch_ugemm_f64(const Wave &w, cudaStream_t st) {

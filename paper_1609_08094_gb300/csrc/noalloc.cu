@@ -52,28 +52,35 @@ __global__ void noalloc_tables_kernel(const InstDesc d, const Seg sg, InstDesc *
     const uint32_t *src = reinterpret_cast<const uint32_t *>(&d);
     uint32_t *dst = reinterpret_cast<uint32_t *>(d_out);
     for (int w = threadIdx.x; w < (int)(sizeof(InstDesc) / 4); w += blockDim.x) dst[w] = src[w];
-    if (threadIdx.x == 0) *sg_out = sg;
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    task[0] = i;
-    task[1] = j;
-    task[2] = k;
+    if (threadIdx.x == 0) {
+        *sg_out = sg;
+        task[0] = i;
+        task[1] = j;
+        task[2] = k;
+    }
+    // thread per (A, B): the triples with this A and B, after those with a smaller
+    // first, then second block
+    const int a = threadIdx.x / NA_NB, b = threadIdx.x % NA_NB;
+    if (a >= nb || b < a || b >= nb) return;
     int n = 0;
-    for (int a = 0; a < nb; a++)
-        for (int b = a; b < nb; b++)
-            for (int c = b; c < nb; c++) {
-                orb[3 * n] = a;
-                orb[3 * n + 1] = b;
-                orb[3 * n + 2] = c;
-                n++;
-            }
+    for (int x = 0; x < a; x++) n += (nb - x) * (nb - x + 1) / 2;
+    for (int x = a; x < b; x++) n += nb - x;
+    for (int c = b; c < nb; c++, n++) {
+        orb[3 * n] = a;
+        orb[3 * n + 1] = b;
+        orb[3 * n + 2] = c;
+    }
 }
+static_assert(NA_NB * NA_NB <= 128, "a thread per (A, B) of the 128");
 
 // U^{s;p,q}[a][b][c] for the three groups of task (i,j,k), FP64, from the
 // canonical arrays (same sums as the layout-based FP64 kernel):
 //   sum_d t2[s][p][a][d] (db|cq) + sum_d t2[s][q][a][d] (dc|bp)
 //   - sum_l (as|lq) t2[p][l][b][c] - sum_l (as|lp) t2[q][l][c][b],
 // with (db|cq) = vvvo[d][b][c][q] and (as|lq) = ooov[l][q][s][a].
-constexpr int CT_P = 128, CT_A = 32, CT_K = 8;
+// Tiles of 32 pairs: at v = 64 the task has 768 of them, 5 on each SM; of 128 pairs
+// there were 192, two on some SMs and one on others (v=61: 323 us, 188 so).
+constexpr int CT_P = 32, CT_A = 32, CT_K = 8;
 __global__ void __launch_bounds__(256) ugemm_f64_canon_kernel(int o, int v, int vc, int64_t ug,
                                                               const double *__restrict__ t2,
                                                               const double *__restrict__ vvvo,
@@ -92,61 +99,53 @@ __global__ void __launch_bounds__(256) ugemm_f64_canon_kernel(int o, int v, int 
     else if (g == 1) { s = tj; pp = ti; q = tk; }
     else { s = tk; pp = ti; q = tj; }
     const int tp = tid & 31, ta = tid >> 5;
-    double acc[4][4] = {};
-    for (int seg = 0; seg < 4; seg++) {
-        const int klen = seg < 2 ? v : o;
-        for (int k0 = 0; k0 < klen; k0 += CT_K) {
-            for (int e = tid; e < CT_P * CT_K; e += 256) {
-                const int r = e / CT_K, kk = e % CT_K, kx = k0 + kk;
-                const int64_t pidx = p0 + r;
-                double x = 0.0;
-                if (pidx < v2 && kx < klen) {
-                    const int64_t b = pidx / v, c = pidx % v;
-                    if (seg == 0) x = vvvo[((kx * (int64_t)v + b) * v + c) * o + q];
-                    else if (seg == 1) x = vvvo[((kx * (int64_t)v + c) * v + b) * o + pp];
-                    else if (seg == 2) x = t2[(((int64_t)pp * o + kx) * v + b) * v + c];
-                    else x = t2[(((int64_t)q * o + kx) * v + c) * v + b];
-                }
-                As[kk][r] = x;
-            }
-            {
-                const int r = tid / CT_K, kk = tid % CT_K, kx = k0 + kk, a = a0 + r;
-                double x = 0.0;
-                if (a < v && kx < klen) {
-                    if (seg == 0) x = t2[(((int64_t)s * o + pp) * v + a) * v + kx];
-                    else if (seg == 1) x = t2[(((int64_t)s * o + q) * v + a) * v + kx];
-                    else if (seg == 2) x = -ooov[(((int64_t)kx * o + q) * o + s) * v + a];
-                    else x = -ooov[(((int64_t)kx * o + pp) * o + s) * v + a];
-                }
-                Bs[kk][r] = x;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < CT_K; kk++) {
-                double av[4], bv[4];
-#pragma unroll
-                for (int r = 0; r < 4; r++) av[r] = As[kk][tp + 32 * r];
-#pragma unroll
-                for (int c = 0; c < 4; c++) bv[c] = Bs[kk][ta * 4 + c];
-#pragma unroll
-                for (int r = 0; r < 4; r++)
-#pragma unroll
-                    for (int c = 0; c < 4; c++) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
-            }
-            __syncthreads();
+    double acc[4] = {};
+    const int r = tid / CT_K, kk = tid % CT_K;  // the row and k that this thread loads of each operand
+    const int64_t pidx = p0 + r;
+    const int64_t b = pidx / v, c = pidx % v;
+    const int a = a0 + r;
+    const int KV = (v + CT_K - 1) / CT_K, KO = (o + CT_K - 1) / CT_K, nch = 2 * KV + 2 * KO;
+    double xa = 0.0, xb = 0.0;
+    auto load = [&](int ch) {  // chunk ch of K = [d | d | l | l]
+        const int seg = ch < KV ? 0 : (ch < 2 * KV ? 1 : (ch < 2 * KV + KO ? 2 : 3));
+        const int kx = (ch - (seg == 0 ? 0 : (seg == 1 ? KV : (seg == 2 ? 2 * KV : 2 * KV + KO)))) * CT_K + kk;
+        const bool k_in = kx < (seg < 2 ? v : o);
+        xa = xb = 0.0;
+        if (k_in && pidx < v2) {
+            if (seg == 0) xa = vvvo[((kx * (int64_t)v + b) * v + c) * o + q];
+            else if (seg == 1) xa = vvvo[((kx * (int64_t)v + c) * v + b) * o + pp];
+            else if (seg == 2) xa = t2[(((int64_t)pp * o + kx) * v + b) * v + c];
+            else xa = t2[(((int64_t)q * o + kx) * v + c) * v + b];
         }
+        if (k_in && a < v) {
+            if (seg == 0) xb = t2[(((int64_t)s * o + pp) * v + a) * v + kx];
+            else if (seg == 1) xb = t2[(((int64_t)s * o + q) * v + a) * v + kx];
+            else if (seg == 2) xb = -ooov[(((int64_t)kx * o + q) * o + s) * v + a];
+            else xb = -ooov[(((int64_t)kx * o + pp) * o + s) * v + a];
+        }
+    };
+    load(0);
+    for (int ch = 0; ch < nch; ch++) {
+        As[kk][r] = xa;
+        Bs[kk][r] = xb;
+        __syncthreads();
+        if (ch + 1 < nch) load(ch + 1);
+        if (a0 + ta * 4 < v) {  // a warp whose four a lie past v issues no FMA
+#pragma unroll
+            for (int k = 0; k < CT_K; k++) {
+                const double av = As[k][tp];
+#pragma unroll
+                for (int x = 0; x < 4; x++) acc[x] = fma(av, Bs[k][ta * 4 + x], acc[x]);
+            }
+        }
+        __syncthreads();
     }
     double *Ug = U + (int64_t)g * ug;
+    const int64_t po = p0 + tp;
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-        const int a = a0 + ta * 4 + c;
-        if (a >= v) continue;
-#pragma unroll
-        for (int r = 0; r < 4; r++) {
-            const int64_t pidx = p0 + tp + 32 * r;
-            if (pidx >= v2) continue;
-            Ug[((int64_t)a * v + pidx / v) * vc + pidx % v] = acc[r][c];
-        }
+    for (int x = 0; x < 4; x++) {
+        const int ax = a0 + ta * 4 + x;
+        if (ax < v && po < v2) Ug[((int64_t)ax * v + po / v) * vc + po % v] = acc[x];
     }
 }
 

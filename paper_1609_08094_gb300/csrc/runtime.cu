@@ -354,7 +354,8 @@ void fill_desc(Exec &ex, Problem &pb, int pbt) {
     d.task_e = pb.task_e;
     pb.u_task = 3 * pb.dm.ug;
     if (ex.prec == TCORR_FP64) {
-        pb.gemm_units = f64_units_per_task(pb.dm);
+        d.f64 = 1;
+        pb.gemm_units = f64_units_per_task(pb.dm, 128);
     } else if (ex.prec == TCORR_FP64_OZ) {
         std::string msg;
         if (oz_fill_desc(d, pb.op, pb.oz_e, msg) != cudaSuccess) throw Fail{TCORR_EUNSUPPORTED, msg};
@@ -389,6 +390,10 @@ int64_t seg_units(const Problem &pb, Seg &sg, PackTabs &tabs) {
     of.ent0 = tabs.ents.size();
     tabs.of.push_back(of);
     const InstDesc &d = pb.desc;
+    if (d.f64) {
+        sg.f64_tp = f64_tile_pairs(pb.dm, sg.ntb);
+        return sg.ntb * f64_units_per_task(pb.dm, sg.f64_tp);
+    }
     if (!d.packw) return sg.ntb * pb.gemm_units;
     // counting sort of the groups (s; p, q) of the tasks by (p, q).  Packed, the
     // passes are 256 columns wide instead of v, so an SM takes in fewer A rows per

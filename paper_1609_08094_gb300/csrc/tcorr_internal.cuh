@@ -93,6 +93,7 @@ struct InstDesc {
     int kind;                 // split-precision operand type: 1 = TF32, 2 = BF16 hi + lo
     int pair;                 // tensor-core tiles on SM pairs (cta_group::2, M = 256)
     int nbt, nct, npass, kv, ko, brows;
+    int f64;                  // FP64 W contractions
     int tblk;                 // SM pairs: tasks that go through the tile pairs together (tc_pair.cuh)
     int packw;                // SM pairs, packed columns (PackRun): columns per entry (v rounded to 16), 0: not packed
     uint32_t stage_tx;        // TMA bytes per pipeline stage
@@ -141,6 +142,7 @@ struct Seg {
     const PackRun *runs;      // packed columns: device tables (nrun runs), else NULL
     const PackEnt *ents;
     int nrun;
+    int f64_tp;               // FP64: pairs per tile
 };
 
 // last segment s with key(s) <= x (segments sorted by key, key(0) = 0)
@@ -193,8 +195,10 @@ cudaError_t launch_epilogue_ff_inputs(double *t1, double *ovov, const double *ep
 cudaError_t launch_build_tables(int o, int nb, int *tasks, int *orbits, cudaStream_t st);
 
 // ---- gemm_f64.cu ---------------------------------------------------------
-// FP64 work units of a segment: ntb * 3 * pair tiles * a tiles
-int64_t f64_units_per_task(const Dims &dm);
+// FP64: pairs per tile of a segment of ntb tasks, and its work units per task
+// (3 * pair tiles * a tiles)
+int f64_tile_pairs(const Dims &dm, int64_t ntb);
+int64_t f64_units_per_task(const Dims &dm, int tp);
 cudaError_t launch_ugemm_f64(const Wave &w, cudaStream_t st);
 
 // ---- epilogue.cu ---------------------------------------------------------
