@@ -462,6 +462,7 @@ struct EpiMeta {
     int smap[6];                 // slot whose cubes hold slot s's data (the first with its block triple)
     int kind;                    // 0: no more orbits, 1: A < B < C, 2: A = B < C, 3: A < B = C, 4: A = B = C
     int v;                       // virtual orbitals of the problem
+    int first;                   // warp that takes the first element orbits of repeated blocks
 };
 
 // Four rows r0..r3 of a 2-D tensor map (box: one row) to dst, back to back.
@@ -622,6 +623,7 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
                 for (int s = 0; s < 6; s++) m.smap[s] = smap[s];
                 m.kind = ob0 == ob1 ? (ob1 == ob2 ? 4 : 2) : (ob1 == ob2 ? 3 : 1);
                 m.v = v;
+                m.first = orb & (EPI_CW - 1);
                 mbar_expect_tx(full, u_bytes + ev_bytes + (EPI_PRODUCERS == 1 ? ovt1_bytes : 0u));
             }
             __syncwarp();
@@ -773,10 +775,10 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
             // where B = C, so that every element of the distinct cubes is met once;
             // of an orbit with equal indices only the slots of its distinct elements
             // count.  Each element's Z W and Z Y are formed in FP32 on their own; the
-            // warps take the orbits in turn (32 each, the first ones by another warp
-            // each time).
+            // warps take 32 orbits each, the first ones a warp given by the block orbit
+            // (by nothing else: the order of the sums must not depend on the wave).
             const int norb = kind == 4 ? 120 : 288;
-            for (int x = ((warp + n) & (EPI_CW - 1)) * 32 + lane; x < norb; x += NT) {
+            for (int x = ((warp + meta[stage].first) & (EPI_CW - 1)) * 32 + lane; x < norb; x += NT) {
                 const int pr = kind == 4 ? trip[x] : trip[120 + (x >> 3)], l8 = x & 7;
                 const int la = kind == 3 ? l8 : pr & 7;
                 const int lb = kind == 3 ? pr & 7 : (pr >> 3) & 7;
