@@ -235,8 +235,7 @@ struct tcorr_mp2_s {
     Exec ex;
     int o = 0, v = 0, naux = 0, kp = 0, nt = 0, ntp = 0;
     int64_t npair = 0, items = 0, nparts = 0;
-    double *Ct = nullptr, *eps_o = nullptr, *eps_v = nullptr, *partials = nullptr, *d_out = nullptr;
-    double *h_out = nullptr;
+    double *Ct = nullptr, *eps_o = nullptr, *eps_v = nullptr, *partials = nullptr;
     int *pairs = nullptr, *tiles = nullptr;
     // split precision (TF32X3 / BF16X3): hi and lo planes of C^T, FP32 eps_v, tensor maps
     void *ct_hi = nullptr, *ct_lo = nullptr;
@@ -341,7 +340,7 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
     // hi + lo operands (same four products, same kernel).
     if (op.prec == TCORR_BF16X3 && (double)o * (o + 1) / 2 * v * v * naux < TCORR_MP2_BF16_MIN_TERMS) op.prec = TCORR_TF32X3;
     try {
-        init_exec(ex, op, stream);  // SM count; split precision only on the sm_103 tensor cores
+        init_exec(ex, op, stream, true);  // SM count; split precision only on the sm_103 tensor cores
         const bool split = op.prec != TCORR_FP64;
         const int tile = split ? MP2_TC_TILE : MT;
         h->o = o;
@@ -362,8 +361,7 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
         h->gram = split && v <= MP2_GRAM_MAX_V;
         if (h->gram) mp2_plan_waves(o, v, ex.sm_count, h->waves, gram_tiles, g_floats, h->nparts);
         const size_t ct_bytes = (size_t)o * v * h->kp * elem_bytes(op.prec) * (split ? 2 : 1);  // hi + lo
-        size_t free_b = 0, total_b = 0;
-        CK(cudaMemGetInfo(&free_b, &total_b));
+        const size_t free_b = free_device_bytes(ex);
         const size_t need = ct_bytes + (size_t)h->nparts * 16 + (size_t)g_floats * 4 + (op.host_inputs ? (size_t)o * v * naux * 8 : 0) +
                             ((size_t)64 << 20);
         if (need > free_b)
@@ -373,15 +371,13 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
             dalloc(ex, h->ct_hi, plane);
             dalloc(ex, h->ct_lo, plane);
             dalloc(ex, h->eps_vf, (size_t)v * sizeof(float));
-            alloc_common(ex);  // device error flag of the bounded waits
         } else {
             dalloc(ex, h->Ct, ct_bytes);
         }
         dalloc(ex, h->eps_o, (size_t)o * sizeof(double));
         dalloc(ex, h->eps_v, (size_t)v * sizeof(double));
         dalloc(ex, h->partials, (size_t)h->nparts * 2 * sizeof(double));
-        dalloc(ex, h->d_out, 3 * sizeof(double));
-        halloc(ex, h->h_out, 3 * sizeof(double));
+        alloc_common(ex, 1);  // error flag of the bounded waits, (E_J, E_K, E)
         const bool host = op.host_inputs == 1;
         const cudaMemcpyKind kd = host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
         CK(cudaMemcpyAsync(h->eps_o, eps_occ, (size_t)o * sizeof(double), kd, ex.stream));
@@ -465,6 +461,7 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
         return f.st;
     } catch (const std::bad_alloc &) {
         g_create_error = "host allocation failed";
+        cudaStreamSynchronize(ex.stream);
         release(ex);
         delete h;
         return TCORR_ENOMEM;
@@ -500,15 +497,12 @@ tcorr_status tcorr_mp2_energy(tcorr_mp2_t h, double *e_out) {
         }
         {
             Timer tm(ex, KC_RED);
-            mp2_sum_kernel<<<1, MNT, 0, ex.stream>>>(h->partials, h->nparts, h->d_out);
+            mp2_sum_kernel<<<1, MNT, 0, ex.stream>>>(h->partials, h->nparts, ex.d_sums);
             CK(cudaGetLastError());
             tm.stop();
         }
-        CK(cudaMemcpyAsync(h->h_out, h->d_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
-        CK(cudaStreamSynchronize(ex.stream));
-        resolve_timers(ex);
-        if (ex.prec != TCORR_FP64) check_err_flag(ex);
-        for (int c = 0; c < 3; c++) e_out[c] = h->h_out[c];
+        finish_call(ex, 1);
+        for (int c = 0; c < 3; c++) e_out[c] = ex.h_sums[c];
     } catch (const Fail &f) {
         ex.last_error = f.msg;
         cudaStreamSynchronize(ex.stream);

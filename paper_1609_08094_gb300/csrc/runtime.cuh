@@ -60,9 +60,12 @@ struct Exec {
     int sm_count = 0, cc_major = 0, cc_minor = 0;
     cudaStream_t stream = nullptr;
     size_t bytes = 0;              // device bytes held
-    std::vector<void *> dev;       // every device allocation
-    std::vector<void *> host;      // every pinned host allocation
-    cudaMemPool_t pool = nullptr;  // set: stream-ordered allocations from this pool (freed in stream order)
+    struct DevPtr { void *p; bool pooled; };
+    std::vector<DevPtr> dev;       // every device allocation
+    struct HostPtr { void *p; size_t bytes; };
+    std::vector<HostPtr> host;     // every pinned host allocation
+    cudaMemPool_t pool = nullptr;  // stream-ordered allocations from this pool (freed in stream order) ...
+    size_t pool_max = SIZE_MAX;    // ... up to this size, larger ones with cudaMalloc
 
     void *U = nullptr;             // wave scratch
     int64_t u_cap = 0;             // elements
@@ -70,11 +73,13 @@ struct Exec {
     int64_t part_cap = 0;          // doubles
     int64_t wave_tasks = 0;        // tasks per wave (cap)
     InstDesc *d_descs = nullptr;   // device [ninst]
-    int *err = nullptr, *h_err = nullptr;
+    int *err = nullptr, *h_err = nullptr;  // device error flag and its copy: first in the returned block
 
     // per-call tables: segments of every wave and the spans to sum
     unsigned char *d_stage = nullptr, *h_stage = nullptr;
     size_t stage_cap = 0;
+    // what a call returns, one block and one copy: the error flag, then the span sums
+    unsigned char *d_ret = nullptr, *h_ret = nullptr;
     double *d_sums = nullptr, *h_sums = nullptr;
     int sums_cap = 0;
 
@@ -85,28 +90,18 @@ struct Exec {
     std::string last_error;
 };
 
+void *dalloc_bytes(Exec &ex, size_t bytes);
 template <typename T>
 void dalloc(Exec &ex, T *&ptr, size_t bytes) {
-    void *p = nullptr;
-    if (bytes == 0) bytes = 16;
-    cudaError_t e = ex.pool ? cudaMallocFromPoolAsync(&p, bytes, ex.pool, ex.stream) : cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        throw Fail{TCORR_ENOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed: " +
-                                     cudaGetErrorString(e)};
-    }
-    ex.dev.push_back(p);
-    ex.bytes += bytes;
-    ptr = static_cast<T *>(p);
+    ptr = static_cast<T *>(dalloc_bytes(ex, bytes));
 }
-
+void *halloc_bytes(Exec &ex, size_t bytes);
 template <typename T>
 void halloc(Exec &ex, T *&ptr, size_t bytes) {
-    void *p = nullptr;
-    CK(cudaMallocHost(&p, bytes ? bytes : 16));
-    ex.host.push_back(p);
-    ptr = static_cast<T *>(p);
+    ptr = static_cast<T *>(halloc_bytes(ex, bytes));
 }
+// Free device memory, what the handles' pool holds unused included
+size_t free_device_bytes(const Exec &ex);
 
 struct Timer {
     Exec &ex;
@@ -200,12 +195,15 @@ int64_t seg_units(const Problem &pb, Seg &sg, PackTabs &tabs);
 void place_tabs(const PackTabs &tabs, std::vector<Seg> &segs, unsigned char *dst, const unsigned char *dev);
 void upload_plan(Exec &ex, Plan &pl, Seg *&d_segs, SumSpan *&d_spans);
 void launch_plan(Exec &ex, const Plan &pl, const Seg *d_segs, const SumSpan *d_spans, cudaStream_t st);
+void raise_err_flag(Exec &ex);   // throws if the flag was set in the last copy
 void check_err_flag(Exec &ex);
 void finish_call(Exec &ex, int nspans);
 tcorr_status check_opts(const tcorr_opts &op, std::string &msg);
 bool sizes_supported(int o, int v);
-void init_exec(Exec &ex, const tcorr_opts &op, void *stream);
-void alloc_common(Exec &ex);
+// pooled: device memory from the handles' pool
+void init_exec(Exec &ex, const tcorr_opts &op, void *stream, bool pooled);
+// The returned block of a handle with nspans span sums
+void alloc_common(Exec &ex, int nspans);
 void upload_descs(Exec &ex, const std::vector<Problem *> &pbs);
 int tuned_pb(Exec &ex, Problem &pb);
 

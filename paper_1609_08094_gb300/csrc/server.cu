@@ -330,7 +330,7 @@ tcorr_status tcorr_server_create(tcorr_server_t *out, const tcorr_opts *opts, in
     }
     Exec &ex = s->ex;
     try {
-        init_exec(ex, op, stream);
+        init_exec(ex, op, stream, false);
         int dev = 0;
         CK(cudaGetDevice(&dev));
         cudaMemPoolProps pp{};
@@ -349,7 +349,7 @@ tcorr_status tcorr_server_create(tcorr_server_t *out, const tcorr_opts *opts, in
         dalloc(ex, ex.U, (size_t)ex.u_cap * ueb);
         dalloc(ex, ex.partials, (size_t)ex.part_cap * sizeof(double));
         dalloc(ex, ex.d_descs, (size_t)MAX_SLOTS * sizeof(InstDesc));
-        alloc_common(ex);
+        alloc_common(ex, 0);
         CK(cudaHostAlloc(&s->h_res, (size_t)MAX_SLOTS * 3 * sizeof(double), cudaHostAllocMapped));
         CK(cudaHostGetDevicePointer(reinterpret_cast<void **>(&s->d_res), s->h_res, 0));
         for (RingSlot &r : s->ring) {

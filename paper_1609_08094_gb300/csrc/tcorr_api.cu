@@ -32,6 +32,11 @@ struct tcorr_s {
     Exec ex;
     Problem pb;
     int batch = 1;  // tasks per wave
+    // the range whose plan is on the device (a repeated call finds it there)
+    int64_t plan_first = -1, plan_count = 0;
+    Plan plan;
+    Seg *d_segs = nullptr;
+    SumSpan *d_spans = nullptr;
 };
 
 struct tcorr_batch_s {
@@ -48,14 +53,19 @@ struct tcorr_batch_s {
 
 namespace {
 
+void place_plan(tcorr_s &hs, int64_t first, int64_t count) {
+    hs.plan_first = -1;
+    std::vector<Problem *> pbs{&hs.pb};
+    hs.plan = make_plan(hs.ex, pbs, {Span{0, first, count}});
+    upload_plan(hs.ex, hs.plan, hs.d_segs, hs.d_spans);
+    hs.plan_first = first;
+    hs.plan_count = count;
+}
+
 void run_range(tcorr_s &hs, int64_t first, int64_t count, double *e_out, double *e_task) {
     Exec &ex = hs.ex;
-    std::vector<Problem *> pbs{&hs.pb};
-    Plan pl = make_plan(ex, pbs, {Span{0, first, count}});
-    Seg *d_segs = nullptr;
-    SumSpan *d_spans = nullptr;
-    upload_plan(ex, pl, d_segs, d_spans);
-    launch_plan(ex, pl, d_segs, d_spans, ex.stream);
+    if (first != hs.plan_first || count != hs.plan_count) place_plan(hs, first, count);
+    launch_plan(ex, hs.plan, hs.d_segs, hs.d_spans, ex.stream);
     if (e_task)
         CK(cudaMemcpyAsync(e_task, hs.pb.task_e + 2 * first, (size_t)count * 2 * sizeof(double),
                            cudaMemcpyDeviceToHost, ex.stream));
@@ -120,13 +130,12 @@ tcorr_status tcorr_create(tcorr_t *out, int o, int v, const double *eps_occ,
     Exec &ex = hs->ex;
     Problem &pb = hs->pb;
     try {
-        init_exec(ex, op, stream);
+        init_exec(ex, op, stream, true);
         const Dims dm = make_dims(o, v);
         const int64_t ntask = (int64_t)o * (o + 1) * (o + 2) / 6;
         const int64_t u_task = 3 * dm.ug;
         const size_t u_task_bytes = (size_t)u_task * u_elem_bytes(ex.prec);
-        size_t free_b = 0, total_b = 0;
-        CK(cudaMemGetInfo(&free_b, &total_b));
+        const size_t free_b = free_device_bytes(ex);
         if (op.batch_tasks > 0) {
             hs->batch = op.batch_tasks;
         } else {
@@ -151,16 +160,12 @@ tcorr_status tcorr_create(tcorr_t *out, int o, int v, const double *eps_occ,
         ex.part_cap = (int64_t)hs->batch * pb.norb * 2;
         dalloc(ex, ex.U, (size_t)ex.u_cap * u_elem_bytes(ex.prec));
         dalloc(ex, ex.partials, (size_t)ex.part_cap * sizeof(double));
-        alloc_common(ex);
+        alloc_common(ex, 1);
         fill_desc(ex, pb, model_pb(v));
         if (is_split(ex.prec) && op.tune == 1) fill_desc(ex, pb, tuned_pb(ex, pb));
         upload_descs(ex, {&pb});
-        {   // staging for the largest plan (the whole task list), so that calls do not allocate
-            Plan pl = make_plan(ex, {&pb}, {Span{0, 0, pb.ntask}});
-            Seg *ds = nullptr;
-            SumSpan *dsp = nullptr;
-            upload_plan(ex, pl, ds, dsp);
-        }
+        // the plan of the whole task list; its staging is the largest, so that calls do not allocate
+        place_plan(*hs, 0, pb.ntask);
         CK(cudaStreamSynchronize(ex.stream));
         CK(cudaGetLastError());
         resolve_timers(ex);
@@ -173,6 +178,7 @@ tcorr_status tcorr_create(tcorr_t *out, int o, int v, const double *eps_occ,
         return f.st;
     } catch (const std::bad_alloc &) {
         g_create_error = "host allocation failed";
+        cudaStreamSynchronize(ex.stream);
         release(ex);
         delete hs;
         return TCORR_ENOMEM;
@@ -299,7 +305,7 @@ tcorr_status tcorr_batch_create(tcorr_batch_t *out, int n, const tcorr_problem *
     }
     Exec &ex = b->ex;
     try {
-        init_exec(ex, op, stream);
+        init_exec(ex, op, stream, true);
         b->eager = op.eager == 1 || op.profile != 0 || op.test_stall != 0;
         const size_t ueb = u_elem_bytes(ex.prec);
         size_t need = 64u << 20, stage = 0;
@@ -326,14 +332,13 @@ tcorr_status tcorr_batch_create(tcorr_batch_t *out, int n, const tcorr_problem *
         const int64_t max_wave_tasks = std::min<int64_t>(ex.wave_tasks, ex.u_cap / u_task_min + 1);
         ex.part_cap = std::max<int64_t>(norb_max * 2, max_wave_tasks * norb_max * 2);
         need += (size_t)ex.u_cap * ueb + (size_t)ex.part_cap * 8 + stage;
-        size_t free_b = 0, total_b = 0;
-        CK(cudaMemGetInfo(&free_b, &total_b));
+        const size_t free_b = free_device_bytes(ex);
         if (need > free_b)
             throw Fail{TCORR_ENOMEM, "footprint " + std::to_string(need) + " bytes exceeds free device memory " +
                                          std::to_string(free_b)};
         dalloc(ex, ex.U, (size_t)ex.u_cap * ueb);
         dalloc(ex, ex.partials, (size_t)ex.part_cap * sizeof(double));
-        alloc_common(ex);
+        alloc_common(ex, n);
         b->pbs.resize(n);
         b->pbt.assign(n, 0);
         for (int m = 0; m < n; m++) {
@@ -371,6 +376,7 @@ tcorr_status tcorr_batch_create(tcorr_batch_t *out, int n, const tcorr_problem *
         return f.st;
     } catch (const std::bad_alloc &) {
         g_create_error = "host allocation failed";
+        cudaStreamSynchronize(ex.stream);
         destroy_batch(b);
         return TCORR_ENOMEM;
     }
