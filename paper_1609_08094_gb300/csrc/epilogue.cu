@@ -92,12 +92,7 @@ __device__ __forceinline__ ff ff_recip(ff d) {
     const float e = fmaf(-d.lo, r, fmaf(-d.hi, r, 1.f));
     return {r, r * e};
 }
-// x * r for an FP32 x: the exact product error of x * r.hi plus x * r.lo
-__device__ __forceinline__ ff ff_mul(float x, ff r) {
-    const float p = x * r.hi;
-    return ff_fast(p, fmaf(x, r.lo, fmaf(x, r.hi, -p)));
-}
-// a * r: as above plus the product with a.lo
+// a * r: the product of the high parts with its exact error, and the cross terms
 __device__ __forceinline__ ff ff_mul2(ff a, ff r) {
     const float p = a.hi * r.hi;
     return ff_fast(p, fmaf(a.lo, r.hi, fmaf(a.hi, r.lo, fmaf(a.hi, r.hi, -p))));
@@ -107,6 +102,34 @@ __device__ __forceinline__ ff ff_of(double x) {  // x rounded to ~48 bits
     return {hi, (float)(x - (double)hi)};
 }
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
+
+// Packed pairs of FP32 values (two operations per instruction, each rounded to
+// nearest as the scalar one is).
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk2(float x, float y) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ f2 dup2(float x) { return pk2(x, x); }
+__device__ __forceinline__ void unpk2(f2 a, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a)); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 neg2(f2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) { return fma2(b, dup2(-1.f), a); }  // exact product: one rounding
 
 // A float-float number with arithmetic operators, the compute type of the
 // FP64-emulation epilogue: W, t1, ovov and the orbital energies arrive as
@@ -397,9 +420,12 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
 // compute warps), and the index arithmetic per element orbit is a handful of
 // precomputed offsets.  Orbits with repeated blocks read the six elements of an
 // element orbit once too.  With swizzled cubes and an element-by-element loop for repeated blocks the kernel
-// took 7.1 ms for 28 tasks of o=50, v=450 (6.6 ms now), 3.93 ms for o=13, v=131
-// (3.01) and 13.7 ms for 24 molecules of v = 20..120 (10.5), where most orbits
-// have repeated blocks.
+// took 7.1 ms for 28 tasks of o=50, v=450, 3.93 ms for o=13, v=131 and 13.7 ms for
+// 24 molecules of v = 20..120, where most orbits have repeated blocks; with scalar
+// arithmetic and the slots found by comparing block triples 6.7, 3.06 and 10.7 ms;
+// as it is 6.2, 2.85 and 10.1 ms.  Loads alone take 4.9, 2.1 and 7.6 ms (U at 5.2 to
+// 6.5 TB/s).  Preparing all of a producer lane's addresses before its wait for the
+// stage was slower (3.03 ms at v=131).
 //
 // The per-orbit sum over the CTA goes through shared memory in a fixed
 // order, summed by one compute warp per orbit in rotation, with
@@ -591,19 +617,12 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
                 break;
             }
             // slot s holds the cube with block pick3(ob, perm_pos(s, d)) along axis d;
-            // a slot whose triple repeats an earlier one's is not loaded
-            int smap[6], loaded = 0, nload = 0;
-#pragma unroll
-            for (int s = 0; s < 6; s++) {
-                smap[s] = s;
-#pragma unroll
-                for (int t = s - 1; t >= 0; t--)
-                    if (pick3(ob0, ob1, ob2, perm_pos(t, 0)) == pick3(ob0, ob1, ob2, perm_pos(s, 0)) &&
-                        pick3(ob0, ob1, ob2, perm_pos(t, 1)) == pick3(ob0, ob1, ob2, perm_pos(s, 1)) &&
-                        pick3(ob0, ob1, ob2, perm_pos(t, 2)) == pick3(ob0, ob1, ob2, perm_pos(s, 2)))
-                        smap[s] = t;
-                if (smap[s] == s) { loaded |= 1 << s; nload++; }
-            }
+            // a slot whose triple repeats an earlier one's reads that one's cube (slots:
+            // one per hex digit, slot 0 lowest) and is not loaded
+            const int kind = ob0 == ob1 ? (ob1 == ob2 ? 4 : 2) : (ob1 == ob2 ? 3 : 1);
+            const uint32_t slots = kind == 1 ? 0x543210u : (kind == 2 ? 0x441010u : (kind == 3 ? 0x323200u : 0u));
+            const uint32_t loaded = kind == 1 ? 0x3fu : (kind == 2 ? 0x13u : (kind == 3 ? 0xdu : 1u));
+            const int nload = __popc(loaded);
             const uint32_t full = smem_u32(&bar_full[stage]);
             // the copies of an orbit: the U cubes of each distinct slot (the three
             // group terms side by side, one 6 KB bulk copy each); the 27 ovov
@@ -620,8 +639,8 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
                 m.eijk = eijk;
                 m.ob[0] = ob0; m.ob[1] = ob1; m.ob[2] = ob2;
 #pragma unroll
-                for (int s = 0; s < 6; s++) m.smap[s] = smap[s];
-                m.kind = ob0 == ob1 ? (ob1 == ob2 ? 4 : 2) : (ob1 == ob2 ? 3 : 1);
+                for (int s = 0; s < 6; s++) m.smap[s] = (slots >> (4 * s)) & 15;
+                m.kind = kind;
                 m.v = v;
                 m.first = orb & (EPI_CW - 1);
                 mbar_expect_tx(full, u_bytes + ev_bytes + (EPI_PRODUCERS == 1 ? ovt1_bytes : 0u));
@@ -718,57 +737,81 @@ __global__ void __launch_bounds__(EPI_THREADS, EPI_CTAS) epilogue_f32_kernel(con
         if (kind == 1) {
             // Distinct blocks: with E and O the sums of W over the even and odd slots,
             // Z at slot q is 6 w_q + 2E - 4O (q even) or 6 w_q + 2O - 4E (q odd), and all
-            // six share one denominator.  What depends only on b and c is read once
-            // for the thread's two orbits.
+            // six share one denominator.  The thread's two orbits go through the
+            // arithmetic side by side, as the halves of packed FP32 pairs; what depends
+            // only on b and c is read once for both.
+            const int la = la0, lA = la0 ^ 4;
+            const bool in0 = B0 + lb < v && C0 + lc < v && A0 + la < v, in1 = B0 + lb < v && C0 + lc < v && A0 + lA < v;
             const float *c0 = S.cube[0][0], *c1 = S.cube[1][0], *c2 = S.cube[2][0];
             const float *c3 = S.cube[3][0], *c4 = S.cube[4][0], *c5 = S.cube[5][0];
-            const float tib = S.t1[0][1][lb], tic = S.t1[0][2][lc];
-            const float tjb = S.t1[1][1][lb], tjc = S.t1[1][2][lc];
-            const float tkb = S.t1[2][1][lb], tkc = S.t1[2][2][lc];
-            const float jk_bc = OVV(0, 1, 2, lb, lc), jk_cb = OVV(0, 2, 1, lc, lb);
-            const float ik_bc = OVV(1, 1, 2, lb, lc), ik_cb = OVV(1, 2, 1, lc, lb);
-            const float ij_bc = OVV(2, 1, 2, lb, lc), ij_cb = OVV(2, 2, 1, lc, lb);
+            // W at slot (x, y, z) = C0 + C1 + C2, each with its group's a (x, y, z)
+            // innermost; x: the bit that tells the two orbits apart there
+#define W2(cq, p0, x0, p1, x1, p2, x2)                                                         \
+    add2(add2(pk2(cq[p0], cq[(p0) ^ (x0)]), pk2(cq[512 + (p1)], cq[512 + ((p1) ^ (x1))])),     \
+         pk2(cq[1024 + (p2)], cq[1024 + ((p2) ^ (x2))]))
+            const f2 w0 = W2(c0, p_bca, 4, p_acb, 256, p_abc, 256), w1 = W2(c1, p_cba, 4, p_abc, 256, p_acb, 256);
+            const f2 w2 = W2(c2, p_acb, 256, p_bca, 4, p_bac, 32), w3 = W2(c3, p_cab, 32, p_bac, 32, p_bca, 4);
+            const f2 w4 = W2(c4, p_abc, 256, p_cba, 4, p_cab, 32), w5 = W2(c5, p_bac, 32, p_cab, 32, p_cba, 4);
+#undef W2
+            // t1 of occupied i, j, k; (j u | k w), (i u | k w), (i u | j w) for the ordered pairs of {a, b, c}
+#define A2(oc) pk2(S.t1[oc][0][la], S.t1[oc][0][lA])
+#define ROW2(sl, pw, lw) pk2(OVV(sl, 0, pw, la, lw), OVV(sl, 0, pw, lA, lw))
+#define COL2(sl, pu, lu) pk2(OVV(sl, pu, 0, lu, la), OVV(sl, pu, 0, lu, lA))
+            const f2 tia = A2(0), tja = A2(1), tka = A2(2);
+            const f2 tib = dup2(S.t1[0][1][lb]), tic = dup2(S.t1[0][2][lc]);
+            const f2 tjb = dup2(S.t1[1][1][lb]), tjc = dup2(S.t1[1][2][lc]);
+            const f2 tkb = dup2(S.t1[2][1][lb]), tkc = dup2(S.t1[2][2][lc]);
+            const f2 jk_bc = dup2(OVV(0, 1, 2, lb, lc)), jk_cb = dup2(OVV(0, 2, 1, lc, lb));
+            const f2 ik_bc = dup2(OVV(1, 1, 2, lb, lc)), ik_cb = dup2(OVV(1, 2, 1, lc, lb));
+            const f2 ij_bc = dup2(OVV(2, 1, 2, lb, lc)), ij_cb = dup2(OVV(2, 2, 1, lc, lb));
+            const f2 jk_ac = ROW2(0, 2, lc), jk_ca = COL2(0, 2, lc), jk_ab = ROW2(0, 1, lb), jk_ba = COL2(0, 1, lb);
+            const f2 ik_ac = ROW2(1, 2, lc), ik_ca = COL2(1, 2, lc), ik_ab = ROW2(1, 1, lb), ik_ba = COL2(1, 1, lb);
+            const f2 ij_ac = ROW2(2, 2, lc), ij_ca = COL2(2, 2, lc), ij_ab = ROW2(2, 1, lb), ij_ba = COL2(2, 1, lb);
+#undef A2
+#undef ROW2
+#undef COL2
+            // Y at each ordering q of (a,b,c): t^{q0}_i (j q1|k q2) + t^{q1}_j (i q0|k q2) + t^{q2}_k (i q0|j q1)
+            const f2 y0 = fma2(tkc, ij_ab, fma2(tia, jk_bc, mul2(tjb, ik_ac)));
+            const f2 y1 = fma2(tkb, ij_ac, fma2(tia, jk_cb, mul2(tjc, ik_ab)));
+            const f2 y2 = fma2(tkc, ij_ba, fma2(tib, jk_ac, mul2(tja, ik_bc)));
+            const f2 y3 = fma2(tka, ij_bc, fma2(tib, jk_ca, mul2(tjc, ik_ba)));
+            const f2 y4 = fma2(tkb, ij_ca, fma2(tic, jk_ab, mul2(tja, ik_cb)));
+            const f2 y5 = fma2(tka, ij_cb, fma2(tic, jk_ba, mul2(tjb, ik_ca)));
+            const f2 E = add2(add2(w0, w3), w4), O = add2(add2(w1, w2), w5);
+            const f2 ww = fma2(w5, w5, fma2(w4, w4, fma2(w3, w3, fma2(w2, w2, fma2(w0, w0, mul2(w1, w1))))));
+            const f2 wy = fma2(w5, y5, fma2(w4, y4, fma2(w3, y3, fma2(w2, y2, fma2(w0, y0, mul2(w1, y1))))));
+            const f2 k2 = dup2(2.f), k4 = dup2(-4.f), k6 = dup2(6.f);
+            // 6 ww + 2 (E^2 + O^2) - 8 E O, 6 wy + (2E - 4O) (y0 + y3 + y4) + (2O - 4E) (y1 + y2 + y5)
+            const f2 s4 = fma2(mul2(dup2(-8.f), E), O, fma2(k6, ww, mul2(k2, fma2(E, E, mul2(O, O)))));
+            const f2 s5 = fma2(fma2(k2, O, mul2(k4, E)), add2(add2(y1, y2), y5),
+                               fma2(k6, wy, mul2(fma2(k2, E, mul2(k4, O)), add2(add2(y0, y3), y4))));
+            // D in float-float (ff_sub), its reciprocal (ff_recip), the products with it (ff_mul)
             const ff evb = {S.ev[1][lb].x, S.ev[1][lb].y}, evc = {S.ev[2][lc].x, S.ev[2][lc].y};
             const ff dbc = ff_sub(ff_sub(eijk, evb), evc);
-            const bool bc_in = B0 + lb < v && C0 + lc < v;
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int la = la0 ^ (4 * h);
-                if (!bc_in || A0 + la >= v) continue;
-                // W at slot (x, y, z) = C0 + C1 + C2, each with its group's a (x, y, z) innermost
-                const int abc = p_abc ^ (h * 256), acb = p_acb ^ (h * 256), bac = p_bac ^ (h * 32);
-                const int bca = p_bca ^ (h * 4), cab = p_cab ^ (h * 32), cba = p_cba ^ (h * 4);
-                const float w0 = c0[bca] + c0[512 + acb] + c0[1024 + abc];
-                const float w1 = c1[cba] + c1[512 + abc] + c1[1024 + acb];
-                const float w2 = c2[acb] + c2[512 + bca] + c2[1024 + bac];
-                const float w3 = c3[cab] + c3[512 + bac] + c3[1024 + bca];
-                const float w4 = c4[abc] + c4[512 + cba] + c4[1024 + cab];
-                const float w5 = c5[bac] + c5[512 + cab] + c5[1024 + cba];
-                // t1 of occupied i, j, k at a (at b and c above)
-                const float tia = S.t1[0][0][la], tja = S.t1[1][0][la], tka = S.t1[2][0][la];
-                // (j u | k w), (i u | k w), (i u | j w) for the ordered pairs of {a, b, c} that hold a
-                const float jk_ac = OVV(0, 0, 2, la, lc), jk_ca = OVV(0, 2, 0, lc, la);
-                const float jk_ab = OVV(0, 0, 1, la, lb), jk_ba = OVV(0, 1, 0, lb, la);
-                const float ik_ac = OVV(1, 0, 2, la, lc), ik_ca = OVV(1, 2, 0, lc, la);
-                const float ik_ab = OVV(1, 0, 1, la, lb), ik_ba = OVV(1, 1, 0, lb, la);
-                const float ij_ac = OVV(2, 0, 2, la, lc), ij_ca = OVV(2, 2, 0, lc, la);
-                const float ij_ab = OVV(2, 0, 1, la, lb), ij_ba = OVV(2, 1, 0, lb, la);
-                // Y at each ordering q of (a,b,c): t^{q0}_i (j q1|k q2) + t^{q1}_j (i q0|k q2) + t^{q2}_k (i q0|j q1)
-                const float y0 = tia * jk_bc + tjb * ik_ac + tkc * ij_ab;
-                const float y1 = tia * jk_cb + tjc * ik_ab + tkb * ij_ac;
-                const float y2 = tib * jk_ac + tja * ik_bc + tkc * ij_ba;
-                const float y3 = tib * jk_ca + tjc * ik_ba + tka * ij_bc;
-                const float y4 = tic * jk_ab + tja * ik_cb + tkb * ij_ca;
-                const float y5 = tic * jk_ba + tjb * ik_ca + tka * ij_cb;
-                const float E = w0 + w3 + w4, O = w1 + w2 + w5;
-                const float ww = w0 * w0 + w1 * w1 + w2 * w2 + w3 * w3 + w4 * w4 + w5 * w5;
-                const float wy = w0 * y0 + w1 * y1 + w2 * y2 + w3 * y3 + w4 * y4 + w5 * y5;
-                const float s4 = 6.f * ww + 2.f * (E * E + O * O) - 8.f * E * O;
-                const float s5 = 6.f * wy + (2.f * E - 4.f * O) * (y0 + y3 + y4) + (2.f * O - 4.f * E) * (y1 + y2 + y5);
-                const ff eva = {S.ev[0][la].x, S.ev[0][la].y};
-                const ff r = ff_recip(ff_sub(dbc, eva));
-                A4 = ff_add(A4, ff_mul(s4, r));
-                A5 = ff_add(A5, ff_mul(s5, r));
+            const float2 ea = S.ev[0][la], eA = S.ev[0][lA];
+            const f2 dh = dup2(dbc.hi), nh = pk2(-ea.x, -eA.x);
+            const f2 sh = add2(dh, nh), sb = sub2(sh, dh);
+            const f2 se = add2(sub2(dh, sub2(sh, sb)), sub2(nh, sb));
+            const f2 sl = add2(se, sub2(dup2(dbc.lo), pk2(ea.y, eA.y)));
+            const f2 Dh = add2(sh, sl), Dl = sub2(sl, sub2(Dh, sh));
+            float d0, d1;
+            unpk2(Dh, d0, d1);
+            const f2 rh = pk2(__fdividef(1.f, d0), __fdividef(1.f, d1));
+            const f2 re = fma2(neg2(Dl), rh, fma2(neg2(Dh), rh, dup2(1.f)));
+            const f2 rl = mul2(rh, re);
+            const f2 m4 = mul2(s4, rh), m5 = mul2(s5, rh);
+            const f2 l4 = fma2(s4, rl, fma2(s4, rh, neg2(m4))), l5 = fma2(s5, rl, fma2(s5, rh, neg2(m5)));
+            const f2 h4 = add2(m4, l4), h5 = add2(m5, l5);
+            const f2 t4 = sub2(l4, sub2(h4, m4)), t5 = sub2(l5, sub2(h5, m5));
+            ff x4, X4, x5, X5;
+            unpk2(h4, x4.hi, X4.hi);
+            unpk2(t4, x4.lo, X4.lo);
+            unpk2(h5, x5.hi, X5.hi);
+            unpk2(t5, x5.lo, X5.lo);
+            if (in0) { A4 = x4; A5 = x5; }
+            if (in1) {
+                A4 = in0 ? ff_add(A4, X4) : X4;
+                A5 = in0 ? ff_add(A5, X5) : X5;
             }
         } else {
             // Repeated blocks: the element orbits with a <= b where A = B and b <= c
