@@ -408,11 +408,13 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_tc_pair_kernel(const __
             const int nbx = uni(sl.nbx);
             const bool boxes = uni(sl.boxes) != 0;
             const uint32_t stage_tx = uni(sl.stage_tx);
-            int bs[PACK_BOXES], ba[PACK_BOXES];
+            int bs[PACK_BOXES], ba[PACK_BOXES], bh[PACK_BOXES], br[PACK_BOXES];
 #pragma unroll
             for (int b = 0; b < PACK_BOXES; b++) {
                 bs[b] = uni(sl.box[b].x);
                 ba[b] = uni(sl.box[b].y);
+                bh[b] = uni(sl.box[b].z);
+                br[b] = uni(sl.box[b].w);
             }
             if (lane == 0) mbar_arrive(smem_u32(&bar_sempty[n % PAIR_SLOTS]));
             for (int seg = 0; seg < 4 && ok; seg++) {
@@ -425,7 +427,6 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_tc_pair_kernel(const __
                     case 2: amap = MAP_T2K_NAT; aslice = pp; bmap = MAP_AON; bmul = 1; badd = q * o; break;
                     default: amap = MAP_T2K_SWP; aslice = q; bmap = MAP_AON; bmul = 1; badd = pp * o; break;
                 }
-                if (boxes) bmap += MAP_T2R_PK - MAP_T2R;
                 // two chunks per stage; the second segment of a kind with an odd chunk
                 // count gives its first chunk to the block that the first one left
                 // half full (a stage of its own: the half that is not used is the next
@@ -457,8 +458,10 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_tc_pair_kernel(const __
                                     if (b < nbx) {
                                         // past the valid columns: a row past the tensor, zero fill
                                         const int brow = bs[b] < 0 ? o * o : bs[b] * bmul + badd;
-                                        tma_load_3d_pair(sB + b * PACK_BOX_BYTES, &d->maps[bmap][0], full_l, k0, ba[b], brow);
-                                        tma_load_3d_pair(sBl + b * PACK_BOX_BYTES, &d->maps[bmap][1], full_l, k0, ba[b], brow);
+                                        const CUtensorMap *m = &d->pmaps[bh[b] & 3][bmap - MAP_T2R][0];
+                                        const uint32_t off = (uint32_t)br[b] * PAIR_ROW;
+                                        tma_load_3d_pair(sB + off, m, full_l, k0, ba[b], brow);
+                                        tma_load_3d_pair(sBl + off, m + 1, full_l, k0, ba[b], brow);
                                     }
                                 }
                             }
@@ -715,18 +718,20 @@ cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int 
             uint64_t st[2] = {dp * eb, V * dp * eb};
             uint32_t box[3] = {bk, brows, 1};
             if (!encode(&d.maps[MAP_T2R][part], dt, 3, src[2], dims, st, box, err, "T2R", swz)) return cudaErrorInvalidValue;
-            box[1] = PACK_ROWS;
-            if (d.packw && !encode(&d.maps[MAP_T2R_PK][part], dt, 3, src[2], dims, st, box, err, "T2R packed", swz))
-                return cudaErrorInvalidValue;
+            for (int h = 0; d.packw && h < 4; h++) {
+                box[1] = (uint32_t)(PACK_ROWS << h);
+                if (!encode(&d.pmaps[h][0][part], dt, 3, src[2], dims, st, box, err, "T2R packed", swz)) return cudaErrorInvalidValue;
+            }
         }
         {   // AoN: (l, a, q*o+s)
             uint64_t dims[3] = {O, V, O * O};
             uint64_t st[2] = {lp * eb, V * lp * eb};
             uint32_t box[3] = {bk, brows, 1};
             if (!encode(&d.maps[MAP_AON][part], dt, 3, src[3], dims, st, box, err, "AoN", swz)) return cudaErrorInvalidValue;
-            box[1] = PACK_ROWS;
-            if (d.packw && !encode(&d.maps[MAP_AON_PK][part], dt, 3, src[3], dims, st, box, err, "AoN packed", swz))
-                return cudaErrorInvalidValue;
+            for (int h = 0; d.packw && h < 4; h++) {
+                box[1] = (uint32_t)(PACK_ROWS << h);
+                if (!encode(&d.pmaps[h][1][part], dt, 3, src[3], dims, st, box, err, "AoN packed", swz)) return cudaErrorInvalidValue;
+            }
         }
     }
     return cudaSuccess;

@@ -18,8 +18,8 @@ constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;  // 2 s of wall time per wait 
 constexpr uint32_t WAIT_MIN_POLLS = 1u << 18;      // ... and at least this many polls, so that time
                                                    // spent off the GPU (pre-emption) never counts
 
-enum { MAP_G_NAT = 0, MAP_G_SWP, MAP_T2K_NAT, MAP_T2K_SWP, MAP_T2R, MAP_AON, MAP_T2R_PK, MAP_AON_PK, NMAP };
-static_assert(NMAP == 8, "InstDesc::maps holds eight operand maps");
+enum { MAP_G_NAT = 0, MAP_G_SWP, MAP_T2K_NAT, MAP_T2K_SWP, MAP_T2R, MAP_AON, NMAP };
+static_assert(NMAP == 6, "InstDesc::maps holds six operand maps");
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));

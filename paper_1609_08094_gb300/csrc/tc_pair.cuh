@@ -19,9 +19,12 @@ constexpr int PAIR_BM = 128;              // pair rows per CTA tile
 constexpr int PAIR_BN = 256;              // widest pass
 constexpr int PAIR_ROW = 128;             // one K block (two chunks) per shared-memory row, 128-byte swizzle
 constexpr int PAIR_A = PAIR_BM * PAIR_ROW;  // 16 KB per A plane
-constexpr int PACK_ROWS = 16;             // rows of a B box of packed columns
-constexpr int PACK_BOXES = PAIR_BN / 2 / PACK_ROWS;  // boxes per CTA and plane at N = 256
-constexpr int PACK_BOX_BYTES = PACK_ROWS * PAIR_ROW;
+// B rows of packed columns come in boxes of 16, 32, 64 or 128 rows, each within one
+// entry: as few as its columns allow.  With boxes of 16 rows only, eight per plane and
+// stage, the contraction of o=13, v=131 took 9.31 ms (9.01 so), of 24 molecules of
+// v = 20..120 17.4 ms (17.0).
+constexpr int PACK_ROWS = 16;
+constexpr int PACK_BOXES = PAIR_BN / 2 / PACK_ROWS;  // most boxes per CTA and plane
 
 struct PairCache {
     SegCache s;
@@ -143,11 +146,11 @@ struct PairSlot {
     int o, v, kv, ko, kind;
     int p, q, N, cb, cc;    // A slices, columns, first b and c of this CTA's tile
     uint32_t stage_tx;      // bytes of a stage, both CTAs'
-    int nbx, boxes;         // B copies per plane and stage; in 16-row boxes?
+    int nbx, boxes;         // B copies per plane and stage; in boxes of packed columns?
     int pc, packed, empty;
     int g, pass0, ncol;     // not packed: group and columns of a
     int scale;              // FP64 emulation: E_A + E_B
-    int2 box[PACK_BOXES];   // (s, first a) of the B copies, s = -1 past the valid columns
+    int4 box[PACK_BOXES];   // B copies: s (-1 past the valid columns), first a, log2(rows / 16), first row
     int2 ent[PAIR_BN / 8];  // packed: (tbg, a) of columns 8 k .. 8 k + 7, a = 2^20 for none
 };
 constexpr int PAIR_SLOTS = 4;
@@ -205,9 +208,7 @@ __device__ __forceinline__ void pair_scheduler(const Wave &wv, uint32_t cid, uin
                 sl.N = w.N;
                 sl.cb = w.bt * d.pb;
                 sl.cc = w.ct * d.pc;
-                sl.nbx = w.boxes ? w.N / (2 * PACK_ROWS) : 1;
-                sl.stage_tx = w.boxes ? 2u * (2u * PAIR_A + 2u * (uint32_t)(w.N / (2 * PACK_ROWS) * PACK_BOX_BYTES))
-                                      : d.stage_tx;
+                sl.stage_tx = w.boxes ? 2u * (2u * PAIR_A + 2u * (uint32_t)(w.N / 2) * PAIR_ROW) : d.stage_tx;
                 sl.boxes = w.boxes;
                 sl.pc = d.pc;
                 sl.packed = w.packed;
@@ -217,17 +218,29 @@ __device__ __forceinline__ void pair_scheduler(const Wave &wv, uint32_t cid, uin
                 sl.ncol = w.ncol;
                 sl.scale = d.oz_e ? d.oz_e[0] + d.oz_e[1] : 0;
             }
-            if (!w.boxes) {
-                if (lane == 0)
-                    sl.box[0] = make_int2(w.packed ? pc.ents[w.ent0].s : w.s, w.pass0 + (int)rank * (w.N / 2));
-            } else if (lane < PACK_BOXES) {
-                const int x = (int)rank * (w.N / 2) + PACK_ROWS * lane;  // column in the pass
-                int2 e = make_int2(-1, 0);
-                if (x < w.ncol && lane < w.N / (2 * PACK_ROWS)) {
-                    const int col = w.pass0 + x, m = col / d.packw;
-                    e = make_int2(pc.ents[w.ent0 + m].s, col - m * d.packw);
+            if (lane == 0) {
+                int nbx = 1;
+                if (!w.boxes) {
+                    sl.box[0] = make_int4(w.packed ? pc.ents[w.ent0].s : w.s, w.pass0 + (int)rank * (w.N / 2), 0, 0);
+                } else {
+                    // the CTA's half of the pass, entry by entry, in the largest boxes that fit
+                    const int half = w.N / 2;
+                    nbx = 0;
+                    for (int row = 0; row < half;) {
+                        const int x = (int)rank * half + row;
+                        int len = half - row, a = 0, s = -1;
+                        if (x < w.ncol) {
+                            const int col = w.pass0 + x, m = col / d.packw;
+                            a = col - m * d.packw;
+                            s = pc.ents[w.ent0 + m].s;
+                            len = min(len, min(d.packw - a, w.ncol - x));
+                        }
+                        const int h = len >= 128 ? 3 : (len >= 64 ? 2 : (len >= 32 ? 1 : 0));
+                        sl.box[nbx++] = make_int4(s, a, h, row);
+                        row += PACK_ROWS << h;
+                    }
                 }
-                sl.box[lane] = e;
+                sl.nbx = nbx;
             }
             if (w.packed) {
                 int2 e = make_int2(0, 1 << 20);

@@ -84,8 +84,8 @@ struct Operands {
 // a single handle has one, a batch one per problem.  Aligned like its tensor
 // maps (alignof(CUtensorMap)), so an array of them keeps every map aligned.
 struct InstDesc {
-    CUtensorMap maps[8][2];   // tensor-core operand maps [G, G swapped, T2K, T2K swapped, T2R, AoN, and T2R, AoN in
-                              // 16-row boxes for packed columns][hi, lo]
+    CUtensorMap maps[6][2];   // tensor-core operand maps [G, G swapped, T2K, T2K swapped, T2R, AoN][hi, lo]
+    CUtensorMap pmaps[4][2][2];  // packed columns: [box of 16, 32, 64, 128 rows][T2R, AoN][hi, lo]
     CUtensorMap emaps[3];     // mixed epilogue row maps for 4-row gathers: ovov 8x8 blocks, t1 rows, eps_v blocks
     Dims dm;
     int pb, pc;               // tensor-core pair tile: pb values of b x pc values of c (pb * pc = 128)
