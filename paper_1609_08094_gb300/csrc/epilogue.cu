@@ -101,6 +101,13 @@ __device__ __forceinline__ ff ff_of(double x) {  // x rounded to ~48 bits
     const float hi = (float)x;
     return {hi, (float)(x - (double)hi)};
 }
+// (double)x from the two formats' fields: a conversion instruction occupies the
+// FP64 pipe as long as an FP64 sum does; zeros, subnormals, infinities and NaN take it
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+    if (e - 1u >= 254u) return (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
 
 // Packed pairs of FP32 values (two operations per instruction, each rounded to
@@ -147,7 +154,7 @@ struct dd {
     }
     __device__ __forceinline__ dd(ff a) : hi(a.hi), lo(a.lo) {}
     __device__ __forceinline__ operator ff() const { return ff{hi, lo}; }
-    __device__ __forceinline__ explicit operator double() const { return (double)hi + (double)lo; }
+    __device__ __forceinline__ explicit operator double() const { return widen(hi) + widen(lo); }
     __device__ __forceinline__ dd &operator+=(dd b) { return *this = dd(ff_add(*this, b)); }
 };
 __device__ __forceinline__ dd operator+(dd a, dd b) { return dd(ff_add(a, b)); }
@@ -207,7 +214,9 @@ template <> __device__ __forceinline__ dd eps_vir<dd>(const InstDesc &p, int x) 
 // share one denominator and the E/O expansion of Z, as in the mixed epilogue; where
 // blocks repeat, only the orbits with a <= b (b <= c), about half of the warps' work
 // of one element at a time (o=4, v=20: 33 us, now 26; 52 tasks of o=40, v=300 in FP64
-// emulation 18.1 ms, now 16.8).  CT = double (FP64 path: U, t1, ovov
+// emulation 18.1 ms, then 16.8; with the sum of the occupied energies formed once, no
+// compensated sum of one term and the energies widened without conversion instructions,
+// 16.0).  CT = double (FP64 path: U, t1, ovov
 // in FP64) or dd (FP64 emulation: all of them float-float pairs, so that no
 // operation per element runs on the FP64 pipe).
 template <typename CT, int TE>
@@ -219,6 +228,7 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
     constexpr int NE = TE * TE * TE;         // elements per cube
     __shared__ short trip[156];
     __shared__ double red[NT][2];
+    __shared__ CT eijk_sh;
 
     const int64_t item = blockIdx.x;
     const Seg sg = wv.segs[seg_find(wv.segs, wv.nseg, item, [](const Seg &x) { return x.epi0; })];
@@ -263,6 +273,7 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
             rc[it] = __ldg(reinterpret_cast<const double2 *>(U2 + ((int64_t)zb * v + xb) * vc + yb));
     }
     if (tid < 64) sorted_entry(trip, tid);
+    if (tid == NT - 1) eijk_sh = CT(p.eps_o[ti] + p.eps_o[tj] + p.eps_o[tkk]);
 #pragma unroll
     for (int it = 0; it < 6; it++) {
         const int e2 = tid + it * NT;
@@ -288,14 +299,14 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
 
     const CT *t1 = static_cast<const CT *>(p.t1);
     const CT *ov = static_cast<const CT *>(p.ovov);
-    const CT eijk = CT(p.eps_o[ti] + p.eps_o[tj] + p.eps_o[tkk]);
+    const CT eijk = eijk_sh;
     // ovov rows used by Y: (j y | k z), (i x | k z), (i x | j y)
     const CT *ov_jk = ov + ((int64_t)tj * v * o + tkk) * v;   // [y][z] stride o*v in y
     const CT *ov_ik = ov + ((int64_t)ti * v * o + tkk) * v;   // [x][z]
     const CT *ov_ij = ov + ((int64_t)ti * v * o + tj) * v;    // [x][y]
     const int64_t ovs = (int64_t)o * v;
 
-    double s4 = 0.0, c4 = 0.0, s5 = 0.0, c5 = 0.0;
+    CT a4 = CT(0), a5 = CT(0);
     if (ob0 < ob1 && ob1 < ob2) {
         // distinct blocks A < B < C: element orbits; slot q holds the element
         // with indices ordered as q (abc, acb, bac, bca, cab, cba); even slots
@@ -306,7 +317,6 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
         const int A0 = ob0 * TE, B0 = ob1 * TE, C0 = ob2 * TE;
         const int lb = (tid / TE) % TE, lc = tid % TE, la0 = tid / (TE * TE);
         const int b = B0 + lb, c = C0 + lc;
-        CT a4 = CT(0), a5 = CT(0);
         if (b < v && c < v) {
         const CT tib = t1[ti * v + b], tic = t1[ti * v + c];
         const CT tjb = t1[tj * v + b], tjc = t1[tj * v + c];
@@ -350,15 +360,12 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
             a5 += q5 * r;
         }
         }
-        kahan_add(s4, c4, double(a4));
-        kahan_add(s5, c5, double(a5));
     } else {
         // repeated blocks: the element orbits with a <= b where A = B and b <= c where
         // B = C; of one with two equal indices the six slots repeat three elements
         // (weight 1/2), with three Z vanishes
         const int kind = ob0 == ob1 ? (ob1 == ob2 ? 4 : 2) : 3;
         const int norb = kind == 4 ? 120 : 288;
-        CT a4 = CT(0), a5 = CT(0);
         for (int x = tid; x < norb; x += NT) {
             const int pr = kind == 4 ? trip[x] : trip[120 + (x >> 3)], l8 = x & 7;
             const int la = kind == 3 ? l8 : pr & 7;
@@ -388,10 +395,8 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
             a4 += q4 * r;
             a5 += q5 * r;
         }
-        kahan_add(s4, c4, double(a4));
-        kahan_add(s5, c5, double(a5));
     }
-    cta_sum2(s4 - c4, s5 - c5, red, out, tid);  // the compensation folded
+    cta_sum2(double(a4), double(a5), red, out, tid);
 }
 
 
