@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cstddef>
 #include <mutex>
+#include <type_traits>
 
 #include "tc_common.cuh"
 
@@ -166,6 +167,45 @@ __device__ __forceinline__ dd operator*(dd a, dd b) {
     return dd(ff_fast(p, e));
 }
 __device__ __forceinline__ dd operator/(dd a, dd b) { return a * dd(ff_recip(b)); }
+// Two independent dd numbers, one per half of the packed FP32 instructions: every
+// operation rounds each half as the scalar one does
+struct dd2 {
+    f2 hi, lo;
+    dd2() = default;
+    __device__ __forceinline__ explicit dd2(int c) : hi(dup2((float)c)), lo(0ull) {}
+    __device__ __forceinline__ dd2(f2 h, f2 l) : hi(h), lo(l) {}
+    __device__ __forceinline__ dd2(dd x, dd y) : hi(pk2(x.hi, y.hi)), lo(pk2(x.lo, y.lo)) {}
+    __device__ __forceinline__ explicit dd2(dd x) : hi(dup2(x.hi)), lo(dup2(x.lo)) {}
+    __device__ __forceinline__ void unpack(dd &x, dd &y) const {
+        unpk2(hi, x.hi, y.hi);
+        unpk2(lo, x.lo, y.lo);
+    }
+};
+__device__ __forceinline__ dd2 fast2(f2 a, f2 b) {  // ff_fast
+    const f2 s = add2(a, b);
+    return dd2(s, sub2(b, sub2(s, a)));
+}
+__device__ __forceinline__ dd2 operator+(dd2 a, dd2 b) {  // ff_add
+    const f2 s = add2(a.hi, b.hi), bb = sub2(s, a.hi);
+    const f2 e = add2(sub2(a.hi, sub2(s, bb)), sub2(b.hi, bb));
+    return fast2(s, add2(e, add2(a.lo, b.lo)));
+}
+__device__ __forceinline__ dd2 operator-(dd2 a, dd2 b) { return a + dd2(neg2(b.hi), neg2(b.lo)); }
+__device__ __forceinline__ dd2 operator*(dd2 a, dd2 b) {
+    const f2 p = mul2(a.hi, b.hi);
+    const f2 e = fma2(a.hi, b.hi, neg2(p));
+    return fast2(p, fma2(a.hi, b.lo, fma2(a.lo, b.hi, e)));
+}
+// The energy sums of one element orbit from its six W and Y (slots abc, acb, bac, bca,
+// cab, cba): even slots 0, 3, 4, odd 1, 2, 5; Z_q = 6 w_q + 2E - 4O (even) or
+// 6 w_q + 2O - 4E (odd)
+template <typename T> __device__ __forceinline__ void orbit_sums(const T (&w)[6], const T (&y)[6], T &q4, T &q5) {
+    const T E = w[0] + w[3] + w[4], O = w[1] + w[2] + w[5];
+    const T ww = w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + w[3] * w[3] + w[4] * w[4] + w[5] * w[5];
+    const T wy = w[0] * y[0] + w[1] * y[1] + w[2] * y[2] + w[3] * y[3] + w[4] * y[4] + w[5] * y[5];
+    q4 = T(6) * ww + T(2) * (E * E + O * O) - T(8) * E * O;
+    q5 = T(6) * wy + (T(2) * E - T(4) * O) * (y[0] + y[3] + y[4]) + (T(2) * O - T(4) * E) * (y[1] + y[2] + y[5]);
+}
 // a U value of the FP64-emulation path: (hi, lo) floats in the 8 bytes of a double
 __device__ __forceinline__ dd dd_bits(double x) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
@@ -216,7 +256,7 @@ template <> __device__ __forceinline__ dd eps_vir<dd>(const InstDesc &p, int x) 
 // of one element at a time (o=4, v=20: 33 us, now 26; 52 tasks of o=40, v=300 in FP64
 // emulation 18.1 ms, then 16.8; with the sum of the occupied energies formed once, no
 // compensated sum of one term and the energies widened without conversion instructions,
-// 16.0).  CT = double (FP64 path: U, t1, ovov
+// 16.0; with the two orbits of a thread in packed FP32 operations, 15.6).  CT = double (FP64 path: U, t1, ovov
 // in FP64) or dd (FP64 emulation: all of them float-float pairs, so that no
 // operation per element runs on the FP64 pipe).
 template <typename CT, int TE>
@@ -226,6 +266,7 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
     constexpr int TP = TE + 1;               // padded innermost extent
     constexpr int CUBE = TE * TE * TP;       // smem elements per cube
     constexpr int NE = TE * TE * TE;         // elements per cube
+    constexpr bool PACKED = std::is_same<CT, dd>::value;
     __shared__ short trip[156];
     __shared__ double red[NT][2];
     __shared__ CT eijk_sh;
@@ -325,6 +366,66 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
         const CT ik_bc = ov_ik[b * ovs + c], ik_cb = ov_ik[c * ovs + b];
         const CT ij_bc = ov_ij[b * ovs + c], ij_cb = ov_ij[c * ovs + b];
         const CT ebc = eijk - eps_vir<CT>(p, b) - eps_vir<CT>(p, c);
+        if constexpr (PACKED) {
+            // both orbits of the thread in the halves of packed FP32 operations (block A,
+            // below B and C, is full); the issue slots bound this kernel
+            const int laA = la0, aA = A0 + laA, laB = la0 + TE / 2, aB = A0 + laB;
+#define W2(s, x, y, z) dd2(Ws[s * CUBE + ((x##A) * TE + (y##A)) * TP + (z##A)], Ws[s * CUBE + ((x##B) * TE + (y##B)) * TP + (z##B)])
+            const int lbA = lb, lbB = lb, lcA = lc, lcB = lc;
+            auto at = [&](const CT *q, int64_t sa) { return dd2(q[aA * sa], q[aB * sa]); };
+            dd2 y[6];
+            {
+                const dd2 ta = at(t1 + ti * v, 1);
+                y[0] = ta * dd2(jk_bc);
+                y[1] = ta * dd2(jk_cb);
+                const dd2 ac = at(ov_ik + c, ovs), ab = at(ov_ik + b, ovs);
+                y[0] = y[0] + dd2(tjb) * ac;
+                y[1] = y[1] + dd2(tjc) * ab;
+            }
+            {
+                const dd2 ac = at(ov_ij + c, ovs), ab = at(ov_ij + b, ovs);
+                y[0] = y[0] + dd2(tkc) * ab;
+                y[1] = y[1] + dd2(tkb) * ac;
+            }
+            {
+                const dd2 ta = at(t1 + tj * v, 1);
+                const dd2 ac = at(ov_jk + c, ovs), ab = at(ov_jk + b, ovs);
+                y[2] = dd2(tib) * ac + ta * dd2(ik_bc);
+                y[4] = dd2(tic) * ab + ta * dd2(ik_cb);
+            }
+            {
+                const dd2 ca = at(ov_jk + c * ovs, 1), ba = at(ov_jk + b * ovs, 1);
+                y[3] = dd2(tib) * ca;
+                y[5] = dd2(tic) * ba;
+            }
+            {
+                const dd2 ca = at(ov_ik + c * ovs, 1), ba = at(ov_ik + b * ovs, 1);
+                y[3] = y[3] + dd2(tjc) * ba;
+                y[5] = y[5] + dd2(tjb) * ca;
+            }
+            {
+                const dd2 ta = at(t1 + tkk * v, 1);
+                y[3] = y[3] + ta * dd2(ij_bc);
+                y[5] = y[5] + ta * dd2(ij_cb);
+                const dd2 ca = at(ov_ij + c * ovs, 1), ba = at(ov_ij + b * ovs, 1);
+                y[2] = y[2] + dd2(tkc) * ba;
+                y[4] = y[4] + dd2(tkb) * ca;
+            }
+            const dd2 w[6] = {W2(0, la, lb, lc), W2(1, la, lc, lb), W2(2, lb, la, lc),
+                              W2(3, lb, lc, la), W2(4, lc, la, lb), W2(5, lc, lb, la)};
+#undef W2
+            dd2 q4, q5;
+            orbit_sums(w, y, q4, q5);
+            dd q4A, q4B, q5A, q5B;
+            q4.unpack(q4A, q4B);
+            q5.unpack(q5A, q5B);
+            const CT rA = CT(1) / (ebc - eps_vir<CT>(p, aA));
+            a4 += q4A * rA;
+            a5 += q5A * rA;
+            const CT rB = CT(1) / (ebc - eps_vir<CT>(p, aB));
+            a4 += q4B * rB;
+            a5 += q5B * rB;
+        } else {
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int la = la0 + h * (TE / 2), a = A0 + la;
@@ -350,14 +451,13 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
             const CT y3 = tib * jk_ca + tjc * ik_ba + tka * ij_bc;
             const CT y4 = tic * jk_ab + tja * ik_cb + tkb * ij_ca;
             const CT y5 = tic * jk_ba + tjb * ik_ca + tka * ij_cb;
-            const CT E = w0 + w3 + w4, O = w1 + w2 + w5;
-            const CT ww = w0 * w0 + w1 * w1 + w2 * w2 + w3 * w3 + w4 * w4 + w5 * w5;
-            const CT wy = w0 * y0 + w1 * y1 + w2 * y2 + w3 * y3 + w4 * y4 + w5 * y5;
-            const CT q4 = CT(6) * ww + CT(2) * (E * E + O * O) - CT(8) * E * O;
-            const CT q5 = CT(6) * wy + (CT(2) * E - CT(4) * O) * (y0 + y3 + y4) + (CT(2) * O - CT(4) * E) * (y1 + y2 + y5);
+            const CT w[6] = {w0, w1, w2, w3, w4, w5}, y[6] = {y0, y1, y2, y3, y4, y5};
+            CT q4, q5;
+            orbit_sums(w, y, q4, q5);
             const CT r = CT(1) / (ebc - eps_vir<CT>(p, a));
             a4 += q4 * r;
             a5 += q5 * r;
+        }
         }
         }
     } else {
@@ -385,11 +485,9 @@ __global__ void __launch_bounds__(NT, 3) epilogue_kernel(const Wave wv) {
             const CT y3 = tib * ov_jk[c * ovs + a] + tjc * ov_ik[b * ovs + a] + tka * ov_ij[b * ovs + c];
             const CT y4 = tic * ov_jk[a * ovs + b] + tja * ov_ik[c * ovs + b] + tkb * ov_ij[c * ovs + a];
             const CT y5 = tic * ov_jk[b * ovs + a] + tjb * ov_ik[c * ovs + a] + tka * ov_ij[c * ovs + b];
-            const CT E = w0 + w3 + w4, O = w1 + w2 + w5;
-            const CT ww = w0 * w0 + w1 * w1 + w2 * w2 + w3 * w3 + w4 * w4 + w5 * w5;
-            const CT wy = w0 * y0 + w1 * y1 + w2 * y2 + w3 * y3 + w4 * y4 + w5 * y5;
-            const CT q4 = CT(6) * ww + CT(2) * (E * E + O * O) - CT(8) * E * O;
-            const CT q5 = CT(6) * wy + (CT(2) * E - CT(4) * O) * (y0 + y3 + y4) + (CT(2) * O - CT(4) * E) * (y1 + y2 + y5);
+            const CT w[6] = {w0, w1, w2, w3, w4, w5}, y[6] = {y0, y1, y2, y3, y4, y5};
+            CT q4, q5;
+            orbit_sums(w, y, q4, q5);
             const CT n = (a == b || b == c) ? CT(2) : CT(1);
             const CT r = CT(1) / (n * (eijk - eps_vir<CT>(p, a) - eps_vir<CT>(p, b) - eps_vir<CT>(p, c)));
             a4 += q4 * r;
