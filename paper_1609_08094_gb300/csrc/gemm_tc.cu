@@ -19,14 +19,17 @@
 // (H0 = TMEM columns [0,256), H1 = [256,512)), so the MMAs of block n+1 run
 // while block n is drained.
 //
-// Kernel structure (one persistent CTA per SM, 10 warps):
+// Kernel structure of the single-SM form (one persistent CTA per SM, 10 warps; the
+// form on SM pairs, the default, adds warp 10, which schedules the items, and is
+// described at its kernel below).  Each role is a whole warp, its copies and MMAs
+// issued by one elected lane:
 //   warp 0  : TMA producer.  Per K chunk it loads A_hi, A_lo (128 pair rows
 //             = 8 b x 16 c, one 4-D box of the K-major layout; the swapped
 //             pair order (c,b) of two segments is a tensor map with permuted
 //             strides, so the tile rows always come out in (b,c) order) and
-//             B_hi, B_lo (up to 256 rows of a) into a 4-stage ring, 64-byte
-//             swizzled rows.
-//   warp 1  : allocates 512 TMEM columns; one thread issues tcgen05.mma
+//             B_hi, B_lo (up to 256 rows of a) into a ring of 4 to 8 stages,
+//             64-byte swizzled rows.
+//   warp 1  : allocates 512 TMEM columns and issues tcgen05.mma
 //             (M = 128, N <= 256, 2 K-steps x 3 products per chunk) into the
 //             accumulator of the current K block of KB = 2 chunks.
 //   warps 2-9: two warps per TMEM lane quarter, 128 columns each: drain each

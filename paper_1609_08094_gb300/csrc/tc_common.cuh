@@ -136,27 +136,6 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
 }
-// K-major operand tile with 64-byte rows and 64-byte swizzle: 8-row groups
-// are 512 bytes apart (SBO); LBO is unused for swizzled K-major layouts.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
-}
-template <int KIND>
-__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                       uint32_t acc) {
-    if constexpr (KIND == 1) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc));
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc));
-    }
-}
 // 16 consecutive accumulator columns of this warp's 32 TMEM lanes (the
 // caller waits with tc_wait_ld before reading r)
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
@@ -238,18 +217,6 @@ __device__ __forceinline__ Item decode(const Wave &w, int64_t it, SegCache &c) {
     return r;
 }
 __device__ __forceinline__ int num_chunks(const InstDesc &d) { return 2 * d.kv + 2 * d.ko; }
-// K steps of chunk ch that carry data: the K extent of each segment is padded
-// only to 16, so the last BF16 chunk of a segment may hold a single K step
-// (the rest of its 64-byte rows is TMA zero fill); a TF32 chunk (16 elements)
-// is always all data.  kind: 1 = TF32, 2 = BF16; kv, ko: chunks of the d and l
-// segments; dp, lp: their padded extents.
-__device__ __forceinline__ int chunk_ksteps(int kind, int kv, int ko, int dp, int lp, int ch) {
-    if (kind == 1) return 2;
-    int kk, kext;
-    if (ch < 2 * kv) { kk = ch < kv ? ch : ch - kv; kext = dp; }
-    else { kk = ch - 2 * kv; kk = kk < ko ? kk : kk - ko; kext = lp; }
-    return kext - kk * 32 >= 32 ? 2 : 1;
-}
 
 // ---- SM pairs (thread-block clusters of 2 CTAs, tcgen05 cta_group::2) -----
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -321,23 +288,6 @@ __device__ __forceinline__ void tma_load_5d_pair(uint32_t dst, const CUtensorMap
         "l"(map), "r"(bar_cl), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
         : "memory");
 }
-// tcgen05.mma over the SM pair (M = 256: A rows 0-127 from this CTA's shared
-// memory, 128-255 from the peer's at the same offsets; B's N columns split in
-// halves the same way; each CTA's tensor memory receives its own 128 rows)
-template <int KIND>
-__device__ __forceinline__ void tc_mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    if constexpr (KIND == 1) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc));
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc));
-    }
-}
 // arrives once on the mbarrier at shared::cta offset bar in every CTA of
 // cta_mask when every pair MMA issued so far by this thread has completed
 __device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t cta_mask) {
@@ -349,19 +299,18 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t cta_mask) 
 }
 
 // ---- lean MMA issue ---------------------------------------------------------
-// One thread issues every MMA of a CTA (or of an SM pair), and between two
-// MMAs it runs a few dependent instructions of its own, each several clocks
+// One warp issues every MMA of a CTA (or of an SM pair, M = 256: A rows 0-127
+// from the leader's shared memory, 128-255 from the peer's at the same offsets,
+// B's N columns split in halves the same way, each CTA's tensor memory receiving
+// its own 128 rows), through one elected lane, and between two MMAs it runs a few dependent instructions of its own, each several clocks
 // long: at M = 128, N = 256, K = 16 an MMA is ~128 tensor clocks, so the
 // issue path has to stay near ten instructions per MMA.  Descriptors are
 // therefore kept as their low 32-bit word (start address >> 4 and the LBO
-// field; one K step of 32 bytes is +2), paired with a constant high word in
+// field, unused for swizzled K-major tiles; one K step of 32 bytes is +2), paired with a constant high word in
 // the asm, and the accumulate flag is a compile-time constant.
 constexpr uint32_t DESC_LO_FLAGS = 1u << 16;                 // LBO = 1 (unused for swizzled K-major tiles)
 constexpr uint32_t DESC_HI = 32u | (1u << 14) | (4u << 29);  // SBO = 512 bytes, bit 46, 64-byte swizzle
 constexpr uint32_t DESC_HI128 = 64u | (1u << 14) | (2u << 29);  // SBO = 1024 bytes, 128-byte swizzle
-static_assert(((uint64_t)DESC_HI << 32 | DESC_LO_FLAGS) == (((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
-                                                             ((uint64_t)1 << 46) | ((uint64_t)4 << 61)),
-              "same descriptor fields as sdesc");
 __device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | DESC_LO_FLAGS; }
 
 #define TCX_MMA_ASM(CGS, KINDS, PRED)                                                             \
@@ -514,14 +463,6 @@ __device__ __forceinline__ bool mma_item_wide(MmaRing &r, uint32_t tmem, uint32_
     return true;
 }
 
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, uint32_t bar,
-                                            int c0, int c1, int c2, int c3, int c4) {
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(dst),
-        "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
-        : "memory");
-}
 // 8 consecutive accumulator columns of this warp's 32 TMEM lanes
 __device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile(
