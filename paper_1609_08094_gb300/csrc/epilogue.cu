@@ -213,28 +213,20 @@ __device__ __forceinline__ dd dd_bits(double x) {
 }
 
 // Sum over the CTA of one (E4, E5) pair per thread, in a fixed order, into
-// out[0..1]: the NT pairs through shared memory, NT / 32 per lane of warp 0,
-// then a shuffle tree.  (A shuffle tree over all NT threads would put ten
-// FP64 adds per thread on the FP64 pipe, which bounds these kernels.)
+// out[0..1]: the NT values through shared memory, NT / 32 per lane of one warp
+// for each of the two, then a shuffle tree.  (A shuffle tree over all NT threads
+// would put ten FP64 adds per thread on the FP64 pipe, which bounds these kernels.)
 __device__ __forceinline__ void cta_sum2(double a4, double a5, double (*red)[2], double *out, int tid) {
     red[tid][0] = a4;
     red[tid][1] = a5;
     __syncthreads();
-    if (tid < 32) {
-        double b4 = red[tid][0], b5 = red[tid][1];
+    if (tid < 64) {
+        const int c = tid >> 5, l = tid & 31;
+        double b = red[l][c];
 #pragma unroll
-        for (int k = 1; k < NT / 32; k++) {
-            b4 += red[tid + 32 * k][0];
-            b5 += red[tid + 32 * k][1];
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            b4 += __shfl_xor_sync(0xffffffffu, b4, off);
-            b5 += __shfl_xor_sync(0xffffffffu, b5, off);
-        }
-        if (tid == 0) {
-            out[0] = b4;
-            out[1] = b5;
-        }
+        for (int k = 1; k < NT / 32; k++) b += red[l + 32 * k][c];
+        for (int off = 16; off > 0; off >>= 1) b += __shfl_xor_sync(0xffffffffu, b, off);
+        if (l == 0) out[c] = b;
     }
 }
 
@@ -256,7 +248,8 @@ template <> __device__ __forceinline__ dd eps_vir<dd>(const InstDesc &p, int x) 
 // of one element at a time (o=4, v=20: 33 us, now 26; 52 tasks of o=40, v=300 in FP64
 // emulation 18.1 ms, then 16.8; with the sum of the occupied energies formed once, no
 // compensated sum of one term and the energies widened without conversion instructions,
-// 16.0; with the two orbits of a thread in packed FP32 operations, 15.6).  CT = double (FP64 path: U, t1, ovov
+// 16.0; with the two orbits of a thread in packed FP32 operations, 15.2; with E4 and
+// E5 summed over the CTA by a warp each, 14.9).  CT = double (FP64 path: U, t1, ovov
 // in FP64) or dd (FP64 emulation: all of them float-float pairs, so that no
 // operation per element runs on the FP64 pipe).
 template <typename CT, int TE>
