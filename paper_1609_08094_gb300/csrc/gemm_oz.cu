@@ -18,10 +18,10 @@
 // weight t and block) is exact: no rounding happens anywhere in the products.
 // The epilogue warps convert each block's P_t to int32 (exact) and add it,
 // shifted by beta (S + 1 - t) bits, into int64 running totals, exact too;
-// the U element is total * 2^{E_A + E_B - beta (S + 1)} rounded once to FP64.
+// the U element is total * 2^{E_A + E_B - beta (S + 1)} as a float-float pair.
 // The error is that of representing each operand with beta S bits below its
 // side's largest magnitude.  U is stored in the FP64 path's layout and the
-// FP64 epilogue does the rest.
+// FP64 epilogue's float-float form does the rest.
 //
 // Kernel structure: SM pairs (tcgen05 cta_group::2, M = 256), the roles of the
 // split-precision pair kernel (gemm_tc.cu, tc_pair.cuh).  Warp 0 loads per chunk
