@@ -20,12 +20,56 @@ thread_local std::string g_create_error;
 // Handles that come and go (one per molecule) spent most of their time in
 // cudaMalloc, cudaFree and the pinned allocations: o=10, v=100 in BF16X3 took 0.83
 // ms to create and 2.65 ms to destroy around 2.1 ms of work.  Their device
-// allocations of up to POOL_KEEP bytes come from one stream-ordered pool per device
-// that keeps at most POOL_KEEP bytes when they are gone (and gives them back when
-// an allocation fails), larger ones from cudaMalloc; pinned blocks of up to 1 MiB
-// are kept for reuse, at most 32 of them.  Pool and list are safe with several
-// threads; a handle frees its memory after it has synchronised its stream.
-constexpr size_t POOL_KEEP = (size_t)4 << 30;
+// allocations of up to POOL_MAX bytes come from one stream-ordered pool per device
+// that keeps at most POOL_KEEP bytes when they are gone; of the larger ones, from
+// cudaMalloc, up to LIST_KEEP bytes per device are kept for a later handle that
+// asks for as much or up to a fifth less, the oldest given back first.  Both are
+// given back when an allocation fails.  (Growing the pool by the gigabytes of a U
+// scratch took 2 ms more than cudaMalloc: o=12, v=82 took 2.8 ms to create and 4.0
+// to destroy while earlier handles were alive, 0.8 and 2.4 with cudaMalloc alone.)
+// Pinned blocks of up to 1 MiB are kept for reuse, at most 32 of them.  Pool and
+// lists are safe with several threads; a block enters a list after its handle's
+// stream has been synchronised.
+constexpr size_t POOL_MAX = (size_t)16 << 20, POOL_KEEP = (size_t)512 << 20, LIST_KEEP = (size_t)3584 << 20;
+namespace {
+struct DevList {
+    std::mutex mu;
+    std::vector<Exec::DevPtr> blocks;  // oldest first
+    size_t kept = 0;
+};
+DevList &dev_list(int dev) {
+    static DevList *l = new DevList[64];  // outlives every handle
+    return l[dev];
+}
+// Gives back the oldest blocks until at most `keep` bytes are kept
+void trim_list(DevList &l, size_t keep) {
+    std::vector<Exec::DevPtr> out;
+    {
+        std::lock_guard<std::mutex> lk(l.mu);
+        size_t n = 0;
+        while (l.kept > keep) {
+            l.kept -= l.blocks[n].bytes;
+            out.push_back(l.blocks[n++]);
+        }
+        l.blocks.erase(l.blocks.begin(), l.blocks.begin() + n);
+    }
+    for (const Exec::DevPtr &d : out) cudaFree(d.p);
+}
+// The smallest kept block of at least `bytes` and at most a quarter more
+bool take_kept(DevList &l, size_t bytes, Exec::DevPtr &d) {
+    std::lock_guard<std::mutex> lk(l.mu);
+    size_t best = l.blocks.size();
+    for (size_t n = 0; n < l.blocks.size(); n++)
+        if (l.blocks[n].bytes >= bytes && l.blocks[n].bytes - bytes <= bytes / 4 &&
+            (best == l.blocks.size() || l.blocks[n].bytes < l.blocks[best].bytes))
+            best = n;
+    if (best == l.blocks.size()) return false;
+    d = l.blocks[best];
+    l.kept -= d.bytes;
+    l.blocks.erase(l.blocks.begin() + best);
+    return true;
+}
+}  // namespace
 static cudaMemPool_t handle_pool(int dev) {
     static std::mutex mu;
     static cudaMemPool_t pools[64] = {};
@@ -50,26 +94,38 @@ static cudaMemPool_t handle_pool(int dev) {
 
 void *dalloc_bytes(Exec &ex, size_t bytes) {
     if (bytes == 0) bytes = 16;
-    void *p = nullptr;
-    const bool pooled = ex.pool && bytes <= ex.pool_max;
+    const bool handle = ex.pool && ex.pool_max != SIZE_MAX;
+    Exec::DevPtr d{nullptr, bytes, ex.pool && bytes <= ex.pool_max, handle && bytes > ex.pool_max};
     cudaError_t e = cudaSuccess;
-    for (int rep = 0; rep < 2; rep++) {
-        e = pooled ? cudaMallocFromPoolAsync(&p, bytes, ex.pool, ex.stream) : cudaMalloc(&p, bytes);
-        if (e == cudaSuccess || ex.pool_max == SIZE_MAX || !ex.pool) break;
-        cudaGetLastError();
-        cudaMemPoolTrimTo(ex.pool, 0);  // what the pool keeps unused, then once more
-    }
+    if (!d.listed || !take_kept(dev_list(ex.device), bytes, d))
+        for (int rep = 0; rep < 2; rep++) {
+            e = d.pooled ? cudaMallocFromPoolAsync(&d.p, bytes, ex.pool, ex.stream) : cudaMalloc(&d.p, bytes);
+            if (e == cudaSuccess || !handle) break;
+            cudaGetLastError();
+            trim_list(dev_list(ex.device), 0);  // what is kept unused, then once more
+            cudaMemPoolTrimTo(ex.pool, 0);
+        }
     if (e != cudaSuccess) {
         cudaGetLastError();
         throw Fail{TCORR_ENOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed: " +
                                      cudaGetErrorString(e)};
     }
-    ex.dev.push_back({p, pooled});
+    ex.dev.push_back(d);
     ex.bytes += bytes;
-    return p;
+    return d.p;
 }
 
 static void dev_free(Exec &ex, const Exec::DevPtr &d) {
+    if (d.listed && d.bytes <= LIST_KEEP && cudaStreamSynchronize(ex.stream) == cudaSuccess) {
+        DevList &l = dev_list(ex.device);
+        trim_list(l, LIST_KEEP - d.bytes);
+        std::lock_guard<std::mutex> lk(l.mu);
+        if (l.kept + d.bytes <= LIST_KEEP) {  // another thread may have filled it
+            l.blocks.push_back(d);
+            l.kept += d.bytes;
+            return;
+        }
+    }
     if (!d.pooled || cudaFreeAsync(d.p, ex.stream) != cudaSuccess) cudaFree(d.p);
 }
 
@@ -92,6 +148,11 @@ size_t free_device_bytes(const Exec &ex) {
         if (cudaMemPoolGetAttribute(ex.pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
             cudaMemPoolGetAttribute(ex.pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
             free_b += reserved - used;
+        if (ex.pool_max != SIZE_MAX) {
+            DevList &l = dev_list(ex.device);
+            std::lock_guard<std::mutex> lk(l.mu);
+            free_b += l.kept;
+        }
     }
     return free_b;
 }
@@ -756,7 +817,8 @@ void init_exec(Exec &ex, const tcorr_opts &op, void *stream, bool pooled) {
     CK(cudaGetDevice(&dev));
     if (pooled) {
         ex.pool = handle_pool(dev);
-        ex.pool_max = POOL_KEEP;
+        ex.pool_max = POOL_MAX;
+        ex.device = dev;
     }
     CK(cudaDeviceGetAttribute(&ex.sm_count, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaDeviceGetAttribute(&ex.cc_major, cudaDevAttrComputeCapabilityMajor, dev));

@@ -60,12 +60,13 @@ struct Exec {
     int sm_count = 0, cc_major = 0, cc_minor = 0;
     cudaStream_t stream = nullptr;
     size_t bytes = 0;              // device bytes held
-    struct DevPtr { void *p; bool pooled; };
+    struct DevPtr { void *p; size_t bytes; bool pooled, listed; };  // from the pool; kept when freed
     std::vector<DevPtr> dev;       // every device allocation
     struct HostPtr { void *p; size_t bytes; };
     std::vector<HostPtr> host;     // every pinned host allocation
     cudaMemPool_t pool = nullptr;  // stream-ordered allocations from this pool (freed in stream order) ...
-    size_t pool_max = SIZE_MAX;    // ... up to this size, larger ones with cudaMalloc
+    size_t pool_max = SIZE_MAX;    // ... up to this size (handles), larger ones with cudaMalloc
+    int device = 0;
 
     void *U = nullptr;             // wave scratch
     int64_t u_cap = 0;             // elements
@@ -100,7 +101,7 @@ template <typename T>
 void halloc(Exec &ex, T *&ptr, size_t bytes) {
     ptr = static_cast<T *>(halloc_bytes(ex, bytes));
 }
-// Free device memory, what the handles' pool holds unused included
+// Free device memory, what the handles' pool and list hold unused included
 size_t free_device_bytes(const Exec &ex);
 
 struct Timer {
