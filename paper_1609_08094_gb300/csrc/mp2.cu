@@ -399,7 +399,7 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
             CK(cudaMemcpyAsync(ev.data(), h->eps_v, (size_t)v * sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
             CK(cudaStreamSynchronize(ex.stream));
             std::vector<float> evf(ev.begin(), ev.end());
-            CK(cudaMemcpy(h->eps_vf, evf.data(), (size_t)v * sizeof(float), cudaMemcpyHostToDevice));
+            copy_in(ex, h->eps_vf, evf.data(), (size_t)v * sizeof(float));
         }
         std::vector<int> pr, tl;
         for (int i = 0; i < o; i++)
@@ -415,8 +415,8 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
         }
         dalloc(ex, h->pairs, pr.size() * sizeof(int));
         dalloc(ex, h->tiles, tl.size() * sizeof(int));
-        CK(cudaMemcpy(h->pairs, pr.data(), pr.size() * sizeof(int), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(h->tiles, tl.data(), tl.size() * sizeof(int), cudaMemcpyHostToDevice));
+        copy_in(ex, h->pairs, pr.data(), pr.size() * sizeof(int));
+        copy_in(ex, h->tiles, tl.data(), tl.size() * sizeof(int));
         if (split) {
             Mp2TcArgs &a = h->tc;
             a.pairs = h->pairs;
@@ -441,7 +441,7 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
                 g.v = v;
                 int2 *tl2 = nullptr;
                 dalloc(ex, tl2, gram_tiles.size() * sizeof(int2));
-                CK(cudaMemcpy(tl2, gram_tiles.data(), gram_tiles.size() * sizeof(int2), cudaMemcpyHostToDevice));
+                copy_in(ex, tl2, gram_tiles.data(), gram_tiles.size() * sizeof(int2));
                 g.tiles = tl2;
                 dalloc(ex, g.g, (size_t)g_floats * sizeof(float));
                 if (mp2_gram_fill(g, op.prec, h->ct_hi, h->ct_lo, o, v, h->kp, err) != cudaSuccess)
@@ -451,6 +451,7 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
             }
         }
         CK(cudaStreamSynchronize(ex.stream));
+        copied_in(ex);
         resolve_timers(ex);
     } catch (const Fail &f) {
         g_create_error = f.msg;

@@ -115,6 +115,14 @@ void *dalloc_bytes(Exec &ex, size_t bytes) {
     return d.p;
 }
 
+void copy_in(Exec &ex, void *dst, const void *src, size_t bytes) {
+    if (bytes == 0) return;
+    const unsigned char *p = static_cast<const unsigned char *>(src);
+    ex.sources.emplace_back(p, p + bytes);
+    CK(cudaMemcpyAsync(dst, ex.sources.back().data(), bytes, cudaMemcpyHostToDevice, ex.stream));
+}
+void copied_in(Exec &ex) { ex.sources.clear(); }
+
 static void dev_free(Exec &ex, const Exec::DevPtr &d) {
     if (d.listed && d.bytes <= LIST_KEEP && cudaStreamSynchronize(ex.stream) == cudaSuccess) {
         DevList &l = dev_list(ex.device);
@@ -859,7 +867,7 @@ void upload_descs(Exec &ex, const std::vector<Problem *> &pbs) {
     std::vector<InstDesc> hd(pbs.size());
     for (size_t n = 0; n < pbs.size(); n++) hd[n] = pbs[n]->desc;
     dalloc(ex, ex.d_descs, hd.size() * sizeof(InstDesc));
-    CK(cudaMemcpy(ex.d_descs, hd.data(), hd.size() * sizeof(InstDesc), cudaMemcpyHostToDevice));
+    copy_in(ex, ex.d_descs, hd.data(), hd.size() * sizeof(InstDesc));
 }
 
 // Measured tile choice: times the W contraction of a few tasks of the problem
@@ -906,9 +914,9 @@ int tuned_pb(Exec &ex, Problem &pb) {
         const int64_t units = seg_units(cp, s, tabs);
         std::vector<unsigned char> ht(tabs.bytes() + 1);
         place_tabs(tabs, sv, ht.data(), d_tab);
-        CK(cudaMemcpy(d_tab, ht.data(), tabs.bytes(), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(d_one, &d, sizeof(InstDesc), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(d_seg, &s, sizeof(Seg), cudaMemcpyHostToDevice));
+        copy_in(ex, d_tab, ht.data(), tabs.bytes());
+        copy_in(ex, d_one, &d, sizeof(InstDesc));
+        copy_in(ex, d_seg, &s, sizeof(Seg));
         Wave w{};
         w.descs = d_one;
         w.segs = d_seg;

@@ -64,6 +64,7 @@ struct Exec {
     std::vector<DevPtr> dev;       // every device allocation
     struct HostPtr { void *p; size_t bytes; };
     std::vector<HostPtr> host;     // every pinned host allocation
+    std::vector<std::vector<unsigned char>> sources;  // host data of copies that may be in flight (copy_in)
     cudaMemPool_t pool = nullptr;  // stream-ordered allocations from this pool (freed in stream order) ...
     size_t pool_max = SIZE_MAX;    // ... up to this size (handles), larger ones with cudaMalloc
     int device = 0;
@@ -101,6 +102,11 @@ template <typename T>
 void halloc(Exec &ex, T *&ptr, size_t bytes) {
     ptr = static_cast<T *>(halloc_bytes(ex, bytes));
 }
+// Copies host data to the device in ex.stream's order, the order in which the
+// blocks of the pool are allocated and given back.  The data is kept until
+// copied_in, which the caller calls after it has synchronised ex.stream.
+void copy_in(Exec &ex, void *dst, const void *src, size_t bytes);
+void copied_in(Exec &ex);
 // Free device memory, what the handles' pool and list hold unused included
 size_t free_device_bytes(const Exec &ex);
 

@@ -167,6 +167,7 @@ tcorr_status tcorr_create(tcorr_t *out, int o, int v, const double *eps_occ,
         // the plan of the whole task list; its staging is the largest, so that calls do not allocate
         place_plan(*hs, 0, pb.ntask);
         CK(cudaStreamSynchronize(ex.stream));
+        copied_in(ex);
         CK(cudaGetLastError());
         resolve_timers(ex);
     } catch (const Fail &f) {
@@ -366,6 +367,7 @@ tcorr_status tcorr_batch_create(tcorr_batch_t *out, int n, const tcorr_problem *
         b->plan = make_plan(ex, pp, spans);
         upload_plan(ex, b->plan, b->d_segs, b->d_spans);
         CK(cudaStreamSynchronize(ex.stream));
+        copied_in(ex);
         CK(cudaGetLastError());
         resolve_timers(ex);
     } catch (const Fail &f) {
