@@ -674,7 +674,7 @@ cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int 
     const int wq = pair ? 32 : 16;
     d.brows = round_up((v + d.npass - 1) / d.npass, wq);
     // SM pairs, v <= PACK_MAX_V: the groups that share (p, q) side by side in passes of up to 256 columns
-    d.packw = pair && v <= PACK_MAX_V ? round_up(v, PACK_ROWS) : 0;
+    d.packw = tc_pack_width(v, pair);
     d.kv = (v + kch - 1) / kch;
     d.ko = (o + kch - 1) / kch;
     // bytes per stage: one CTA's (single SM), or both CTAs' (the pair's leader expects them all)
@@ -745,6 +745,7 @@ int64_t tc_units_per_task(const InstDesc &d) {
     return (int64_t)3 * (d.pair ? (tiles + 1) / 2 : tiles) * d.npass;
 }
 
+int tc_pack_width(int v, bool pair) { return pair && v <= PACK_MAX_V ? round_up(v, PACK_ROWS) : 0; }
 int tc_tile_pairs(const InstDesc &d) { return (d.nbt * d.nct + 1) / 2; }
 
 cudaError_t tc_prepare(int) {

@@ -705,6 +705,37 @@ Plan make_plan(const Exec &ex, const std::vector<Problem *> &pbs, const std::vec
     return pl;
 }
 
+size_t stage_bytes_max(const Exec &ex, const Problem &pb) {
+    const int64_t per_wave = std::max<int64_t>(
+        1, std::min({ex.u_cap / pb.u_task, ex.part_cap / ((int64_t)pb.norb * 2), ex.wave_tasks, (int64_t)0x7fffffff / pb.norb}));
+    const int64_t nseg = (pb.ntask + per_wave - 1) / per_wave + 1;
+    return ((size_t)nseg * sizeof(Seg) + 255) / 256 * 256 + 256 + table_bytes_max(pb.dm, ex.prec, ex.pair);
+}
+
+size_t table_bytes_max(const Dims &d, int prec, bool pair) {
+    // packing has to save a quarter of the passes (seg_units), so packed columns
+    // are at most three quarters of a pass wide; a segment has an entry for each of
+    // a task's three groups and at most a run per entry
+    const int w = is_split(prec) ? tc_pack_width(d.v, pair) : 0;
+    if (w == 0 || 4 * w > 3 * 256) return 0;
+    const size_t o = d.o;
+    return o * (o + 1) * (o + 2) / 6 * 3 * (sizeof(PackRun) + sizeof(PackEnt));
+}
+
+void reserve_stage(Exec &ex, size_t bytes) {
+    if (bytes <= ex.stage_cap) return;
+    CK(cudaStreamSynchronize(ex.stream));  // the old tables may still be in use
+    const size_t old = ex.stage_cap;
+    unsigned char *d = ex.d_stage, *h = ex.h_stage;
+    ex.d_stage = ex.h_stage = nullptr;  // nothing left to write to where an allocation fails
+    ex.stage_cap = 0;
+    dfree(ex, d, old);
+    hfree(ex, h);
+    dalloc(ex, ex.d_stage, bytes);
+    halloc(ex, ex.h_stage, bytes);
+    ex.stage_cap = bytes;
+}
+
 // Uploads the plan's tables (one copy from pinned staging); returns the
 // device segment and span arrays.
 void upload_plan(Exec &ex, Plan &pl, Seg *&d_segs, SumSpan *&d_spans) {
@@ -713,14 +744,7 @@ void upload_plan(Exec &ex, Plan &pl, Seg *&d_segs, SumSpan *&d_spans) {
     const size_t tab_off = (span_off + pl.sums.size() * sizeof(SumSpan) + 255) / 256 * 256;
     const size_t total = tab_off + pl.tabs.bytes();
     if ((int)pl.sums.size() > ex.sums_cap) throw Fail{TCORR_EINVAL, "more spans than the handle was made for"};
-    if (total > ex.stage_cap) {
-        CK(cudaStreamSynchronize(ex.stream));  // the old tables may still be in use
-        dfree(ex, ex.d_stage, ex.stage_cap);
-        dalloc(ex, ex.d_stage, total);
-        hfree(ex, ex.h_stage);
-        halloc(ex, ex.h_stage, total);
-        ex.stage_cap = total;
-    }
+    reserve_stage(ex, total);
     for (size_t n = 0; n < pl.sums.size(); n++) pl.sums[n].out = ex.d_sums + 3 * n;
     place_tabs(pl.tabs, pl.segs, ex.h_stage + tab_off, ex.d_stage + tab_off);
     memcpy(ex.h_stage, pl.segs.data(), seg_b);

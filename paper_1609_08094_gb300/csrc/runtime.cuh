@@ -200,6 +200,12 @@ Plan make_plan(const Exec &ex, const std::vector<Problem *> &pbs, const std::vec
 int64_t seg_units(const Problem &pb, Seg &sg, PackTabs &tabs);
 // Copies the tables to dst (host) and points the segments at their device copy
 void place_tabs(const PackTabs &tabs, std::vector<Seg> &segs, unsigned char *dst, const unsigned char *dev);
+// Room for the plan tables, on the device and pinned; and the most that a plan of
+// any range of pb's task list takes (which segments have tables, and how large,
+// depends on where the range is cut into waves), of it the tables of packed columns
+void reserve_stage(Exec &ex, size_t bytes);
+size_t stage_bytes_max(const Exec &ex, const Problem &pb);
+size_t table_bytes_max(const Dims &d, int prec, bool pair);
 void upload_plan(Exec &ex, Plan &pl, Seg *&d_segs, SumSpan *&d_spans);
 void launch_plan(Exec &ex, const Plan &pl, const Seg *d_segs, const SumSpan *d_spans, cudaStream_t st);
 void raise_err_flag(Exec &ex);   // throws if the flag was set in the last copy

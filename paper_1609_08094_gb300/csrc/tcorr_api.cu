@@ -164,7 +164,7 @@ tcorr_status tcorr_create(tcorr_t *out, int o, int v, const double *eps_occ,
         fill_desc(ex, pb, model_pb(v));
         if (is_split(ex.prec) && op.tune == 1) fill_desc(ex, pb, tuned_pb(ex, pb));
         upload_descs(ex, {&pb});
-        // the plan of the whole task list; its staging is the largest, so that calls do not allocate
+        reserve_stage(ex, stage_bytes_max(ex, pb));  // for the plan of any range: calls do not allocate
         place_plan(*hs, 0, pb.ntask);
         CK(cudaStreamSynchronize(ex.stream));
         copied_in(ex);

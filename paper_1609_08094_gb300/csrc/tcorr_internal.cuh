@@ -229,6 +229,8 @@ cudaError_t tc_fill_desc(InstDesc &d, int prec, const Operands &op, int pb, int 
 // per column pass of a packed one (tile pairs)
 int64_t tc_units_per_task(const InstDesc &d);
 int tc_tile_pairs(const InstDesc &d);
+// columns of an entry of packed columns (InstDesc::packw); 0: never packed
+int tc_pack_width(int v, bool pair);
 // sets the kernel attributes once per process (call before any stream capture)
 cudaError_t tc_prepare(int prec);
 
