@@ -149,7 +149,7 @@ tcorr_status tcorr_create(tcorr_t *out, int o, int v, const double *eps_occ,
         if (hs->batch > ntask) hs->batch = (int)ntask;
         const int norb = epilogue_orbits(v);
         const size_t need = problem_bytes(dm, ex.prec) + (size_t)hs->batch * u_task_bytes +
-                            (size_t)hs->batch * norb * 16 + (op.host_inputs ? host_staging_bytes(dm) : 0) +
+                            (size_t)hs->batch * norb * 16 + table_bytes_max(dm, ex.prec, ex.pair) + (op.host_inputs ? host_staging_bytes(dm) : 0) +
                             (64u << 20);
         if (need > free_b)
             throw Fail{TCORR_ENOMEM, "footprint " + std::to_string(need) + " bytes exceeds free device memory " +
@@ -313,7 +313,7 @@ tcorr_status tcorr_batch_create(tcorr_batch_t *out, int n, const tcorr_problem *
         int64_t u_task_max = 0, norb_max = 0;
         for (int m = 0; m < n; m++) {
             const Dims dm = make_dims(problems[m].o, problems[m].v);
-            need += problem_bytes(dm, ex.prec);
+            need += problem_bytes(dm, ex.prec) + table_bytes_max(dm, ex.prec, ex.pair);
             if (op.host_inputs) stage = std::max(stage, host_staging_bytes(dm));
             u_task_max = std::max<int64_t>(u_task_max, 3 * dm.ug);
             norb_max = std::max<int64_t>(norb_max, epilogue_orbits(dm.v));
