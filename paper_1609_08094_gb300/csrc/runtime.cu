@@ -306,6 +306,9 @@ struct CopyPipe {
     cudaStream_t cs = nullptr;
     cudaEvent_t ev[5] = {};  // start, copied[2], used[2]
     ~CopyPipe() {
+        // also where an error ends the streaming: the staging blocks may go to
+        // another handle, so no copy into them may be left
+        if (cs) cudaStreamSynchronize(cs);
         for (cudaEvent_t e : ev)
             if (e) cudaEventDestroy(e);
         if (cs) cudaStreamDestroy(cs);

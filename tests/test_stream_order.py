@@ -53,3 +53,17 @@ def test_batch(lib, prec):
     assert dev.lib.tcorr_batch_energy(h, (ctypes.c_double * 9)()) == fd.OK
     assert dev.lib.tcorr_batch_destroy(h) == fd.OK
     assert dev.bad() == ""
+
+
+@pytest.mark.parametrize("prec", [0, 2, 3])
+@pytest.mark.parametrize("fn", ["cudaStreamWaitEvent", "cudaEventRecord"])
+def test_no_copy_is_left_in_a_block_given_back(lib, prec, fn):
+    """An error between a chunk's copy and the stream's wait for it ends the
+    creation; the staging block (20 MB, kept for reuse) then goes to the next one."""
+    dev = fd.Device(lib)
+    o, v = 12, 60
+    dev.fail(fn, nth=2, code=fd.LAUNCH_FAILURE)
+    assert fd.Handle(dev, o, v, prec=prec).status == fd.ECUDA
+    h = fd.Handle(dev, o, v, prec=prec)
+    assert h.status == fd.OK and h.close() == fd.OK
+    assert dev.bad() == ""
