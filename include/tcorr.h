@@ -166,11 +166,22 @@ tcorr_status tcorr_energy_range(tcorr_t h, int64_t first, int64_t count,
  */
 tcorr_status tcorr_kernel_times(tcorr_t h, double *ms, int64_t *launches, int reset);
 
-/* Device bytes held by the handle. */
+/* Device bytes held by the handle: the sizes of its blocks, of which one that an
+ * earlier handle left may be up to a quarter larger than what it is used for. */
 int64_t tcorr_device_bytes(tcorr_t h);
 
-/* Release every resource of the handle.  NULL is accepted (no-op). */
+/* Release every resource of the handle.  NULL is accepted (no-op).
+ *
+ * Closed handles (of a problem, a batch or RI-MP2) leave memory for later ones:
+ * per device at most 512 MiB of small blocks and 3.5 GiB of larger ones, and 32
+ * pinned host blocks of at most 1 MiB.  It goes back to the device when an
+ * allocation of this library fails, when a server is created, and with
+ * tcorr_trim, for a program whose other parts need it. */
 tcorr_status tcorr_destroy(tcorr_t h);
+
+/* Gives back what closed handles left on the current device (see tcorr_destroy).
+ * Safe beside other calls; open handles keep their memory.  ECUDA without a device. */
+tcorr_status tcorr_trim(void);
 
 /* Text of the last failure on h (h = NULL: last failure of tcorr_create on
  * this thread).  Never NULL; owned by the library. */

@@ -393,7 +393,7 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
                                      ex.stream));
             tm.stop();
         }
-        free_tmp(ex, tmp, (size_t)o * v * naux);
+        free_tmp(ex, tmp);
         if (split) {  // FP32 copy of the virtual energies for the FP32 denominators
             std::vector<double> ev(v);
             CK(cudaMemcpyAsync(ev.data(), h->eps_v, (size_t)v * sizeof(double), cudaMemcpyDeviceToHost, ex.stream));

@@ -24,7 +24,8 @@ thread_local std::string g_create_error;
 // that keeps at most POOL_KEEP bytes when they are gone; of the larger ones, from
 // cudaMalloc, up to LIST_KEEP bytes per device are kept for a later handle that
 // asks for as much or up to a fifth less, the oldest given back first.  Both are
-// given back when an allocation fails.  (Growing the pool by the gigabytes of a U
+// given back when an allocation of a handle or a server fails, when a server is
+// created, and by tcorr_trim; another user of the device has the latter.  (Growing the pool by the gigabytes of a U
 // scratch took 2 ms more than cudaMalloc: o=12, v=82 took 2.8 ms to create and 4.0
 // to destroy while earlier handles were alive, 0.8 and 2.4 with cudaMalloc alone.)
 // Pinned blocks of up to 1 MiB are kept for reuse, at most 32 of them.  Pool and
@@ -70,12 +71,21 @@ bool take_kept(DevList &l, size_t bytes, Exec::DevPtr &d) {
     return true;
 }
 }  // namespace
+namespace {
+struct Pools {
+    std::mutex mu;
+    cudaMemPool_t p[64] = {};
+};
+Pools &pools() {
+    static Pools *l = new Pools();
+    return *l;
+}
+}  // namespace
 static cudaMemPool_t handle_pool(int dev) {
-    static std::mutex mu;
-    static cudaMemPool_t pools[64] = {};
     if (dev < 0 || dev >= 64) return nullptr;
-    std::lock_guard<std::mutex> lk(mu);
-    if (!pools[dev]) {
+    Pools &l = pools();
+    std::lock_guard<std::mutex> lk(l.mu);
+    if (!l.p[dev]) {
         cudaMemPoolProps pp{};
         pp.allocType = cudaMemAllocationTypePinned;
         pp.location.type = cudaMemLocationTypeDevice;
@@ -87,9 +97,17 @@ static cudaMemPool_t handle_pool(int dev) {
             cudaGetLastError();
             return nullptr;  // plain cudaMalloc instead
         }
-        pools[dev] = p;
+        l.p[dev] = p;
     }
-    return pools[dev];
+    return l.p[dev];
+}
+
+void give_back_kept(int dev) {
+    if (dev < 0 || dev >= 64) return;
+    trim_list(dev_list(dev), 0);
+    Pools &l = pools();
+    std::lock_guard<std::mutex> lk(l.mu);
+    if (l.p[dev]) cudaMemPoolTrimTo(l.p[dev], 0);
 }
 
 void *dalloc_bytes(Exec &ex, size_t bytes) {
@@ -100,10 +118,9 @@ void *dalloc_bytes(Exec &ex, size_t bytes) {
     if (!d.listed || !take_kept(dev_list(ex.device), bytes, d))
         for (int rep = 0; rep < 2; rep++) {
             e = d.pooled ? cudaMallocFromPoolAsync(&d.p, bytes, ex.pool, ex.stream) : cudaMalloc(&d.p, bytes);
-            if (e == cudaSuccess || !handle) break;
+            if (e == cudaSuccess) break;
             cudaGetLastError();
-            trim_list(dev_list(ex.device), 0);  // what is kept unused, then once more
-            cudaMemPoolTrimTo(ex.pool, 0);
+            give_back_kept(ex.device);  // then once more, the server's allocations too
         }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -111,7 +128,7 @@ void *dalloc_bytes(Exec &ex, size_t bytes) {
                                      cudaGetErrorString(e)};
     }
     ex.dev.push_back(d);
-    ex.bytes += bytes;
+    ex.bytes += d.bytes;  // of a kept block its size, up to a quarter more than asked for
     return d.p;
 }
 
@@ -137,13 +154,13 @@ static void dev_free(Exec &ex, const Exec::DevPtr &d) {
     if (!d.pooled || cudaFreeAsync(d.p, ex.stream) != cudaSuccess) cudaFree(d.p);
 }
 
-void dfree(Exec &ex, void *p, size_t bytes) {
+void dfree(Exec &ex, void *p) {
     if (!p) return;
     for (size_t n = 0; n < ex.dev.size(); n++)
         if (ex.dev[n].p == p) {
+            ex.bytes -= ex.dev[n].bytes;
             dev_free(ex, ex.dev[n]);
             ex.dev.erase(ex.dev.begin() + n);
-            ex.bytes -= (bytes ? bytes : 16);
             return;
         }
 }
@@ -194,6 +211,16 @@ void *halloc_bytes(Exec &ex, size_t bytes) {
     if (!h.p) CK(cudaHostAlloc(&h.p, bytes, cudaHostAllocPortable));
     ex.host.push_back(h);
     return h.p;
+}
+
+void give_back_pinned() {
+    PinList &l = pin_list();
+    std::vector<Exec::HostPtr> out;
+    {
+        std::lock_guard<std::mutex> lk(l.mu);
+        out.swap(l.blocks);
+    }
+    for (const Exec::HostPtr &h : out) cudaFreeHost(h.p);
 }
 
 static void host_free(const Exec::HostPtr &h) {
@@ -252,10 +279,10 @@ const double *device_view(Exec &ex, const double *src, size_t n, bool host, doub
     return tmp;
 }
 
-void free_tmp(Exec &ex, double *&tmp, size_t n) {
+void free_tmp(Exec &ex, double *&tmp) {
     if (!tmp) return;
     CK(cudaStreamSynchronize(ex.stream));
-    dfree(ex, tmp, n * sizeof(double));
+    dfree(ex, tmp);
     tmp = nullptr;
 }
 
@@ -339,7 +366,7 @@ static void stream_rows(Exec &ex, const double *host, size_t row, int v, F consu
         consume(stage[b], d0, nr);
         CK(cudaEventRecord(cp.ev[3 + b], ex.stream));
     }
-    for (int b = 0; b < nbuf; b++) free_tmp(ex, stage[b], rows_per * row);  // synchronises ex.stream
+    for (int b = 0; b < nbuf; b++) free_tmp(ex, stage[b]);  // synchronises ex.stream
     CK(cudaStreamSynchronize(cp.cs));
 }
 
@@ -414,8 +441,8 @@ static void build_operands_oz(Exec &ex, Problem &pb, const double *t2, const dou
     layout_g(ex, pb, 3, (int64_t)nG, eA, vvvo, host);
     layout_small(ex, pb, 3, (int64_t)nT2K, (int64_t)nT2R, (int64_t)nAoN, eA, eB, dt2, doo);
     tm.stop();
-    free_tmp(ex, tmp_t2, (size_t)o * o * v2);
-    free_tmp(ex, tmp_oo, (size_t)o * o * o * v);
+    free_tmp(ex, tmp_t2);
+    free_tmp(ex, tmp_oo);
 }
 
 void build_operands(Exec &ex, Problem &pb, const double *t2, const double *vvvo, const double *ooov,
@@ -450,8 +477,8 @@ void build_operands(Exec &ex, Problem &pb, const double *t2, const double *vvvo,
     const double *doo = device_view(ex, ooov, (size_t)o * o * o * v, host, tmp_oo);
     layout_small(ex, pb, kind, 0, 0, 0, nullptr, nullptr, dt2, doo);
     tm.stop();
-    free_tmp(ex, tmp_t2, (size_t)o * o * v2);
-    free_tmp(ex, tmp_oo, (size_t)o * o * o * v);
+    free_tmp(ex, tmp_t2);
+    free_tmp(ex, tmp_oo);
 }
 
 void build_epilogue_inputs(Exec &ex, Problem &pb, const double *eps_occ, const double *eps_vir,
@@ -483,8 +510,8 @@ void build_epilogue_inputs(Exec &ex, Problem &pb, const double *eps_occ, const d
         const double *d2 = device_view(ex, ovov, nov2, host, tmp2);
         CK(launch_epilogue_f32_inputs(d1, d2, pb.eps_v, static_cast<float *>(pb.t1), static_cast<float *>(pb.ovov),
                                       pb.evf, o, v, (int)vp, ex.stream));
-        free_tmp(ex, tmp1, (size_t)o * v);
-        free_tmp(ex, tmp2, nov2);
+        free_tmp(ex, tmp1);
+        free_tmp(ex, tmp2);
     }
 }
 
@@ -728,11 +755,10 @@ size_t table_bytes_max(const Dims &d, int prec, bool pair) {
 void reserve_stage(Exec &ex, size_t bytes) {
     if (bytes <= ex.stage_cap) return;
     CK(cudaStreamSynchronize(ex.stream));  // the old tables may still be in use
-    const size_t old = ex.stage_cap;
     unsigned char *d = ex.d_stage, *h = ex.h_stage;
     ex.d_stage = ex.h_stage = nullptr;  // nothing left to write to where an allocation fails
     ex.stage_cap = 0;
-    dfree(ex, d, old);
+    dfree(ex, d);
     hfree(ex, h);
     dalloc(ex, ex.d_stage, bytes);
     halloc(ex, ex.h_stage, bytes);
@@ -850,10 +876,10 @@ void init_exec(Exec &ex, const tcorr_opts &op, void *stream, bool pooled) {
     ex.pair = op.single_sm == 0;
     int dev = 0;
     CK(cudaGetDevice(&dev));
+    ex.device = dev;
     if (pooled) {
         ex.pool = handle_pool(dev);
         ex.pool_max = POOL_MAX;
-        ex.device = dev;
     }
     CK(cudaDeviceGetAttribute(&ex.sm_count, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaDeviceGetAttribute(&ex.cc_major, cudaDevAttrComputeCapabilityMajor, dev));
@@ -966,9 +992,9 @@ int tuned_pb(Exec &ex, Problem &pb) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    dfree(ex, d_one, sizeof(InstDesc));
-    dfree(ex, d_seg, sizeof(Seg));
-    dfree(ex, d_tab, tab_cap);
+    dfree(ex, d_one);
+    dfree(ex, d_seg);
+    dfree(ex, d_tab);
     check_err_flag(ex);
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune_cache[key] = best;

@@ -59,7 +59,7 @@ struct Exec {
     bool pair = true;              // split precisions: tensor-core tiles on SM pairs
     int sm_count = 0, cc_major = 0, cc_minor = 0;
     cudaStream_t stream = nullptr;
-    size_t bytes = 0;              // device bytes held
+    size_t bytes = 0;              // device bytes held (the sizes of its blocks)
     struct DevPtr { void *p; size_t bytes; bool pooled, listed; };  // from the pool; kept when freed
     std::vector<DevPtr> dev;       // every device allocation
     struct HostPtr { void *p; size_t bytes; };
@@ -107,6 +107,9 @@ void halloc(Exec &ex, T *&ptr, size_t bytes) {
 // copied_in, which the caller calls after it has synchronised ex.stream.
 void copy_in(Exec &ex, void *dst, const void *src, size_t bytes);
 void copied_in(Exec &ex);
+// Gives back to the device (and the host) what closed handles left for later ones
+void give_back_kept(int dev);
+void give_back_pinned();
 // Free device memory, what the handles' pool and list hold unused included
 size_t free_device_bytes(const Exec &ex);
 
@@ -159,11 +162,11 @@ struct Plan {
     std::vector<SumSpan> sums;  // span n sums into d_sums[3n .. 3n+2] (out set at upload)
 };
 
-void dfree(Exec &ex, void *p, size_t bytes);
+void dfree(Exec &ex, void *p);
 void hfree(Exec &ex, void *p);
 void release(Exec &ex);
 const double *device_view(Exec &ex, const double *src, size_t n, bool host, double *&tmp);
-void free_tmp(Exec &ex, double *&tmp, size_t n);
+void free_tmp(Exec &ex, double *&tmp);
 void resolve_timers(Exec &ex);
 // Algorithmic flops of a problem: 12 v^3 (v + o) per task, i = j = k excluded.
 double problem_flops(int o, int v);

@@ -154,6 +154,7 @@ void admit(tcorr_server_s &s) {
         j->ex.pair = s.ex.pair;
         j->ex.stream = s.ex.stream;
         j->ex.pool = s.pool;
+        j->ex.device = s.ex.device;
         j->ex.sm_count = s.ex.sm_count;
         const tcorr_problem &p = j->in;
         try {
@@ -252,7 +253,7 @@ void launch_wave(tcorr_server_s &s) {
     const size_t tab_off = (span_off + std::max<size_t>(1, sums.size()) * sizeof(SumSpan) + 255) / 256 * 256;
     const size_t total = tab_off + tabs.bytes();
     if (total > r.cap) {  // the slot's previous wave has retired (ring discipline)
-        dfree(ex, r.d_tab, r.cap);
+        dfree(ex, r.d_tab);
         hfree(ex, r.h_tab);
         r.cap = 0;
         const size_t cap = std::max<size_t>(total, (size_t)512 << 10);  // above a wave of 4096 tasks
@@ -331,8 +332,8 @@ tcorr_status tcorr_server_create(tcorr_server_t *out, const tcorr_opts *opts, in
     Exec &ex = s->ex;
     try {
         init_exec(ex, op, stream, false);
-        int dev = 0;
-        CK(cudaGetDevice(&dev));
+        const int dev = ex.device;
+        give_back_kept(dev);  // the budget below is of what is free then
         cudaMemPoolProps pp{};
         pp.allocType = cudaMemAllocationTypePinned;
         pp.location.type = cudaMemLocationTypeDevice;

@@ -88,6 +88,17 @@ extern "C" {
 
 int tcorr_version(void) { return 3; }
 
+tcorr_status tcorr_trim(void) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return TCORR_ECUDA;
+    }
+    give_back_kept(dev);
+    give_back_pinned();
+    return TCORR_OK;
+}
+
 const char *tcorr_status_string(tcorr_status s) {
     if ((int)s < 0 || (int)s > 5) return "TCORR_UNKNOWN";
     return kStatusNames[(int)s];

@@ -78,6 +78,8 @@ def load():
         lib.tcorr_device_bytes.argtypes = [vp]
         lib.tcorr_destroy.restype = ctypes.c_int
         lib.tcorr_destroy.argtypes = [vp]
+        lib.tcorr_trim.restype = ctypes.c_int
+        lib.tcorr_trim.argtypes = []
         lib.tcorr_last_error.restype = ctypes.c_char_p
         lib.tcorr_last_error.argtypes = [vp]
         lib.tcorr_status_string.restype = ctypes.c_char_p
@@ -154,7 +156,7 @@ EXPORTS = ("tcorr_create", "tcorr_energy", "tcorr_energy_range", "tcorr_num_task
            "tcorr_server_destroy",
            "tcorr_mp2_create", "tcorr_mp2_energy", "tcorr_mp2_kernel_times", "tcorr_mp2_device_bytes",
            "tcorr_mp2_last_error", "tcorr_mp2_destroy",
-           "tcorr_task_energy_noalloc")
+           "tcorr_task_energy_noalloc", "tcorr_trim")
 JOB_STATES = ("queued", "running", "done", "failed")
 SERVER_STATS = ("submitted", "done", "failed", "running", "queued", "bytes", "peak_bytes", "waves")
 NOALLOC_MAX_V = 64
@@ -192,6 +194,14 @@ def _pointer(name, a, on_device: bool):
     if a.dtype != np.float64 or not a.flags.c_contiguous:
         raise ValueError(f"{name}: needs a C-contiguous float64 array")
     return a.ctypes.data
+
+
+def trim():
+    """Give back the memory that closed handles left on the current device for
+    later ones (at most 4 GiB); open handles are not touched."""
+    st = load().tcorr_trim()
+    if st != 0:
+        raise TcorrError(st, "no device")
 
 
 class Tcorr:

@@ -101,3 +101,33 @@ class Mp2:
 
     def close(self):
         return self.dev.lib.tcorr_mp2_destroy(self.h)
+
+
+class Server:
+    def __init__(self, dev, prec=1, hbm=0, **opts):
+        self.dev, self.keep = dev, []
+        self.opts = tcorr.Opts(prec=prec, **opts)
+        self.h = ctypes.c_void_p()
+        self.status = dev.lib.tcorr_server_create(ctypes.byref(self.h), ctypes.byref(self.opts), ctypes.c_int64(hbm),
+                                                  dev.stream)
+
+    def submit(self, o, v):
+        a = [np.zeros(n) for n in (o, v, o * v, o * o * v * v, v ** 3 * o, o ** 3 * v, o * v * o * v)]
+        self.keep.append(a)
+        p, i = tcorr.Problem(o, v, *[x.ctypes.data for x in a]), ctypes.c_int64()
+        assert self.dev.lib.tcorr_server_submit(self.h, ctypes.byref(p), ctypes.byref(i)) == OK
+        return i.value
+
+    def step(self):
+        return self.dev.lib.tcorr_server_step(self.h, None)
+
+    def drain(self):
+        return self.dev.lib.tcorr_server_drain(self.h)
+
+    def state(self, i):
+        st, js = ctypes.c_int(), ctypes.c_int()
+        assert self.dev.lib.tcorr_server_poll(self.h, ctypes.c_int64(i), ctypes.byref(st), None, ctypes.byref(js)) == OK
+        return tcorr.JOB_STATES[st.value], js.value
+
+    def close(self):
+        return self.dev.lib.tcorr_server_destroy(self.h)
