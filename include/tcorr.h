@@ -338,8 +338,9 @@ tcorr_status tcorr_server_destroy(tcorr_server_t s);
  * precision (all four products: the lo*lo term is kept, as the same-index
  * elements of i = j pairs are sums of squares; FP32 accumulation, FP32 energy
  * terms, FP64 sums).  The split precisions form g in waves of at most 1 GiB of
- * the handle's scratch and sum the energy in a second kernel (up to v = 8192;
- * beyond that in one kernel, without storing g).  TCORR_BF16X3 problems with fewer than 2^24
+ * the handle's scratch (less where less memory is free, which changes the last
+ * bits of the FP64 sums) and sum the energy in a second kernel; beyond v = 8192,
+ * and where not even two pairs of it fit, in one kernel without storing g.  TCORR_BF16X3 problems with fewer than 2^24
  * (pair i <= j, a, b, gamma) terms run on TF32 hi + lo operands instead (the
  * BF16 split's residual averages below 1e-6 only over more terms); their
  * results are identical to TCORR_TF32X3's.

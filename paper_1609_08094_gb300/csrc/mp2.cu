@@ -250,16 +250,18 @@ struct tcorr_mp2_s {
 namespace {
 
 // The Gram form of the split precisions keeps g of a wave in scratch: at most
-// MP2_GRAM_BYTES, which holds at least one pair up to v = MP2_GRAM_MAX_V.
+// MP2_GRAM_BYTES, which holds at least one pair up to v = MP2_GRAM_MAX_V; less
+// where less memory is free (mp2_fit_waves).
 constexpr int64_t MP2_GRAM_BYTES = (int64_t)1 << 30;
 constexpr int MP2_GRAM_MAX_V = 8192;
 
 // Waves over the pairs i <= j (pair list lexicographic, so that each wave's
 // pairs are consecutive): ni values of i with every j >= the first of them, or
 // one i with some j; and their tiles, skipping those left of the pairs i <= j.
-void mp2_plan_waves(int o, int v, int sm_count, std::vector<Mp2Wave> &waves, std::vector<int2> &tiles, int64_t &g_floats,
-                    int64_t &nparts) {
-    const int64_t cap = MP2_GRAM_BYTES / 4;
+void mp2_plan_waves(int o, int v, int sm_count, int64_t cap, std::vector<Mp2Wave> &waves, std::vector<int2> &tiles,
+                    int64_t &g_floats, int64_t &nparts) {
+    waves.clear();
+    tiles.clear();
     g_floats = nparts = 0;
     auto pair_index = [&](int64_t i, int64_t j) { return i * o - i * (i - 1) / 2 + (j - i); };
     for (int i0 = 0; i0 < o;) {
@@ -294,6 +296,19 @@ void mp2_plan_waves(int o, int v, int sm_count, std::vector<Mp2Wave> &waves, std
         }
         i0 += ni;
     }
+}
+
+// The largest waves (of MP2_GRAM_BYTES, halved down to two pairs) that fit `avail`
+// device bytes with their tile list and partials; false where none do.
+bool mp2_fit_waves(int o, int v, int sm_count, size_t avail, std::vector<Mp2Wave> &waves, std::vector<int2> &tiles,
+                   int64_t &g_floats, int64_t &nparts) {
+    for (int64_t cap = MP2_GRAM_BYTES / 4; cap >= 2 * (int64_t)v * v; cap /= 2) {
+        mp2_plan_waves(o, v, sm_count, cap, waves, tiles, g_floats, nparts);
+        if ((size_t)g_floats * 4 + tiles.size() * sizeof(int2) + (size_t)nparts * 16 <= avail) return true;
+    }
+    waves.clear();
+    tiles.clear();
+    return false;
 }
 
 }  // namespace
@@ -358,12 +373,18 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
         h->nparts = split ? std::min<int64_t>(ex.sm_count, h->items) : h->items;
         std::vector<int2> gram_tiles;
         int64_t g_floats = 0;
-        h->gram = split && v <= MP2_GRAM_MAX_V;
-        if (h->gram) mp2_plan_waves(o, v, ex.sm_count, h->waves, gram_tiles, g_floats, h->nparts);
         const size_t ct_bytes = (size_t)o * v * h->kp * elem_bytes(op.prec) * (split ? 2 : 1);  // hi + lo
         const size_t free_b = free_device_bytes(ex);
-        const size_t need = ct_bytes + (size_t)h->nparts * 16 + (size_t)g_floats * 4 + (op.host_inputs ? (size_t)o * v * naux * 8 : 0) +
-                            ((size_t)64 << 20);
+        // 64 MiB for the small arrays, or what the pair and tile lists take where that is more
+        size_t need = ct_bytes + (op.host_inputs ? (size_t)o * v * naux * 8 : 0) +
+                      std::max<size_t>((size_t)64 << 20, ((size_t)16 << 20) + (size_t)(h->npair + h->ntp) * 8);
+        if (split && v <= MP2_GRAM_MAX_V && need < free_b) {
+            int64_t np = 0;
+            h->gram = mp2_fit_waves(o, v, ex.sm_count, free_b - need, h->waves, gram_tiles, g_floats, np);
+            if (h->gram) h->nparts = np;
+        }
+        need += (size_t)h->nparts * 16;
+        if (h->gram) need += (size_t)g_floats * 4 + gram_tiles.size() * sizeof(int2);
         if (need > free_b)
             throw Fail{TCORR_ENOMEM, "footprint " + std::to_string(need) + " bytes exceeds free device memory"};
         if (split) {
@@ -404,7 +425,7 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
         std::vector<int> pr, tl;
         for (int i = 0; i < o; i++)
             for (int j = i; j < o; j++) { pr.push_back(i); pr.push_back(j); }
-        for (int a = 0; a < h->nt; a++)
+        for (int a = 0; a < h->nt && !h->gram; a++)  // tile pairs: of the forms that keep no g
             for (int b = a; b < h->nt; b++) { tl.push_back(a); tl.push_back(b); }
         if (!split) {  // columns of the last tile that hold data, in units of a warp's 6; a diagonal pair forms G only
             auto work = [&](int a, int b) { return std::min(8, (std::min(MT, v - b * MT) + 5) / 6) * (a == b ? 1 : 2); };
@@ -414,8 +435,8 @@ tcorr_status tcorr_mp2_create(tcorr_mp2_t *out, int o, int v, int naux, const do
             for (size_t n = 0; n < t.size(); n++) { tl[2 * n] = t[n].first; tl[2 * n + 1] = t[n].second; }
         }
         dalloc(ex, h->pairs, pr.size() * sizeof(int));
-        dalloc(ex, h->tiles, tl.size() * sizeof(int));
         copy_in(ex, h->pairs, pr.data(), pr.size() * sizeof(int));
+        dalloc(ex, h->tiles, tl.size() * sizeof(int));
         copy_in(ex, h->tiles, tl.data(), tl.size() * sizeof(int));
         if (split) {
             Mp2TcArgs &a = h->tc;

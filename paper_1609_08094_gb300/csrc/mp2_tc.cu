@@ -1,8 +1,9 @@
 // RI-MP2 correlation energy in mixed precision on the tcgen05 tensor cores, in
 // two forms.  The first (up to v = MP2_GRAM_MAX_V, tcorr_mp2_create) forms g of
 // a block of the problem as one Gram matrix and sums the energy in a second
-// pass (mp2_gram_kernel, further down); the second, for larger v, whose blocks
-// would not fit its scratch, forms and sums g tile pair by tile pair:
+// pass (mp2_gram_kernel, further down); the second, where the blocks do not fit
+// its scratch (larger v, or little free memory), forms and sums g tile pair by
+// tile pair:
 // the paper's mixed-precision variant of the RI-MP2 kernel (Sec. 2.1, with
 // the dgemm of the integral assembly done in reduced precision, Sec. 3),
 // re-designed with the split-precision scheme of the (T) contractions.

@@ -160,8 +160,8 @@ tcorr_status tcorr_create(tcorr_t *out, int o, int v, const double *eps_occ,
         if (hs->batch > ntask) hs->batch = (int)ntask;
         const int norb = epilogue_orbits(v);
         const size_t need = problem_bytes(dm, ex.prec) + (size_t)hs->batch * u_task_bytes +
-                            (size_t)hs->batch * norb * 16 + table_bytes_max(dm, ex.prec, ex.pair) + (op.host_inputs ? host_staging_bytes(dm) : 0) +
-                            (64u << 20);
+                            (size_t)hs->batch * norb * 16 + (op.host_inputs ? host_staging_bytes(dm) : 0) +
+                            std::max<size_t>(64u << 20, (16u << 20) + table_bytes_max(dm, ex.prec, ex.pair));
         if (need > free_b)
             throw Fail{TCORR_ENOMEM, "footprint " + std::to_string(need) + " bytes exceeds free device memory " +
                                          std::to_string(free_b)};
@@ -320,11 +320,12 @@ tcorr_status tcorr_batch_create(tcorr_batch_t *out, int n, const tcorr_problem *
         init_exec(ex, op, stream, true);
         b->eager = op.eager == 1 || op.profile != 0 || op.test_stall != 0;
         const size_t ueb = u_elem_bytes(ex.prec);
-        size_t need = 64u << 20, stage = 0;
+        size_t need = 0, stage = 0, tables = 0;
         int64_t u_task_max = 0, norb_max = 0;
         for (int m = 0; m < n; m++) {
             const Dims dm = make_dims(problems[m].o, problems[m].v);
-            need += problem_bytes(dm, ex.prec) + table_bytes_max(dm, ex.prec, ex.pair);
+            need += problem_bytes(dm, ex.prec);
+            tables += table_bytes_max(dm, ex.prec, ex.pair);
             if (op.host_inputs) stage = std::max(stage, host_staging_bytes(dm));
             u_task_max = std::max<int64_t>(u_task_max, 3 * dm.ug);
             norb_max = std::max<int64_t>(norb_max, epilogue_orbits(dm.v));
@@ -343,7 +344,7 @@ tcorr_status tcorr_batch_create(tcorr_batch_t *out, int n, const tcorr_problem *
         }
         const int64_t max_wave_tasks = std::min<int64_t>(ex.wave_tasks, ex.u_cap / u_task_min + 1);
         ex.part_cap = std::max<int64_t>(norb_max * 2, max_wave_tasks * norb_max * 2);
-        need += (size_t)ex.u_cap * ueb + (size_t)ex.part_cap * 8 + stage;
+        need += (size_t)ex.u_cap * ueb + (size_t)ex.part_cap * 8 + stage + std::max<size_t>(64u << 20, (16u << 20) + tables);
         const size_t free_b = free_device_bytes(ex);
         if (need > free_b)
             throw Fail{TCORR_ENOMEM, "footprint " + std::to_string(need) + " bytes exceeds free device memory " +
