@@ -19,7 +19,7 @@ def test_tile_pair_form_matches_the_fp64_kernel(o, v, naux):
         ref = h.energy()
     for prec in ("tf32x3", "bf16x3"):
         with tcorr.Mp2(o, v, naux, eo, ev, C, prec=prec) as h:
-            assert h.device_bytes < 4 * v * v  # no room for g of a pair
+            assert tcorr.load().tcorr_mp2_device_bytes(h._h) < 4 * v * v  # no room for g of a pair
             e = h.energy()
             assert h.energy() == e
         for a, b in zip(e, ref):
