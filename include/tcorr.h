@@ -67,7 +67,8 @@ typedef enum {
                           chunk and in int64 across chunks, U rounded once to FP64 and stored as
                           a float-float (hi, lo) pair (~48 significant bits); the energy epilogue
                           in float-float arithmetic on the FP32 pipe (relative error ~2^-44 per
-                          operation) with FP64 sums from the orbit on.  sm_103 only; device or
+                          operation) with FP64 sums from the orbit on; an infinity or a NaN in vvvo,
+                          t2 or ooov makes the problem's energies NaN.  sm_103 only; device or
                           host inputs; batch and server too */
 } tcorr_precision;
 

@@ -430,8 +430,9 @@ __global__ void oz_exponents_kernel(const unsigned long long *m, int *e) {
     const double a = fmax(__longlong_as_double((long long)m[0]), __longlong_as_double((long long)m[1]));
     const double b = fmax(__longlong_as_double((long long)m[1]), __longlong_as_double((long long)m[2]));
     int ea = 0, eb = 0;
-    if (a > 0.0) frexp(a, &ea);  // a = f 2^ea, f in [0.5, 1): a < 2^ea
-    if (b > 0.0) frexp(b, &eb);
+    // infinite or NaN: any exponent, the energies are NaN (eps_ff_kernel)
+    if (a > 0.0 && isfinite(a)) frexp(a, &ea);  // a = f 2^ea, f in [0.5, 1): a < 2^ea
+    if (b > 0.0 && isfinite(b)) frexp(b, &eb);
     e[0] = ea;
     e[1] = eb;
 }

@@ -44,7 +44,7 @@ __device__ __forceinline__ int64_t oz_fixed(double x, int e) {
     const int64_t bits = __double_as_longlong(x);
     const int ex = (int)((bits >> 52) & 0x7ff);
     const int s = 1075 - 35 + e - ex;
-    // zero and values below any digit; s < 1 is no finite value of this side
+    // zero and values below any digit; s < 1: infinity or NaN (eps_ff_kernel answers)
     if (ex == 0 || s > 60 || s < 1) return 0;
     const int64_t m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
     // |x| = m 2^(ex - 1075) < 2^e: T = m 2^-s, s >= 18
@@ -231,10 +231,19 @@ __global__ void ovov_blocks_kernel(const double *__restrict__ in, float *__restr
 
 // eps_v as float-float pairs: hi = eps rounded to FP32, lo = the rest rounded
 // to FP32 (about 48 significant bits together); zero for x >= v
-__global__ void eps_ff_kernel(const double *__restrict__ e, float2 *__restrict__ out, int v, int vp) {
+// eps_v as float-float pairs.  m (FP64 emulation, else NULL): the bits of the largest
+// |vvvo|, |t2| and |ooov|.  A digit plane has no infinity or NaN, so such a value
+// would leave finite energies behind: eps_v[0], which every task's denominators
+// read, becomes NaN then, and with it every energy of the problem.
+__global__ void eps_ff_kernel(const double *__restrict__ e, const unsigned long long *__restrict__ m,
+                              float2 *__restrict__ out, int v, int vp) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= vp) return;
-    const double d = x < v ? e[x] : 0.0;
+    double d = x < v ? e[x] : 0.0;
+    if (m && x == 0) {
+        const unsigned long long inf = 0x7ff0000000000000ull;
+        if (m[0] >= inf || m[1] >= inf || m[2] >= inf) d = __longlong_as_double(0x7ff8000000000000ll);
+    }
     const float hi = static_cast<float>(d);
     out[x] = make_float2(hi, static_cast<float>(d - static_cast<double>(hi)));
 }
@@ -295,12 +304,12 @@ cudaError_t launch_pad_convert_rows(int kind, const double *in, void *out_hi, vo
     return cudaGetLastError();
 }
 
-cudaError_t launch_epilogue_ff_inputs(double *t1, double *ovov, const double *eps_v, float2 *evf, int o, int v,
-                                      cudaStream_t st) {
+cudaError_t launch_epilogue_ff_inputs(double *t1, double *ovov, const double *eps_v, const unsigned long long *m,
+                                      float2 *evf, int o, int v, cudaStream_t st) {
     const int64_t n = (int64_t)o * v * o * v, blocks = (n + 255) / 256;
     to_ff_kernel<<<(unsigned)(blocks < 65536 ? blocks : 65536), 256, 0, st>>>(ovov, n);
     to_ff_kernel<<<(unsigned)(((int64_t)o * v + 255) / 256), 256, 0, st>>>(t1, (int64_t)o * v);
-    eps_ff_kernel<<<(v + 255) / 256, 256, 0, st>>>(eps_v, evf, v, v);
+    eps_ff_kernel<<<(v + 255) / 256, 256, 0, st>>>(eps_v, m, evf, v, v);
     return cudaGetLastError();
 }
 
@@ -310,7 +319,7 @@ cudaError_t launch_epilogue_f32_inputs(const double *t1, const double *ovov, con
     const int64_t n = (int64_t)o * o * vp * vp, blocks = (n + 255) / 256;
     ovov_blocks_kernel<<<(unsigned)(blocks < 65536 ? blocks : 65536), 256, 0, st>>>(ovov, ovf, o, v, vp);
     pad_rows_kernel<<<(unsigned)((o * (int64_t)vp + 255) / 256), 256, 0, st>>>(t1, t1f, o, v, vp);
-    eps_ff_kernel<<<(vp + 255) / 256, 256, 0, st>>>(eps_v, evf, v, vp);
+    eps_ff_kernel<<<(vp + 255) / 256, 256, 0, st>>>(eps_v, nullptr, evf, v, vp);
     return cudaGetLastError();
 }
 

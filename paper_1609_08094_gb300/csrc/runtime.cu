@@ -3,6 +3,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <limits>
 #include <map>
 #include <mutex>
 #include <new>
@@ -431,8 +432,13 @@ static void build_operands_oz(Exec &ex, Problem &pb, const double *t2, const dou
         CK(launch_maxabs(vvvo, (int64_t)(row * v), pb.oz_max, ex.stream));
     } else {
         double m = 0.0;
-        for (size_t k = 0; k < row * v; k++) m = std::max(m, std::fabs(vvvo[k]));
-        CK(launch_seed_max(pb.oz_max, m, ex.stream));
+        bool finite = true;  // std::max passes a NaN over
+        for (size_t k = 0; k < row * v; k++) {
+            const double a = std::fabs(vvvo[k]);
+            m = std::max(m, a);
+            finite &= a <= std::numeric_limits<double>::max();
+        }
+        CK(launch_seed_max(pb.oz_max, finite ? m : std::numeric_limits<double>::infinity(), ex.stream));
     }
     CK(launch_maxabs(dt2, (int64_t)o * o * v2, pb.oz_max + 1, ex.stream));
     CK(launch_maxabs(doo, (int64_t)o * o * o * v, pb.oz_max + 2, ex.stream));
@@ -498,7 +504,7 @@ void build_epilogue_inputs(Exec &ex, Problem &pb, const double *eps_occ, const d
         if (ex.prec == TCORR_FP64_OZ) {  // the emulation's epilogue works in float-float
             dalloc(ex, pb.evf, (size_t)v * sizeof(float2));
             CK(launch_epilogue_ff_inputs(static_cast<double *>(pb.t1), static_cast<double *>(pb.ovov), pb.eps_v,
-                                         pb.evf, o, v, ex.stream));
+                                         pb.oz_max, pb.evf, o, v, ex.stream));
         }
     } else {
         const size_t vp = epi_vp(v);

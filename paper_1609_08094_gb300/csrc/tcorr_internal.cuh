@@ -186,9 +186,10 @@ cudaError_t launch_pad_convert_rows(int kind, const double *in, void *out_hi, vo
 cudaError_t launch_epilogue_f32_inputs(const double *t1, const double *ovov, const double *eps_v, float *t1f,
                                        float *ovf, float2 *evf, int o, int v, int vp, cudaStream_t st);
 // FP64-emulation epilogue inputs: t1 [o][v] and ovov [o][v][o][v] converted in
-// place to float-float (hi, lo) pairs; evf[x] = eps_v[x] as a pair, x < v
-cudaError_t launch_epilogue_ff_inputs(double *t1, double *ovov, const double *eps_v, float2 *evf, int o, int v,
-                                      cudaStream_t st);
+// place to float-float (hi, lo) pairs; evf[x] = eps_v[x] as a pair, x < v, with
+// evf[0] NaN where one of the maxima m[0..2] (bits) is infinite or NaN
+cudaError_t launch_epilogue_ff_inputs(double *t1, double *ovov, const double *eps_v, const unsigned long long *m,
+                                      float2 *evf, int o, int v, cudaStream_t st);
 // tasks[n] = (i, j, k): the sorted occupied triples i <= j <= k of o orbitals
 // in lexicographic order; orbits[n] = (A, B, C): the sorted block triples
 // A <= B <= C of nb virtual blocks, lexicographic
