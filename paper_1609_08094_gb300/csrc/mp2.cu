@@ -530,6 +530,10 @@ tcorr_status tcorr_mp2_energy(tcorr_mp2_t h, double *e_out) {
         cudaStreamSynchronize(ex.stream);
         cudaGetLastError();
         return f.st;
+    } catch (const std::bad_alloc &) {
+        ex.last_error = "host allocation failed";
+        cudaStreamSynchronize(ex.stream);
+        return TCORR_ENOMEM;
     }
     return TCORR_OK;
 }

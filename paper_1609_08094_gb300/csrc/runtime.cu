@@ -45,21 +45,22 @@ DevList &dev_list(int dev) {
 }
 // Gives back the oldest blocks until at most `keep` bytes are kept
 void trim_list(DevList &l, size_t keep) {
-    std::vector<Exec::DevPtr> out;
-    {
-        std::lock_guard<std::mutex> lk(l.mu);
-        size_t n = 0;
-        while (l.kept > keep) {
-            l.kept -= l.blocks[n].bytes;
-            out.push_back(l.blocks[n++]);
+    for (;;) {
+        Exec::DevPtr d;
+        {
+            std::lock_guard<std::mutex> lk(l.mu);
+            if (l.kept <= keep) return;
+            d = l.blocks.front();
+            l.kept -= d.bytes;
+            l.blocks.erase(l.blocks.begin());
         }
-        l.blocks.erase(l.blocks.begin(), l.blocks.begin() + n);
+        cudaFree(d.p);
     }
-    for (const Exec::DevPtr &d : out) cudaFree(d.p);
 }
 // The smallest kept block of at least `bytes` and at most a quarter more
 bool take_kept(DevList &l, size_t bytes, Exec::DevPtr &d) {
     std::lock_guard<std::mutex> lk(l.mu);
+    l.blocks.reserve(LIST_KEEP / POOL_MAX + 1);  // giving a block back must not allocate (dev_free)
     size_t best = l.blocks.size();
     for (size_t n = 0; n < l.blocks.size(); n++)
         if (l.blocks[n].bytes >= bytes && l.blocks[n].bytes - bytes <= bytes / 4 &&
@@ -111,9 +112,16 @@ void give_back_kept(int dev) {
     if (l.p[dev]) cudaMemPoolTrimTo(l.p[dev], 0);
 }
 
+// Room for one more element: what is noted after an allocation cannot fail then
+template <typename T>
+static void reserve_one(std::vector<T> &v) {
+    if (v.size() == v.capacity()) v.reserve(2 * v.size() + 16);
+}
+
 void *dalloc_bytes(Exec &ex, size_t bytes) {
     if (bytes == 0) bytes = 16;
     const bool handle = ex.pool && ex.pool_max != SIZE_MAX;
+    reserve_one(ex.dev);
     Exec::DevPtr d{nullptr, bytes, ex.pool && bytes <= ex.pool_max, handle && bytes > ex.pool_max};
     cudaError_t e = cudaSuccess;
     if (!d.listed || !take_kept(dev_list(ex.device), bytes, d))
@@ -199,9 +207,11 @@ constexpr size_t PIN_UNIT = (size_t)64 << 10, PIN_MAX = (size_t)1 << 20, PIN_BLO
 void *halloc_bytes(Exec &ex, size_t bytes) {
     bytes = std::max<size_t>(1, (bytes + PIN_UNIT - 1) / PIN_UNIT) * PIN_UNIT;
     Exec::HostPtr h{nullptr, bytes};
+    reserve_one(ex.host);
     if (bytes <= PIN_MAX) {
         PinList &l = pin_list();
         std::lock_guard<std::mutex> lk(l.mu);
+        l.blocks.reserve(PIN_BLOCKS);  // giving a block back must not allocate (host_free)
         for (size_t n = 0; n < l.blocks.size(); n++)
             if (l.blocks[n].bytes == bytes) {
                 h = l.blocks[n];
@@ -216,12 +226,16 @@ void *halloc_bytes(Exec &ex, size_t bytes) {
 
 void give_back_pinned() {
     PinList &l = pin_list();
-    std::vector<Exec::HostPtr> out;
-    {
-        std::lock_guard<std::mutex> lk(l.mu);
-        out.swap(l.blocks);
+    for (;;) {
+        Exec::HostPtr h;
+        {
+            std::lock_guard<std::mutex> lk(l.mu);
+            if (l.blocks.empty()) return;
+            h = l.blocks.back();
+            l.blocks.pop_back();
+        }
+        cudaFreeHost(h.p);
     }
-    for (const Exec::HostPtr &h : out) cudaFreeHost(h.p);
 }
 
 static void host_free(const Exec::HostPtr &h) {

@@ -157,6 +157,14 @@ void admit(tcorr_server_s &s) {
         j->ex.device = s.ex.device;
         j->ex.sm_count = s.ex.sm_count;
         const tcorr_problem &p = j->in;
+        auto fail_admission = [&](tcorr_status st) {
+            release(j->ex);
+            s.used -= j->bytes;
+            s.free_slots.push_back(j->slot);
+            j->state = TCORR_JOB_FAILED;
+            j->status = st;
+            s.n_failed++;
+        };
         try {
             build_problem(j->ex, j->pb, p.o, p.v, p.eps_occ, p.eps_vir, p.t1, p.t2, p.vvvo, p.ooov, p.ovov,
                           false);
@@ -164,13 +172,11 @@ void admit(tcorr_server_s &s) {
             store_desc_kernel<<<1, 128, 0, s.ex.stream>>>(j->pb.desc, s.ex.d_descs + j->slot);
             CK(cudaGetLastError());
         } catch (const Fail &f) {
-            release(j->ex);
-            s.used -= j->bytes;
-            s.free_slots.push_back(j->slot);
-            j->state = TCORR_JOB_FAILED;
-            j->status = f.st;
-            s.n_failed++;
+            fail_admission(f.st);
             if (f.st == TCORR_ECUDA) throw;
+            continue;
+        } catch (const std::bad_alloc &) {
+            fail_admission(TCORR_ENOMEM);
             continue;
         }
         j->state = TCORR_JOB_RUNNING;
@@ -444,6 +450,9 @@ tcorr_status tcorr_server_poll(tcorr_server_t s, int64_t id, int *state, double 
     } catch (const Fail &f) {
         s->ex.last_error = f.msg;
         return f.st;
+    } catch (const std::bad_alloc &) {
+        s->ex.last_error = "host allocation failed";
+        return TCORR_ENOMEM;
     }
     const Job &j = *it->second;
     *state = j.state;
@@ -469,6 +478,9 @@ tcorr_status tcorr_server_drain(tcorr_server_t s) {
         s->ex.last_error = f.msg;
         cudaGetLastError();
         return f.st;
+    } catch (const std::bad_alloc &) {
+        s->ex.last_error = "host allocation failed";
+        return TCORR_ENOMEM;
     }
     return TCORR_OK;
 }

@@ -245,6 +245,10 @@ tcorr_status tcorr_energy_range(tcorr_t hh, int64_t first, int64_t count, double
         cudaStreamSynchronize(ex.stream);
         cudaGetLastError();
         return f.st;
+    } catch (const std::bad_alloc &) {
+        ex.last_error = "host allocation failed";
+        cudaStreamSynchronize(ex.stream);
+        return TCORR_ENOMEM;
     }
     return TCORR_OK;
 }
@@ -439,6 +443,10 @@ tcorr_status tcorr_batch_energy(tcorr_batch_t b, double *e_out) {
         cudaStreamSynchronize(ex.stream);
         cudaGetLastError();
         return f.st;
+    } catch (const std::bad_alloc &) {
+        ex.last_error = "host allocation failed";
+        cudaStreamSynchronize(ex.stream);
+        return TCORR_ENOMEM;
     }
     return TCORR_OK;
 }
