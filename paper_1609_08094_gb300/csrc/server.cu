@@ -245,9 +245,8 @@ void launch_wave(tcorr_server_s &s) {
         wr.n_red += take[n];
         u_off += take[n] * j->pb.u_task;
         p_off += take[n] * (int64_t)j->pb.norb * 2;
-        j->next += take[n];
         members.push_back(j);
-        if (j->next == j->pb.ntask) {
+        if (j->next + take[n] == j->pb.ntask) {
             sums.push_back(SumSpan{j->pb.task_e, 0, j->pb.ntask, s.d_res + 3 * j->slot});
             finishing.push_back(j);
         }
@@ -261,27 +260,38 @@ void launch_wave(tcorr_server_s &s) {
     if (total > r.cap) {  // the slot's previous wave has retired (ring discipline)
         dfree(ex, r.d_tab);
         hfree(ex, r.h_tab);
+        r.d_tab = r.h_tab = nullptr;
         r.cap = 0;
         const size_t cap = std::max<size_t>(total, (size_t)512 << 10);  // above a wave of 4096 tasks
         dalloc(ex, r.d_tab, cap);
         halloc(ex, r.h_tab, cap);
         r.cap = cap;
     }
-    place_tabs(tabs, segs, r.h_tab + tab_off, r.d_tab + tab_off);
-    memcpy(r.h_tab, segs.data(), seg_b);
-    if (!sums.empty()) memcpy(r.h_tab + span_off, sums.data(), sums.size() * sizeof(SumSpan));
-    CK(cudaMemcpyAsync(r.d_tab, r.h_tab, total, cudaMemcpyHostToDevice, ex.stream));
     Plan pl;
     wr.seg0 = 0;
     pl.waves.push_back(wr);
     pl.sums = sums;
-    launch_plan(ex, pl, reinterpret_cast<Seg *>(r.d_tab), reinterpret_cast<SumSpan *>(r.d_tab + span_off),
-                ex.stream);
-    CK(cudaMemcpyAsync(r.h_err, ex.err, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
-    CK(cudaEventRecord(r.ev, ex.stream));
+    // From here on the stream may read the slot's tables, so where an error ends the
+    // wave's launch, what was launched has to be done before they are written again.
+    // The jobs' tasks count as scheduled only when the whole wave is (a repeated one
+    // gives the same energies); an error before leaves them to the next step.
+    try {
+        place_tabs(tabs, segs, r.h_tab + tab_off, r.d_tab + tab_off);
+        memcpy(r.h_tab, segs.data(), seg_b);
+        if (!sums.empty()) memcpy(r.h_tab + span_off, sums.data(), sums.size() * sizeof(SumSpan));
+        CK(cudaMemcpyAsync(r.d_tab, r.h_tab, total, cudaMemcpyHostToDevice, ex.stream));
+        launch_plan(ex, pl, reinterpret_cast<Seg *>(r.d_tab), reinterpret_cast<SumSpan *>(r.d_tab + span_off),
+                    ex.stream);
+        CK(cudaMemcpyAsync(r.h_err, ex.err, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
+        CK(cudaEventRecord(r.ev, ex.stream));
+    } catch (...) {
+        cudaStreamSynchronize(ex.stream);
+        throw;
+    }
+    for (size_t n = 0; n < act.size(); n++) act[n]->next += take[n];
     r.wave = s.waves_issued++;
-    r.finishing = finishing;
-    r.members = members;
+    r.finishing.swap(finishing);
+    r.members.swap(members);
 }
 
 void server_step(tcorr_server_s &s) {
@@ -365,6 +375,7 @@ tcorr_status tcorr_server_create(tcorr_server_t *out, const tcorr_opts *opts, in
             *r.h_err = 0;
         }
         for (int k = MAX_SLOTS - 1; k >= 0; k--) s->free_slots.push_back(k);
+        s->running.reserve(MAX_SLOTS);  // an admitted job is noted without an allocation
         CK(cudaStreamSynchronize(ex.stream));
         size_t free_b = 0, total_b = 0;
         CK(cudaMemGetInfo(&free_b, &total_b));

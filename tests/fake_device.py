@@ -131,3 +131,8 @@ class Server:
 
     def close(self):
         return self.dev.lib.tcorr_server_destroy(self.h)
+
+    def waves(self):
+        st = (ctypes.c_int64 * 8)()
+        assert self.dev.lib.tcorr_server_stats(self.h, st) == OK
+        return st[7]
