@@ -49,9 +49,8 @@ namespace {
 // relative, with integer and FP32 operations only: t = t2 2^48 + t1 2^24 + t0
 // with |t2| < 2^15 and 0 <= t1, t0 < 2^24, each part exact in FP32; Knuth's
 // TwoSum of the two largest, then the smallest added (one rounding, of the
-// small parts only); the power-of-two scale 2^k, as two factors (pow2_factors), is
-// exact in the normal range.
-__device__ __forceinline__ float2 int64_to_ff(long long t, float k1, float k2) {
+// small parts only); the power-of-two scale is exact in the normal range.
+__device__ __forceinline__ float2 int64_to_ff(long long t, int k) {
     const long long t2 = t >> 48;
     const long long rem = t - (t2 << 48);
     const float f2 = (float)(int)t2 * 0x1p48f, f1 = (float)(int)(rem >> 24) * 0x1p24f;
@@ -61,16 +60,7 @@ __device__ __forceinline__ float2 int64_to_ff(long long t, float k1, float k2) {
     const float s2 = s + f0, b2 = s2 - s;
     e += (s - (s2 - b2)) + (f0 - b2);       // s2 + e == t up to the rounding of e
     const float hi = s2 + e, lo = e - (hi - s2);
-    return make_float2(hi * k1 * k2, lo * k1 * k2);
-}
-// 2^k = k1 k2 for factors in FP32's normal range, beyond which any integer times 2^k
-// is 0 or infinite.  x k1 k2 with an integer |x| < 2^63 is rounded at most once, as
-// ldexpf(x, k) is: x k1 is exact, or as infinite as the result.
-__device__ __forceinline__ void pow2_factors(int k, float &k1, float &k2) {
-    k = min(254, max(-252, k));
-    const int h = k / 2;
-    k1 = __int_as_float((h + 127) << 23);
-    k2 = __int_as_float((k - h + 127) << 23);
+    return make_float2(ldexpf(hi, k), ldexpf(lo, k));
 }
 
 
@@ -397,16 +387,17 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_oz_kernel(const __grid_
             const int v = sl.v, pc = sl.pc, vc = round_up(v, UPAD);
             const int b = sl.cb + row / pc, c = sl.cc + row % pc;
             if (!sl.empty && b < v && c < v) {
-                float k1, k2;
-                pow2_factors(sl.scale - OZ_BETA * (OZ_S + 1), k1, k2);
+                const int scale_exp = sl.scale - OZ_BETA * (OZ_S + 1);
                 const int a0 = sl.pass0 + half * hw;
                 const int64_t stride = (int64_t)v * vc;
-                // Columns in eights and few instructions per value: at small v an item is
-                // so short that fetching the instructions of this part bounds it, and a
-                // branch past every column cost as much as the column (contraction of
-                // o=30: v=17 6.13 ms with ldexpf and a branch per column, 3.31 so; v=33
-                // 18.0 and 10.4; v=48 14.4 and 11.3; o=4, v=300 20.6 and 20.5.  A loop
-                // over the weights that is not unrolled is 5% slower from v=72 on).
+                // One branch past eight columns: at small v an item is so short that
+                // fetching the instructions of this part bounds it, and a branch past
+                // every column cost as much as the column (contraction of o=30: v=17
+                // 6.12 ms with those, 3.32 so; v=33 18.0 and 10.3; o=12: v=48 1.00 and
+                // 0.85, v=72 3.37 and 3.34; 52 tasks of o=40, v=300 70.66 both.  A
+                // multiplication by two powers of two in place of ldexpf gave no more
+                // and made the last 71.0; a loop over the weights that is not unrolled
+                // is 5% slower from v=72 on).
                 float2 *Ug = static_cast<float2 *>(wv.U) + sl.u_off + (int64_t)sl.g * (sl.ug3 / 3) + (int64_t)b * vc + c +
                              (int64_t)a0 * stride;
 #pragma unroll
@@ -414,7 +405,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) ugemm_oz_kernel(const __grid_
                     if (c8 * 8 < hw && a0 + c8 * 8 < v) {
 #pragma unroll
                         for (int j = 0; j < 8; j++) {
-                            if (a0 + c8 * 8 + j < v) *Ug = int64_to_ff(tot[c8 * 8 + j], k1, k2);
+                            if (a0 + c8 * 8 + j < v) *Ug = int64_to_ff(tot[c8 * 8 + j], scale_exp);
                             Ug += stride;
                         }
                     }

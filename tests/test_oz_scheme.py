@@ -66,20 +66,3 @@ def test_recombination_error_bound():
                  + 2.0 ** (ex + ey - BETA * (S + 2)) * S * S * 128 * 128)
     assert np.abs(u - ref).max() <= bound
     assert np.abs(u - ref).max() / np.abs(ref).max() < 1e-9
-
-
-def test_scale_of_two_factors_equals_ldexp():
-    """The drain scales the exact int64 totals' float parts by 2^k as x k1 k2 with two
-    powers of two in FP32's normal range: the same float as ldexp gives, for every
-    integer-valued float below 2^63 and every exponent, over- and underflow included."""
-    f = np.float32
-    g = np.random.default_rng(4)
-    x = np.concatenate([[0, 1, 3, 2 ** 24 - 1, 2 ** 47, 2 ** 62], g.integers(1, 2 ** 62, 200), g.integers(1, 2 ** 24, 200)])
-    x = np.concatenate([x, -x]).astype(f)
-    with np.errstate(over="ignore", under="ignore"):
-        for k in range(-700, 700):
-            c = min(254, max(-252, k))
-            h = int(c / 2)
-            k1, k2 = [np.array((e + 127) << 23, np.uint32).view(f) for e in (h, c - h)]
-            assert -126 <= h <= 127 and -126 <= c - h <= 127
-            assert np.array_equal(x * k1 * k2, np.ldexp(x, k)), k
