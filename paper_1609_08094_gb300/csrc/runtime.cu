@@ -26,7 +26,9 @@ thread_local std::string g_create_error;
 // cudaMalloc, up to LIST_KEEP bytes per device are kept for a later handle that
 // asks for as much or up to a fifth less, the oldest given back first.  Both are
 // given back when an allocation of a handle or a server fails, when a server is
-// created, and by tcorr_trim; another user of the device has the latter.  (Growing the pool by the gigabytes of a U
+// created, and by tcorr_trim; another user of the device has the latter.  The two
+// bounds are 4 GiB together, 1.5% of the device: a U scratch above 3.5 GiB (up to
+// 16 GiB) goes back when its handle is closed, as all did before.  (Growing the pool by the gigabytes of a U
 // scratch took 2 ms more than cudaMalloc: o=12, v=82 took 2.8 ms to create and 4.0
 // to destroy while earlier handles were alive, 0.8 and 2.4 with cudaMalloc alone.)
 // Pinned blocks of up to 1 MiB are kept for reuse, at most 32 of them.  Pool and
